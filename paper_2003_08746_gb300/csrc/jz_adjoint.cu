@@ -403,13 +403,13 @@ __global__ void k_adj_inout(Dims d, Consts c, Inflow in, State q, Adj64 a, doubl
       if (sup) {
         utb = lb[1] + lb[4] * ut;
       } else {
-        const double rho1 = Q1[0];
-        const double u1 = Q1[1] / rho1;
-        const double pr1 = c.gm1 * (Q1[4] - 0.5 * (Q1[1] * Q1[1] + Q1[2] * Q1[2] + Q1[3] * Q1[3]) / rho1);
-        const double a1 = sqrt(c.gamma * pr1 / rho1);
+        const double ir1 = rcp64(Q1[0]);
+        const double u1 = Q1[1] * ir1;
+        const double pr1 = c.gm1 * (Q1[4] - 0.5 * (Q1[1] * Q1[1] + Q1[2] * Q1[2] + Q1[3] * Q1[3]) * ir1);
+        const double a1 = sqrt64(c.gamma * pr1 * ir1);
         const double Rm = u1 - 2.0 * a1 / c.gm1, Rp = ut + 2.0 * 1.0 / c.gm1;
         const double ub = 0.5 * (Rp + Rm), ab = 0.25 * c.gm1 * (Rp - Rm);
-        const double rs = pow(ab * ab / (c.gamma * c.p_inf), 1.0 / c.gm1);
+        const double rs = isentrope(c, fabs(ab));
         const double rhob = lb[0] + lb[1] * ub + 0.5 * lb[4] * ub * ub;
         const double ubb = lb[1] * rs + lb[4] * rs * ub;
         const double pbb = lb[4] / c.gm1;
@@ -421,8 +421,8 @@ __global__ void k_adj_inout(Dims d, Consts c, Inflow in, State q, Adj64 a, doubl
         utb = Rpb;
         double u1b[3] = {Rmb, 0.0, 0.0};
         const double a1b = -2.0 * Rmb / c.gm1;
-        const double p1b = a1b * c.gamma / (2.0 * a1 * rho1);
-        double q1b[5] = {-a1b * c.gamma * pr1 / (2.0 * a1 * rho1 * rho1), 0, 0, 0, 0};
+        const double p1b = a1b * c.gamma * 0.5 * rcp64(a1) * ir1;
+        double q1b[5] = {-p1b * pr1 * ir1, 0, 0, 0, 0};
         prim_bar(c, Q1, u1b, p1b, q1b);
         for (int m = 0; m < 5; ++m) a.lam[m][p1] += q1b[m];
       }
@@ -476,22 +476,21 @@ __global__ void k_adj_farfield(Dims d, Consts c, GridDev g, State q, Adj64 a) {
   const long long pb = pidx(d, i, jb, k), pi = pidx(d, i, jb - 1, k);
   const long long nsurf = (long long)d.nk * d.ni, isurf = (long long)k * d.ni + i;
   const double sx = g.Sb[isurf], sy = g.Sb[nsurf + isurf], sz = g.Sb[2 * nsurf + isurf];
-  const double nm = sqrt(sx * sx + sy * sy + sz * sz);
-  const double n[3] = {sx / nm, sy / nm, sz / nm};
+  const double im = rcp64(sqrt64(sx * sx + sy * sy + sz * sz));
+  const double n[3] = {sx * im, sy * im, sz * im};
   double Qi[5];
   load5(q, pi, Qi);
-  const double rho_i = Qi[0];
-  const double ui[3] = {Qi[1] / rho_i, Qi[2] / rho_i, Qi[3] / rho_i};
+  const double rho_i = Qi[0], ir = rcp64(rho_i);
+  const double ui[3] = {Qi[1] * ir, Qi[2] * ir, Qi[3] * ir};
   const double p_i = c.gm1 * (Qi[4] - 0.5 * (Qi[1] * ui[0] + Qi[2] * ui[1] + Qi[3] * ui[2]));
-  const double a_i = sqrt(c.gamma * p_i / rho_i);
+  const double a_i = sqrt64(c.gamma * p_i * ir), ia = rcp64(a_i);
   const double un_i = ui[0] * n[0] + ui[1] * n[1] + ui[2] * n[2];
   const double Rp = un_i + 2.0 * a_i / c.gm1, Rm = -2.0 / c.gm1;
   const double un = 0.5 * (Rp + Rm), ab = 0.25 * c.gm1 * (Rp - Rm);
   const bool out = un > 0.0;
   double ut[3];
   for (int x = 0; x < 3; ++x) ut[x] = out ? ui[x] - un_i * n[x] : 0.0;
-  const double s = out ? p_i / pow(rho_i, c.gamma) : c.p_inf;
-  const double rho = pow(ab * ab / (c.gamma * s), 1.0 / c.gm1);
+  const double rho = out ? rho_i * isentrope(c, fabs(ab) * ia) : isentrope(c, fabs(ab));
   double ubv[3];
   for (int x = 0; x < 3; ++x) ubv[x] = ut[x] + un * n[x];
   double lb[5];
@@ -506,7 +505,6 @@ __global__ void k_adj_farfield(Dims d, Consts c, GridDev g, State q, Adj64 a) {
   rhob += pbb * ab * ab / c.gamma;
   double abb = pbb * 2.0 * rho * ab / c.gamma;
   abb += rhob * 2.0 * rho / (c.gm1 * ab);
-  const double sb = -rhob * rho / (c.gm1 * s);
   double unb = 0.0;
   for (int x = 0; x < 3; ++x) unb += ubb[x] * n[x];
   const double Rpb = 0.5 * unb + 0.25 * c.gm1 * abb;
@@ -522,13 +520,15 @@ __global__ void k_adj_farfield(Dims d, Consts c, GridDev g, State q, Adj64 a) {
       tn += ubb[x] * n[x];
     }
     un_ib += -tn;
-    const double rg = pow(rho_i, -c.gamma);
-    p_ib += sb * rg;
-    qb[0] += -c.gamma * sb * s / rho_i;
+    // through the entropy s = p_i / rho_i^gamma: s_bar = -rho_bar rho / ((gamma-1) s)
+    const double sb = -rhob * rho * c.Cp;
+    p_ib += sb * rcp64(p_i);
+    qb[0] += -c.gamma * sb * ir;
   }
   for (int x = 0; x < 3; ++x) uib[x] += un_ib * n[x];
-  p_ib += a_ib * c.gamma / (2.0 * a_i * rho_i);
-  qb[0] += -a_ib * c.gamma * p_i / (2.0 * a_i * rho_i * rho_i);
+  const double apb = a_ib * c.gamma * 0.5 * ia * ir;
+  p_ib += apb;
+  qb[0] += -apb * p_i * ir;
   prim_bar(c, Qi, uib, p_ib, qb);
   for (int m = 0; m < 5; ++m) {
     a.lam[m][pi] += qb[m];
@@ -576,13 +576,6 @@ __global__ void k_observer(Dims d, Consts c, State q, const double* w, int j0, d
     double x = 0.0;
     for (int w2 = 0; w2 < kTPB / 32; ++w2) x += red[w2];
     if (!want_grad) atomicAdd(a.J, x);
-  }
-}
-
-__global__ void k_set_time(Scalars* sc, double t, double dt) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    sc->t = t;
-    sc->dt = dt;
   }
 }
 
@@ -637,11 +630,6 @@ cudaError_t observer(const Dims& d, const Consts& c, const State& q, const doubl
                      double dt, const Adj64& a, int want_grad, cudaStream_t st) {
   const long long n = (long long)d.ni * d.nk;
   k_observer<<<blocks_for(n, kTPB), kTPB, 0, st>>>(d, c, q, w, j0, beta, dt, a, want_grad);
-  return cudaGetLastError();
-}
-
-cudaError_t set_time(Scalars* sc, double t, double dt, cudaStream_t st) {
-  k_set_time<<<1, 32, 0, st>>>(sc, t, dt);
   return cudaGetLastError();
 }
 

@@ -199,9 +199,8 @@ int load_state(jz_solver* s, const double* src, jz::State& q) {
       dev = s->staging;
     }
   }
-  JZ_CK(jz::pack_real(d, q.q, dev, 5, s->st));
-  JZ_CK(jz::ghost_fill(d, q.q, 5, s->st));
-  if (s->fp32) JZ_CK(jz::shadow_refresh(d, s->c, q, 1, s->st));
+  JZ_CK(jz::pack_state(d, s->c, q, dev, s->st));
+  JZ_CK(jz::ghost_fill_state(d, q, nullptr, s->st));
   if (host) JZ_CK(cudaStreamSynchronize(s->st));           // the caller may reuse its host buffer
   return JZ_OK;
 }
@@ -245,17 +244,27 @@ int run_stage64(jz_solver* s, const jz::State& in, const jz::State& out, double 
   if (s->pair) {
     JZ_RUN(JZ_PROF_NODAL, jz::nodal_df(d, s->c, s->mdf, s->w, s->qdf, in, s->st,
                                        cfl_first ? &s->sc->rate_max : nullptr));
-    if (cfl_first) JZ_RUN(JZ_PROF_REDUCE, jz::set_dt(s->c, s->sc, 0, s->st));
+    if (cfl_first) JZ_RUN(JZ_PROF_REDUCE, jz::set_dt(s->c, s->in, s->sc, s->st));
     JZ_RUN(JZ_PROF_VISCOUS, jz::viscous_df(d, s->c, s->mdf, s->w, s->qdf, s->st));
     JZ_RUN(JZ_PROF_FACES, jz::faces_update_df(d, s->c, g, s->w, s->qdf, in, s->qn, out, s->sc, alpha, want_res,
                                               rhs_flat, s->st));
     return JZ_OK;
   }
   JZ_RUN(JZ_PROF_NODAL, jz::nodal64(d, s->c, g, s->w, in, s->st, cfl_first ? &s->sc->rate_max : nullptr));
-  if (cfl_first) JZ_RUN(JZ_PROF_REDUCE, jz::set_dt(s->c, s->sc, 0, s->st));
+  if (cfl_first) JZ_RUN(JZ_PROF_REDUCE, jz::set_dt(s->c, s->in, s->sc, s->st));
   JZ_RUN(JZ_PROF_VISCOUS, jz::viscous64(d, s->c, g, s->w, in, s->st));
   JZ_RUN(JZ_PROF_FACES, jz::faces64(d, s->c, s->w, in, s->st));
   JZ_RUN(JZ_PROF_UPDATE, jz::update64(d, g, s->w, in, s->qn, out, s->sc, alpha, want_res, rhs_flat, s->st));
+  return JZ_OK;
+}
+
+// After stage l (0 .. 4): the boundary nodes and ghosts of its state; last: the step ends, t += dt.
+int run_shell(jz_solver* s, const jz::State& q, int l, int last) {
+  const jz::Dims& d = s->grid->d;
+  if (d.topo == JZ_TOPO_JET)
+    JZ_RUN(JZ_PROF_BC, jz::jet_shell(d, s->c, s->grid->g, s->in, q, s->sc, l, last, s->st));
+  else
+    JZ_RUN(JZ_PROF_GHOST, jz::ghost_fill_state(d, q, last ? s->sc : nullptr, s->st));
   return JZ_OK;
 }
 
@@ -268,7 +277,7 @@ int run_step(jz_solver* s) {
   // jz_set_state it is reduced here.
   if (s->fp32 || !cfl) {
     if (cfl && !s->rate_ready) JZ_RUN(JZ_PROF_REDUCE, jz::cfl_rate(d, s->c, g, s->qn, s->sc, s->st));
-    JZ_RUN(JZ_PROF_REDUCE, jz::set_dt(s->c, s->sc, 0, s->st));
+    JZ_RUN(JZ_PROF_REDUCE, jz::set_dt(s->c, s->in, s->sc, s->st));
   }
   jz::State in = s->qn;
   for (int l = 0; l < 5; ++l) {
@@ -280,26 +289,20 @@ int run_step(jz_solver* s) {
     else
       r = run_stage64(s, in, out, kAlpha[l], l == 0, nullptr, l == 0 && cfl);
     if (r) return r;
-    if (d.topo == JZ_TOPO_JET) {
-      JZ_RUN(JZ_PROF_BC, jz::bc_farfield(d, s->c, g, out, s->st));
-      JZ_RUN(JZ_PROF_BC, jz::bc_inout(d, s->c, s->in, out, s->sc, kAlpha[l], s->st));
-      JZ_RUN(JZ_PROF_BC, jz::bc_axis(d, out, s->st));
-    }
-    JZ_RUN(JZ_PROF_GHOST, jz::ghost_fill(d, out.q, 5, s->st));
-    if (s->fp32) JZ_RUN(JZ_PROF_GHOST, jz::shadow_refresh(d, s->c, out, 0, s->st));
+    r = run_shell(s, out, l, l == 4);
+    if (r) return r;
     in = out;
   }
   // Q^{n+1} is in qa (stage 5 wrote it); it becomes Q^n.
   jz::State t = s->qn;
   s->qn = s->qa;
   s->qa = t;
-  JZ_RUN(JZ_PROF_REDUCE, jz::set_dt(s->c, s->sc, 1, s->st));
   s->steps += 1;
   s->rate_ready = s->fp32 && cfl;
   return JZ_OK;
 }
 
-// Two time steps replayed as one CUDA graph.  A step launches 27 (FP32-flux form) or 43
+// Two time steps replayed as one CUDA graph.  A jet step launches 11 (FP32-flux form) or 26
 // (FP64 form) small kernels whose parameters never change between steps, except that the
 // roles of the Q^n and stage buffers swap every step and come back after two; so two steps
 // are captured once per starting buffer (on a private stream, nothing executes while
@@ -387,18 +390,12 @@ int fwd_stage(jz_solver* s, const jz::State& in, const jz::State& qn, const jz::
     JZ_RUN(JZ_PROF_FACES, jz::faces64(d, s->c, s->w, in, s->st));
     JZ_RUN(JZ_PROF_UPDATE, jz::update64(d, g, s->w, in, qn, out, s->sc, kAlpha[l], 0, nullptr, s->st));
   }
-  if (d.topo == JZ_TOPO_JET) {
-    JZ_RUN(JZ_PROF_BC, jz::bc_farfield(d, s->c, g, out, s->st));
-    JZ_RUN(JZ_PROF_BC, jz::bc_inout(d, s->c, s->in, out, s->sc, kAlpha[l], s->st));
-    JZ_RUN(JZ_PROF_BC, jz::bc_axis(d, out, s->st));
-  }
-  JZ_RUN(JZ_PROF_GHOST, jz::ghost_fill(d, out.q, 5, s->st));
-  return JZ_OK;
+  return run_shell(s, out, l, 0);
 }
 
 // One time step in -> out (in, out distinct from the solver's stage buffers).
 int fwd_step(jz_solver* s, const jz::State& in, const jz::State& out, double t, double dt) {
-  JZ_CK(jz::set_time(s->sc, t, dt, s->st));
+  JZ_CK(jz::set_time(s->in, s->sc, t, dt, s->st));
   const jz::State* src = &in;
   for (int l = 0; l < 5; ++l) {
     const jz::State& dst = l == 4 ? out : ((l % 2 == 0) ? s->qa : s->qb);
@@ -412,7 +409,7 @@ int fwd_step(jz_solver* s, const jz::State& in, const jz::State& out, double t, 
 // One time step in -> out that leaves the four intermediate stage states in keep[0..3].
 int fwd_step_keep(jz_solver* s, const jz::State& in, const jz::State& out, double t, double dt,
                   const jz::State keep[4]) {
-  JZ_CK(jz::set_time(s->sc, t, dt, s->st));
+  JZ_CK(jz::set_time(s->in, s->sc, t, dt, s->st));
   const jz::State* src = &in;
   for (int l = 0; l < 5; ++l) {
     const jz::State& dst = l == 4 ? out : keep[l];
@@ -683,6 +680,7 @@ int jz_create(jz_grid* g, const jz_params* p, void* stream, jz_solver** out) {
   if (d.topo == JZ_TOPO_JET) {
     A(s->in.u0, (size_t)d.nj * d.nk);
     A(s->in.Gf, (size_t)jz::kNF * d.nj * d.nk);
+    A(s->in.sn, 5 * (size_t)jz::kNF);
   }
   if (e != cudaSuccess) {
     delete s;
@@ -941,11 +939,11 @@ int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ck
   struct RestoreTime {
     jz_solver* s;
     double t, dt;
-    ~RestoreTime() { jz::set_time(s->sc, t, dt, s->st); }
+    ~RestoreTime() { jz::set_time(s->in, s->sc, t, dt, s->st); }
   } restore_time{s, h0.t, h0.dt};
   // frozen time step and start time
   if (s->c.dt_fixed <= 0.0) JZ_RUN(JZ_PROF_REDUCE, jz::cfl_rate(d, s->c, g, s->qn, s->sc, s->st));
-  JZ_RUN(JZ_PROF_REDUCE, jz::set_dt(s->c, s->sc, 0, s->st));
+  JZ_RUN(JZ_PROF_REDUCE, jz::set_dt(s->c, s->in, s->sc, s->st));
   jz::Scalars h;
   JZ_CK(cudaMemcpyAsync(&h, s->sc, sizeof h, cudaMemcpyDeviceToHost, s->st));
   JZ_CK(cudaStreamSynchronize(s->st));
@@ -995,7 +993,7 @@ int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ck
       const jz::State* sv = kept.empty() ? stg.data() : &kept[(size_t)(n - n0) * 4];
       const jz::State* st[6] = {&Qn, &sv[0], &sv[1], &sv[2], &sv[3], &Qn1};
       if (kept.empty()) {
-        JZ_CK(jz::set_time(s->sc, tn, dt, s->st));
+        JZ_CK(jz::set_time(s->in, s->sc, tn, dt, s->st));
         for (int l = 0; l < 4; ++l) {
           r = fwd_stage(s, *st[l], Qn, *st[l + 1], l);
           if (r) return r;

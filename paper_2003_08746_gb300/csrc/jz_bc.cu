@@ -1,127 +1,269 @@
 // Boundary conditions of the jet (paper Sec. "Large Eddy Simulation
-// Formulation": entrance, far field, exit, azimuthal periodicity, centerline),
-// applied after every Runge-Kutta stage (Algorithm 2: Update(B.C., Visc.)).
-// Order: far field (j = nj-1), then entrance (i = 0) and exit (i = ni-1),
-// then the axis average (j = 0).  The ghost points are filled afterwards by
-// the caller.
-#include "jz_internal.cuh"
+// Formulation": entrance, far field, exit, azimuthal periodicity, centerline)
+// and its ghost points, applied after every Runge-Kutta stage (Algorithm 2:
+// Update(B.C., Visc.), Create(Ghost)) by one kernel.
+//
+// In order the conditions are: far field (j = nj-1), entrance (i = 0) and exit
+// (i = ni-1), axis average (j = 0), then every ghost copies its source node.
+// Each reads only nodes the stage advanced or the condition before it, and the
+// values that are read across conditions are few (the far field at i = 1 and
+// i = ni-2 by the corners of the entrance and exit planes, the corners of the
+// ring j = 1 by the axis ends), so each thread forms those again and the whole
+// shell needs no order between blocks: a thread that owns a boundary node
+// computes it and writes it with all its ghost images, and the ghosts of
+// advanced nodes (across the axis, around the azimuth) are copied beside them.
+#include "jz_shadow.cuh"
 
 namespace jz {
 namespace {
 
 constexpr int kTPB = 128;
 
-__device__ __forceinline__ void store_cons(const State& q, long long p, double rho, double u, double v, double w,
-                                           double pr, double gm1) {
-  q.q[0][p] = rho;
-  q.q[1][p] = rho * u;
-  q.q[2][p] = rho * v;
-  q.q[3][p] = rho * w;
-  q.q[4][p] = pr / gm1 + 0.5 * rho * (u * u + v * v + w * w);
+// What the kernel needs of the state: the FP64 fields and, for the FP32-flux form, the shadow.
+struct ShellArgs {
+  Dims d;
+  Consts c;
+  ConstsF cf;
+  const double* Sb;      // far-field normals [3][nk][ni]
+  const double* u0;      // entrance profile [nk][nj]
+  const double* Gf;      // forcing shapes [32][nk][nj]
+  double amp[kNF];
+  State q;
+  const double* sn;      // temporal factors of the forcing at this stage's time
+  Scalars* sc;
+  int advance;           // last stage of a step: t += dt
+  unsigned bA, bE, bX, bF, bR;   // first block after the axis, entrance, exit, far-field and row roles
+};
+
+struct Prim {
+  double u[3], p, ir, rho;
+};
+__device__ __forceinline__ Prim prim_of(const Consts& c, const double q[5]) {
+  Prim r;
+  r.rho = q[0];
+  r.ir = rcp64(q[0]);
+  for (int a = 0; a < 3; ++a) r.u[a] = q[a + 1] * r.ir;
+  r.p = fma(-c.gm1_half, q[1] * r.u[0] + q[2] * r.u[1] + q[3] * r.u[2], c.gm1 * q[4]);
+  return r;
+}
+__device__ __forceinline__ void cons_of(const Consts& c, double rho, double u, double v, double w, double pr,
+                                        double out[5]) {
+  out[0] = rho;
+  out[1] = rho * u;
+  out[2] = rho * v;
+  out[3] = rho * w;
+  out[4] = fma(pr, c.Cp, 0.5 * (out[1] * u + out[2] * v + out[3] * w));   // p / (gamma-1) + rho |u|^2 / 2
+}
+__device__ __forceinline__ void load_q(const State& q, long long p, double v[5]) {
+#pragma unroll
+  for (int m = 0; m < 5; ++m) v[m] = q.q[m][p];
 }
 
-// Riemann-invariant far field on j = nj-1, 1 <= i <= ni-2.
-__global__ void k_farfield(Dims d, Consts c, GridDev g, State q) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const int ni2 = d.ni - 2;
-  if (t >= (long long)ni2 * d.nk) return;
-  const int i = 1 + (int)(t % ni2), k = (int)(t / ni2);
-  const int jb = d.nj - 1;
-  const long long pb = pidx(d, i, jb, k), pi = pidx(d, i, jb - 1, k);
-  const long long nb = (long long)d.nk * d.ni, sb = (long long)k * d.ni + i;
-  const double sx = g.Sb[sb], sy = g.Sb[nb + sb], sz = g.Sb[2 * nb + sb];
-  const double nm = sqrt(sx * sx + sy * sy + sz * sz);
-  const double n[3] = {sx / nm, sy / nm, sz / nm};
-  const double rho_i = q.q[0][pi];
-  const double ui[3] = {q.q[1][pi] / rho_i, q.q[2][pi] / rho_i, q.q[3][pi] / rho_i};
-  const double p_i = c.gm1 * (q.q[4][pi] - 0.5 * (q.q[1][pi] * ui[0] + q.q[2][pi] * ui[1] + q.q[3][pi] * ui[2]));
-  const double a_i = sqrt(c.gamma * p_i / rho_i);
-  const double un_i = ui[0] * n[0] + ui[1] * n[1] + ui[2] * n[2];
-  const double Rp = un_i + 2.0 * a_i / c.gm1;
-  const double Rm = -2.0 / c.gm1;
-  const double un = 0.5 * (Rp + Rm);
-  const double ab = 0.25 * c.gm1 * (Rp - Rm);
-  const bool out = un > 0.0;
-  double ut[3];
-  for (int a = 0; a < 3; ++a) ut[a] = out ? ui[a] - un_i * n[a] : 0.0;
-  const double s = out ? p_i / pow(rho_i, c.gamma) : c.p_inf;
-  const double rho = pow(ab * ab / (c.gamma * s), 1.0 / c.gm1);
-  const double pr = rho * ab * ab / c.gamma;
-  store_cons(q, pb, rho, ut[0] + un * n[0], ut[1] + un * n[1], ut[2] + un * n[2], pr, c.gm1);
+// Riemann-invariant far field of the node (i, nj-1, k) from its inner neighbour qi = Q(i, nj-2, k).
+__device__ void farfield_value(const ShellArgs& A, int i, int k, const double qi[5], double out[5]) {
+  const Consts& c = A.c;
+  const long long nb = (long long)A.d.nk * A.d.ni, sb = (long long)k * A.d.ni + i;
+  const double sx = A.Sb[sb], sy = A.Sb[nb + sb], sz = A.Sb[2 * nb + sb];
+  const double im = rcp64(sqrt64(sx * sx + sy * sy + sz * sz));
+  const double n[3] = {sx * im, sy * im, sz * im};
+  const Prim r = prim_of(c, qi);
+  const double a_i = sqrt64(c.gamma * r.p * r.ir);
+  const double un_i = r.u[0] * n[0] + r.u[1] * n[1] + r.u[2] * n[2];
+  const double two = 2.0 * c.Cp;                           // 2 / (gamma - 1)
+  const double Rp = fma(two, a_i, un_i), Rm = -two;
+  const double un = 0.5 * (Rp + Rm), ab = 0.25 * c.gm1 * (Rp - Rm);
+  const bool outflow = un > 0.0;
+  // density of the isentrope through (rho_s, a_s), interior or ambient, at sound speed ab:
+  // rho_s |ab / a_s|^(2 / (gamma-1))
+  const double rho = outflow ? r.rho * isentrope(c, fabs(ab) * rcp64(a_i)) : isentrope(c, fabs(ab));
+  const double pr = rho * ab * ab * c.p_inf;               // rho a^2 / gamma
+  double v[3];
+  for (int x = 0; x < 3; ++x) v[x] = outflow ? fma(un - un_i, n[x], r.u[x]) : un * n[x];
+  cons_of(c, rho, v[0], v[1], v[2], pr, out);
 }
 
-// Entrance (i = 0) and exit (i = ni-1) for 1 <= j <= nj-1, every k.
-__global__ void k_inout(Dims d, Consts c, Inflow in, State q, const Scalars* sc, double alpha) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const int nj1 = d.nj - 1;
-  const long long nface = (long long)nj1 * d.nk;
-  // the 32 temporal factors sin(omega_f t + psi_mf) at t_n + alpha dt are the same at every
-  // entrance node: one evaluation each per block
-  __shared__ double sn[kNF];
-  if (threadIdx.x < kNF) sn[threadIdx.x] = sin(in.omega[threadIdx.x % JZ_N_FREQ] * (sc->t + alpha * sc->dt) +
-                                               in.psi[threadIdx.x]);
-  __syncthreads();
-  if (t >= 2 * nface) return;
-  const bool exit_plane = t >= nface;
-  const long long tt = exit_plane ? t - nface : t;
-  const int j = 1 + (int)(tt % nj1), k = (int)(tt / nj1);
-  if (!exit_plane) {
-    // target: tanh profile + forcing at t_n + alpha dt
-    const long long tab = (long long)k * d.nj + j;
-    const long long plane = (long long)d.nk * d.nj;
-    double f = 0.0;
-    for (int mf = 0; mf < kNF; ++mf) f = f + in.amp[mf] * in.Gf[mf * plane + tab] * sn[mf];
-    const double ut = in.u0[tab] + c.jet_mach * f;
-    const long long p1 = pidx(d, 1, j, k), pb = pidx(d, 0, j, k);
-    const double rho1 = q.q[0][p1];
-    const double u1[3] = {q.q[1][p1] / rho1, q.q[2][p1] / rho1, q.q[3][p1] / rho1};
-    const double p1v = c.gm1 * (q.q[4][p1] - 0.5 * (q.q[1][p1] * u1[0] + q.q[2][p1] * u1[1] + q.q[3][p1] * u1[2]));
-    const double a1 = sqrt(c.gamma * p1v / rho1);
-    const double Rm = u1[0] - 2.0 * a1 / c.gm1;
-    const double Rp = ut + 2.0 * 1.0 / c.gm1;
-    const double ub = 0.5 * (Rp + Rm);
-    const double ab = 0.25 * c.gm1 * (Rp - Rm);
-    const double rho_sub = pow(ab * ab / (c.gamma * c.p_inf), 1.0 / c.gm1);
-    const double p_sub = rho_sub * ab * ab / c.gamma;
-    const bool sup = ut >= 1.0;
-    store_cons(q, pb, sup ? 1.0 : rho_sub, sup ? ut : ub, 0.0, 0.0, sup ? c.p_inf : p_sub, c.gm1);
+// Entrance node (0, j, k) by 1-D characteristics: tanh profile + forcing at the stage time; am the
+// amplitudes times their temporal factors, q1 = Q(1, j, k).
+__device__ void entrance_value(const ShellArgs& A, const double* am, int j, int k, const double q1[5], double out[5]) {
+  const Consts& c = A.c;
+  const long long tab = (long long)k * A.d.nj + j, plane = (long long)A.d.nk * A.d.nj;
+  double f = 0.0;
+#pragma unroll 8
+  for (int mf = 0; mf < kNF; ++mf) f = fma(am[mf], __ldg(A.Gf + mf * plane + tab), f);
+  const double ut = fma(c.jet_mach, f, A.u0[tab]);
+  if (ut >= 1.0) {                                          // supersonic: all imposed
+    cons_of(c, 1.0, ut, 0.0, 0.0, c.p_inf, out);
+    return;
+  }
+  const Prim r = prim_of(c, q1);
+  const double two = 2.0 * c.Cp;
+  const double Rm = fma(-two, sqrt64(c.gamma * r.p * r.ir), r.u[0]), Rp = ut + two;
+  const double ub = 0.5 * (Rp + Rm), ab = 0.25 * c.gm1 * (Rp - Rm);
+  const double rho = isentrope(c, fabs(ab));
+  cons_of(c, rho, ub, 0.0, 0.0, rho * ab * ab * c.p_inf, out);
+}
+
+// Exit node (ni-1, j, k): ambient pressure, velocity and internal energy of qi = Q(ni-2, j, k).
+__device__ void exit_value(const ShellArgs& A, const double qi[5], double out[5]) {
+  const Prim r = prim_of(A.c, qi);
+  cons_of(A.c, A.c.p_inf * r.rho * rcp64(r.p), r.u[0], r.u[1], r.u[2], A.c.p_inf, out);
+}
+
+// The inner neighbour of an entrance or exit node (i = 1 or ni-2): an advanced node, or for
+// j = nj-1 the far-field node formed from the one below it.
+__device__ __forceinline__ void inner_neighbour(const ShellArgs& A, int i, int j, int k, double q[5]) {
+  if (j < A.d.nj - 1) {
+    load_q(A.q, pidx(A.d, i, j, k), q);
   } else {
-    const long long pi = pidx(d, d.ni - 2, j, k), pb = pidx(d, d.ni - 1, j, k);
-    const double rho_i = q.q[0][pi];
-    const double ui[3] = {q.q[1][pi] / rho_i, q.q[2][pi] / rho_i, q.q[3][pi] / rho_i};
-    const double p_i = c.gm1 * (q.q[4][pi] - 0.5 * (q.q[1][pi] * ui[0] + q.q[2][pi] * ui[1] + q.q[3][pi] * ui[2]));
-    const double eint = p_i / (c.gm1 * rho_i);
-    const double pr = c.p_inf;
-    const double rho = pr / (c.gm1 * eint);
-    store_cons(q, pb, rho, ui[0], ui[1], ui[2], pr, c.gm1);
+    double t[5];
+    load_q(A.q, pidx(A.d, i, j - 1, k), t);
+    farfield_value(A, i, k, t, q);
   }
 }
 
-// Axis j = 0: the ring j = 1 averaged over the azimuth, one block per i.
-__global__ void k_axis(Dims d, State q) {
-  const int i = blockIdx.x;
-  double s[5] = {0, 0, 0, 0, 0};
-  for (int k = threadIdx.x; k < d.nk; k += blockDim.x) {
-    const long long p = pidx(d, i, 1, k);
-    for (int m = 0; m < 5; ++m) s[m] += q.q[m][p];
+// Write a value at (i, j, k) and at its azimuthal images.
+template <bool SH>
+__device__ __forceinline__ void put(const ShellArgs& A, const double v[5], const float2 s[NSH], int i, int j, int k) {
+  const Dims& d = A.d;
+  const long long turn = (long long)d.nk * d.sk;
+  long long p = pidx(d, i, j, k);
+  const int before = k >= d.nk - kG, after = k < kG;       // images at k - nk and k + nk
+  if (before) p -= turn;
+  for (int n = 0; n < 1 + before + after; ++n, p += turn) {
+#pragma unroll
+    for (int m = 0; m < 5; ++m) A.q.q[m][p] = v[m];
+    if (SH) {
+#pragma unroll
+      for (int m = 0; m < NSH; ++m) A.q.sh[m * d.Np + p] = s[m];
+    }
   }
-  __shared__ double red[5][kTPB / 32];
-  for (int m = 0; m < 5; ++m) {
-    double x = s[m];
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if ((threadIdx.x & 31) == 0) red[m][threadIdx.x >> 5] = x;
+}
+
+// Write the value of a boundary node (i, j, k), real, with every ghost that copies it: beyond the
+// entrance and exit (zero order in i), beyond the far field (zero order in j), across the axis
+// (rows -1 and -2 hold nodes (i, 1 | 2, k + nk/2)) and around the azimuth.
+template <bool SH>
+__device__ void put_node(const ShellArgs& A, const double v[5], int i, int j, int k) {
+  const Dims& d = A.d;
+  float2 s[NSH];
+  if (SH) shadow_of(A.cf, v, s);
+  const int i0 = i == 0 ? -kG : i, i1 = i == d.ni - 1 ? i + kG : i;
+  const int j1 = j == d.nj - 1 ? j + kG : j;
+  const bool mirror = j >= 1 && j <= kG;
+  const int half = d.nk / 2, km = k >= half ? k - half : k + half;
+  for (int ii = i0; ii <= i1; ++ii) {
+    for (int jj = j; jj <= j1; ++jj) put<SH>(A, v, s, ii, jj, k);
+    if (mirror) put<SH>(A, v, s, ii, -j, km);
   }
-  __syncthreads();
-  double mean[5];
-  for (int m = 0; m < 5; ++m) {
-    double x = 0.0;
-    for (int w = 0; w < kTPB / 32; ++w) x += red[m][w];
-    mean[m] = x / d.nk;
+}
+
+// Copy a source node to a ghost (state and shadow as they are).
+template <bool SH>
+__device__ __forceinline__ void copy_node(const ShellArgs& A, long long p, long long src) {
+#pragma unroll
+  for (int m = 0; m < 5; ++m) A.q.q[m][p] = A.q.q[m][src];
+  if (SH) {
+#pragma unroll
+    for (int m = 0; m < NSH; ++m) A.q.sh[m * A.d.Np + p] = A.q.sh[m * A.d.Np + src];
   }
-  for (int k = threadIdx.x; k < d.nk; k += blockDim.x) {
-    const long long p = pidx(d, i, 0, k);
-    for (int m = 0; m < 5; ++m) q.q[m][p] = mean[m];
+}
+
+// Boundary nodes and ghosts of the jet, by block roles: axis (one block per i), entrance, exit,
+// far field, ghost rows across the axis, ghost planes around the azimuth.  Latency bounds it (a
+// chain of dependent FP64 operations per node on a few thousand nodes).
+template <bool SH>
+__global__ void __launch_bounds__(kTPB) k_jet_shell(const __grid_constant__ ShellArgs A) {
+  const Dims& d = A.d;
+  const unsigned b = blockIdx.x, th = threadIdx.x;
+  __shared__ double am[kNF];
+  if (b < A.bE) {                                          // axis and entrance blocks
+    if (th < kNF) am[th] = A.amp[th] * A.sn[th];
+    __syncthreads();
   }
+  if (b < A.bA) {
+    // axis: the ring j = 1 averaged over the azimuth
+    const int i = (int)b;
+    double s[5] = {0, 0, 0, 0, 0};
+    for (int k = th; k < d.nk; k += kTPB) {
+      double v[5], t[5];
+      if (i == 0) {
+        inner_neighbour(A, 1, 1, k, t);
+        entrance_value(A, am, 1, k, t, v);
+      } else if (i == d.ni - 1) {
+        inner_neighbour(A, i - 1, 1, k, t);
+        exit_value(A, t, v);
+      } else {
+        load_q(A.q, pidx(d, i, 1, k), v);
+      }
+#pragma unroll
+      for (int m = 0; m < 5; ++m) s[m] += v[m];
+    }
+    __shared__ double red[5][kTPB / 32];
+#pragma unroll
+    for (int m = 0; m < 5; ++m) {
+      double x = s[m];
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      if ((th & 31) == 0) red[m][th >> 5] = x;
+    }
+    __syncthreads();
+    double mean[5];
+#pragma unroll
+    for (int m = 0; m < 5; ++m) {
+      double x = 0.0;
+      for (int w = 0; w < kTPB / 32; ++w) x += red[m][w];
+      mean[m] = x / d.nk;
+    }
+    for (int k = th; k < d.nk; k += kTPB) put_node<SH>(A, mean, i, 0, k);
+    if (b == 0 && th == 0 && A.advance) A.sc->t = A.sc->t + A.sc->dt;
+    return;
+  }
+  if (b < A.bX) {
+    // entrance (i = 0) and exit (i = ni-1), 1 <= j <= nj-1
+    const bool ent = b < A.bE;
+    const unsigned t = (b - (ent ? A.bA : A.bE)) * kTPB + th, nj1 = d.nj - 1;
+    if (t >= nj1 * (unsigned)d.nk) return;
+    const int j = 1 + (int)(t % nj1), k = (int)(t / nj1);
+    double qi[5], v[5];
+    inner_neighbour(A, ent ? 1 : d.ni - 2, j, k, qi);
+    if (ent)
+      entrance_value(A, am, j, k, qi, v);
+    else
+      exit_value(A, qi, v);
+    put_node<SH>(A, v, ent ? 0 : d.ni - 1, j, k);
+    return;
+  }
+  const unsigned ni2 = d.ni - 2;
+  if (b < A.bF) {
+    // far field j = nj-1, 1 <= i <= ni-2
+    const unsigned t = (b - A.bX) * kTPB + th;
+    if (t >= ni2 * (unsigned)d.nk) return;
+    const int i = 1 + (int)(t % ni2), k = (int)(t / ni2);
+    double qi[5], v[5];
+    load_q(A.q, pidx(d, i, d.nj - 2, k), qi);
+    farfield_value(A, i, k, qi, v);
+    put_node<SH>(A, v, i, d.nj - 1, k);
+    return;
+  }
+  if (b < A.bR) {
+    // ghost rows across the axis, 1 <= i <= ni-2, every padded k
+    const unsigned t = (b - A.bF) * kTPB + th, ek = d.nk + 2 * kG;
+    if (t >= 2 * ni2 * ek) return;
+    const int i = 1 + (int)(t % ni2);
+    const unsigned r = t / ni2;
+    const int m = 1 + (int)(r & 1), k = (int)(r >> 1) - kG;
+    int ks = k + d.nk / 2;
+    ks = ks < 0 ? ks + d.nk : (ks >= d.nk ? ks - d.nk : ks);
+    copy_node<SH>(A, pidx(d, i, -m, k), pidx(d, i, m, ks));
+    return;
+  }
+  // ghost planes around the azimuth, 1 <= i <= ni-2, 1 <= j <= nj-2
+  const unsigned t = (b - A.bR) * kTPB + th, nj2 = d.nj - 2;
+  if (t >= 4 * ni2 * nj2) return;
+  const int i = 1 + (int)(t % ni2);
+  const unsigned r = t / ni2;
+  const int j = 1 + (int)(r % nj2), s = (int)(r / nj2);    // k = -2, -1, nk, nk+1
+  const int k = s < 2 ? s - kG : d.nk + s - kG;
+  copy_node<SH>(A, pidx(d, i, j, k), pidx(d, i, j, s < 2 ? k + d.nk : k - d.nk));
 }
 
 struct Phases {
@@ -150,21 +292,32 @@ __global__ void k_build_inflow(Dims d, Consts c, GridDev g, double* u0, double* 
 
 }  // namespace
 
-cudaError_t bc_farfield(const Dims& d, const Consts& c, const GridDev& g, const State& q, cudaStream_t st) {
-  const long long nf = (long long)(d.ni - 2) * d.nk;
-  k_farfield<<<blocks_for(nf, kTPB), kTPB, 0, st>>>(d, c, g, q);
-  return cudaGetLastError();
-}
-
-cudaError_t bc_inout(const Dims& d, const Consts& c, const Inflow& in, const State& q, const Scalars* sc,
-                     double alpha, cudaStream_t st) {
-  const long long nio = 2LL * (d.nj - 1) * d.nk;
-  k_inout<<<blocks_for(nio, kTPB), kTPB, 0, st>>>(d, c, in, q, sc, alpha);
-  return cudaGetLastError();
-}
-
-cudaError_t bc_axis(const Dims& d, const State& q, cudaStream_t st) {
-  k_axis<<<d.ni, kTPB, 0, st>>>(d, q);
+cudaError_t jet_shell(const Dims& d, const Consts& c, const GridDev& g, const Inflow& in, const State& q,
+                      Scalars* sc, int stage, int advance, cudaStream_t st) {
+  ShellArgs A;
+  A.d = d;
+  A.c = c;
+  A.cf = make_constsf(c);
+  A.Sb = g.Sb;
+  A.u0 = in.u0;
+  A.Gf = in.Gf;
+  for (int mf = 0; mf < kNF; ++mf) A.amp[mf] = in.amp[mf];
+  A.q = q;
+  A.sc = sc;
+  A.sn = in.sn + stage * kNF;
+  A.advance = advance;
+  const long long ni2 = d.ni - 2;
+  const unsigned nio = blocks_for((long long)(d.nj - 1) * d.nk, kTPB);
+  A.bA = (unsigned)d.ni;
+  A.bE = A.bA + nio;
+  A.bX = A.bE + nio;
+  A.bF = A.bX + blocks_for(ni2 * d.nk, kTPB);
+  A.bR = A.bF + blocks_for(2 * ni2 * (d.nk + 2 * kG), kTPB);
+  const unsigned n = A.bR + blocks_for(4 * ni2 * (d.nj - 2), kTPB);
+  if (q.sh)
+    k_jet_shell<true><<<n, kTPB, 0, st>>>(A);
+  else
+    k_jet_shell<false><<<n, kTPB, 0, st>>>(A);
   return cudaGetLastError();
 }
 

@@ -1,7 +1,7 @@
 // Grid set-up kernels: ghost coordinates, metrics of the curvilinear
 // transformation (Algorithm 2: Calc(Jacob., Metric)), ghost fills and the
 // copies between unpadded caller arrays and the padded device layout.
-#include "jz_internal.cuh"
+#include "jz_shadow.cuh"
 
 namespace jz {
 namespace {
@@ -172,6 +172,22 @@ __global__ void k_ghost_fill(Dims d, Ptrs16 f, int nvar) {
   for (int v = 0; v < nvar; ++v) f.p[v][p] = f.p[v][q];
 }
 
+// Ghosts of a state (and of its shadow).
+__global__ void k_ghost_state(Dims d, State q, Scalars* advance) {
+  if (advance && blockIdx.x == 0 && threadIdx.x == 0) advance->t = advance->t + advance->dt;
+  int i, j, k;
+  if (!ghost_coord(d, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
+  int si, sj, sk;
+  ghost_source(d, i, j, k, si, sj, sk);
+  const long long p = pidx(d, i, j, k), s = pidx(d, si, sj, sk);
+#pragma unroll
+  for (int m = 0; m < 5; ++m) q.q[m][p] = q.q[m][s];
+  if (q.sh) {
+#pragma unroll
+    for (int m = 0; m < NSH; ++m) q.sh[m * d.Np + p] = q.sh[m * d.Np + s];
+  }
+}
+
 // FP32 metric records: kMF floats per padded node from kMF FP64 arrays.
 __global__ void k_to_f32(Dims d, Ptrs16 src, float* __restrict__ dst) {
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -184,13 +200,24 @@ __global__ void k_to_f32(Dims d, Ptrs16 src, float* __restrict__ dst) {
   o[2] = make_float4(r[8], r[9], r[10], r[11]);
 }
 
-__global__ void k_pack(Dims d, Ptrs16 padded, const double* __restrict__ flat, int nvar) {
+// A flat [5][N] array into the real nodes of a state (and their shadow).
+__global__ void k_pack_state(Dims d, ConstsF c, State q, const double* __restrict__ flat) {
   Box b{0, 0, 0, d.ni, d.nj, d.nk};
   int i, j, k;
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (!box_coord(b, t, i, j, k)) return;
   const long long N = (long long)d.ni * d.nj * d.nk, p = pidx(d, i, j, k);
-  for (int v = 0; v < nvar; ++v) padded.p[v][p] = flat[v * N + t];
+  double v[5];
+#pragma unroll
+  for (int m = 0; m < 5; ++m) v[m] = flat[m * N + t];
+#pragma unroll
+  for (int m = 0; m < 5; ++m) q.q[m][p] = v[m];
+  if (q.sh) {
+    float2 s[NSH];
+    shadow_of(c, v, s);
+#pragma unroll
+    for (int m = 0; m < NSH; ++m) q.sh[m * d.Np + p] = s[m];
+  }
 }
 
 __global__ void k_unpack(Dims d, Ptrs16 padded, double* __restrict__ flat, int nvar) {
@@ -299,9 +326,16 @@ cudaError_t metrics_to_f32(const Dims& d, const GridDev& g, float* Mf, cudaStrea
   return cudaGetLastError();
 }
 
-cudaError_t pack_real(const Dims& d, double* const* padded, const double* flat, int nvar, cudaStream_t st) {
+cudaError_t pack_state(const Dims& d, const Consts& c, const State& q, const double* flat, cudaStream_t st) {
   const long long nr = (long long)d.ni * d.nj * d.nk;
-  k_pack<<<blocks_for(nr, kTPB), kTPB, 0, st>>>(d, ptrs(padded, nvar), flat, nvar);
+  k_pack_state<<<blocks_for(nr, kTPB), kTPB, 0, st>>>(d, make_constsf(c), q, flat);
+  return cudaGetLastError();
+}
+
+cudaError_t ghost_fill_state(const Dims& d, const State& q, Scalars* advance, cudaStream_t st) {
+  const long long ei = d.ni + 2 * kG, ej = d.nj + 2 * kG;
+  const long long ng = 4 * ei * ej + 4 * ei * d.nk + 4LL * d.nj * d.nk;
+  k_ghost_state<<<blocks_for(ng, kTPB), kTPB, 0, st>>>(d, q, advance);
   return cudaGetLastError();
 }
 

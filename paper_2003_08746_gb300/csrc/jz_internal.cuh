@@ -155,7 +155,24 @@ struct Consts {
   double cfl, dt_fixed;
   double p_inf;
   double jet_mach, theta_mom;
+  double isen;                      // 2 / (gamma - 1): exponent of rho along an isentrope in a
+  int isen_n;                       // that exponent if it is a small whole number (5 for air), else 0
 };
+
+// (a / a_s)^(2 / (gamma-1)) = rho / rho_s along an isentrope, x = a / a_s >= 0.  Whole exponents by
+// products: for air x^5 is 3 FP64 instructions where the library pow takes well over a hundred.
+__device__ __forceinline__ double isentrope(const Consts& c, double x) {
+  if (c.isen_n == 5) {
+    const double x2 = x * x;
+    return x2 * x2 * x;
+  }
+  if (c.isen_n > 0) {
+    double r = x;
+    for (int n = 1; n < c.isen_n; ++n) r *= x;
+    return r;
+  }
+  return pow(x, c.isen);
+}
 
 // Derived constants from the caller's parameters.
 inline Consts make_consts(const jz_params& p) {
@@ -180,6 +197,9 @@ inline Consts make_consts(const jz_params& p) {
   c.p_inf = 1.0 / p.gamma;
   c.jet_mach = p.jet_mach;
   c.theta_mom = p.theta_mom;
+  c.isen = 2.0 / c.gm1;
+  const int n = c.isen < 8.5 ? (int)(c.isen + 0.5) : 0;
+  c.isen_n = n > 0 && fabs(c.isen - n) <= 1e-14 * n ? n : 0;
   return c;
 }
 
@@ -282,6 +302,8 @@ struct Inflow {
   double amp[kNF];
   double psi[kNF];
   double omega[JZ_N_FREQ];       // 2 pi St_f U_j
+  double* sn;                    // [5][32] temporal factors sin(omega_f (t + alpha_l dt) + psi_mf) of the
+                                 // current step's stages, written with dt (device)
 };
 
 // ---- kernels' host launchers -------------------------------------------
@@ -291,14 +313,16 @@ cudaError_t pad_coordinates(const Dims& d, const double* xyz_real, const double*
 cudaError_t compute_metrics(const Dims& d, GridDev& g, double* scratch9[9], cudaStream_t st);
 // ghost fill of nvar padded fields by the state's ghost map
 cudaError_t ghost_fill(const Dims& d, double* const* f, int nvar, cudaStream_t st);
+// ghosts of a state and of its shadow; advance: the scalars of a solver whose step ends here, t += dt
+cudaError_t ghost_fill_state(const Dims& d, const State& q, Scalars* advance, cudaStream_t st);
 // FP32 copy of the metrics S (9) and V; dst_dev is a device array of 10 pointers
 cudaError_t boundary_copies(const Dims& d, const GridDev& g, cudaStream_t st);
 cudaError_t metrics_to_f32(const Dims& d, const GridDev& g, float* Mf, cudaStream_t st);
-// copy between unpadded [nvar][N] and padded real region
-cudaError_t pack_real(const Dims& d, double* const* padded, const double* flat, int nvar,
-                      cudaStream_t st);
+// padded real region of nvar fields to a flat [nvar][N] array
 cudaError_t unpack_real(const Dims& d, double* const* padded, double* flat, int nvar,
                         cudaStream_t st);
+// real nodes of a state from a flat [5][N] array, with their shadow in the FP32-flux form
+cudaError_t pack_state(const Dims& d, const Consts& c, const State& q, const double* flat, cudaStream_t st);
 // FP64 stage passes (one kernel each)
 // rate_max != nullptr: also reduce the CFL rate of qin over the advanced nodes into
 // *rate_max (max of (sum_dir lambda_dir) / V; the caller has left it 0)
@@ -317,10 +341,6 @@ cudaError_t update64(const Dims& d, const GridDev& g, const Work64& w, const Sta
 cudaError_t fused32(const Dims& d, const Consts& c, const float* Mf, const State& qin, const void* tm_in,
                     const State& qn, const State& qout, Scalars* sc, double alpha, int want_res, int want_rate,
                     double* rhs_flat, int kchunk, cudaStream_t st);
-// FP32 shadow of q from its FP64 values: every padded node (full) or only the shell that the
-// boundary conditions and the ghost fill rewrite after a stage (ghost layers and the planes
-// i = 0, ni-1, j = 0, nj-1).
-cudaError_t shadow_refresh(const Dims& d, const Consts& c, const State& q, int full, cudaStream_t st);
 // TMA descriptor (CUtensorMap, 128 bytes, 64-byte aligned) of a shadow: 4-D (Pi, Pj, Pk, 3)
 // of 8-byte elements; returns cudaErrorInvalidValue if the encoder is unavailable or refuses.
 cudaError_t make_shadow_map(const Dims& d, float2* sh, void* tmap128);
@@ -339,17 +359,19 @@ cudaError_t viscous_df(const Dims& d, const Consts& c, const DFMetrics& M, const
 cudaError_t faces_update_df(const Dims& d, const Consts& c, const GridDev& g, const Work64& w, const QDF& qdf,
                             const State& qin, const State& qn, const State& qout, const Scalars* sc, double alpha,
                             int want_res, double* rhs_flat, cudaStream_t st);
-// boundary conditions (jet), in this order after every stage
-cudaError_t bc_farfield(const Dims& d, const Consts& c, const GridDev& g, const State& q, cudaStream_t st);
-cudaError_t bc_inout(const Dims& d, const Consts& c, const Inflow& in, const State& q, const Scalars* sc,
-                     double alpha, cudaStream_t st);
-cudaError_t bc_axis(const Dims& d, const State& q, cudaStream_t st);
+// boundary conditions and ghost points of the jet after stage `stage` (one kernel); advance: last
+// stage of a step, t += dt.  Needs the temporal factors that set_dt or set_time left for the step.
+cudaError_t jet_shell(const Dims& d, const Consts& c, const GridDev& g, const Inflow& in, const State& q,
+                      Scalars* sc, int stage, int advance, cudaStream_t st);
 cudaError_t build_inflow(const Dims& d, const Consts& c, const GridDev& g, const jz_params& p,
                          Inflow& in, cudaStream_t st);
 // reductions
 cudaError_t cfl_rate(const Dims& d, const Consts& c, const GridDev& g, const State& q,
                      Scalars* sc, cudaStream_t st);
-cudaError_t set_dt(const Consts& c, Scalars* sc, int advance_time, cudaStream_t st);
+// time step of the current step from the reduced rate (or dt_fixed), and the forcing's temporal factors
+cudaError_t set_dt(const Consts& c, const Inflow& in, Scalars* sc, cudaStream_t st);
+// t and dt given (the adjoint's sweeps), and the forcing's temporal factors
+cudaError_t set_time(const Inflow& in, Scalars* sc, double t, double dt, cudaStream_t st);
 int stat_partial_count();
 cudaError_t stats_with(const Dims& d, const Consts& c, const GridDev& g, const State& q, Scalars* sc,
                        double* part, cudaStream_t st);
@@ -383,7 +405,6 @@ cudaError_t adj_bcs(const Dims& d, const Consts& c, const GridDev& g, const Infl
                     const Adj64& a, double ts, cudaStream_t st);
 cudaError_t observer(const Dims& d, const Consts& c, const State& q, const double* w, int j0, double beta,
                      double dt, const Adj64& a, int want_grad, cudaStream_t st);
-cudaError_t set_time(Scalars* sc, double t, double dt, cudaStream_t st);
 
 // ---- shared with the C ABI layer ------------------------------------------
 // Record an error message for jz_last_error(); returns code.

@@ -133,8 +133,8 @@ extern "C" int jz_residual_noalloc(const jz_grid* g, const jz_params* p, const d
   // Every scratch element a kernel reads is written earlier in this call;
   // only the scalar block is cleared (the previous call's values stay in the rest).
   e = cudaMemsetAsync(sc, 0, sizeof(Scalars), st);
-  if (e == cudaSuccess) e = pack_real(d, qp.q, q, 5, st);
-  if (e == cudaSuccess) e = ghost_fill(d, qp.q, 5, st);
+  if (e == cudaSuccess) e = pack_state(d, c, qp, q, st);
+  if (e == cudaSuccess) e = ghost_fill_state(d, qp, nullptr, st);
   if (e == cudaSuccess) e = nodal64(d, c, gd, w, qp, st);
   if (e == cudaSuccess) e = viscous64(d, c, gd, w, qp, st);
   if (e == cudaSuccess) e = faces64(d, c, w, qp, st);

@@ -36,16 +36,43 @@ __global__ void k_cfl_rate(Dims d, GridDev g, State q, Consts c, Scalars* sc) {
   }
 }
 
-__global__ void k_set_dt(Consts c, Scalars* sc) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  sc->dt = c.dt_fixed > 0.0 ? c.dt_fixed : c.cfl / sc->rate_max;
+// Temporal factors of the entrance forcing at the five stage times of the step (t, dt), one
+// thread each; a step evaluates them once instead of once per entrance block and stage.
+struct Forcing {
+  double psi[kNF], omega[JZ_N_FREQ];
+  double* sn;                    // null off the jet
+};
+constexpr int kForcing = 5 * kNF;
+__device__ __forceinline__ void stage_forcing(const Forcing& f, double t, double dt) {
+  const double alpha[5] = {0.25, 1.0 / 6.0, 0.375, 0.5, 1.0};
+  const int l = threadIdx.x / kNF, mf = threadIdx.x % kNF;
+  if (f.sn && l < 5) f.sn[threadIdx.x] = sin(f.omega[mf % JZ_N_FREQ] * (t + alpha[l] * dt) + f.psi[mf]);
+}
+
+__global__ void k_set_dt(Consts c, Forcing f, Scalars* sc) {
+  const double dt = c.dt_fixed > 0.0 ? c.dt_fixed : c.cfl / sc->rate_max;
+  stage_forcing(f, sc->t, dt);
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  sc->dt = dt;
   sc->rate_max = 0.0;
   sc->res_sum = 0.0;
 }
 
-__global__ void k_end_step(Scalars* sc) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  sc->t = sc->t + sc->dt;
+__global__ void k_set_time(Forcing f, Scalars* sc, double t, double dt) {
+  stage_forcing(f, t, dt);
+  if (threadIdx.x == 0) {
+    sc->t = t;
+    sc->dt = dt;
+  }
+}
+
+Forcing forcing_of(const Inflow& in) {
+  Forcing f;
+  f.sn = in.sn;
+  for (int mf = 0; mf < kNF; ++mf) f.psi[mf] = in.psi[mf];
+  for (int q = 0; q < JZ_N_FREQ; ++q) f.omega[q] = in.omega[q];
+  return f;
 }
 
 // Totals sum Q_m V, min rho, min p, non-finite flag; grid-stride with a fixed
@@ -127,11 +154,13 @@ cudaError_t cfl_rate(const Dims& d, const Consts& c, const GridDev& g, const Sta
   return cudaGetLastError();
 }
 
-cudaError_t set_dt(const Consts& c, Scalars* sc, int advance_time, cudaStream_t st) {
-  if (advance_time)
-    k_end_step<<<1, 32, 0, st>>>(sc);
-  else
-    k_set_dt<<<1, 32, 0, st>>>(c, sc);
+cudaError_t set_dt(const Consts& c, const Inflow& in, Scalars* sc, cudaStream_t st) {
+  k_set_dt<<<1, kForcing, 0, st>>>(c, forcing_of(in), sc);
+  return cudaGetLastError();
+}
+
+cudaError_t set_time(const Inflow& in, Scalars* sc, double t, double dt, cudaStream_t st) {
+  k_set_time<<<1, kForcing, 0, st>>>(forcing_of(in), sc, t, dt);
   return cudaGetLastError();
 }
 

@@ -9,8 +9,8 @@
 // beside the FP64 state in three float2 arrays per padded node:
 // (rho - 1, e - e_inf), (rho u, rho v), (rho w, p - p_inf).  The offsets keep
 // the FP32 values small in the ambient flow.  The stage that writes Q^(l)
-// writes its shadow; after the boundary conditions and the ghost fill a shell
-// kernel refreshes the shadow of the nodes they rewrote.
+// writes its shadow, and the kernels that set boundary nodes, fill ghosts or
+// load a state write the shadow of what they set.
 //
 // Each CTA owns a TX x TY tile of (i, j) columns and marches in k.  Shared
 // memory holds a ring of four planes of the shadow (tile + 2-node halo; each
@@ -38,7 +38,7 @@
 #include <algorithm>
 #include <cstring>
 
-#include "jz_internal.cuh"
+#include "jz_shadow.cuh"
 
 namespace jz {
 namespace {
@@ -61,7 +61,6 @@ constexpr int NIR = (NP2 + NT - 1) / NT;                     // halo-2 points pe
 // shadow ring: per halo-2 point three float2 pairs, as in global memory
 // (rho' = rho - 1, e' = e - e_inf), (m1, m2), (m3, p' = p - p_inf), and 1/rho beside them
 // (u = m/rho and T = gamma p/rho are formed where they are used)
-constexpr int NSH = 3;
 constexpr int NRING = 4;           // planes k-1 .. k+2: the next plane's request needs no barrier
 constexpr int BOX_BYTES = NSH * NP2 * 8;                       // one TMA box (34 x 12 x 1 x 3 float2)
 constexpr int SLOT = ((BOX_BYTES + 127) / 128) * 128 / 8;      // float2 per ring slot, 128-byte aligned
@@ -83,23 +82,6 @@ struct Smem {
   int fail;                        // a bounded wait ran out in this CTA
 };
 
-struct ConstsF {
-  float gamma, gm1, mu_ref, S_hat, sut_num, k_lam, k_sgs, C_s, kappa2, kappa4;
-  float p_inf, ep_inf;     // p_inf, e_inf + p_inf
-  double e_inf;            // p_inf / (gamma - 1), subtracted in FP64
-};
-
-// FP64 -> FP32 by bit manipulation (truncation toward zero; magnitudes below
-// 2^-126 flush to signed zero).  Valid for finite |x| < 2^128.  Re-biasing the
-// exponent on the high word (e - 896 fits in 8 bits) lets one funnel shift pick
-// the FP32 exponent and the top 23 mantissa bits at once.
-__device__ __forceinline__ float f64_to_f32(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned f = __funnelshift_l(lo, hi - (896u << 20), 3);
-  const unsigned r = (f & 0x7FFFFFFFu) | (hi & 0x80000000u);
-  return __uint_as_float((hi << 1) >= (897u << 21) ? r : (hi & 0x80000000u));
-}
-
 // FP32 -> FP64, exact (subnormals flush to zero; Inf/NaN kept).
 __device__ __forceinline__ double f32_to_f64(float f) {
   const unsigned b = __float_as_uint(f);
@@ -109,13 +91,7 @@ __device__ __forceinline__ double f32_to_f64(float f) {
   return __hiloint2double((int)(s | (e11 << 20) | (m >> 3)), (int)(m << 29));
 }
 
-// Single MUFU approximations (relative error ~2^-22), far inside the FP32-flux
-// form's error budget.
-__device__ __forceinline__ float f_rcp(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
+// Single MUFU approximations as f_rcp (relative error ~2^-22).
 __device__ __forceinline__ float f_sqrt(float x) {
   float r;
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -226,18 +202,6 @@ __device__ __forceinline__ void inv_rho(Smem& sm, int slot) {
     const int t = threadIdx.x + r * NT;
     if (t < NP2) sm.ir[slot][t] = f_rcp(sm.sh[slot][t].x + 1.f);
   }
-}
-
-// The three shadow pairs of an FP64 state node (the FP32 values the stage arithmetic uses).
-__device__ __forceinline__ void shadow_of(const ConstsF& c, const double q[5], float2 out[NSH]) {
-  const float rp = f64_to_f32(q[0] - 1.0);
-  const float m1 = f64_to_f32(q[1]), m2 = f64_to_f32(q[2]), m3 = f64_to_f32(q[3]);
-  const float ep = f64_to_f32(q[4] - c.e_inf);
-  const float ir = f_rcp(rp + 1.f);
-  const float pp = c.gm1 * (ep - 0.5f * ir * (m1 * m1 + m2 * m2 + m3 * m3));
-  out[0] = make_float2(rp, ep);
-  out[1] = make_float2(m1, m2);
-  out[2] = make_float2(m3, pp);
 }
 
 // Metric record of one node (three 16-byte loads).
@@ -633,53 +597,6 @@ __global__ void __launch_bounds__(NT, kMinBlocks) k_fused32(const __grid_constan
 }
 
 
-// FP32 shadow of the FP64 state on every padded node (full) or on the shell that the boundary
-// conditions and the ghost fill rewrite: i in {-2, -1, 0, ni-1, ni, ni+1} (all j, k), then j in
-// {-2, -1, 0, nj-1, nj, nj+1} and k in {-2, -1, nk, nk+1} over the remaining nodes.
-__global__ void k_shadow(Dims d, ConstsF c, State q, int full) {
-  long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  int i, j, k;
-  if (full) {
-    const Box b{-kG, -kG, -kG, d.ni + 2 * kG, d.nj + 2 * kG, d.nk + 2 * kG};
-    if (!box_coord(b, t, i, j, k)) return;
-  } else {
-    const int ii = max(d.ni - 2, 0), ij = max(d.nj - 2, 0);
-    const long long cI = 6LL * (d.nj + 2 * kG) * (d.nk + 2 * kG);
-    const long long cJ = 6LL * ii * (d.nk + 2 * kG);
-    const long long cK = 4LL * ii * ij;
-    int a;
-    if (t < cI) {
-      a = (int)(t % 6);
-      const long long r = t / 6;
-      j = (int)(r % (d.nj + 2 * kG)) - kG;
-      k = (int)(r / (d.nj + 2 * kG)) - kG;
-      i = a < 3 ? a - kG : d.ni - 1 + (a - 3);
-    } else if ((t -= cI) < cJ) {
-      a = (int)(t % 6);
-      const long long r = t / 6;
-      i = 1 + (int)(r % ii);
-      k = (int)(r / ii) - kG;
-      j = a < 3 ? a - kG : d.nj - 1 + (a - 3);
-    } else if ((t -= cJ) < cK) {
-      a = (int)(t % 4);
-      const long long r = t / 4;
-      i = 1 + (int)(r % ii);
-      j = 1 + (int)(r / ii);
-      k = a < 2 ? a - kG : d.nk + (a - 2);
-    } else {
-      return;
-    }
-  }
-  const long long p = pidx(d, i, j, k);
-  double v[5];
-#pragma unroll
-  for (int m = 0; m < 5; ++m) v[m] = q.q[m][p];
-  float2 s[NSH];
-  shadow_of(c, v, s);
-#pragma unroll
-  for (int m = 0; m < NSH; ++m) q.sh[m * d.Np + p] = s[m];
-}
-
 // Self-check of the bounded wait: one warp initialises an mbarrier that nothing ever arrives at
 // and waits for it with the stage kernel's bounded poll; the wait must run out and return.
 __global__ void k_wait_check(int* timed_out, long long* cycles) {
@@ -696,16 +613,6 @@ __global__ void k_wait_check(int* timed_out, long long* cycles) {
     *timed_out = ok ? 0 : 1;
     *cycles = t1 - t0;
   }
-}
-
-ConstsF make_constsf(const Consts& c) {
-  ConstsF f;
-  f.gamma = (float)c.gamma; f.gm1 = (float)c.gm1; f.mu_ref = (float)c.mu_ref; f.S_hat = (float)c.S_hat;
-  f.sut_num = (float)c.sut_num; f.k_lam = (float)c.k_lam; f.k_sgs = (float)c.k_sgs; f.C_s = (float)c.C_s;
-  f.kappa2 = (float)c.kappa2; f.kappa4 = (float)c.kappa4; f.p_inf = (float)c.p_inf;
-  f.e_inf = c.p_inf / c.gm1;
-  f.ep_inf = (float)(f.e_inf + c.p_inf);
-  return f;
 }
 
 constexpr int kSmemBytes = (int)sizeof(Smem) + 128;    // + room to align the ring to 128 bytes
@@ -759,18 +666,6 @@ cudaError_t make_shadow_map(const Dims& d, float2* sh, void* tmap128) {
                             box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
-}
-
-cudaError_t shadow_refresh(const Dims& d, const Consts& c, const State& q, int full, cudaStream_t st) {
-  long long n;
-  if (full) {
-    n = (long long)(d.ni + 2 * kG) * (d.nj + 2 * kG) * (d.nk + 2 * kG);
-  } else {
-    const long long ii = std::max(d.ni - 2, 0), ij = std::max(d.nj - 2, 0);
-    n = 6LL * (d.nj + 2 * kG) * (d.nk + 2 * kG) + 6LL * ii * (d.nk + 2 * kG) + 4LL * ii * ij;
-  }
-  k_shadow<<<blocks_for(n, 256), 256, 0, st>>>(d, make_constsf(c), q, full);
-  return cudaGetLastError();
 }
 
 cudaError_t fused32(const Dims& d, const Consts& c, const float* Mf, const State& qin, const void* tm_in,
