@@ -242,10 +242,8 @@ int run_stage64(jz_solver* s, const jz::State& in, const jz::State& out, double 
   const jz::Dims& d = s->grid->d;
   const jz::GridDev& g = s->grid->g;
   if (s->pair) {
-    JZ_RUN(JZ_PROF_NODAL, jz::nodal_df(d, s->c, s->mdf, s->w, s->qdf, in, s->st,
-                                       cfl_first ? &s->sc->rate_max : nullptr));
+    JZ_RUN(JZ_PROF_VISCOUS, jz::flux_df(d, s->c, s->mdf, s->w, s->qdf, in, s->sc, s->st, cfl_first));
     if (cfl_first) JZ_RUN(JZ_PROF_REDUCE, jz::set_dt(s->c, s->in, s->sc, s->st));
-    JZ_RUN(JZ_PROF_VISCOUS, jz::viscous_df(d, s->c, s->mdf, s->w, s->qdf, s->st));
     JZ_RUN(JZ_PROF_FACES, jz::faces_update_df(d, s->c, g, s->w, s->qdf, in, s->qn, out, s->sc, alpha, want_res,
                                               rhs_flat, s->st));
     return JZ_OK;
@@ -380,8 +378,7 @@ int fwd_stage(jz_solver* s, const jz::State& in, const jz::State& qn, const jz::
   const jz::Dims& d = s->grid->d;
   const jz::GridDev& g = s->grid->g;
   if (s->pair) {
-    JZ_RUN(JZ_PROF_NODAL, jz::nodal_df(d, s->c, s->mdf, s->w, s->qdf, in, s->st));
-    JZ_RUN(JZ_PROF_VISCOUS, jz::viscous_df(d, s->c, s->mdf, s->w, s->qdf, s->st));
+    JZ_RUN(JZ_PROF_VISCOUS, jz::flux_df(d, s->c, s->mdf, s->w, s->qdf, in, s->sc, s->st));
     JZ_RUN(JZ_PROF_FACES, jz::faces_update_df(d, s->c, g, s->w, s->qdf, in, qn, out, s->sc, kAlpha[l], 0, nullptr,
                                               s->st));
   } else {
@@ -1006,7 +1003,7 @@ int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ck
         // the forward intermediates the transposed passes read, regenerated in the solver's form
         if (s->pair) {
           JZ_RUN(JZ_PROF_NODAL, jz::nodal_df(d, s->c, s->mdf, s->w, s->qdf, *st[l], s->st));
-          JZ_RUN(JZ_PROF_VISCOUS, jz::viscous_df(d, s->c, s->mdf, s->w, s->qdf, s->st));
+          JZ_RUN(JZ_PROF_VISCOUS, jz::sensor_df_pass(d, s->w, s->st));
         } else {
           JZ_RUN(JZ_PROF_NODAL, jz::nodal64(d, s->c, g, s->w, *st[l], s->st));
           JZ_RUN(JZ_PROF_VISCOUS, jz::viscous64(d, s->c, g, s->w, *st[l], s->st));

@@ -18,6 +18,7 @@ namespace jz {
 namespace {
 
 constexpr int kTPB = 128;
+constexpr int AXI = 8, AXK = kTPB / AXI;   // axis blocks: lines of i, threads along k
 
 // What the kernel needs of the state: the FP64 fields and, for the FP32-flux form, the shadow.
 struct ShellArgs {
@@ -87,10 +88,11 @@ __device__ void farfield_value(const ShellArgs& A, int i, int k, const double qi
 __device__ void entrance_value(const ShellArgs& A, const double* am, int j, int k, const double q1[5], double out[5]) {
   const Consts& c = A.c;
   const long long tab = (long long)k * A.d.nj + j, plane = (long long)A.d.nk * A.d.nj;
-  double f = 0.0;
-#pragma unroll 8
-  for (int mf = 0; mf < kNF; ++mf) f = fma(am[mf], __ldg(A.Gf + mf * plane + tab), f);
-  const double ut = fma(c.jet_mach, f, A.u0[tab]);
+  // four partial sums: the FP64 latency of one chain of 32 would set the kernel's time
+  double f[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+  for (int mf = 0; mf < kNF; ++mf) f[mf & 3] = fma(am[mf], __ldg(A.Gf + mf * plane + tab), f[mf & 3]);
+  const double ut = fma(c.jet_mach, (f[0] + f[1]) + (f[2] + f[3]), A.u0[tab]);
   if (ut >= 1.0) {                                          // supersonic: all imposed
     cons_of(c, 1.0, ut, 0.0, 0.0, c.p_inf, out);
     return;
@@ -168,7 +170,7 @@ __device__ __forceinline__ void copy_node(const ShellArgs& A, long long p, long 
   }
 }
 
-// Boundary nodes and ghosts of the jet, by block roles: axis (one block per i), entrance, exit,
+// Boundary nodes and ghosts of the jet, by block roles: axis (eight lines of i per block), entrance, exit,
 // far field, ghost rows across the axis, ghost planes around the azimuth.  Latency bounds it (a
 // chain of dependent FP64 operations per node on a few thousand nodes).
 template <bool SH>
@@ -181,39 +183,43 @@ __global__ void __launch_bounds__(kTPB) k_jet_shell(const __grid_constant__ Shel
     __syncthreads();
   }
   if (b < A.bA) {
-    // axis: the ring j = 1 averaged over the azimuth
-    const int i = (int)b;
+    // axis: the ring j = 1 averaged over the azimuth, AXI lines of i by AXK threads along k
+    const int i = (int)(b * AXI + th % AXI), ky = th / AXI;
+    const bool in = i < d.ni;
     double s[5] = {0, 0, 0, 0, 0};
-    for (int k = th; k < d.nk; k += kTPB) {
-      double v[5], t[5];
-      if (i == 0) {
-        inner_neighbour(A, 1, 1, k, t);
-        entrance_value(A, am, 1, k, t, v);
-      } else if (i == d.ni - 1) {
-        inner_neighbour(A, i - 1, 1, k, t);
-        exit_value(A, t, v);
-      } else {
-        load_q(A.q, pidx(d, i, 1, k), v);
-      }
+    if (in) {
+      for (int k = ky; k < d.nk; k += AXK) {
+        double v[5], t[5];
+        if (i == 0) {
+          inner_neighbour(A, 1, 1, k, t);
+          entrance_value(A, am, 1, k, t, v);
+        } else if (i == d.ni - 1) {
+          inner_neighbour(A, i - 1, 1, k, t);
+          exit_value(A, t, v);
+        } else {
+          load_q(A.q, pidx(d, i, 1, k), v);
+        }
 #pragma unroll
-      for (int m = 0; m < 5; ++m) s[m] += v[m];
+        for (int m = 0; m < 5; ++m) s[m] += v[m];
+      }
     }
-    __shared__ double red[5][kTPB / 32];
+    __shared__ double red[5][kTPB / 32][AXI];
 #pragma unroll
     for (int m = 0; m < 5; ++m) {
       double x = s[m];
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-      if ((th & 31) == 0) red[m][th >> 5] = x;
+      for (int o = 16; o >= AXI; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      if ((th & 31) < AXI) red[m][th >> 5][th & 31] = x;
     }
     __syncthreads();
     double mean[5];
 #pragma unroll
     for (int m = 0; m < 5; ++m) {
       double x = 0.0;
-      for (int w = 0; w < kTPB / 32; ++w) x += red[m][w];
+      for (int w = 0; w < kTPB / 32; ++w) x += red[m][w][th % AXI];
       mean[m] = x / d.nk;
     }
-    for (int k = th; k < d.nk; k += kTPB) put_node<SH>(A, mean, i, 0, k);
+    if (in)
+      for (int k = ky; k < d.nk; k += AXK) put_node<SH>(A, mean, i, 0, k);
     if (b == 0 && th == 0 && A.advance) A.sc->t = A.sc->t + A.sc->dt;
     return;
   }
@@ -308,7 +314,7 @@ cudaError_t jet_shell(const Dims& d, const Consts& c, const GridDev& g, const In
   A.advance = advance;
   const long long ni2 = d.ni - 2;
   const unsigned nio = blocks_for((long long)(d.nj - 1) * d.nk, kTPB);
-  A.bA = (unsigned)d.ni;
+  A.bA = blocks_for(d.ni, AXI);
   A.bE = A.bA + nio;
   A.bX = A.bE + nio;
   A.bF = A.bX + blocks_for(ni2 * d.nk, kTPB);

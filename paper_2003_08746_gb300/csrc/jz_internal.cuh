@@ -349,13 +349,15 @@ cudaError_t fused32_slots(int* slots);
 cudaError_t wait_check(int* dev_timed_out, long long* dev_cycles, cudaStream_t st);
 int fused32_tile_x();
 int fused32_tile_y();
-// Pair form of the FP64 stage (jz_stagedf.cu): the four passes in double-float arithmetic,
-// the stage combination in FP64.
+// Pair form of the FP64 stage (jz_stagedf.cu) in double-float arithmetic, the stage combination in
+// FP64: flux_df and faces_update_df; nodal_df and sensor_df_pass regenerate what the adjoint's
+// transposed kernels read (want_rate: reduce the CFL rate of qin into sc->rate_max, left 0 before).
 cudaError_t metrics_to_df(const Dims& d, const GridDev& g, const DFMetrics& M, cudaStream_t st);
 cudaError_t nodal_df(const Dims& d, const Consts& c, const DFMetrics& M, const Work64& w, const QDF& qdf,
-                     const State& qin, cudaStream_t st, double* rate_max = nullptr);
-cudaError_t viscous_df(const Dims& d, const Consts& c, const DFMetrics& M, const Work64& w, const QDF& qdf,
-                       cudaStream_t st);
+                     const State& qin, cudaStream_t st);
+cudaError_t flux_df(const Dims& d, const Consts& c, const DFMetrics& M, const Work64& w, const QDF& qdf,
+                    const State& qin, Scalars* sc, cudaStream_t st, int want_rate = 0);
+cudaError_t sensor_df_pass(const Dims& d, const Work64& w, cudaStream_t st);
 cudaError_t faces_update_df(const Dims& d, const Consts& c, const GridDev& g, const Work64& w, const QDF& qdf,
                             const State& qin, const State& qn, const State& qout, const Scalars* sc, double alpha,
                             int want_res, double* rhs_flat, cudaStream_t st);

@@ -38,6 +38,7 @@
 #include <algorithm>
 #include <cstring>
 
+#include "jz_mbar.cuh"
 #include "jz_shadow.cuh"
 
 namespace jz {
@@ -154,13 +155,7 @@ struct Args {
   int want_rate;
 };
 
-// ---- TMA and mbarrier (inline PTX) ----
-__device__ __forceinline__ unsigned smem_u32(const void* p) {
-  return (unsigned)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void bar_init(unsigned long long* b, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
-}
+// ---- TMA (inline PTX) ----
 // Request the shadow of plane k (padded plane k + 2) of this CTA's halo-2 box into a ring slot;
 // the mbarrier completes when its BOX_BYTES have landed.  Called by one thread.
 __device__ __forceinline__ void request_plane(const Args& A, Smem& sm, int slot, int x0, int y0, int k) {
@@ -174,21 +169,6 @@ __device__ __forceinline__ void request_plane(const Args& A, Smem& sm, int slot,
       "%5}], [%6];" ::"r"(smem_u32(&sm.sh[slot][0])),
       "l"(reinterpret_cast<unsigned long long>(&A.tm)), "r"(x0), "r"(y0), "r"(k + kG), "r"(0), "r"(smem_u32(b))
       : "memory");
-}
-// Wait for an mbarrier phase with a bounded number of polls; false if it never completed.
-constexpr int kWaitPolls = 1 << 18;   // ~1 s on GB300 (each unanswered try_wait suspends a few microseconds)
-__device__ __forceinline__ bool wait_bar(unsigned long long* bar, unsigned parity) {
-  const unsigned b = smem_u32(bar);
-  for (int it = 0; it < kWaitPolls; ++it) {
-    unsigned ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(ok)
-        : "r"(b), "r"(parity)
-        : "memory");
-    if (ok) return true;
-  }
-  return false;
 }
 __device__ __forceinline__ bool wait_slot(Smem& sm, int slot, unsigned parity) { return wait_bar(&sm.bar[slot], parity); }
 

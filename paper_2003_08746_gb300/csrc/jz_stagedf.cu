@@ -1,16 +1,16 @@
 // Pair form of the FP64 stage: the work of the four passes of jz_stage64.cu (nodal, viscous,
 // faces, update; Algorithm 2's inviscid flux, dissipation, viscous flux, RHS and
-// Update(Cons, alpha_l)) in three kernels, with every flux, dissipation and SGS operation in
+// Update(Cons, alpha_l)) in two kernels, with every flux, dissipation and SGS operation in
 // double-float arithmetic (jz_df.cuh: pairs of FP32 numbers, ~48 significant bits) and the stage
-// combination Q^n - alpha dt RHS in FP64.  The state stays FP64; the nodal pass reads it once and
-// leaves a double-float copy for the dissipation; the intermediate fields are double-float pairs
+// combination Q^n - alpha dt RHS in FP64.  The state stays FP64; the flux kernel reads it once and
+// leaves a double-float copy for the dissipation; the fields it hands on are double-float pairs
 // (float2) in the FP64 form's work arrays (same size); the metrics are a double-float copy made
-// when the solver is created.  The last kernel forms the face fluxes and sums them into the RHS
-// of each node without storing them, so the pair form's results are those of separate faces and
-// update passes bit for bit.
+// when the solver is created.  The second kernel forms the dissipative face fluxes, sums them and
+// the flux differences into the RHS of each node, and updates the state.
 //
-// The nodal and viscous passes are launched on 3-D grids (64 x 4 threads per block along i and j,
-// one block row per k), so no pass divides a flat index.
+// The adjoint of a pair-form solver regenerates the primitives, spectral radii and sensors of a
+// stage with the nodal and sensor passes below, on 3-D launches (64 x 4 threads per block along i
+// and j, one block row per k), so that no pass divides a flat index.
 #include "jz_dfconsts.cuh"
 
 namespace jz {
@@ -33,253 +33,399 @@ __device__ __forceinline__ bool advanced(const Dims& d, int i, int j) {
 }
 
 
-// A: every padded node.  Primitives, Sutherland mu, spectral radii and their anisotropic
-// scaling; the double-float copy of Q for the viscous and faces passes; at stage 1 also the CFL
-// rate of Q^n (block max, one atomic per block).
-// Five blocks per SM (48 registers): the pass is bound by DRAM traffic and gains from the extra
-// warps (11.3 against 12.8 ms per launch on 1000 x 400 x 500); the viscous pass loses from the same.
+// Every padded node: primitives, Sutherland mu, spectral radii and their anisotropic scaling, the
+// double-float copy of Q.  Five blocks per SM (48 registers): the pass is bound by DRAM traffic and
+// gains from the extra warps (11.3 against 12.8 ms per launch on 1000 x 400 x 500).
 __global__ void __launch_bounds__(BX* BY, 5) k_nodal_df(Dims d, ConstsDF c, DFMetrics M, Work64 w, State q,
-                                                     QDF qdf, double* rate_max) {
+                                                     QDF qdf) {
   int i, j, k;
-  double rate = 0.0;
-  if (node3(-kG, -kG, -kG, d.ni + 2 * kG, d.nj + 2 * kG, i, j, k)) {
-    const long long p = pidx(d, i, j, k);
-    const dfl rho = df_of(q.q[0][p]), m1 = df_of(q.q[1][p]), m2 = df_of(q.q[2][p]), m3 = df_of(q.q[3][p]),
-              e = df_of(q.q[4][p]);
-    st(qdf.q[0], p, rho); st(qdf.q[1], p, m1); st(qdf.q[2], p, m2); st(qdf.q[3], p, m3); st(qdf.q[4], p, e);
-    const dfl ir = df_rcp(rho);
-    const dfl u = df_mul(m1, ir), v = df_mul(m2, ir), ww = df_mul(m3, ir);
-    const dfl ke = df_fma(m3, ww, df_fma(m2, v, df_mul(m1, u)));            // rho |u|^2
-    const dfl pr = df_sub(df_mul(e, c.gm1), df_mul(ke, c.gm1_half));    // (gamma-1)(e - rho|u|^2/2)
-    const dfl T = df_mul(df_mul(pr, c.gamma), ir);
-    const dfl a = df_sqrt(T);
-    // Sutherland, eq. (sutherland), with T_inf = 1
-    const dfl mu = df_mul(df_mul(c.mu_sut, df_mul(T, a)), df_rcp(df_add(T, c.S_hat)));
-    st(w.u, p, u); st(w.v, p, v); st(w.w, p, ww); st(w.T, p, T); st(w.p, p, pr); st(w.mu, p, mu);
-    dfl lam[3];
-    for (int dir = 0; dir < 3; ++dir) {
-      const dfl sx = df_load(M.S[3 * dir], p), sy = df_load(M.S[3 * dir + 1], p), sz = df_load(M.S[3 * dir + 2], p);
-      const dfl U = df_fma(sz, ww, df_fma(sy, v, df_mul(sx, u)));
-      lam[dir] = df_fma(a, df_load(M.Smag[dir], p), df_abs(U));
-    }
-    if (rate_max && i >= 0 && i < d.ni && j >= 0 && j < d.nj && k >= 0 && k < d.nk && advanced(d, i, j))
-      rate = df_to_f64(df_mul(df_add(df_add(lam[0], lam[1]), lam[2]), df_load(M.invV, p)));
-    dfl Lam[3];
-    aniso_df(c, lam, Lam);
-    st(w.Lam[0], p, Lam[0]); st(w.Lam[1], p, Lam[1]); st(w.Lam[2], p, Lam[2]);
+  if (!node3(-kG, -kG, -kG, d.ni + 2 * kG, d.nj + 2 * kG, i, j, k)) return;
+  const long long p = pidx(d, i, j, k);
+  const dfl rho = df_of(q.q[0][p]), m1 = df_of(q.q[1][p]), m2 = df_of(q.q[2][p]), m3 = df_of(q.q[3][p]),
+            e = df_of(q.q[4][p]);
+  st(qdf.q[0], p, rho); st(qdf.q[1], p, m1); st(qdf.q[2], p, m2); st(qdf.q[3], p, m3); st(qdf.q[4], p, e);
+  const dfl ir = df_rcp(rho);
+  const dfl u = df_mul(m1, ir), v = df_mul(m2, ir), ww = df_mul(m3, ir);
+  const dfl ke = df_fma(m3, ww, df_fma(m2, v, df_mul(m1, u)));            // rho |u|^2
+  const dfl pr = df_sub(df_mul(e, c.gm1), df_mul(ke, c.gm1_half));    // (gamma-1)(e - rho|u|^2/2)
+  const dfl T = df_mul(df_mul(pr, c.gamma), ir);
+  const dfl a = df_sqrt(T);
+  // Sutherland, eq. (sutherland), with T_inf = 1
+  const dfl mu = df_mul(df_mul(c.mu_sut, df_mul(T, a)), df_rcp(df_add(T, c.S_hat)));
+  st(w.u, p, u); st(w.v, p, v); st(w.w, p, ww); st(w.T, p, T); st(w.p, p, pr); st(w.mu, p, mu);
+  dfl lam[3];
+  for (int dir = 0; dir < 3; ++dir) {
+    const dfl sx = df_load(M.S[3 * dir], p), sy = df_load(M.S[3 * dir + 1], p), sz = df_load(M.S[3 * dir + 2], p);
+    const dfl U = df_fma(sz, ww, df_fma(sy, v, df_mul(sx, u)));
+    lam[dir] = df_fma(a, df_load(M.Smag[dir], p), df_abs(U));
   }
-  if (rate_max) {
-    // block max -> one atomic per block (non-negative doubles order like their bits)
-    __shared__ double redm[BX * BY / 32];
-    const int tid = threadIdx.y * BX + threadIdx.x;
-    for (int o = 16; o > 0; o >>= 1) rate = fmax(rate, __shfl_xor_sync(0xffffffffu, rate, o));
-    if ((tid & 31) == 0) redm[tid >> 5] = rate;
-    __syncthreads();
-    if (tid < 32) {
-      double x = tid < BX * BY / 32 ? redm[tid] : 0.0;
-      for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
-      if (tid == 0 && x > 0.0)
-        atomicMax(reinterpret_cast<unsigned long long*>(rate_max), (unsigned long long)__double_as_longlong(x));
-    }
-  }
+  dfl Lam[3];
+  aniso_df(c, lam, Lam);
+  st(w.Lam[0], p, Lam[0]); st(w.Lam[1], p, Lam[1]); st(w.Lam[2], p, Lam[2]);
 }
 
-// B: nodes within one layer of the real region (the nodes whose fluxes the faces read).
-// Gradients by the chain rule, strain rate, Smagorinsky eddy viscosity, stresses and heat flux;
-// the transformed flux H^dir = E^dir - S^dir_j F_j, inviscid part E^dir from the nodal
-// primitives and the pair copy of Q, written once; pressure sensors.  Forming E^dir here rather
-// than in the nodal pass saves its store there and the load of it here (160 bytes per node):
-// 17.1 against 20.2 + 3.2 ms per launch on 1000 x 400 x 500.  Four blocks per SM (64 registers,
-// a few spilled): 17.1 against 17.6 ms at 80 registers.  Unnormalized sums and products inside
-// each chain (normalized before stores, roots and reciprocals; jz_df.cuh): 15.2 against 17.1 ms,
-// ~20% fewer FP32 operations; residuals move by up to 5e-13 of their norm, states by 2e-15.
-__global__ void __launch_bounds__(BX* BY, 4) k_viscous_df(Dims d, ConstsDF c, DFMetrics M, Work64 w, QDF qdf) {
+// Pressure sensors |p+ - 2p + p-| / (p+ + 2p + p-) of the nodes within one layer of the real region,
+// from the nodal pass's pressures: with that pass, what the adjoint's transposed kernels read of a
+// stage (they form the gradients and stresses again themselves).
+__device__ __forceinline__ dfl sensor_df(dfl pc, dfl pm, dfl pp) {
+  const dfl pc2 = df_scale(pc, 2.f), sum = df_add_l(pp, pm);
+  return df_n(df_mul_l(df_abs(df_n(df_sub_l(sum, pc2))), df_rcp(df_n(df_add_l(sum, pc2)))));
+}
+__global__ void __launch_bounds__(BX* BY) k_sensor_df(Dims d, Work64 w) {
   int i, j, k;
   if (!node3(-1, -1, -1, d.ni + 2, d.nj + 2, i, j, k)) return;
   const long long p = pidx(d, i, j, k);
   const long long s[3] = {1, d.sj, d.sk};
-  const double* f[4] = {w.u, w.v, w.w, w.T};
-  dfl S[3][3];
-  for (int dir = 0; dir < 3; ++dir)
-    for (int cc = 0; cc < 3; ++cc) S[dir][cc] = df_load(M.S[3 * dir + cc], p);
-  const dfl iV = df_load(M.invV, p);
-  // G[n][j] = sum_dir S^dir_j (f_n[+dir] - f_n[-dir]); the gradient is h G with h = 1/(2V)
-  dfl G[4][3];
-  for (int n = 0; n < 4; ++n) {
-    dfl dd[3];
-    for (int dir = 0; dir < 3; ++dir) dd[dir] = df_sub_l(ld(f[n], p + s[dir]), ld(f[n], p - s[dir]));
-    for (int jj = 0; jj < 3; ++jj)
-      G[n][jj] = df_n(df_fma_l(S[2][jj], dd[2], df_fma_l(S[1][jj], dd[1], df_mul_l(S[0][jj], dd[0]))));
-  }
-  const dfl h = df_scale(iV, 0.5f);
-  // |S| = h sqrt(2 sum G_ii^2 + sum_{i<j} A_ij^2), A_ij = G_ij + G_ji
-  const dfl A12 = df_add_l(G[0][1], G[1][0]), A13 = df_add_l(G[0][2], G[2][0]), A23 = df_add_l(G[1][2], G[2][1]);
-  const dfl Gd = df_add_l(df_add_l(G[0][0], G[1][1]), G[2][2]);
-  const dfl DG = df_fma_l(G[2][2], G[2][2], df_fma_l(G[1][1], G[1][1], df_mul_l(G[0][0], G[0][0])));
-  const dfl AA = df_fma_l(A23, A23, df_fma_l(A13, A13, df_mul_l(A12, A12)));
-  const dfl mu = ld(w.mu, p);
-  const dfl csd = df_mul_l(df_load(M.Delta, p), c.C_s);
-  // Smagorinsky eddy viscosity rho (C_s Delta)^2 |S|
-  const dfl rho = ld(qdf.q[0], p);
-  const dfl mu_sgs = df_n(df_mul_l(df_mul_l(rho, df_mul_l(csd, csd)),
-                                   df_mul_l(h, df_sqrt(df_n(df_add_l(df_scale(DG, 2.f), AA))))));
-  const dfl mt = df_add_l(mu, mu_sgs);
-  const dfl mV = df_mul_l(mt, iV), mh = df_mul_l(mt, h);
-  const dfl kh = df_mul_l(df_add_l(df_mul_l(mu, c.k_lam), df_mul_l(mu_sgs, c.k_sgs)), h);   // k_eff h
-  const dfl d3 = df_mul_l(Gd, c.third);                                                       // Gd / 3
-  const dfl t11 = df_mul_l(mV, df_sub_l(G[0][0], d3)), t22 = df_mul_l(mV, df_sub_l(G[1][1], d3)),
-            t33 = df_mul_l(mV, df_sub_l(G[2][2], d3));
-  const dfl t12 = df_mul_l(mh, A12), t13 = df_mul_l(mh, A13), t23 = df_mul_l(mh, A23);
-  const dfl tau[3][3] = {{t11, t12, t13}, {t12, t22, t23}, {t13, t23, t33}};
-  const dfl vel[3] = {ld(w.u, p), ld(w.v, p), ld(w.w, p)};
-  dfl F[3][4];
-  for (int jj = 0; jj < 3; ++jj) {
-    F[jj][0] = tau[0][jj];
-    F[jj][1] = tau[1][jj];
-    F[jj][2] = tau[2][jj];
-    F[jj][3] = df_fma_l(kh, G[3][jj],
-                        df_fma_l(vel[2], tau[2][jj], df_fma_l(vel[1], tau[1][jj], df_mul_l(vel[0], tau[0][jj]))));
-  }
   const dfl pc = ld(w.p, p);
-  const dfl mq[3] = {ld(qdf.q[1], p), ld(qdf.q[2], p), ld(qdf.q[3], p)};
-  const dfl h0 = df_add_l(ld(qdf.q[4], p), pc);                                               // e + p
-  for (int dir = 0; dir < 3; ++dir) {
-    const dfl U = df_fma_l(S[dir][2], vel[2], df_fma_l(S[dir][1], vel[1], df_mul_l(S[dir][0], vel[0])));
-    dfl E[5];
-    E[0] = df_mul_l(rho, U);
-    for (int jj = 0; jj < 3; ++jj) E[jj + 1] = df_fma_l(mq[jj], U, df_mul_l(pc, S[dir][jj]));
-    E[4] = df_mul_l(h0, U);
-    st(w.H[dir][0], p, df_n(E[0]));
-    for (int m = 0; m < 4; ++m) {
-      const dfl sf = df_fma_l(S[dir][2], F[2][m], df_fma_l(S[dir][1], F[1][m], df_mul_l(S[dir][0], F[0][m])));
-      st(w.H[dir][m + 1], p, df_n(df_sub_l(E[m + 1], sf)));
+#pragma unroll
+  for (int dir = 0; dir < 3; ++dir) st(w.nu[dir], p, sensor_df(pc, ld(w.p, p - s[dir]), ld(w.p, p + s[dir])));
+}
+
+// Fluxes of a stage: primitives, Sutherland's viscosity, spectral radii and their anisotropic scaling,
+// gradients by the chain rule, Smagorinsky eddy viscosity, stresses and heat flux, the transformed
+// fluxes H^dir = E^dir - S^dir_j F_j and the pressure sensors of the nodes within one layer of the
+// real region, and the pair copy of Q on every padded node; at stage 1 also the CFL rate of Q^n
+// (block max, one atomic per block).  A block of 32 x VY threads marches along k; per plane every
+// thread forms u, v, w, T, p of its node into shared memory (three planes in turn), and the inner
+// 30 x (VY - 2) nodes form their fluxes from the neighbours there, so the primitives and the
+// viscosity never reach HBM (360 bytes per node against 568 for a nodal and a viscous pass).
+// The momentum and energy fluxes are contracted as H_m = m_m U + S_j P_jm, P = p I - tau, and
+// H_e = e U + S_j (u_m P_jm - k dT/dx_j).
+// FP32 issue bounds it: 10.7 ms per launch on 512 x 512 x 360 (the two passes before: 11.4); 32 x 10
+// at three blocks per SM as 32 x 16 at two, 11.3 for 32 x 8 at four, 10.9 for 32 x 12 at two with 80
+// registers.  Split arrivals instead of a barrier per plane (warps drifting by a plane): 12.0.
+constexpr int VX = 32, VY = 10;
+
+// Element of a field at a 32-bit byte offset (every field of a pair solver is below 4 GB: its 632
+// bytes per padded node reach the GPU's memory first): the address is a uniform base plus one
+// register, and the offsets of a node's neighbours are shared by all fields.
+__device__ __forceinline__ dfl ldo(const float2* f, unsigned off) {
+  const float2 v = *reinterpret_cast<const float2*>(reinterpret_cast<const char*>(f) + off);
+  return df_make(v.x, v.y);
+}
+__device__ __forceinline__ double ldo(const double* f, unsigned off) {
+  return *reinterpret_cast<const double*>(reinterpret_cast<const char*>(f) + off);
+}
+__device__ __forceinline__ void sto(float2* f, unsigned off, dfl v) {
+  *reinterpret_cast<float2*>(reinterpret_cast<char*>(f) + off) = make_float2(v.hi, v.lo);
+}
+inline cudaError_t offsets_fit(const Dims& d) { return d.Np < (1LL << 29) ? cudaSuccess : cudaErrorInvalidValue; }
+
+struct StageArgs {
+  Dims d;
+  ConstsDF c;
+  const float2* S[9];
+  const float2* Smag[3];
+  const float2* invV;
+  const float2* Delta;
+  const double* q[5];
+  float2* qdf[5];
+  float2* H[3][5];
+  float2* nu[3];
+  float2* Lam[3];
+  double* rate_max;      // non-null: also the CFL rate of q over the advanced nodes
+  int kchunk;
+  unsigned nbx;
+};
+
+struct PlaneDF {
+  float2 f[5][VY][VX];   // u, v, w, T, p
+};
+__device__ __forceinline__ dfl sm(const PlaneDF& P, int n, int y, int x) {
+  const float2 t = P.f[n][y][x];
+  return df_make(t.x, t.y);
+}
+
+__global__ void __launch_bounds__(VX* VY, 3) k_flux_df(const __grid_constant__ StageArgs A) {
+  __shared__ PlaneDF pl[3];
+  const Dims& d = A.d;
+  const ConstsDF& c = A.c;
+  const int x = threadIdx.x, y = threadIdx.y;
+  const unsigned by = blockIdx.x / A.nbx, bx = blockIdx.x - by * A.nbx;
+  const int i = (int)bx * (VX - 2) - 2 + x, j = (int)by * (VY - 2) - 2 + y;
+  const int k0 = (int)blockIdx.y * A.kchunk - 1, k1 = min(k0 + A.kchunk, d.nk + 1);   // planes [k0, k1) of -1 .. nk
+  const bool inside = i <= d.ni + 1 && j <= d.nj + 1;      // i, j >= -2 by construction
+  const bool inner = x > 0 && x < VX - 1 && y > 0 && y < VY - 1;
+  const bool out = inner && i <= d.ni && j <= d.nj;        // a node this block forms the fluxes of
+  // nodes whose pair copy of Q this thread writes: the block's own and the outermost ghosts
+  const bool own = inside && (x > 0 || i == -2) && (x < VX - 1 || i == d.ni + 1) && (y > 0 || j == -2) &&
+                   (y < VY - 1 || j == d.nj + 1);
+  double rate = 0.0;
+  int s0 = 0, s1 = 1, s2 = 2;                               // slots of planes k - 1, k, k + 1
+  const unsigned sk = (unsigned)d.sk * 8u;                  // bytes
+  unsigned p = (unsigned)pidx(d, i, j, k0 - 2) * 8u;        // (k0 - 2 may lie below the array: only p + sk is read then)
+  for (int k = k0 - 2; k < k1; ++k, p += sk) {
+    dfl S[3][3] = {}, iV = {}, Delta = {};
+    if (out && k >= k0) {
+      // the metrics of plane k, requested before the primitives of plane k + 1 that hide their latency
+#pragma unroll
+      for (int dir = 0; dir < 3; ++dir)
+#pragma unroll
+        for (int cc = 0; cc < 3; ++cc) S[dir][cc] = ldo(A.S[3 * dir + cc], p);
+      iV = ldo(A.invV, p);
+      Delta = ldo(A.Delta, p);
+    }
+    if (inside) {
+      // primitives of plane k + 1
+      const unsigned pn = p + sk;
+      const dfl rho = df_of(ldo(A.q[0], pn)), m1 = df_of(ldo(A.q[1], pn)), m2 = df_of(ldo(A.q[2], pn)), m3 = df_of(ldo(A.q[3], pn)),
+                e = df_of(ldo(A.q[4], pn));
+      if (own && ((k + 1 >= k0 && k + 1 < k1) || k + 1 == -2 || k + 1 == d.nk + 1)) {
+        sto(A.qdf[0], pn, rho);
+        sto(A.qdf[1], pn, m1);
+        sto(A.qdf[2], pn, m2);
+        sto(A.qdf[3], pn, m3);
+        sto(A.qdf[4], pn, e);
+      }
+      const dfl ir = df_rcp(rho);
+      const dfl u = df_mul(m1, ir), v = df_mul(m2, ir), w = df_mul(m3, ir);
+      const dfl ke = df_fma(m3, w, df_fma(m2, v, df_mul(m1, u)));         // rho |u|^2
+      const dfl pr = df_sub(df_mul(e, c.gm1), df_mul(ke, c.gm1_half));    // (gamma-1)(e - rho|u|^2/2)
+      const dfl T = df_mul(df_mul(pr, c.gamma), ir);
+      PlaneDF& P = pl[s2];
+      P.f[0][y][x] = make_float2(u.hi, u.lo);
+      P.f[1][y][x] = make_float2(v.hi, v.lo);
+      P.f[2][y][x] = make_float2(w.hi, w.lo);
+      P.f[3][y][x] = make_float2(T.hi, T.lo);
+      P.f[4][y][x] = make_float2(pr.hi, pr.lo);
+    }
+    if (k >= k0) {
+      // plane k + 1 before its neighbours read it one iteration later, and every thread done with
+      // plane k - 1 as neighbours; planes k - 1 and k + 1 are read by their own column only
+      __syncthreads();
+      if (out) {
+        const PlaneDF &Pm = pl[s0], &P0 = pl[s1], &Pp = pl[s2];
+        // G[n][j] = sum_dir S^dir_j (f_n[+dir] - f_n[-dir]); the gradient is h G with h = 1/(2V)
+        dfl G[4][3];
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+          const dfl dx = df_sub_l(sm(P0, n, y, x + 1), sm(P0, n, y, x - 1));
+          const dfl dy = df_sub_l(sm(P0, n, y + 1, x), sm(P0, n, y - 1, x));
+          const dfl dz = df_sub_l(sm(Pp, n, y, x), sm(Pm, n, y, x));
+#pragma unroll
+          for (int jj = 0; jj < 3; ++jj)
+            G[n][jj] = df_n(df_fma_l(S[2][jj], dz, df_fma_l(S[1][jj], dy, df_mul_l(S[0][jj], dx))));
+        }
+        const dfl h = df_scale(iV, 0.5f);
+        // |S| = h sqrt(2 sum G_ii^2 + sum_{i<j} A_ij^2), A_ij = G_ij + G_ji
+        const dfl A12 = df_add_l(G[0][1], G[1][0]), A13 = df_add_l(G[0][2], G[2][0]), A23 = df_add_l(G[1][2], G[2][1]);
+        const dfl Gd = df_add_l(df_add_l(G[0][0], G[1][1]), G[2][2]);
+        const dfl DG = df_fma_l(G[2][2], G[2][2], df_fma_l(G[1][1], G[1][1], df_mul_l(G[0][0], G[0][0])));
+        const dfl AA = df_fma_l(A23, A23, df_fma_l(A13, A13, df_mul_l(A12, A12)));
+        const dfl csd = df_mul_l(Delta, c.C_s);
+        const dfl rho = ldo(A.qdf[0], p);
+        // Smagorinsky eddy viscosity rho (C_s Delta)^2 |S|
+        const dfl mu_sgs = df_n(df_mul_l(df_mul_l(rho, df_mul_l(csd, csd)),
+                                         df_mul_l(h, df_sqrt(df_n(df_add_l(df_scale(DG, 2.f), AA))))));
+        // Sutherland, eq. (sutherland), with T_inf = 1
+        const dfl T = sm(P0, 3, y, x), a = df_sqrt(T);
+        const dfl mu = df_mul(df_mul(c.mu_sut, df_mul(T, a)), df_rcp(df_add(T, c.S_hat)));
+        const dfl mt = df_add_l(mu, mu_sgs);
+        const dfl mV = df_mul_l(mt, iV), mh = df_neg(df_mul_l(mt, h));
+        const dfl kh = df_neg(df_mul_l(df_add_l(df_mul_l(mu, c.k_lam), df_mul_l(mu_sgs, c.k_sgs)), h));  // -k_eff h
+        const dfl d3 = df_mul_l(Gd, c.third);                                                              // Gd / 3
+        // P_jm = p delta_jm - tau_jm (symmetric)
+        const dfl pc = sm(P0, 4, y, x);
+        const dfl P11 = df_fma_l(mV, df_sub_l(d3, G[0][0]), pc), P22 = df_fma_l(mV, df_sub_l(d3, G[1][1]), pc),
+                  P33 = df_fma_l(mV, df_sub_l(d3, G[2][2]), pc);
+        const dfl P12 = df_mul_l(mh, A12), P13 = df_mul_l(mh, A13), P23 = df_mul_l(mh, A23);
+        const dfl u = sm(P0, 0, y, x), v = sm(P0, 1, y, x), w = sm(P0, 2, y, x);
+        // X_j = sum_m u_m P_jm - k dT/dx_j: what remains of the energy flux beside e U
+        const dfl X1 = df_fma_l(kh, G[3][0], df_fma_l(w, P13, df_fma_l(v, P12, df_mul_l(u, P11))));
+        const dfl X2 = df_fma_l(kh, G[3][1], df_fma_l(w, P23, df_fma_l(v, P22, df_mul_l(u, P12))));
+        const dfl X3 = df_fma_l(kh, G[3][2], df_fma_l(w, P33, df_fma_l(v, P23, df_mul_l(u, P13))));
+        const dfl m1 = ldo(A.qdf[1], p), m2 = ldo(A.qdf[2], p), m3 = ldo(A.qdf[3], p),
+                  e = ldo(A.qdf[4], p);
+        dfl lam[3];
+#pragma unroll
+        for (int dir = 0; dir < 3; ++dir) {
+          const dfl sx = S[dir][0], sy = S[dir][1], sz = S[dir][2];
+          const dfl U = df_n(df_fma_l(sz, w, df_fma_l(sy, v, df_mul_l(sx, u))));
+          lam[dir] = df_fma(a, ldo(A.Smag[dir], p), df_abs(U));
+          // H^dir = [rho U, m_i U + S_j P_ji, e U + S_j X_j]
+          auto flux = [&](dfl q, dfl f1, dfl f2, dfl f3) {
+            return df_n(df_fma_l(q, U, df_fma_l(sz, f3, df_fma_l(sy, f2, df_mul_l(sx, f1)))));
+          };
+          sto(A.H[dir][0], p, df_mul(rho, U));
+          sto(A.H[dir][1], p, flux(m1, P11, P12, P13));
+          sto(A.H[dir][2], p, flux(m2, P12, P22, P23));
+          sto(A.H[dir][3], p, flux(m3, P13, P23, P33));
+          sto(A.H[dir][4], p, flux(e, X1, X2, X3));
+        }
+        if (A.rate_max && i >= 0 && i < d.ni && j >= 0 && j < d.nj && k >= 0 && k < d.nk && advanced(d, i, j))
+          rate = fmax(rate, df_to_f64(df_mul(df_add(df_add(lam[0], lam[1]), lam[2]), iV)));
+        dfl L[3];
+        aniso_df(c, lam, L);
+        sto(A.nu[0], p, sensor_df(pc, sm(P0, 4, y, x - 1), sm(P0, 4, y, x + 1)));
+        sto(A.nu[1], p, sensor_df(pc, sm(P0, 4, y - 1, x), sm(P0, 4, y + 1, x)));
+        sto(A.nu[2], p, sensor_df(pc, sm(Pm, 4, y, x), sm(Pp, 4, y, x)));
+#pragma unroll
+        for (int dir = 0; dir < 3; ++dir) sto(A.Lam[dir], p, L[dir]);
+      }
+    }
+    const int t = s0;
+    s0 = s1;
+    s1 = s2;
+    s2 = t;
+  }
+  if (A.rate_max) {
+    // block max -> one atomic per block (non-negative doubles order like their bits)
+    __shared__ double redm[VY];
+    for (int o = 16; o > 0; o >>= 1) rate = fmax(rate, __shfl_xor_sync(0xffffffffu, rate, o));
+    if (x == 0) redm[y] = rate;
+    __syncthreads();
+    if (x == 0 && y == 0) {
+      for (int n = 1; n < VY; ++n) rate = fmax(rate, redm[n]);
+      if (rate > 0.0)
+        atomicMax(reinterpret_cast<unsigned long long*>(A.rate_max), (unsigned long long)__double_as_longlong(rate));
     }
   }
-  // pressure sensor along each direction: |p+ - 2p + p-| / (p+ + 2p + p-)
-  const dfl pc2 = df_scale(pc, 2.f);
-  for (int dir = 0; dir < 3; ++dir) {
-    const dfl sum = df_add_l(ld(w.p, p + s[dir]), ld(w.p, p - s[dir]));
-    st(w.nu[dir], p, df_n(df_mul_l(df_abs(df_n(df_sub_l(sum, pc2))), df_rcp(df_n(df_add_l(sum, pc2))))));
-  }
 }
 
-// C + D: Turkel-Vatsa dissipation combined with the face sum of H into the doubled total face
-// flux G = H_n + H_(n+1) - 2 d_(n+1/2), and, in the same kernel, 2 V RHS = sum_dir (G(p) -
-// G(p - s_dir)) in double-float with the stage combination Q^n - alpha dt RHS in FP64 (mode 0)
-// or the RHS itself (mode 1).  The face fluxes never leave the SM: a block of 32 x 16 threads
-// marches along k over a chunk of planes; the thread at (i, j) forms the three faces i + 1/2,
-// j + 1/2, k + 1/2 of its node, takes the face i - 1/2 from the lane below it (shuffle), the face
-// j - 1/2 from the row below it (shared memory) and the face k - 1/2 from its own previous plane.
-// Column 0 and row 0 of the block are that halo (31 x 15 nodes updated per block and plane).
-constexpr int FX = 32, FY = 16;
-
-template <int DIR>
-__device__ __forceinline__ void face_df(const ConstsDF& c, const Work64& w, const QDF& qdf, long long p,
-                                        long long sd, dfl G[5]) {
-  const dfl eps2 = df_mul(df_max(ld(w.nu[DIR], p), ld(w.nu[DIR], p + sd)), c.kappa2);
+// C + D: Turkel-Vatsa dissipation, RHS and stage update in one kernel.  Per node and variable
+//   2 V RHS = sum_dir [ H(n+1) - H(n-1) - (D(n+1/2) - D(n-1/2)) ],  D = 2 d,
+// in double-float, then Q^n - alpha dt RHS in FP64 (mode 0) or the RHS itself (mode 1).  Neither the
+// faces nor their sums leave the SM.
+// 2 d = a32 d1 - b2 e3 on the face between p and p + sd, with d1 and e3 the differences of Q over the
+// face (one and three spacings): Ls = 2 L_f, b2 = Ls eps4, a32 = 3 b2 + Ls eps2, as (a32, b2).
+__device__ __forceinline__ float4 face_coef(const ConstsDF& c, const float2* nu, const float2* Lam, long long p,
+                                            long long sd) {
+  const dfl eps2 = df_mul(df_max(df_load(nu, p), df_load(nu, p + sd)), c.kappa2);
   const dfl k4 = df_sub(c.kappa4, eps2);
   const dfl eps4 = df_gt0(k4) ? k4 : df_make(0.f, 0.f);
-  // 2 d = a32 d1 - b2 e3 with Ls = 2 L_f, b2 = Ls eps4, a32 = 3 b2 + Ls eps2
-  const dfl Ls = df_add(ld(w.Lam[DIR], p), ld(w.Lam[DIR], p + sd));
+  const dfl Ls = df_add(df_load(Lam, p), df_load(Lam, p + sd));
   const dfl b2 = df_mul(Ls, eps4);
   const dfl a32 = df_fma(Ls, eps2, df_mul_f(b2, 3.f));
-#pragma unroll
-  for (int m = 0; m < 5; ++m) {
-    const double* Q = qdf.q[m];
-    const dfl d1 = df_sub(ld(Q, p + sd), ld(Q, p));
-    const dfl e3 = df_sub(ld(Q, p + 2 * sd), ld(Q, p - sd));
-    const dfl hs = df_add(ld(w.H[DIR][m], p), ld(w.H[DIR][m], p + sd));
-    G[m] = df_sub(df_fma(b2, e3, hs), df_mul(a32, d1));
-  }
+  return make_float4(a32.hi, a32.lo, b2.hi, b2.lo);
+}
+__device__ __forceinline__ dfl face_diss(float4 k, dfl qm, dfl q0, dfl q1, dfl q2) {
+  const dfl d1 = df_sub_l(q1, q0), e3 = df_sub_l(q2, qm);
+  return df_fma_l(df_make(-k.z, -k.w), e3, df_mul_l(df_make(k.x, k.y), d1));
 }
 
-// Blocks of 32 x 16 threads, two per SM (64 registers): 19.2 ms per launch on 1000 x 400 x 500,
-// against 19.9 for 32 x 8 at five per SM (48 registers, a few spilled), 20.0 for 32 x 12 at
-// three, 21.3 for 32 x 4 at ten, 22.7 for 32 x 16 at three (40 registers) and 31.9 for 32 x 8
-// at three when the face fluxes of the three directions were held in registers across the
-// barrier (80 registers).
+struct FacesArgs {
+  Dims d;
+  ConstsDF c;
+  const float2* nu[3];
+  const float2* Lam[3];
+  const float2* H[3][5];
+  const float2* Q[5];
+  const double* invV;
+  const double* qin[5];
+  const double* qn[5];
+  double* qout[5];
+  const Scalars* sc;
+  double alpha;
+  double* rhs;           // [5][N] (mode 1)
+  double* res_sum;       // non-null: add the sum of RHS_rho^2
+  int kchunk;
+  unsigned nbx;          // blocks along i (blockIdx.x = by * nbx + bx)
+};
+
+
+// A block of 32 x FY nodes marches along k over a chunk of planes; a thread forms the faces i + 1/2,
+// j + 1/2, k + 1/2 of its node for the five variables, takes i - 1/2 from the lane below it (shuffle),
+// j - 1/2 from the row below it (shared memory) and k - 1/2 from its own previous plane.  Column 0
+// and row 0 of the block are that halo (31 x (FY - 1) nodes updated per plane).  The fluxes enter as
+// the difference of their neighbours, not as face sums: fewer operations and a smaller rounding
+// error (H(n+1) - H(n-1) cancels before anything is rounded), and the dissipation, small beside the
+// flux, is summed in unnormalized pairs.
+// Issue-bound (62%) with load latency behind it: 8.1 ms per launch on 512 x 512 x 360 with 32 x 8
+// blocks at four per SM (8.3 for 32 x 16 at two, 8.1 for 32 x 12 at three), 9.2 before with face sums.
+// One variable per thread (five times the threads, coefficients through shared memory) took 16.9.
+constexpr int FX = 32, FY = 8;
 template <int MODE>
-__global__ void __launch_bounds__(FX* FY, 2) k_faces_update_df(Dims d, ConstsDF c, Work64 w, QDF qdf, const double* invV,
-                                                            State qin, State qn, State qout, const Scalars* sc,
-                                                            double alpha, int want_res, double* rhs_flat,
-                                                            double* res_sum, int kchunk) {
+__global__ void __launch_bounds__(FX* FY, 4) k_faces_update_df(const __grid_constant__ FacesArgs A) {
+  const Dims& d = A.d;
+  const ConstsDF& c = A.c;
   __shared__ float2 g1s[2][5][FY][FX];   // faces j + 1/2 of the plane, two planes in turn
   __shared__ float2 g2s[5][FY][FX];      // each thread's face k - 1/2
   const int x = threadIdx.x, y = threadIdx.y;
-  const int i = (int)blockIdx.x * (FX - 1) - 1 + x, j = (int)blockIdx.y * (FY - 1) - 1 + y;
-  const int k0 = (int)blockIdx.z * kchunk, k1 = min(k0 + kchunk, d.nk);
-  const bool inside = i <= d.ni - 1 && j <= d.nj - 1;     // i, j >= -1 by construction
-  const bool need0 = inside && y > 0;                      // face i + 1/2: halo column and body
-  const bool need1 = inside && x > 0;                      // face j + 1/2: halo row and body
-  const bool node = need0 && x > 0;                        // a real node this block updates
+  const unsigned by = blockIdx.x / A.nbx, bx = blockIdx.x - by * A.nbx;
+  const int i = (int)bx * (FX - 1) - 1 + x, j = (int)by * (FY - 1) - 1 + y;
+  const int k0 = (int)blockIdx.y * A.kchunk, k1 = min(k0 + A.kchunk, d.nk);
+  const bool inside = i <= d.ni - 1 && j <= d.nj - 1;
+  const bool need0 = inside && y > 0, need1 = inside && x > 0, node = need0 && x > 0;
   const bool adv = advanced(d, i, j);
-  const long long N = (long long)d.ni * d.nj * d.nk;
+  const long long sj = d.sj, sk = d.sk;
+  long long p = pidx(d, i, j, k0);
   double r2 = 0.0;
   if (node) {
-    dfl g[5];
-    face_df<2>(c, w, qdf, pidx(d, i, j, k0 - 1), d.sk, g);
-#pragma unroll
-    for (int m = 0; m < 5; ++m) g2s[m][y][x] = make_float2(g[m].hi, g[m].lo);
-  }
-  for (int k = k0; k < k1; ++k) {
-    const long long p = pidx(d, i, j, k);
-    const int b = k & 1;
-    dfl g[5] = {}, a[5], cc[5];
-    if (need0) face_df<0>(c, w, qdf, p, 1, g);
+    const float4 cf = face_coef(c, A.nu[2], A.Lam[2], p - sk, sk);
 #pragma unroll
     for (int m = 0; m < 5; ++m) {
-      const float lh = __shfl_up_sync(0xffffffffu, g[m].hi, 1), ll = __shfl_up_sync(0xffffffffu, g[m].lo, 1);
-      a[m] = df_sub(g[m], df_make(lh, ll));
+      const float2* Q = A.Q[m] + p;
+      const dfl D = face_diss(cf, df_load(Q, -2 * sk), df_load(Q, -sk), df_load(Q, 0), df_load(Q, sk));
+      g2s[m][y][x] = make_float2(D.hi, D.lo);
+    }
+  }
+  for (int k = k0; k < k1; ++k, p += sk) {
+    const int b = k & 1;
+    dfl R[5];
+    float4 cf = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (need0) cf = face_coef(c, A.nu[0], A.Lam[0], p, 1);
+#pragma unroll
+    for (int m = 0; m < 5; ++m) {
+      dfl D = df_make(0.f, 0.f);
+      if (need0) {
+        const float2* Q = A.Q[m] + p;
+        D = face_diss(cf, df_load(Q, -1), df_load(Q, 0), df_load(Q, 1), df_load(Q, 2 * 1));
+      }
+      const float mh = __shfl_up_sync(0xffffffffu, D.hi, 1), ml = __shfl_up_sync(0xffffffffu, D.lo, 1);
+      R[m] = df_sub_l(df_make(mh, ml), D);
     }
     if (need1) {
-      face_df<1>(c, w, qdf, p, d.sj, g);
-#pragma unroll
-      for (int m = 0; m < 5; ++m) g1s[b][m][y][x] = make_float2(g[m].hi, g[m].lo);
-    }
-    if (node) {
-      face_df<2>(c, w, qdf, p, d.sk, g);
+      cf = face_coef(c, A.nu[1], A.Lam[1], p, sj);
 #pragma unroll
       for (int m = 0; m < 5; ++m) {
+        const float2* Q = A.Q[m] + p;
+        const dfl D = face_diss(cf, df_load(Q, -sj), df_load(Q, 0), df_load(Q, sj), df_load(Q, 2 * sj));
+        g1s[b][m][y][x] = make_float2(D.hi, D.lo);
+      }
+    }
+    if (node) {
+      cf = face_coef(c, A.nu[2], A.Lam[2], p, sk);
+#pragma unroll
+      for (int m = 0; m < 5; ++m) {
+        const float2* Q = A.Q[m] + p;
+        const dfl D = face_diss(cf, df_load(Q, -sk), df_load(Q, 0), df_load(Q, sk), df_load(Q, 2 * sk));
         const float2 o = g2s[m][y][x];
-        cc[m] = df_sub(g[m], df_make(o.x, o.y));
-        g2s[m][y][x] = make_float2(g[m].hi, g[m].lo);
+        g2s[m][y][x] = make_float2(D.hi, D.lo);
+        const float2 *H0 = A.H[0][m] + p, *H1 = A.H[1][m] + p, *H2 = A.H[2][m] + p;
+        R[m] = df_add_l(R[m], df_sub_l(df_load(H0, 1), df_load(H0, -1)));
+        R[m] = df_add_l(R[m], df_sub_l(df_sub_l(df_load(H2, sk), df_load(H2, -sk)), df_sub_l(D, df_make(o.x, o.y))));
+        R[m] = df_add_l(R[m], df_sub_l(df_load(H1, sj), df_load(H1, -sj)));
       }
     }
     __syncthreads();
     if (node) {
-      double R[5];
+      const double hV = 0.5 * A.invV[p];
 #pragma unroll
       for (int m = 0; m < 5; ++m) {
         const float2 t1 = g1s[b][m][y][x], t0 = g1s[b][m][y - 1][x];
-        const dfl bb = df_sub(df_make(t1.x, t1.y), df_make(t0.x, t0.y));
-        R[m] = df_to_f64(df_add(df_add(a[m], bb), cc[m]));
-      }
-      const double hV = 0.5 * invV[p];
-      if (MODE == 0) {
-        const double adtV = alpha * sc->dt * hV;
-#pragma unroll
-        for (int m = 0; m < 5; ++m) qout.q[m][p] = adv ? fma(-adtV, R[m], qn.q[m][p]) : qin.q[m][p];
-      } else {
-        const long long t = ((long long)k * d.nj + j) * d.ni + i;
-#pragma unroll
-        for (int m = 0; m < 5; ++m) rhs_flat[m * N + t] = adv ? R[m] * hV : 0.0;
-      }
-      if (adv) {
-        const double r0 = R[0] * hV;
-        r2 += r0 * r0;
+        const double R64 = df_to_f64(df_sub_l(R[m], df_sub_l(df_make(t1.x, t1.y), df_make(t0.x, t0.y))));
+        if (MODE == 0) {
+          A.qout[m][p] = adv ? fma(-(A.alpha * A.sc->dt * hV), R64, A.qn[m][p]) : A.qin[m][p];
+        } else {
+          const long long N = (long long)d.ni * d.nj * d.nk, t = ((long long)k * d.nj + j) * d.ni + i;
+          A.rhs[m * N + t] = adv ? R64 * hV : 0.0;
+        }
+        if (adv && m == 0) {
+          const double r0 = R64 * hV;
+          r2 += r0 * r0;
+        }
       }
     }
   }
-  if (want_res) {
-    __shared__ double red[FX * FY / 32];
-    const int tid = y * FX + x;
+  if (A.res_sum) {
+    __shared__ double red[FY];
     for (int o = 16; o > 0; o >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, o);
-    if ((tid & 31) == 0) red[tid >> 5] = r2;
+    if (x == 0) red[y] = r2;
     __syncthreads();
-    if (tid < 32) {
-      double v = tid < FX * FY / 32 ? red[tid] : 0.0;
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (tid == 0) atomicAdd(res_sum, v);
+    if (x == 0 && y == 0) {
+      double t = 0.0;
+      for (int q = 0; q < FY; ++q) t += red[q];
+      atomicAdd(A.res_sum, t);
     }
   }
 }
@@ -305,39 +451,88 @@ cudaError_t metrics_to_df(const Dims& d, const GridDev& g, const DFMetrics& M, c
 }
 
 cudaError_t nodal_df(const Dims& d, const Consts& c, const DFMetrics& M, const Work64& w, const QDF& qdf,
-                     const State& qin, cudaStream_t st, double* rate_max) {
+                     const State& qin, cudaStream_t st) {
   k_nodal_df<<<grid3(d.ni + 2 * kG, d.nj + 2 * kG, d.nk + 2 * kG), dim3(BX, BY), 0, st>>>(d, make_cdf(c), M, w, qin,
-                                                                                          qdf, rate_max);
+                                                                                          qdf);
   return cudaGetLastError();
 }
 
-cudaError_t viscous_df(const Dims& d, const Consts& c, const DFMetrics& M, const Work64& w, const QDF& qdf,
-                       cudaStream_t st) {
-  k_viscous_df<<<grid3(d.ni + 2, d.nj + 2, d.nk + 2), dim3(BX, BY), 0, st>>>(d, make_cdf(c), M, w, qdf);
+cudaError_t sensor_df_pass(const Dims& d, const Work64& w, cudaStream_t st) {
+  k_sensor_df<<<grid3(d.ni + 2, d.nj + 2, d.nk + 2), dim3(BX, BY), 0, st>>>(d, w);
   return cudaGetLastError();
 }
 
-// planes per block of the faces-update kernel: enough blocks for several waves, one extra
-// k-face per chunk
-int faces_kchunk(const Dims& d) {
-  const long long tiles = (long long)((d.ni + FX - 2) / (FX - 1)) * ((d.nj + FY - 2) / (FY - 1));
+// Planes per block of a marching kernel with `tiles` tiles in the plane: 32 where the grid gives two
+// waves of blocks over the SMs all the same, less on small grids (down to one plane, with its priming
+// work again for every block): a 32 x 24 x 16 grid has 16 tiles, and its faces kernel takes 8 us in
+// blocks of one plane against 25 in blocks of four.
+int march_kchunk(long long tiles, int planes) {
   int kc = 32;
-  while (kc > 4 && tiles * ((d.nk + kc - 1) / kc) < 8 * 152) kc /= 2;
+  while (kc > 1 && tiles * ((planes + kc - 1) / kc) < 8 * 152) kc /= 2;
   return kc;
+}
+
+cudaError_t flux_df(const Dims& d, const Consts& c, const DFMetrics& M, const Work64& w, const QDF& qdf,
+                    const State& qin, Scalars* sc, cudaStream_t st, int want_rate) {
+  const cudaError_t fit = offsets_fit(d);
+  if (fit != cudaSuccess) return fit;
+  StageArgs A;
+  A.d = d;
+  A.c = make_cdf(c);
+  auto f2 = [](double* x) { return reinterpret_cast<float2*>(x); };
+  for (int n = 0; n < 9; ++n) A.S[n] = M.S[n];
+  for (int dir = 0; dir < 3; ++dir) {
+    A.Smag[dir] = M.Smag[dir];
+    A.nu[dir] = f2(w.nu[dir]);
+    A.Lam[dir] = f2(w.Lam[dir]);
+    for (int m = 0; m < 5; ++m) A.H[dir][m] = f2(w.H[dir][m]);
+  }
+  A.invV = M.invV;
+  A.Delta = M.Delta;
+  for (int m = 0; m < 5; ++m) {
+    A.q[m] = qin.q[m];
+    A.qdf[m] = f2(qdf.q[m]);
+  }
+  A.rate_max = want_rate ? &sc->rate_max : nullptr;
+  A.nbx = (d.ni + VX - 1) / (VX - 2);
+  const long long tiles = (long long)A.nbx * ((d.nj + VY - 1) / (VY - 2));
+  A.kchunk = march_kchunk(tiles, d.nk + 2);
+  const dim3 gr((unsigned)tiles, (d.nk + 1 + A.kchunk) / A.kchunk);
+  k_flux_df<<<gr, dim3(VX, VY), 0, st>>>(A);
+  return cudaGetLastError();
 }
 
 cudaError_t faces_update_df(const Dims& d, const Consts& c, const GridDev& g, const Work64& w, const QDF& qdf,
                             const State& qin, const State& qn, const State& qout, const Scalars* sc, double alpha,
                             int want_res, double* rhs_flat, cudaStream_t st) {
-  double* res_sum = const_cast<double*>(&sc->res_sum);
-  const int kc = faces_kchunk(d);
-  const dim3 gr((d.ni + FX - 2) / (FX - 1), (d.nj + FY - 2) / (FY - 1), (d.nk + kc - 1) / kc), blk(FX, FY);
-  const ConstsDF cdf = make_cdf(c);
+  FacesArgs A;
+  A.d = d;
+  A.c = make_cdf(c);
+  auto f2 = [](const double* x) { return reinterpret_cast<const float2*>(x); };
+  for (int dir = 0; dir < 3; ++dir) {
+    A.nu[dir] = f2(w.nu[dir]);
+    A.Lam[dir] = f2(w.Lam[dir]);
+    for (int m = 0; m < 5; ++m) A.H[dir][m] = f2(w.H[dir][m]);
+  }
+  for (int m = 0; m < 5; ++m) {
+    A.Q[m] = f2(qdf.q[m]);
+    A.qin[m] = qin.q[m];
+    A.qn[m] = qn.q[m];
+    A.qout[m] = qout.q[m];
+  }
+  A.invV = g.invV;
+  A.sc = sc;
+  A.alpha = alpha;
+  A.rhs = rhs_flat;
+  A.res_sum = want_res && !rhs_flat ? const_cast<double*>(&sc->res_sum) : nullptr;
+  A.nbx = (d.ni + FX - 2) / (FX - 1);
+  const long long tiles = (long long)A.nbx * ((d.nj + FY - 2) / (FY - 1));
+  A.kchunk = march_kchunk(tiles, d.nk);
+  const dim3 gr((unsigned)tiles, (d.nk + A.kchunk - 1) / A.kchunk), blk(FX, FY);
   if (rhs_flat)
-    k_faces_update_df<1><<<gr, blk, 0, st>>>(d, cdf, w, qdf, g.invV, qin, qn, qout, sc, alpha, 0, rhs_flat, res_sum, kc);
+    k_faces_update_df<1><<<gr, blk, 0, st>>>(A);
   else
-    k_faces_update_df<0><<<gr, blk, 0, st>>>(d, cdf, w, qdf, g.invV, qin, qn, qout, sc, alpha, want_res, nullptr,
-                                             res_sum, kc);
+    k_faces_update_df<0><<<gr, blk, 0, st>>>(A);
   return cudaGetLastError();
 }
 
