@@ -274,7 +274,7 @@ int run_step(jz_solver* s) {
   // spectral radii anyway; the FP32-flux form's stage 5 left it behind, and after
   // jz_set_state it is reduced here.
   if (s->fp32 || !cfl) {
-    if (cfl && !s->rate_ready) JZ_RUN(JZ_PROF_REDUCE, jz::cfl_rate(d, s->c, g, s->qn, s->sc, s->st));
+    if (cfl && !s->rate_ready) JZ_RUN(JZ_PROF_REDUCE, jz::cfl_rate(d, s->c, g, s->Mf, s->qn, s->sc, s->st));
     JZ_RUN(JZ_PROF_REDUCE, jz::set_dt(s->c, s->in, s->sc, s->st));
   }
   jz::State in = s->qn;
@@ -939,7 +939,7 @@ int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ck
     ~RestoreTime() { jz::set_time(s->in, s->sc, t, dt, s->st); }
   } restore_time{s, h0.t, h0.dt};
   // frozen time step and start time
-  if (s->c.dt_fixed <= 0.0) JZ_RUN(JZ_PROF_REDUCE, jz::cfl_rate(d, s->c, g, s->qn, s->sc, s->st));
+  if (s->c.dt_fixed <= 0.0) JZ_RUN(JZ_PROF_REDUCE, jz::cfl_rate(d, s->c, g, s->Mf, s->qn, s->sc, s->st));
   JZ_RUN(JZ_PROF_REDUCE, jz::set_dt(s->c, s->in, s->sc, s->st));
   jz::Scalars h;
   JZ_CK(cudaMemcpyAsync(&h, s->sc, sizeof h, cudaMemcpyDeviceToHost, s->st));

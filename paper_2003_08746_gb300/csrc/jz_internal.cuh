@@ -368,8 +368,10 @@ cudaError_t jet_shell(const Dims& d, const Consts& c, const GridDev& g, const In
 cudaError_t build_inflow(const Dims& d, const Consts& c, const GridDev& g, const jz_params& p,
                          Inflow& in, cudaStream_t st);
 // reductions
-cudaError_t cfl_rate(const Dims& d, const Consts& c, const GridDev& g, const State& q,
-                     Scalars* sc, cudaStream_t st);
+// largest CFL rate of q over the advanced nodes into sc->rate_max (the caller has left it 0); Mf: FP32 metric
+// records, null: none at hand
+cudaError_t cfl_rate(const Dims& d, const Consts& c, const GridDev& g, const float* Mf, const State& q, Scalars* sc,
+                     cudaStream_t st);
 // time step of the current step from the reduced rate (or dt_fixed), and the forcing's temporal factors
 cudaError_t set_dt(const Consts& c, const Inflow& in, Scalars* sc, cudaStream_t st);
 // t and dt given (the adjoint's sweeps), and the forcing's temporal factors

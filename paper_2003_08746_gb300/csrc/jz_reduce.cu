@@ -1,6 +1,8 @@
 // Reductions: the CFL time step, the conservation totals and the state
 // checks (minimum density and pressure, non-finite values).
-#include "jz_internal.cuh"
+#include <algorithm>
+
+#include "jz_shadow.cuh"
 
 namespace jz {
 namespace {
@@ -8,31 +10,94 @@ namespace {
 constexpr int kTPB = 256;
 constexpr int kStatBlocks = 1216;   // 8 x 152 SMs; fixed so the sums are reproducible
 
-__device__ __forceinline__ double warp_max(double x) {
-  for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
-  return x;
+// CFL rate of the advanced nodes, max of (lambda_xi + lambda_eta + lambda_zeta) / V in FP64, found
+// with FP32 bounds.  The exact rate costs ~45 FP64 instructions, an SM retires one per warp in 16
+// clocks, and a plain sweep is bound by that (26 ms on 1024 x 512 x 360 where its bytes take 2.5).
+// So every node gets an interval [lo, hi] around its rate in FP32, and only nodes whose interval
+// reaches the largest rate known so far (this warp's lower bounds, its exact values, what other
+// warps have published) are evaluated exactly: the node of the maximum is always among them, so the
+// result is the plain sweep's bit for bit.  Values outside FP32's range and NaN count as reaching it.
+struct RateBounds {
+  float lo, hi;
+};
+__device__ __forceinline__ RateBounds rate_bounds(const ConstsF& c, const double q[5], const float S[9], float iV) {
+  unsigned big = 0;
+#pragma unroll
+  for (int m = 0; m < 5; ++m) big = max(big, (unsigned)__double2hiint(q[m]) & 0x7FFFFFFFu);
+  if (big >= 0x45E00000u) return RateBounds{0.f, __int_as_float(0x7F800000)};   // some |q| >= 2^95
+  // each quantity below is within kRel of its FP64 value relative to the magnitudes summed in it:
+  // truncated conversions (2^-23 each), a few roundings, one hardware reciprocal and square root
+  constexpr float kRel = 4e-6f;
+  const float ir = f_rcp(f64_to_f32(q[0]));
+  const float m1 = f64_to_f32(q[1]), m2 = f64_to_f32(q[2]), m3 = f64_to_f32(q[3]), e = f64_to_f32(q[4]);
+  const float u = m1 * ir, v = m2 * ir, w = m3 * ir;
+  const float ke = 0.5f * (m1 * u + m2 * v + m3 * w);
+  const float p = c.gm1 * (e - ke), dp = kRel * c.gm1 * (fabsf(e) + fabsf(ke));
+  const float a_hi = sqrtf(c.gamma * fabsf(ir) * (fabsf(p) + dp)), a_lo = ir > 0.f ? sqrtf(fmaxf(c.gamma * ir * (p - dp), 0.f)) : 0.f;
+  float lo = 0.f, hi = 0.f;
+#pragma unroll
+  for (int dir = 0; dir < 3; ++dir) {
+    const float sx = S[3 * dir], sy = S[3 * dir + 1], sz = S[3 * dir + 2];
+    const float U = fabsf(sx * u + sy * v + sz * w), dU = kRel * (fabsf(sx * u) + fabsf(sy * v) + fabsf(sz * w));
+    const float smag = sqrtf(sx * sx + sy * sy + sz * sz);
+    lo += fmaxf(U - dU, 0.f) + a_lo * smag;
+    hi += U + dU + a_hi * smag;
+  }
+  const float inf = __int_as_float(0x7F800000), top = hi * iV * (1.f + kRel);
+  // (sums so small that flushed conversions could matter decide nothing)
+  if (!(hi > 1e-25f) || !(top > 1e-25f)) return RateBounds{0.f, inf};
+  return RateBounds{lo * iV * (1.f - kRel), top};
 }
 
-// max over the advanced nodes of (lambda_xi + lambda_eta + lambda_zeta)/V.
-__global__ void k_cfl_rate(Dims d, GridDev g, State q, Consts c, Scalars* sc) {
-  Box b{0, 0, 0, d.ni, d.nj, d.nk};
-  int i, j, k;
-  double rate = 0.0;
-  if (box_coord(b, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k) &&
-      (d.topo != JZ_TOPO_JET || (i >= 1 && i <= d.ni - 2 && j >= 1 && j <= d.nj - 2))) {
-    const long long p = pidx(d, i, j, k);
-    rate = node_rate(g, c, p, q.q[0][p], q.q[1][p], q.q[2][p], q.q[3][p], q.q[4][p]);
-  }
-  __shared__ double red[kTPB / 32];
-  rate = warp_max(rate);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = rate;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double x = threadIdx.x < kTPB / 32 ? red[threadIdx.x] : 0.0;
-    x = warp_max(x);
-    // non-negative doubles order like their bit patterns
-    if (threadIdx.x == 0 && x > 0.0)
-      atomicMax(reinterpret_cast<unsigned long long*>(&sc->rate_max), (unsigned long long)__double_as_longlong(x));
+// Mf: FP32 metric records where the solver or the grid has them, else the FP64 metrics.
+__global__ void __launch_bounds__(kTPB) k_cfl_rate(Dims d, GridDev g, State q, Consts c, ConstsF cf, const float* Mf,
+                                                   Scalars* sc) {
+  const volatile double* known = &sc->rate_max;
+  const unsigned lane = threadIdx.x & 31;
+  const long long warps = (long long)gridDim.x * (kTPB / 32);
+  // rows of the advanced nodes in turns of 32 along i
+  const bool jet = d.topo == JZ_TOPO_JET;
+  const int i0 = jet ? 1 : 0, i1 = jet ? d.ni - 1 : d.ni, j0 = jet ? 1 : 0, ej = jet ? d.nj - 2 : d.nj;
+  const int segs = (i1 - i0 + 31) / 32;
+  const long long n = (long long)segs * ej * d.nk;
+  double rate = 0.0, cut = 0.0;            // this thread's largest exact rate; no node below cut is the maximum
+  for (long long t = blockIdx.x * (long long)(kTPB / 32) + threadIdx.x / 32; t < n; t += warps) {
+    const int sgm = (int)(t % segs);
+    const long long r = t / segs;
+    const int i = i0 + sgm * 32 + (int)lane, j = j0 + (int)(r % ej), k = (int)(r / ej);
+    const bool in = i < i1;
+    const long long p = pidx(d, in ? i : i0, j, k);
+    double v[5];
+    float S[9], iV;
+#pragma unroll
+    for (int m = 0; m < 5; ++m) v[m] = q.q[m][p];
+    if (Mf) {
+      const float4* M = reinterpret_cast<const float4*>(Mf + p * kMF);
+      const float4 a = __ldg(M), b = __ldg(M + 1), e = __ldg(M + 2);
+      S[0] = a.x; S[1] = a.y; S[2] = a.z; S[3] = a.w; S[4] = b.x; S[5] = b.y; S[6] = b.z; S[7] = b.w;
+      S[8] = e.x;
+      iV = e.z;
+    } else {
+#pragma unroll
+      for (int m = 0; m < 9; ++m) S[m] = f64_to_f32(g.S[m][p]);
+      const double w = g.invV[p];
+      iV = w < 1e30 ? f64_to_f32(w) : __int_as_float(0x7F800000);
+    }
+    cut = fmax(cut, *known);
+    const RateBounds b = rate_bounds(cf, v, S, iV);
+    float best = in && b.lo > 0.f ? b.lo : 0.f;            // (a NaN bound claims nothing)
+    for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
+    // compared in FP32: the cut rounded down
+    const float cutf = fmaxf(best, __double2float_rd(cut));
+    if (in && !(b.hi < cutf)) rate = fmax(rate, node_rate(g, c, p, v[0], v[1], v[2], v[3], v[4]));
+    double x = rate;
+    if (__any_sync(0xffffffffu, x > cut)) {
+      for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
+      // non-negative doubles order like their bit patterns
+      if (lane == 0)
+        atomicMax(reinterpret_cast<unsigned long long*>(&sc->rate_max), (unsigned long long)__double_as_longlong(x));
+      cut = x;
+    }
   }
 }
 
@@ -147,10 +212,12 @@ __global__ void k_stats_final(const double* part, int nblk, Scalars* sc) {
 
 int stat_partial_count() { return kStatBlocks; }
 
-cudaError_t cfl_rate(const Dims& d, const Consts& c, const GridDev& g, const State& q, Scalars* sc,
+cudaError_t cfl_rate(const Dims& d, const Consts& c, const GridDev& g, const float* Mf, const State& q, Scalars* sc,
                      cudaStream_t st) {
-  const long long nr = (long long)d.ni * d.nj * d.nk;
-  k_cfl_rate<<<blocks_for(nr, kTPB), kTPB, 0, st>>>(d, g, q, c, sc);
+  // eight blocks per SM keep the sweep going; fewer where the grid has fewer turns of 32 nodes
+  const long long turns = (long long)((d.ni + 31) / 32) * d.nj * d.nk;
+  const unsigned blocks = (unsigned)std::min<long long>(8 * 152, (turns + kTPB / 32 - 1) / (kTPB / 32));
+  k_cfl_rate<<<blocks, kTPB, 0, st>>>(d, g, q, c, make_constsf(c), Mf, sc);
   return cudaGetLastError();
 }
 
