@@ -13,6 +13,8 @@
 // first argument on ties, |x| and sqrt(x) at 0 have derivative 0, cbrt'(0)
 // is 0, and the supersonic/subsonic and inflow/outflow switches take the
 // branch the forward pass took.
+#include <cmath>
+
 #include "jz_adjgather.cuh"
 
 namespace jz {
@@ -291,41 +293,9 @@ __global__ void __launch_bounds__(kTPBN, 3) k_adj_nodal(Dims d, Consts c, GridDe
 }
 
 // ---- transposed ghost map: ghost adjoint added onto its source node --------------
-__device__ __forceinline__ bool ghost_coord_adj(const Dims& d, long long t, int& i, int& j, int& k) {
-  const long long ei = d.ni + 2 * kG, ej = d.nj + 2 * kG;
-  const long long nA = 4 * ei * ej, nB = 4 * ei * d.nk, nC = 4LL * d.nj * d.nk;
-  if (t < nA) {
-    i = (int)(t % ei) - kG;
-    const long long r = t / ei;
-    j = (int)(r % ej) - kG;
-    const int s = (int)(r / ej);
-    k = s < 2 ? s - 2 : d.nk + s - 2;
-    return true;
-  }
-  t -= nA;
-  if (t < nB) {
-    i = (int)(t % ei) - kG;
-    const long long r = t / ei;
-    const int s = (int)(r % 4);
-    k = (int)(r / 4);
-    j = s < 2 ? s - 2 : d.nj + s - 2;
-    return true;
-  }
-  t -= nB;
-  if (t < nC) {
-    const int s = (int)(t % 4);
-    const long long r = t / 4;
-    j = (int)(r % d.nj);
-    k = (int)(r / d.nj);
-    i = s < 2 ? s - 2 : d.ni + s - 2;
-    return true;
-  }
-  return false;
-}
-
 __global__ void k_adj_ghost(Dims d, Adj64 a) {
   int i, j, k;
-  if (!ghost_coord_adj(d, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
+  if (!ghost_coord(d, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
   int si, sj, sk;
   ghost_source(d, i, j, k, si, sj, sk);
   const long long p = pidx(d, i, j, k), q = pidx(d, si, sj, sk);
@@ -372,28 +342,35 @@ __global__ void k_adj_axis(Dims d, Adj64 a) {
   }
 }
 
-__global__ void k_adj_inout(Dims d, Consts c, Inflow in, State q, Adj64 a, double ts) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+// Entrance and exit, blocks of kTPBS threads (a few thousand nodes of long FP64 chains: small blocks
+// spread them over the SMs).  The forcing's temporal factors come from the host, which knows the
+// stage time: sn, and am = amplitude times factor.
+constexpr int kTPBS = 64;
+struct ForcingAt {
+  double sn[kNF], am[kNF];
+};
+__global__ void __launch_bounds__(kTPBS) k_adj_inout(Dims d, Consts c, Inflow in, State q, Adj64 a,
+                                                     const __grid_constant__ ForcingAt F, unsigned ent_blocks) {
   const int nj1 = d.nj - 1;
   const long long nface = (long long)nj1 * d.nk;
   const long long plane = (long long)d.nk * d.nj;
+  const bool exit_plane = blockIdx.x >= ent_blocks;
+  const long long tt = (blockIdx.x - (exit_plane ? ent_blocks : 0u)) * (long long)kTPBS + threadIdx.x;
   double g0 = 0.0;                 // d J / d u_target (times U_j) at this entrance node
-  long long tab = 0;
-  // temporal factors sin(omega_f t + psi_mf), uniform over the entrance: once per block
-  __shared__ double sn[kNF];
-  if (threadIdx.x < kNF) sn[threadIdx.x] = sin(in.omega[threadIdx.x % JZ_N_FREQ] * ts + in.psi[threadIdx.x]);
-  __syncthreads();
-  if (t < 2 * nface) {
-    const bool exit_plane = t >= nface;
-    const long long tt = exit_plane ? t - nface : t;
+  __shared__ double Gs[kNF][kTPBS + 1];        // this block's forcing shapes
+  if (tt < nface) {
     const int j = 1 + (int)(tt % nj1), k = (int)(tt / nj1);
     if (!exit_plane) {
       const long long pb = pidx(d, 0, j, k), p1 = pidx(d, 1, j, k);
-      tab = (long long)k * d.nj + j;
-      double f = 0.0;
-      for (int mf = 0; mf < kNF; ++mf)
-        f = f + in.amp[mf] * in.Gf[mf * plane + tab] * sn[mf];
-      const double ut = in.u0[tab] + c.jet_mach * f;
+      const long long tab = (long long)k * d.nj + j;
+      double f[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+      for (int mf = 0; mf < kNF; ++mf) {
+        const double G = __ldg(in.Gf + mf * plane + tab);
+        Gs[mf][threadIdx.x] = G;
+        f[mf & 3] = fma(F.am[mf], G, f[mf & 3]);
+      }
+      const double ut = in.u0[tab] + c.jet_mach * ((f[0] + f[1]) + (f[2] + f[3]));
       double Q1[5];
       load5(q, p1, Q1);
       double lb[5];
@@ -451,21 +428,26 @@ __global__ void k_adj_inout(Dims d, Consts c, Inflow in, State q, Adj64 a, doubl
       }
     }
   }
-  // dJ/dA_mf = sum over the entrance of g0 G_mf sin(omega_f t + psi_mf): block sums,
-  // one atomic per parameter per block
-  __shared__ double red[kNF][kTPB / 32];
-  for (int f = 0; f < kNF; ++f) {
-    double x = g0 != 0.0 ? g0 * in.Gf[f * plane + tab] * sn[f] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if ((threadIdx.x & 31) == 0) red[f][threadIdx.x >> 5] = x;
-  }
+  if (exit_plane) return;
+  // dJ/dA_mf = sum over the entrance of g0 G_mf sin(omega_f t + psi_mf): one parameter per lane, the
+  // block's nodes in halves, one atomic per parameter per block
+  __shared__ double gs[kTPBS], half[kNF];
+  gs[threadIdx.x] = g0;
+  if (tt >= nface)
+    for (int mf = 0; mf < kNF; ++mf) Gs[mf][threadIdx.x] = 0.0;
   __syncthreads();
-  if (threadIdx.x < kNF) {
-    double x = 0.0;
-    for (int w = 0; w < kTPB / 32; ++w) x += red[threadIdx.x][w];
-    if (x != 0.0) atomicAdd(&a.abar[threadIdx.x], x);
+  const int mf = threadIdx.x % kNF, n0 = threadIdx.x / kNF * (kTPBS / 2);
+  double x = 0.0;
+#pragma unroll 8
+  for (int n = n0; n < n0 + kTPBS / 2; ++n) x = fma(gs[n], Gs[mf][n], x);
+  if (n0) half[mf] = x;
+  __syncthreads();
+  if (n0 == 0) {
+    x = (x + half[mf]) * F.sn[mf];
+    if (x != 0.0) atomicAdd(&a.abar[mf], x);
   }
 }
+static_assert(kTPBS == 2 * kNF, "two halves of the block's nodes, one lane per parameter");
 
 __global__ void k_adj_farfield(Dims d, Consts c, GridDev g, State q, Adj64 a) {
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -603,9 +585,7 @@ cudaError_t adj_stage(const Dims& d, const Consts& c, const GridDev& g, const Wo
     k_adj_visc<<<blocks_for(n1, kTPB), kTPB, 0, st>>>(d, c, g, w, q, a);
     k_adj_nodal<<<blocks_for(n0, kTPBN), kTPBN, 0, st>>>(d, c, g, w, q, a);
   }
-  const long long ei = d.ni + 2 * kG, ej = d.nj + 2 * kG;
-  const long long ng = 4 * ei * ej + 4 * ei * d.nk + 4LL * d.nj * d.nk;
-  k_adj_ghost<<<blocks_for(ng, kTPB), kTPB, 0, st>>>(d, a);
+  k_adj_ghost<<<blocks_for(ghost_count(d), kTPB), kTPB, 0, st>>>(d, a);
   return cudaGetLastError();
 }
 
@@ -619,10 +599,15 @@ cudaError_t adj_bcs(const Dims& d, const Consts& c, const GridDev& g, const Infl
                     const Adj64& a, double ts, cudaStream_t st) {
   if (d.topo != JZ_TOPO_JET) return cudaSuccess;
   k_adj_axis<<<d.ni, 128, 0, st>>>(d, a);
-  const long long nio = 2LL * (d.nj - 1) * d.nk;
-  k_adj_inout<<<blocks_for(nio, kTPB), kTPB, 0, st>>>(d, c, in, q, a, ts);
+  ForcingAt F;
+  for (int mf = 0; mf < kNF; ++mf) {
+    F.sn[mf] = std::sin(in.omega[mf % JZ_N_FREQ] * ts + in.psi[mf]);
+    F.am[mf] = in.amp[mf] * F.sn[mf];
+  }
+  const unsigned nio = blocks_for((long long)(d.nj - 1) * d.nk, kTPBS);
+  k_adj_inout<<<2 * nio, kTPBS, 0, st>>>(d, c, in, q, a, F, nio);
   const long long nf = (long long)(d.ni - 2) * d.nk;
-  k_adj_farfield<<<blocks_for(nf, kTPB), kTPB, 0, st>>>(d, c, g, q, a);
+  k_adj_farfield<<<blocks_for(nf, kTPBS), kTPBS, 0, st>>>(d, c, g, q, a);
   return cudaGetLastError();
 }
 

@@ -13,19 +13,30 @@
 namespace jz {
 namespace {
 
+// Node of a launch over the box [o, o + ei) x [o, o + ej) x [o, o + ek): the plane's nodes in a row
+// along blockIdx.x (no lanes lost to tiles that overhang it: 64 x 4 tiles cost the 130 nodes along i
+// of a 128-node grid a third), k along blockIdx.y; one 32-bit division.
+__device__ __forceinline__ bool plane_node(int o, int ei, int ej, int& i, int& j, int& k) {
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x, y = t / (unsigned)ei;
+  i = o + (int)(t - y * (unsigned)ei);
+  j = o + (int)y;
+  k = o + (int)blockIdx.y;
+  return y < (unsigned)ej;
+}
+dim3 plane_grid(int ei, int ej, int ek, int tpb) { return dim3(blocks_for((long long)ei * ej, tpb), ek); }
+
 // Adjoint of the stage update: Qn_bar += lambda (FP64), acc = -alpha dt lambda / V as a pair, on
 // advanced real nodes (acc stays 0 elsewhere).
 __global__ void k_adj_update_df(Dims d, GridDev g, Adj64 a, double adt) {
-  Box b{0, 0, 0, d.ni, d.nj, d.nk};
   int i, j, k;
-  if (!box_coord(b, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
+  if (!plane_node(0, d.ni, d.nj, i, j, k)) return;
   const long long p = pidx(d, i, j, k);
   const bool adv = d.topo != JZ_TOPO_JET || (i >= 1 && i <= d.ni - 2 && j >= 1 && j <= d.nj - 2);
-  const double iV = g.invV[p];
+  const double f = -adt * g.invV[p];
   for (int m = 0; m < 5; ++m) {
     const double l = a.lam[m][p];
     if (adv) a.qnbar[m][p] += l;
-    st(a.acc[m], p, adv ? df_of(-adt * l * iV) : df_from(0.f));
+    st(a.acc[m], p, adv ? df_of(f * l) : df_from(0.f));
   }
 }
 
@@ -33,9 +44,8 @@ __global__ void k_adj_update_df(Dims d, GridDev g, Adj64 a, double adt) {
 // pair-form solver, in double-float arithmetic on the pair copies of Q, the sensors and Lambda.
 // Faces n + 1/2, n in [-1, n_dir - 1].
 __global__ void k_adj_faces_df(Dims d, ConstsDF c, Work64 w, QDF qdf, Adj64 a) {
-  Box b{-1, -1, -1, d.ni + 1, d.nj + 1, d.nk + 1};
   int i, j, k;
-  if (!box_coord(b, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
+  if (!plane_node(-1, d.ni + 1, d.nj + 1, i, j, k)) return;
   const long long p = pidx(d, i, j, k);
   const long long s[3] = {1, d.sj, d.sk};
   for (int dir = 0; dir < 3; ++dir) {
@@ -75,9 +85,8 @@ __global__ void k_adj_faces_df(Dims d, ConstsDF c, Work64 w, QDF qdf, Adj64 a) {
 // passes regenerated (u, v, w, T, p, mu, the pair copies of Q and of the metrics).  Nodes within
 // one layer of the real region.
 __global__ void k_adj_visc_df(Dims d, ConstsDF c, DFMetrics M, Work64 w, QDF qdf, Adj64 a) {
-  Box b{-1, -1, -1, d.ni + 2, d.nj + 2, d.nk + 2};
   int i, j, k;
-  if (!box_coord(b, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
+  if (!plane_node(-1, d.ni + 2, d.nj + 2, i, j, k)) return;
   const long long p = pidx(d, i, j, k);
   const long long s[3] = {1, d.sj, d.sk};
   // adjoint of H^dir (components 1..4 carry the viscous flux)
@@ -180,39 +189,50 @@ __global__ void k_adj_visc_df(Dims d, ConstsDF c, DFMetrics M, Work64 w, QDF qdf
 }
 
 
-// A pair adjoint array at (i, j, k) + offset along dir, 0 outside the padded box.
-__device__ __forceinline__ dfl nbp(const Dims& d, const double* f, int i, int j, int k, int dir, int off) {
-  int ii = i, jj = j, kk = k;
-  if (dir == 0) ii += off; else if (dir == 1) jj += off; else kk += off;
-  return in_box(d, ii, jj, kk) ? ld(f, pidx(d, ii, jj, kk)) : df_from(0.f);
-}
+// Neighbours of a padded node in the pair adjoint arrays, `off` nodes along `dir` (up to two), read by
+// offset.  Beyond the padded box along i or j the offset lands in the next or previous row or plane,
+// on elements that no pass writes: acc is 0 off the real nodes, the face arrays off [-1, n), the
+// viscous and sensor arrays off [-1, n], and what an offset of one or two can reach from the outer
+// ghosts lies outside those ranges at the other end (padding columns, i = -2, -1 or i >= n, and the
+// same for j); before the first and after the last row of an array stand rows of zeros
+// (jz_adjoint_step).  Along k the neighbour is tested.
+struct PaddedNode {
+  int p, sj, sk;
+  bool m2, m1, p1, p2;             // k - 2, k - 1, k + 1, k + 2 lie in the padded box
+  __device__ __forceinline__ PaddedNode(const Dims& d, int i, int j, int k)
+      : p((int)pidx(d, i, j, k)), sj((int)d.sj), sk((int)d.sk), m2(k >= 0), m1(k >= -1), p1(k <= d.nk), p2(k < d.nk) {}
+  __device__ __forceinline__ dfl operator()(const double* f, int dir, int off) const {
+    if (dir < 2 || off == 0) return ld(f, p + off * (dir == 0 ? 1 : sj));
+    const bool in = off == -2 ? m2 : (off == -1 ? m1 : (off == 1 ? p1 : p2));
+    return in ? ld(f, p + off * sk) : df_from(0.f);
+  }
+};
 
 // The gathers of the transposed nodal pass (as nodal_gathers, jz_adjgather.cuh) on the pair
 // adjoint arrays, summed in double-float.
 struct NodalGathersDF {
   dfl fb[4], pb, Eb[3][5], Lamb[3], qb[5], mub;
 };
-__device__ __forceinline__ void nodal_gathers_df(const Dims& d, const Adj64& a, int i, int j, int k,
-                                                 NodalGathersDF& G) {
+__device__ __forceinline__ void nodal_gathers_df(const Adj64& a, const PaddedNode& nb, NodalGathersDF& G) {
 #pragma unroll
   for (int n = 0; n < 4; ++n) {
-    dfl v = n < 3 ? nbp(d, a.ubd[n], i, j, k, 0, 0) : df_from(0.f);
+    dfl v = n < 3 ? nb(a.ubd[n], 0, 0) : df_from(0.f);
 #pragma unroll
     for (int dir = 0; dir < 3; ++dir)
-      v = df_add(v, df_scale(df_sub(nbp(d, a.G[n][dir], i, j, k, dir, -1), nbp(d, a.G[n][dir], i, j, k, dir, 1)), 0.5f));
+      v = df_add(v, df_scale(df_sub(nb(a.G[n][dir], dir, -1), nb(a.G[n][dir], dir, 1)), 0.5f));
     G.fb[n] = v;
   }
   G.pb = df_from(0.f);
 #pragma unroll
   for (int dir = 0; dir < 3; ++dir)
-    G.pb = df_add(G.pb, df_add(df_add(nbp(d, a.c0[dir], i, j, k, 0, 0), nbp(d, a.cpm[dir], i, j, k, dir, -1)),
-                               nbp(d, a.cpm[dir], i, j, k, dir, 1)));
+    G.pb = df_add(G.pb, df_add(df_add(nb(a.c0[dir], 0, 0), nb(a.cpm[dir], dir, -1)),
+                               nb(a.cpm[dir], dir, 1)));
 #pragma unroll
   for (int dir = 0; dir < 3; ++dir) {
 #pragma unroll
     for (int m = 0; m < 5; ++m)
-      G.Eb[dir][m] = df_scale(df_sub(nbp(d, a.acc[m], i, j, k, dir, -1), nbp(d, a.acc[m], i, j, k, dir, 1)), 0.5f);
-    G.Lamb[dir] = df_add(nbp(d, a.lfh[dir], i, j, k, 0, 0), nbp(d, a.lfh[dir], i, j, k, dir, -1));
+      G.Eb[dir][m] = df_scale(df_sub(nb(a.acc[m], dir, -1), nb(a.acc[m], dir, 1)), 0.5f);
+    G.Lamb[dir] = df_add(nb(a.lfh[dir], 0, 0), nb(a.lfh[dir], dir, -1));
   }
 #pragma unroll
   for (int m = 0; m < 5; ++m) G.qb[m] = df_from(0.f);
@@ -221,14 +241,14 @@ __device__ __forceinline__ void nodal_gathers_df(const Dims& d, const Adj64& a, 
     dfl c2[4], c4[4];              // faces n-2, n-1, n, n+1
 #pragma unroll
     for (int o = 0; o < 4; ++o) {
-      c2[o] = nbp(d, a.ca2[dir], i, j, k, dir, o - 2);
-      c4[o] = nbp(d, a.ca4[dir], i, j, k, dir, o - 2);
+      c2[o] = nb(a.ca2[dir], dir, o - 2);
+      c4[o] = nb(a.ca4[dir], dir, o - 2);
     }
 #pragma unroll
     for (int m = 0; m < 5; ++m) {
-      const dfl am2 = nbp(d, a.acc[m], i, j, k, dir, -2), am1 = nbp(d, a.acc[m], i, j, k, dir, -1),
-                a0 = nbp(d, a.acc[m], i, j, k, 0, 0), ap1 = nbp(d, a.acc[m], i, j, k, dir, 1),
-                ap2 = nbp(d, a.acc[m], i, j, k, dir, 2);
+      const dfl am2 = nb(a.acc[m], dir, -2), am1 = nb(a.acc[m], dir, -1),
+                a0 = nb(a.acc[m], 0, 0), ap1 = nb(a.acc[m], dir, 1),
+                ap2 = nb(a.acc[m], dir, 2);
       const dfl D0 = df_sub(am1, am2), D1 = df_sub(a0, am1), D2 = df_sub(ap1, a0), D3 = df_sub(ap2, ap1);
       // -D0 c4(n-2) + D1 (c2(n-1) + 3 c4(n-1)) - D2 (c2(n) + 3 c4(n)) + D3 c4(n+1)
       dfl v = df_sub(df_mul(D3, c4[3]), df_mul(D0, c4[0]));
@@ -237,23 +257,27 @@ __device__ __forceinline__ void nodal_gathers_df(const Dims& d, const Adj64& a, 
       G.qb[m] = df_add(G.qb[m], v);
     }
   }
-  G.qb[0] = df_add(G.qb[0], nbp(d, a.rhob, i, j, k, 0, 0));
-  G.mub = nbp(d, a.mub, i, j, k, 0, 0);
+  G.qb[0] = df_add(G.qb[0], nb(a.rhob, 0, 0));
+  G.mub = nb(a.mub, 0, 0);
 }
 
 // Transposed nodal pass (jz_adjoint.cu, k_adj_nodal) for a pair-form solver: the gathers, then
 // the reverse of the anisotropic spectral radii, the inviscid fluxes, Sutherland's law and the
 // primitives, all in double-float arithmetic (the gathers on the pair adjoint arrays).
-// Every padded node.  Three 128-thread blocks per SM (168 registers): 1.49 s per 200-step
-// gradient on 128 x 96 x 64, against 1.51 at four (128, spilling) and 1.55 at two (188).
+// Every padded node.  Issue and load latency bound it at the 12 warps per SM that 168 registers
+// leave: 0.21 ms per launch on 128 x 96 x 64, against 0.29 with a bounds check and 64-bit indices for
+// each of the ~140 gathers (more than half of its 6770 instructions per node).
 constexpr int kTPBN = 128;
-__global__ void __launch_bounds__(kTPBN, 3) k_adj_nodal_df(Dims d, ConstsDF c, DFMetrics M, QDF qdf, Adj64 a) {
-  Box b{-kG, -kG, -kG, d.ni + 2 * kG, d.nj + 2 * kG, d.nk + 2 * kG};
+__global__ void __launch_bounds__(kTPBN, 3) k_adj_nodal_df(const __grid_constant__ Dims d, const __grid_constant__ ConstsDF c,
+                                                           const __grid_constant__ DFMetrics M,
+                                                           const __grid_constant__ QDF qdf,
+                                                           const __grid_constant__ Adj64 a) {
   int i, j, k;
-  if (!box_coord(b, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
-  const long long p = pidx(d, i, j, k);
+  if (!plane_node(-kG, d.ni + 2 * kG, d.nj + 2 * kG, i, j, k)) return;
+  const PaddedNode nb(d, i, j, k);
+  const int p = nb.p;
   NodalGathersDF G;
-  nodal_gathers_df(d, a, i, j, k, G);
+  nodal_gathers_df(a, nb, G);
   dfl ub[3] = {G.fb[0], G.fb[1], G.fb[2]};
   dfl Tb = G.fb[3];
   dfl pb = G.pb;
@@ -368,29 +392,27 @@ __global__ void __launch_bounds__(kTPBN, 3) k_adj_nodal_df(Dims d, ConstsDF c, D
 }  // namespace
 
 cudaError_t adj_update_df(const Dims& d, const GridDev& g, const Adj64& a, double adt, cudaStream_t st) {
-  const long long nr = (long long)d.ni * d.nj * d.nk;
-  k_adj_update_df<<<blocks_for(nr, 256), 256, 0, st>>>(d, g, a, adt);
+  k_adj_update_df<<<plane_grid(d.ni, d.nj, d.nk, 256), 256, 0, st>>>(d, g, a, adt);
   return cudaGetLastError();
 }
 
 cudaError_t adj_nodal_df(const Dims& d, const Consts& c, const DFMetrics& M, const QDF& qdf, const Adj64& a,
                          cudaStream_t st) {
-  const long long n0 = (long long)(d.ni + 2 * kG) * (d.nj + 2 * kG) * (d.nk + 2 * kG);
-  k_adj_nodal_df<<<blocks_for(n0, kTPBN), kTPBN, 0, st>>>(d, make_cdf(c), M, qdf, a);
+  if (d.Np >= (1LL << 31)) return cudaErrorInvalidValue;      // (the adjoint's arrays reach the memory long before)
+  k_adj_nodal_df<<<plane_grid(d.ni + 2 * kG, d.nj + 2 * kG, d.nk + 2 * kG, kTPBN), kTPBN, 0, st>>>(d, make_cdf(c), M,
+                                                                                                    qdf, a);
   return cudaGetLastError();
 }
 
 cudaError_t adj_faces_df(const Dims& d, const Consts& c, const Work64& w, const QDF& qdf, const Adj64& a,
                          cudaStream_t st) {
-  const long long nf = (long long)(d.ni + 1) * (d.nj + 1) * (d.nk + 1);
-  k_adj_faces_df<<<blocks_for(nf, 256), 256, 0, st>>>(d, make_cdf(c), w, qdf, a);
+  k_adj_faces_df<<<plane_grid(d.ni + 1, d.nj + 1, d.nk + 1, 256), 256, 0, st>>>(d, make_cdf(c), w, qdf, a);
   return cudaGetLastError();
 }
 
 cudaError_t adj_visc_df(const Dims& d, const Consts& c, const DFMetrics& M, const Work64& w, const QDF& qdf,
                         const Adj64& a, cudaStream_t st) {
-  const long long n1 = (long long)(d.ni + 2) * (d.nj + 2) * (d.nk + 2);
-  k_adj_visc_df<<<blocks_for(n1, 256), 256, 0, st>>>(d, make_cdf(c), M, w, qdf, a);
+  k_adj_visc_df<<<plane_grid(d.ni + 2, d.nj + 2, d.nk + 2, 256), 256, 0, st>>>(d, make_cdf(c), M, w, qdf, a);
   return cudaGetLastError();
 }
 

@@ -18,7 +18,7 @@ namespace jz {
 namespace {
 
 constexpr int kTPB = 128;
-constexpr int AXI = 8, AXK = kTPB / AXI;   // axis blocks: lines of i, threads along k
+constexpr int AXI = 8;                     // lines of i per axis block
 
 // What the kernel needs of the state: the FP64 fields and, for the FP32-flux form, the shadow.
 struct ShellArgs {
@@ -170,7 +170,7 @@ __device__ __forceinline__ void copy_node(const ShellArgs& A, long long p, long 
   }
 }
 
-// Boundary nodes and ghosts of the jet, by block roles: axis (eight lines of i per block), entrance, exit,
+// Boundary nodes and ghosts of the jet, by block roles: axis, entrance, exit,
 // far field, ghost rows across the axis, ghost planes around the azimuth.  Latency bounds it (a
 // chain of dependent FP64 operations per node on a few thousand nodes).
 template <bool SH>
@@ -183,17 +183,20 @@ __global__ void __launch_bounds__(kTPB) k_jet_shell(const __grid_constant__ Shel
     __syncthreads();
   }
   if (b < A.bA) {
-    // axis: the ring j = 1 averaged over the azimuth, AXI lines of i by AXK threads along k
-    const int i = (int)(b * AXI + th % AXI), ky = th / AXI;
-    const bool in = i < d.ni;
+    // axis: the ring j = 1 averaged over the azimuth; the two ends, whose ring is entrance and exit
+    // nodes, by a block each with all its threads along k, the lines between AXI to a block
+    const bool end = b < 2;
+    const int nx = end ? 1 : AXI, ix = end ? 0 : (int)(th % AXI), ky = end ? (int)th : (int)(th / AXI), nky = kTPB / nx;
+    const int i = end ? (b == 0 ? 0 : d.ni - 1) : (int)((b - 2) * AXI) + 1 + ix;
+    const bool in = end || i < d.ni - 1;
     double s[5] = {0, 0, 0, 0, 0};
     if (in) {
-      for (int k = ky; k < d.nk; k += AXK) {
+      for (int k = ky; k < d.nk; k += nky) {
         double v[5], t[5];
-        if (i == 0) {
+        if (b == 0) {
           inner_neighbour(A, 1, 1, k, t);
           entrance_value(A, am, 1, k, t, v);
-        } else if (i == d.ni - 1) {
+        } else if (b == 1) {
           inner_neighbour(A, i - 1, 1, k, t);
           exit_value(A, t, v);
         } else {
@@ -207,19 +210,19 @@ __global__ void __launch_bounds__(kTPB) k_jet_shell(const __grid_constant__ Shel
 #pragma unroll
     for (int m = 0; m < 5; ++m) {
       double x = s[m];
-      for (int o = 16; o >= AXI; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-      if ((th & 31) < AXI) red[m][th >> 5][th & 31] = x;
+      for (int o = 16; o >= nx; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      if ((th & 31) < nx) red[m][th >> 5][th & 31] = x;
     }
     __syncthreads();
     double mean[5];
 #pragma unroll
     for (int m = 0; m < 5; ++m) {
       double x = 0.0;
-      for (int w = 0; w < kTPB / 32; ++w) x += red[m][w][th % AXI];
+      for (int w = 0; w < kTPB / 32; ++w) x += red[m][w][ix];
       mean[m] = x / d.nk;
     }
     if (in)
-      for (int k = ky; k < d.nk; k += AXK) put_node<SH>(A, mean, i, 0, k);
+      for (int k = ky; k < d.nk; k += nky) put_node<SH>(A, mean, i, 0, k);
     if (b == 0 && th == 0 && A.advance) A.sc->t = A.sc->t + A.sc->dt;
     return;
   }
@@ -314,7 +317,7 @@ cudaError_t jet_shell(const Dims& d, const Consts& c, const GridDev& g, const In
   A.advance = advance;
   const long long ni2 = d.ni - 2;
   const unsigned nio = blocks_for((long long)(d.nj - 1) * d.nk, kTPB);
-  A.bA = blocks_for(d.ni, AXI);
+  A.bA = 2 + blocks_for(ni2, AXI);
   A.bE = A.bA + nio;
   A.bX = A.bE + nio;
   A.bF = A.bX + blocks_for(ni2 * d.nk, kTPB);

@@ -128,41 +128,6 @@ __global__ void k_derived(Dims d, Ptrs16 M, Ptrs16 out) {
   out.p[4][p] = cbrt(V);
 }
 
-// Ghost shell enumerated directly: the four k-ghost planes (with their i/j
-// ghosts), then the four j-ghost rows of every real k, then the four i-ghost
-// columns of every real (j, k).  Every ghost copies from a real node.
-__device__ __forceinline__ bool ghost_coord(const Dims& d, long long t, int& i, int& j, int& k) {
-  const long long ei = d.ni + 2 * kG, ej = d.nj + 2 * kG;
-  const long long nA = 4 * ei * ej, nB = 4 * ei * d.nk, nC = 4LL * d.nj * d.nk;
-  if (t < nA) {
-    i = (int)(t % ei) - kG;
-    const long long r = t / ei;
-    j = (int)(r % ej) - kG;
-    const int s = (int)(r / ej);                 // 0..3
-    k = s < 2 ? s - 2 : d.nk + s - 2;
-    return true;
-  }
-  t -= nA;
-  if (t < nB) {
-    i = (int)(t % ei) - kG;
-    const long long r = t / ei;
-    const int s = (int)(r % 4);
-    k = (int)(r / 4);
-    j = s < 2 ? s - 2 : d.nj + s - 2;
-    return true;
-  }
-  t -= nB;
-  if (t < nC) {
-    const int s = (int)(t % 4);
-    const long long r = t / 4;
-    j = (int)(r % d.nj);
-    k = (int)(r / d.nj);
-    i = s < 2 ? s - 2 : d.ni + s - 2;
-    return true;
-  }
-  return false;
-}
-
 __global__ void k_ghost_fill(Dims d, Ptrs16 f, int nvar) {
   int i, j, k;
   if (!ghost_coord(d, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
@@ -285,9 +250,7 @@ cudaError_t check_volume(const Dims& d, const GridDev& g, int* bad, cudaStream_t
 }
 
 cudaError_t ghost_fill(const Dims& d, double* const* f, int nvar, cudaStream_t st) {
-  const long long ei = d.ni + 2 * kG, ej = d.nj + 2 * kG;
-  const long long ng = 4 * ei * ej + 4 * ei * d.nk + 4LL * d.nj * d.nk;
-  k_ghost_fill<<<blocks_for(ng, kTPB), kTPB, 0, st>>>(d, ptrs(f, nvar), nvar);
+  k_ghost_fill<<<blocks_for(ghost_count(d), kTPB), kTPB, 0, st>>>(d, ptrs(f, nvar), nvar);
   return cudaGetLastError();
 }
 
@@ -333,9 +296,7 @@ cudaError_t pack_state(const Dims& d, const Consts& c, const State& q, const dou
 }
 
 cudaError_t ghost_fill_state(const Dims& d, const State& q, Scalars* advance, cudaStream_t st) {
-  const long long ei = d.ni + 2 * kG, ej = d.nj + 2 * kG;
-  const long long ng = 4 * ei * ej + 4 * ei * d.nk + 4LL * d.nj * d.nk;
-  k_ghost_state<<<blocks_for(ng, kTPB), kTPB, 0, st>>>(d, q, advance);
+  k_ghost_state<<<blocks_for(ghost_count(d), kTPB), kTPB, 0, st>>>(d, q, advance);
   return cudaGetLastError();
 }
 

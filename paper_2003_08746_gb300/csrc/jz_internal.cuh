@@ -453,4 +453,44 @@ __host__ __device__ inline void ghost_source(const Dims& d, int i, int j, int k,
   sk = ((kk % d.nk) + d.nk) % d.nk;
 }
 
+// Ghost shell enumerated directly: the four k-ghost planes (with their i/j
+// ghosts), then the four j-ghost rows of every real k, then the four i-ghost
+// columns of every real (j, k).  Every ghost copies from a real node.
+__device__ __forceinline__ bool ghost_coord(const Dims& d, long long t, int& i, int& j, int& k) {
+  const long long ei = d.ni + 2 * kG, ej = d.nj + 2 * kG;
+  const long long nA = 4 * ei * ej, nB = 4 * ei * d.nk, nC = 4LL * d.nj * d.nk;
+  if (t < nA) {
+    i = (int)(t % ei) - kG;
+    const long long r = t / ei;
+    j = (int)(r % ej) - kG;
+    const int s = (int)(r / ej);                 // 0..3
+    k = s < 2 ? s - 2 : d.nk + s - 2;
+    return true;
+  }
+  t -= nA;
+  if (t < nB) {
+    i = (int)(t % ei) - kG;
+    const long long r = t / ei;
+    const int s = (int)(r % 4);
+    k = (int)(r / 4);
+    j = s < 2 ? s - 2 : d.nj + s - 2;
+    return true;
+  }
+  t -= nB;
+  if (t < nC) {
+    const int s = (int)(t % 4);
+    const long long r = t / 4;
+    j = (int)(r % d.nj);
+    k = (int)(r / d.nj);
+    i = s < 2 ? s - 2 : d.ni + s - 2;
+    return true;
+  }
+  return false;
+}
+
+inline long long ghost_count(const Dims& d) {
+  const long long ei = d.ni + 2 * kG, ej = d.nj + 2 * kG;
+  return 4 * ei * ej + 4 * ei * d.nk + 4LL * d.nj * d.nk;
+}
+
 }  // namespace jz
