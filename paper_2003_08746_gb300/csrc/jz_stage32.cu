@@ -12,19 +12,25 @@
 // writes its shadow, and the kernels that set boundary nodes, fill ghosts or
 // load a state write the shadow of what they set.
 //
-// Each CTA owns a TX x TY tile of (i, j) columns and marches in k.  Shared
-// memory holds a ring of four planes of the shadow (tile + 2-node halo; each
-// plane is one 4-D TMA box of 34 x 12 x 1 x 3 float2 landing on an mbarrier),
-// a ring of two planes of in-plane nodal fluxes, spectral radii and sensors
-// (tile + 1-node halo), the same for the zeta direction (tile only), and the
-// xi/eta dissipation faces of one plane.  Per plane:
-//   (a) wait for the shadow of plane k+2 (requested one plane earlier) and
-//       form 1/rho on its points; one thread then requests plane k+3,
-//   (b) every node of plane k+1 within one node of the tile gets its
-//       gradients, viscous and inviscid transformed fluxes H^dir, spectral
-//       radii Lambda^dir and pressure sensors nu^dir; the same threads then
-//       compute each xi and eta dissipation face of plane k once,
-//   (c) the tile of plane k gets its zeta face, RHS and update.
+// Each CTA owns a TX x TY tile of (i, j) columns and marches in k; a thread
+// owns the column of one node of the tile or of its one-node halo, a warp one
+// row of them.  Shared memory holds a ring of four planes of the shadow (tile +
+// 2-node halo; each plane is one 4-D TMA box of 34 x 12 x 1 x 3 float2 landing
+// on an mbarrier) with 1/rho beside them, and the eta quantities that rows
+// exchange (H^eta, Lambda^eta, nu^eta of one plane, two planes in turn).
+// Everything else stays with its thread.  Per plane p:
+//   (a) wait for the shadow of plane p+2 (requested one plane earlier) and
+//       form 1/rho on its points;
+//   (b) the node of plane p+1 gets its gradients, viscous and inviscid
+//       transformed fluxes H^dir, spectral radii Lambda^dir and pressure
+//       sensors nu^dir; its eta quantities go to shared memory, its xi faces
+//       and the xi part of its RHS are formed from the neighbouring lanes
+//       (shuffles);
+//       one barrier; one thread requests plane p+3;
+//   (c) the node of plane p gets its zeta face, which completes its RHS (xi
+//       and eta part from the iteration before), and its update;
+//   (d) the eta faces below and above the node of plane p+1 (each face formed
+//       by both its nodes: cheaper than a second exchange) and the eta part.
 //
 // On a GB300 the FP64 pipe (DADD/DFMA, and also the F2F conversions between
 // FP64 and FP32) issues ~2 instructions per SM per clock against 128 for
@@ -44,19 +50,11 @@
 namespace jz {
 namespace {
 
-#ifndef JZ_FUSED_TX
-#define JZ_FUSED_TX 30
-#endif
-#ifndef JZ_FUSED_TY
-#define JZ_FUSED_TY 8
-#endif
-constexpr int TX = JZ_FUSED_TX, TY = JZ_FUSED_TY;
+constexpr int TX = 30, TY = 8;
 constexpr int H1X = TX + 2, H1Y = TY + 2, NP1 = H1X * H1Y;   // 32 x 10
 constexpr int H2X = TX + 4, H2Y = TY + 4, NP2 = H2X * H2Y;   // 34 x 12
 constexpr int NT = NP1;                                      // threads per CTA
-constexpr int NOUT = TX * TY;
-constexpr int NOT = 32 * TY;                                 // output threads: one warp per row
-static_assert(TX <= 32 && NOT <= NT, "one warp per output row");
+static_assert(TX == 30, "a warp holds a row of the tile and its halo");
 constexpr int NIR = (NP2 + NT - 1) / NT;                     // halo-2 points per thread (1/rho pass)
 
 // shadow ring: per halo-2 point three float2 pairs, as in global memory
@@ -65,20 +63,14 @@ constexpr int NIR = (NP2 + NT - 1) / NT;                     // halo-2 points pe
 constexpr int NRING = 4;           // planes k-1 .. k+2: the next plane's request needs no barrier
 constexpr int BOX_BYTES = NSH * NP2 * 8;                       // one TMA box (34 x 12 x 1 x 3 float2)
 constexpr int SLOT = ((BOX_BYTES + 127) / 128) * 128 / 8;      // float2 per ring slot, 128-byte aligned
-// in-plane flux ring (tile + 1 halo): H^xi(5), H^eta(5), Lambda^xi, Lambda^eta, nu^xi, nu^eta
-constexpr int X_HX = 0, X_HY = 5, X_LX = 10, X_LY = 11, X_NX = 12, X_NY = 13, NXF = 14;
-// zeta ring (tile): H^zeta(5), Lambda^zeta, nu^zeta, 1/V
-constexpr int Z_HZ = 0, Z_L = 5, Z_N = 6, Z_IV = 7, NZF = 8;
-// xi faces: TY rows of TX+1; eta faces: TY+1 rows of TX
-constexpr int NFX = TY * (TX + 1), NFY = (TY + 1) * TX;
+// eta exchange between rows, two planes in turn: H^eta(5), Lambda^eta, nu^eta
+constexpr int E_H = 0, E_L = 5, E_N = 6, NEF = 7;
 
 struct Smem {
   float2 sh[NRING][SLOT];          // TMA destinations (first member: 128-byte aligned)
   float ir[NRING][NP2];
-  float fxy[2][NXF][NP1];
-  float fz[2][NZF][NOUT];
-  float dx[5][NFX];
-  float dy[5][NFY];
+  float eta[2][NEF][NP1];
+  float carry[5][NP1];             // H^zeta(p-1) of each thread's column
   unsigned long long bar[NRING];   // one mbarrier per ring slot
   int fail;                        // a bounded wait ran out in this CTA
 };
@@ -108,11 +100,6 @@ __device__ __forceinline__ float f_lg2(float x) {
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-// Ask L2 to fetch the sector holding p (no register, no wait).
-__device__ __forceinline__ void prefetch_l2(const void* p) {
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-
 __device__ __forceinline__ float cbrt_pos(float x) {   // x >= 0; 0 -> 0
   return x > 0.f ? f_ex2(f_lg2(x) * (1.f / 3.f)) : 0.f;
 }
@@ -145,8 +132,7 @@ struct Args {
   const double* qin[5];      // FP64 Q^(l-1): copied on the nodes the stage does not advance
   const double* qn[5];
   double* qout[5];
-  float2* sout;              // shadow of Q^(l) [3][Np] (null with rhs)
-  long long Np;
+  float2* sout[NSH];         // shadow of Q^(l) (not used with rhs)
   double* rhs;               // non-null: write RHS [5][N] instead of updating
   Scalars* sc;
   double alpha;
@@ -185,22 +171,17 @@ __device__ __forceinline__ void inv_rho(Smem& sm, int slot) {
 }
 
 // Metric record of one node (three 16-byte loads).
-__device__ __forceinline__ void load_record(const float* M, long long p, float met[kMF]) {
-  const float4* r = reinterpret_cast<const float4*>(M + p * kMF);
+__device__ __forceinline__ void load_record(const float* M, unsigned p, float met[kMF]) {
+  const float4* r = reinterpret_cast<const float4*>(M) + (unsigned long long)p * (kMF / 4);
   const float4 a = __ldg(r), b = __ldg(r + 1), c = __ldg(r + 2);
   met[0] = a.x; met[1] = a.y; met[2] = a.z; met[3] = a.w;
   met[4] = b.x; met[5] = b.y; met[6] = b.z; met[7] = b.w;
   met[8] = c.x; met[9] = c.y; met[10] = c.z; met[11] = c.w;
 }
 
-// Metric record of this thread's halo-1 node of plane q (nb < 0: outside, zeros).
-__device__ __forceinline__ void load_metrics(const Args& A, long long nb, int q, float met[kMF]) {
-  if (nb < 0) {
-#pragma unroll
-    for (int f = 0; f < kMF; ++f) met[f] = 0.f;
-    return;
-  }
-  load_record(A.M, nb + (long long)q * A.d.sk, met);
+// Ask L2 to fetch the sector holding p (no register, no wait).
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
 // A landed ring slot: the shadow pairs and 1/rho of its halo-2 points.
@@ -218,25 +199,15 @@ __device__ __forceinline__ void load_q(const Plane& P, int c, float q[5]) {
   q[0] = a.x; q[1] = b.x; q[2] = b.y; q[3] = d.x; q[4] = a.y;
 }
 
-// Nodal fluxes, spectral radii and sensors of one node of plane q (slots
-// s_m, s_0, s_p of planes q-1, q, q+1) at halo-1 index t, into ring slot g.
-__device__ void nodal(const Args& A, Smem& sm, long long nb, const float met[kMF], int s_m, int s_0, int s_p, int g) {
+// Transformed fluxes, anisotropic spectral radii and pressure sensors of one node, and 1/V.
+struct Node {
+  float H[3][5], lam[3], nu[3], iV;
+};
+
+// ... of one node of plane q (slots s_m, s_0, s_p of planes q-1, q, q+1) at halo-2 index c2.
+__device__ __forceinline__ void nodal(const Args& A, const Smem& sm, const float met[kMF], int s_m, int s_0, int s_p,
+                                      int c2, Node& N) {
   const ConstsF& c = A.c;
-  const int t = threadIdx.x;
-  const int x1 = t % H1X, y1 = t / H1X;
-  const bool tile = x1 >= 1 && x1 <= TX && y1 >= 1 && y1 <= TY;
-  const int o = (y1 - 1) * TX + (x1 - 1);
-  const int c2 = (y1 + 1) * H2X + (x1 + 1);
-  float* Fx = &sm.fxy[g][0][0];
-  float* Fz = &sm.fz[g][0][0];
-  if (nb < 0) {
-#pragma unroll 1
-    for (int f = 0; f < NXF; ++f) Fx[f * NP1 + t] = 0.f;
-    if (tile)
-#pragma unroll 1
-      for (int f = 0; f < NZF; ++f) Fz[f * NOUT + o] = 0.f;
-    return;
-  }
   float S[3][3];
 #pragma unroll
   for (int dir = 0; dir < 3; ++dir)
@@ -244,9 +215,9 @@ __device__ void nodal(const Args& A, Smem& sm, long long nb, const float met[kMF
     for (int cc = 0; cc < 3; ++cc) S[dir][cc] = met[3 * dir + cc];
   const float iV = met[MF_IV];
   const Plane P0 = plane(sm, s_0), Pm = plane(sm, s_m), Pp = plane(sm, s_p);
-  // u, v, w, T at a node of the ring (plane P, halo-2 index cc)
-  auto uvwT = [&](const Plane& P, int cc, float f[4]) {
-    const float ir = P.ir[cc];
+  // u, v, w, T at a node of the ring (plane P, halo-2 index cc, 1/rho there; that of plane q+1 is only
+  // being written by others and formed again)
+  auto uvwT = [&](const Plane& P, int cc, float ir, float f[4]) {
     const float2 a = P_m12(P, cc), b = P_m3p(P, cc);
     f[0] = a.x * ir;
     f[1] = a.y * ir;
@@ -256,12 +227,12 @@ __device__ void nodal(const Args& A, Smem& sm, long long nb, const float met[kMF
   // gradients of u, v, w, T: L[n][j] = sum_dir (S^dir_j / (2V)) (f_{+} - f_{-})
   const float h = 0.5f * iV;
   float fxp[4], fxm[4], fyp[4], fym[4], fzp[4], fzm[4];
-  uvwT(P0, c2 + 1, fxp);
-  uvwT(P0, c2 - 1, fxm);
-  uvwT(P0, c2 + H2X, fyp);
-  uvwT(P0, c2 - H2X, fym);
-  uvwT(Pp, c2, fzp);
-  uvwT(Pm, c2, fzm);
+  uvwT(P0, c2 + 1, P0.ir[c2 + 1], fxp);
+  uvwT(P0, c2 - 1, P0.ir[c2 - 1], fxm);
+  uvwT(P0, c2 + H2X, P0.ir[c2 + H2X], fyp);
+  uvwT(P0, c2 - H2X, P0.ir[c2 - H2X], fym);
+  uvwT(Pp, c2, f_rcp(P_re(Pp, c2).x + 1.f), fzp);
+  uvwT(Pm, c2, Pm.ir[c2], fzm);
   float L[4][3];
 #pragma unroll
   for (int n = 0; n < 4; ++n) {
@@ -273,7 +244,7 @@ __device__ void nodal(const Args& A, Smem& sm, long long nb, const float met[kMF
   const float rho = re0.x + 1.f;
   const float m1 = m12.x, m2 = m12.y, m3 = m3p.x;
   float f0[4];
-  uvwT(P0, c2, f0);
+  uvwT(P0, c2, P0.ir[c2], f0);
   const float u = f0[0], v = f0[1], w = f0[2], T = f0[3];
   const float pp = m3p.y;
   const float ep = re0.y;
@@ -297,7 +268,8 @@ __device__ void nodal(const Args& A, Smem& sm, long long nb, const float met[kMF
                          {t12, t22, t23, u * t12 + v * t22 + w * t23 + k_eff * L[3][1]},
                          {t13, t23, t33, u * t13 + v * t23 + w * t33 + k_eff * L[3][2]}};
   const float h0 = ep + pp + c.ep_inf;   // e + p
-  float lam[3], H[3][5];
+  float lam[3];
+  float (*H)[5] = N.H;
 #pragma unroll
   for (int dir = 0; dir < 3; ++dir) {
     const float U = S[dir][0] * u + S[dir][1] * v + S[dir][2] * w;
@@ -315,71 +287,22 @@ __device__ void nodal(const Args& A, Smem& sm, long long nb, const float met[kMF
   const float pym = P_m3p(P0, c2 - H2X).y, pyp = P_m3p(P0, c2 + H2X).y;
   const float pzm = P_m3p(Pm, c2).y, pzp = P_m3p(Pp, c2).y;
   const float p4 = 4.f * c.p_inf;
-#pragma unroll
-  for (int m = 0; m < 5; ++m) {
-    Fx[(X_HX + m) * NP1 + t] = H[0][m];
-    Fx[(X_HY + m) * NP1 + t] = H[1][m];
-  }
-  Fx[X_LX * NP1 + t] = lam[0] + r0 * (r1 * r1 + r2 * r2);
-  Fx[X_LY * NP1 + t] = lam[1] + r1 * (r0 * r0 + r2 * r2);
-  Fx[X_NX * NP1 + t] = fabsf(pxp - 2.f * pp + pxm) * f_rcp(pxp + 2.f * pp + pxm + p4);
-  Fx[X_NY * NP1 + t] = fabsf(pyp - 2.f * pp + pym) * f_rcp(pyp + 2.f * pp + pym + p4);
-  if (tile) {
-#pragma unroll
-    for (int m = 0; m < 5; ++m) Fz[(Z_HZ + m) * NOUT + o] = H[2][m];
-    Fz[Z_L * NOUT + o] = lam[2] + r2 * (r0 * r0 + r1 * r1);
-    Fz[Z_N * NOUT + o] = fabsf(pzp - 2.f * pp + pzm) * f_rcp(pzp + 2.f * pp + pzm + p4);
-    Fz[Z_IV * NOUT + o] = iV;
-  }
+  N.lam[0] = lam[0] + r0 * (r1 * r1 + r2 * r2);
+  N.lam[1] = lam[1] + r1 * (r0 * r0 + r2 * r2);
+  N.lam[2] = lam[2] + r2 * (r0 * r0 + r1 * r1);
+  N.nu[0] = fabsf(pxp - 2.f * pp + pxm) * f_rcp(pxp + 2.f * pp + pxm + p4);
+  N.nu[1] = fabsf(pyp - 2.f * pp + pym) * f_rcp(pyp + 2.f * pp + pym + p4);
+  N.nu[2] = fabsf(pzp - 2.f * pp + pzm) * f_rcp(pzp + 2.f * pp + pzm + p4);
+  N.iV = iV;
 }
 
-// The xi and eta dissipation faces of one plane (ring slots: prim s_0, fluxes g),
-// each computed once by one thread.  Tasks are laid out one 32-lane row per
-// face row so that a warp touches one shared-memory row (no bank conflicts).
-constexpr int NTX = 32 * TY, NTY = 32 * (TY + 1);
-static_assert(TX + 1 <= 32, "xi face row fits a warp");
-
-__device__ void plane_faces(const Args& A, Smem& sm, int s_0, int g) {
-  const Plane P = plane(sm, s_0);
-  const float* Fx = &sm.fxy[g][0][0];
-  for (int task = threadIdx.x; task < NTX + NTY; task += NT) {
-    float qm[5], q0[5], q1[5], q2[5], out[5];
-    if (task < NTX) {
-      const int oy = task >> 5, fx = task & 31;
-      if (fx > TX) continue;
-      const int e = oy * (TX + 1) + fx;
-      const int a = (oy + 1) * H1X + fx;           // halo-1 index of the left node
-      const int cq = (oy + 2) * H2X + fx + 1;      // halo-2 index of the left node
-      load_q(P, cq - 1, qm);
-      load_q(P, cq, q0);
-      load_q(P, cq + 1, q1);
-      load_q(P, cq + 2, q2);
-      face_flux(A.c, Fx[X_LX * NP1 + a], Fx[X_LX * NP1 + a + 1], Fx[X_NX * NP1 + a], Fx[X_NX * NP1 + a + 1],
-                qm, q0, q1, q2, out);
-#pragma unroll
-      for (int m = 0; m < 5; ++m) sm.dx[m][e] = out[m];
-    } else {
-      const int fy = (task - NTX) >> 5, ox = (task - NTX) & 31;
-      if (ox >= TX) continue;
-      const int e2 = fy * TX + ox;
-      const int a = fy * H1X + ox + 1;             // halo-1 index of the lower node
-      const int cq = (fy + 1) * H2X + ox + 2;      // halo-2 index of the lower node
-      load_q(P, cq - H2X, qm);
-      load_q(P, cq, q0);
-      load_q(P, cq + H2X, q1);
-      load_q(P, cq + 2 * H2X, q2);
-      face_flux(A.c, Fx[X_LY * NP1 + a], Fx[X_LY * NP1 + a + H1X], Fx[X_NY * NP1 + a], Fx[X_NY * NP1 + a + H1X],
-                qm, q0, q1, q2, out);
-#pragma unroll
-      for (int m = 0; m < 5; ++m) sm.dy[m][e2] = out[m];
-    }
-  }
-}
-
-
-constexpr int kMinBlocks = NT <= 320 ? 2 : 1;
-
-__global__ void __launch_bounds__(NT, kMinBlocks) k_fused32(const __grid_constant__ Args A) {
+// Latency and issue bound it (58% of the cycles issue, 20 warps per SM): 9.9 ms per launch on
+// 1024 x 512 x 360, 2.9 TB/s of algorithmic bytes, against 13.0 with the zeta and xi quantities and
+// the faces in shared memory too and two barriers per plane.  Rows per tile: 8 (96 registers, two
+// CTAs per SM); 6: 11.7, 9 (88 registers, spills): 17.5, 12 at one CTA: 12.8.  H^zeta(p-1) in shared
+// memory instead of registers (spills): 10.8 against 12.0; metric records and Q^n a plane ahead by
+// cp.async: 11.8 against 10.3.
+__global__ void __launch_bounds__(NT, 2) k_fused32(const __grid_constant__ Args A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   // TMA destinations need 128-byte alignment; the launch adds 128 bytes of room for it
   Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~(uintptr_t)127);
@@ -389,24 +312,21 @@ __global__ void __launch_bounds__(NT, kMinBlocks) k_fused32(const __grid_constan
   const int k0 = blockIdx.z * A.kchunk;
   const int k1 = min(k0 + A.kchunk, d.nk);          // output planes [k0, k1)
   const int t = threadIdx.x;
-  const int ox = t & 31, oy = t >> 5;
-  const bool outth = t < NOT && ox < TX;
-  const int o = oy * TX + ox;                       // tile index of the output node
-  const int oi = i0 + ox, oj = j0 + oy;
-  const bool outv = outth && oi < d.ni && oj < d.nj;
+  // this thread's node: one row of the tile and its one-node halo per warp
+  const int x1 = t & 31, y1 = t >> 5;
+  const int oi = i0 - 1 + x1, oj = j0 - 1 + y1;
+  const int c2 = (y1 + 1) * H2X + (x1 + 1);         // its halo-2 index
+  const bool valid = in_padded(d, oi, oj);
+  const bool rowt = y1 >= 1 && y1 <= TY;            // (uniform in a warp)
+  const bool outv = rowt && x1 >= 1 && x1 <= TX && oi < d.ni && oj < d.nj;   // an output node
   const bool adv = outv && (d.topo != JZ_TOPO_JET || (oi >= 1 && oi <= d.ni - 2 && oj >= 1 && oj <= d.nj - 2));
-  const int c1 = (oy + 1) * H1X + (ox + 1);
-  const int c2 = (oy + 2) * H2X + (ox + 2);
   // the halo-2 box starts at real (i0 - 2, j0 - 2): padded (i0, j0); x0 * 8 bytes is a multiple
   // of 16 because TX is even
   const int x0 = i0, y0 = j0;
-
-  long long nb;                                    // halo-1 node of this thread (nodal work)
-  {
-    const int i = i0 - 1 + t % H1X, j = j0 - 1 + t / H1X;
-    nb = in_padded(d, i, j) ? pidx(d, i, j, 0) : -1;
-  }
-  const long long ob = outv ? pidx(d, oi, oj, 0) : 0;   // output node
+  // its element in plane p of a padded field (32 bits: a field's Np nodes at 168 bytes each reach the
+  // GPU's memory before 2^32), here for p = k0 - 2
+  const unsigned sk = (unsigned)d.sk;
+  unsigned pp = (unsigned)(valid ? pidx(d, oi, oj, k0 - 2) : 0);
   // prime: mbarriers, then planes k0-2 .. k0 requested; k0-2 and k0-1 waited for
   int last_req = k0 - 3;                           // thread 0: last plane requested
   if (t == 0) {
@@ -423,84 +343,99 @@ __global__ void __launch_bounds__(NT, kMinBlocks) k_fused32(const __grid_constan
     if (!wait_slot(sm, ring(q), plane_parity(q, k0))) sm.fail = q + 1000000;
     inv_rho(sm, ring(q));
   }
+  __syncthreads();                                 // 1/rho of the first two planes
 
-  float Hz_prev[5] = {0, 0, 0, 0, 0};   // H^zeta(p-1)
+  // marching state of the thread's column: plane p-1 (fluxes, Q, face p-1/2) and plane p (zeta
+  // quantities, and the xi and eta part of its RHS)
+  float Hz_0[5] = {0, 0, 0, 0, 0};      // H^zeta(p); H^zeta(p-1) is kept in shared memory
   float Dz_prev[5] = {0, 0, 0, 0, 0};   // d^zeta(p-1/2)
+  for (int m = 0; m < 5; ++m) sm.carry[m][t] = 0.f;
   float Qz_prev[5] = {0, 0, 0, 0, 0};   // Q(p-1), FP32
-  float Lz = 0.f, Nz = 0.f;             // Lambda^zeta(p), nu^zeta(p)
+  float acc[5] = {0, 0, 0, 0, 0};       // xi and eta part of plane p
+  float Lz = 0.f, Nz = 0.f, iV0 = 0.f;  // Lambda^zeta(p), nu^zeta(p), 1/V(p)
   const float adt = f64_to_f32(A.alpha * A.sc->dt);
   float res = 0.f, rate = 0.f;
 
-  for (int p = k0 - 2; p < k1; ++p) {
-    // (a) metrics of plane p+1 (used in (b)); the shadow of plane p+2 (requested one plane
-    // earlier) and its 1/rho
-    float met[kMF];
-    load_metrics(A, nb, p + 1, met);
-    // L2 hints one plane ahead: metrics of plane p+2 (next iteration's nodal work)
-    // and Q^n of plane p+1 (next iteration's update)
-    if (nb >= 0 && p + 2 <= k1) {
-      // a 48-byte record spans two 32-byte sectors; with the neighbours' requests every
-      // sector of the row is asked for
-      const float* pm = A.M + (nb + (long long)(p + 2) * d.sk) * kMF;
-      prefetch_l2(pm);
-      prefetch_l2(pm + 8);
-    }
-    if (adv && !A.rhs && p + 1 < k1) {
-      const long long pq = ob + (long long)(p + 1) * d.sk;
-#pragma unroll
-      for (int m = 0; m < 5; ++m) prefetch_l2(A.qn[m] + pq);
+  for (int p = k0 - 2; p < k1; ++p, pp += sk) {
+    const Plane P0 = plane(sm, ring(p)), P1 = plane(sm, ring(p + 1)), P2 = plane(sm, ring(p + 2));
+    // (a) metrics of plane p+1; the shadow of plane p+2 (requested one plane earlier) and its 1/rho
+    float met[kMF] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (valid) {
+      load_record(A.M, pp + sk, met);
+      if (p + 2 <= k1) {
+        // the next plane's record: it spans two 32-byte sectors, and with the neighbours' requests
+        // every sector of the row is asked for
+        const float* pm = A.M + (unsigned long long)(pp + 2 * sk) * kMF;
+        prefetch_l2(pm);
+        prefetch_l2(pm + 8);
+      }
     }
     // after a wait ran out no plane is requested or waited for any more (the CTA finishes on
     // stale data and the host reports the error)
     if (sm.fail == 0 && !wait_slot(sm, ring(p + 2), plane_parity(p + 2, k0))) sm.fail = p + 2 + 1000000;
-    inv_rho(sm, ring(p + 2));
+    inv_rho(sm, ring(p + 2));                      // (neighbours read it one plane later)
+    // (b) the node of plane p+1; its eta quantities for the rows above and below
+    // Q^n of the output node of plane p, requested before the work that hides its latency
+    double qn_r[5];
+    if (p >= k0 && adv && !A.rhs) {
+#pragma unroll
+      for (int m = 0; m < 5; ++m) qn_r[m] = __ldg(A.qn[m] + pp);
+    }
+    Node N;                                        // (zeros outside the padded box, as its metrics)
+    nodal(A, sm, met, ring(p), ring(p + 1), ring(p + 2), c2, N);
+    float* E = &sm.eta[p & 1][0][0];
+    const bool inplane = p + 1 >= k0 && p + 1 < k1;   // plane p+1 is an output plane
+    float ax[5] = {0.f, 0.f, 0.f, 0.f, 0.f};          // its xi (and then eta) part
+    if (inplane) {
+#pragma unroll
+      for (int m = 0; m < 5; ++m) E[(E_H + m) * NP1 + t] = N.H[1][m];
+      E[E_L * NP1 + t] = N.lam[1];
+      E[E_N * NP1 + t] = N.nu[1];
+      if (rowt) {
+        // xi faces: each lane the face to its right neighbour, the left one from the lane before
+        float qm[5], q0[5], q1[5], q2[5], out[5];
+        load_q(P1, c2 - 1, qm);
+        load_q(P1, c2, q0);
+        load_q(P1, c2 + 1, q1);
+        load_q(P1, c2 + 2, q2);
+        const unsigned all = 0xffffffffu;
+        face_flux(c, N.lam[0], __shfl_down_sync(all, N.lam[0], 1), N.nu[0], __shfl_down_sync(all, N.nu[0], 1), qm, q0, q1,
+                  q2, out);
+#pragma unroll
+        for (int m = 0; m < 5; ++m) {
+          const float hp = __shfl_down_sync(all, N.H[0][m], 1), hm = __shfl_up_sync(all, N.H[0][m], 1);
+          ax[m] = 0.5f * (hp - hm) - (out[m] - __shfl_up_sync(all, out[m], 1));
+        }
+      }
+    }
+    // The one barrier of a plane: 1/rho of plane p+2 and the eta quantities of plane p+1 are there;
+    // every thread is done with plane p-1 of the ring and with the eta quantities of plane p.
     __syncthreads();
-    // the slot of plane p-1 is free: request plane p+3 into it
     if (t == 0 && p + 3 <= k1 + 1 && sm.fail == 0) {
       request_plane(A, sm, ring(p + 3), x0, y0, p + 3);
       last_req = p + 3;
     }
-    // (b) nodal quantities of plane p+1, then the xi/eta faces of plane p
-    nodal(A, sm, nb, met, ring(p), ring(p + 1), ring(p + 2), (p + 1) & 1);
-    plane_faces(A, sm, ring(p), p & 1);
-    __syncthreads();
-    // (c) zeta face p+1/2 and the output plane p
-    if (outth) {
-      const float* Z0 = &sm.fz[p & 1][0][0];
-      const float* Z1 = &sm.fz[(p + 1) & 1][0][0];
-      const Plane P0 = plane(sm, ring(p)), P1 = plane(sm, ring(p + 1)), P2 = plane(sm, ring(p + 2));
-      const float Lz1 = Z1[Z_L * NOUT + o], Nz1 = Z1[Z_N * NOUT + o];
-      // Q^n of this output node, requested before the zeta-face work that hides its latency
-      double qn_r[5];
-      const long long pp = ob + (long long)p * d.sk;
-      if (p >= k0 && adv && !A.rhs) {
-#pragma unroll
-        for (int m = 0; m < 5; ++m) qn_r[m] = __ldg(A.qn[m] + pp);
-      }
+    // metrics of plane p+2 (those of plane p+1 have been used)
+    if (rowt) {
+      // (c) zeta face p+1/2, RHS and update of plane p
       float q0[5], q1[5], q2[5], Dz[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
       load_q(P0, c2, q0);
       load_q(P1, c2, q1);
       load_q(P2, c2, q2);
-      if (p >= k0 - 1) face_flux(c, Lz, Lz1, Nz, Nz1, Qz_prev, q0, q1, q2, Dz);
+      if (p >= k0 - 1) face_flux(c, Lz, N.lam[2], Nz, N.nu[2], Qz_prev, q0, q1, q2, Dz);
       if (p >= k0 && outv) {
-        const float* F0 = &sm.fxy[p & 1][0][0];
-        const int ex = oy * (TX + 1) + ox, ey = oy * TX + ox;
-        const float iV = Z0[Z_IV * NOUT + o];
         float R[5];
 #pragma unroll
         for (int m = 0; m < 5; ++m) {
-          float acc = 0.5f * (F0[(X_HX + m) * NP1 + c1 + 1] - F0[(X_HX + m) * NP1 + c1 - 1]) -
-                      (sm.dx[m][ex + 1] - sm.dx[m][ex]);
-          acc += 0.5f * (F0[(X_HY + m) * NP1 + c1 + H1X] - F0[(X_HY + m) * NP1 + c1 - H1X]) -
-                 (sm.dy[m][ey + TX] - sm.dy[m][ey]);
-          acc += 0.5f * (Z1[(Z_HZ + m) * NOUT + o] - Hz_prev[m]) - (Dz[m] - Dz_prev[m]);
-          R[m] = acc * iV;
+          float a = acc[m];
+                    a += 0.5f * (N.H[2][m] - sm.carry[m][t]) - (Dz[m] - Dz_prev[m]);
+          R[m] = a * iV0;
         }
         if (A.rhs) {
-          const long long N = (long long)d.ni * d.nj * d.nk;
+          const long long Nr = (long long)d.ni * d.nj * d.nk;
           const long long ridx = ((long long)p * d.nj + oj) * d.ni + oi;
 #pragma unroll
-          for (int m = 0; m < 5; ++m) A.rhs[m * N + ridx] = adv ? f32_to_f64(R[m]) : 0.0;
+          for (int m = 0; m < 5; ++m) A.rhs[m * Nr + ridx] = adv ? f32_to_f64(R[m]) : 0.0;
         } else if (adv) {
           double qnew[5];
 #pragma unroll
@@ -511,7 +446,7 @@ __global__ void __launch_bounds__(NT, kMinBlocks) k_fused32(const __grid_constan
           float2 shn[NSH];
           shadow_of(c, qnew, shn);
 #pragma unroll
-          for (int m = 0; m < NSH; ++m) A.sout[m * A.Np + pp] = shn[m];
+          for (int m = 0; m < NSH; ++m) A.sout[m][pp] = shn[m];
           if (A.want_rate) {
             const float rho = f64_to_f32(qnew[0]);
             const float ir = f_rcp(rho);
@@ -519,36 +454,54 @@ __global__ void __launch_bounds__(NT, kMinBlocks) k_fused32(const __grid_constan
             const float u = m1 * ir, v = m2 * ir, w = m3 * ir;
             const float pr = c.gm1 * (f64_to_f32(qnew[4] - c.e_inf) - 0.5f * (m1 * u + m2 * v + m3 * w)) + c.p_inf;
             const float a = f_sqrt(c.gamma * pr * ir);
-            float ls = 0.f;            float mr[kMF];
+            float ls = 0.f;
+            float mr[kMF];
             load_record(A.M, pp, mr);
 #pragma unroll
             for (int dir = 0; dir < 3; ++dir) {
               const float sx = mr[3 * dir], sy = mr[3 * dir + 1], sz = mr[3 * dir + 2];
               ls += fabsf(sx * u + sy * v + sz * w) + a * f_sqrt(sx * sx + sy * sy + sz * sz);
             }
-            rate = fmaxf(rate, ls * iV);
+            rate = fmaxf(rate, ls * iV0);
           }
         } else {
 #pragma unroll
           for (int m = 0; m < 5; ++m) A.qout[m][pp] = A.qin[m][pp];
-          A.sout[pp] = P_re(P0, c2);
-          A.sout[A.Np + pp] = P_m12(P0, c2);
-          A.sout[2 * A.Np + pp] = P_m3p(P0, c2);
+          A.sout[0][pp] = P_re(P0, c2);
+          A.sout[1][pp] = P_m12(P0, c2);
+          A.sout[2][pp] = P_m3p(P0, c2);
         }
         if (adv) res += R[0] * R[0];
       }
-      // rotate the zeta registers
+      // (d) eta faces of plane p+1, both of the node's, and its xi and eta part
+      if (inplane) {
+        float qa[5], qb[5], qc[5], qd[5], lo[5], hi[5];
+        load_q(P1, c2 - 2 * H2X, qa);
+        load_q(P1, c2 - H2X, qb);
+        load_q(P1, c2 + H2X, qc);
+        load_q(P1, c2 + 2 * H2X, qd);
+        face_flux(c, E[E_L * NP1 + t - 32], N.lam[1], E[E_N * NP1 + t - 32], N.nu[1], qa, qb, q1, qc, lo);
+        face_flux(c, N.lam[1], E[E_L * NP1 + t + 32], N.nu[1], E[E_N * NP1 + t + 32], qb, q1, qc, qd, hi);
+#pragma unroll
+        for (int m = 0; m < 5; ++m) {
+          float a = ax[m];
+          a += 0.5f * (E[(E_H + m) * NP1 + t + 32] - E[(E_H + m) * NP1 + t - 32]) - (hi[m] - lo[m]);
+          ax[m] = a;
+        }
+      }
+      // rotate the marching state
 #pragma unroll
       for (int m = 0; m < 5; ++m) {
-        Hz_prev[m] = Z0[(Z_HZ + m) * NOUT + o];
+        sm.carry[m][t] = Hz_0[m];
+        Hz_0[m] = N.H[2][m];
         Dz_prev[m] = Dz[m];
         Qz_prev[m] = q0[m];
+        acc[m] = ax[m];
       }
-      Lz = Lz1;
-      Nz = Nz1;
+      Lz = N.lam[2];
+      Nz = N.nu[2];
+      iV0 = N.iV;
     }
-    // no barrier here: the next iteration's phase (a) writes 1/rho of ring slot p+3, which no
-    // thread reads in this iteration; the barrier after it orders the flux rings.
   }
   if (t == 0 && sm.fail != 0) {
     // a wait ran out: give the copies still in flight a bounded time to land before the CTA's
@@ -663,8 +616,8 @@ cudaError_t fused32(const Dims& d, const Consts& c, const float* Mf, const State
     A.qn[m] = qn.q[m];
     A.qout[m] = qout.q[m];
   }
-  A.sout = qout.sh;
-  A.Np = d.Np;
+  if (d.Np >= (1LL << 32)) return cudaErrorInvalidValue;
+  for (int m = 0; m < NSH; ++m) A.sout[m] = qout.sh + m * d.Np;
   A.rhs = rhs_flat;
   A.sc = sc;
   A.alpha = alpha;
