@@ -85,16 +85,18 @@ __global__ void __launch_bounds__(BX* BY) k_sensor_df(Dims d, Work64 w) {
 // gradients by the chain rule, Smagorinsky eddy viscosity, stresses and heat flux, the transformed
 // fluxes H^dir = E^dir - S^dir_j F_j and the pressure sensors of the nodes within one layer of the
 // real region, and the pair copy of Q on every padded node; at stage 1 also the CFL rate of Q^n
-// (block max, one atomic per block).  A block of 32 x VY threads marches along k; per plane every
-// thread forms u, v, w, T, p of its node into shared memory (three planes in turn), and the inner
-// 30 x (VY - 2) nodes form their fluxes from the neighbours there, so the primitives and the
-// viscosity never reach HBM (360 bytes per node against 568 for a nodal and a viscous pass).
+// (block max, one atomic per block).  A block of VY - 2 warps marches along k; per plane every thread
+// forms u, v, w, T, p of its node into shared memory (three planes in turn; the first and the last
+// warp also of the tile's halo rows), and 30 x (VY - 2) nodes form their fluxes from the neighbours
+// there, so the primitives and the viscosity never reach HBM (360 bytes per node against 568 for a
+// nodal and a viscous pass).
 // The momentum and energy fluxes are contracted as H_m = m_m U + S_j P_jm, P = p I - tau, and
 // H_e = e U + S_j (u_m P_jm - k dT/dx_j).
-// FP32 issue bounds it: 10.7 ms per launch on 512 x 512 x 360 (the two passes before: 11.4); 32 x 10
-// at three blocks per SM as 32 x 16 at two, 11.3 for 32 x 8 at four, 10.9 for 32 x 12 at two with 80
-// registers.  Split arrivals instead of a barrier per plane (warps drifting by a plane): 12.0.
-constexpr int VX = 32, VY = 10;
+// FP32 issue bounds it: 10.2 ms per launch on 512 x 512 x 360 (the two passes before: 11.4) with 8
+// rows at three blocks per SM (80 registers); at four (64, spills) 11.2, at two (128) 11.5; 14 rows at
+// two 10.1, but slower on small grids.  Warps for the halo rows that then idle through the fluxes:
+// 10.7.  Split arrivals instead of a barrier per plane (warps drifting by a plane): 12.0.
+constexpr int VX = 32, VY = 10;      // nodes of the tile with its one-node halo
 
 // Element of a field at a 32-bit byte offset (every field of a pair solver is below 4 GB: its 632
 // bytes per padded node reach the GPU's memory first): the address is a uniform base plus one
@@ -136,23 +138,21 @@ __device__ __forceinline__ dfl sm(const PlaneDF& P, int n, int y, int x) {
   return df_make(t.x, t.y);
 }
 
-__global__ void __launch_bounds__(VX* VY, 3) k_flux_df(const __grid_constant__ StageArgs A) {
+__global__ void __launch_bounds__(VX*(VY - 2), 3) k_flux_df(const __grid_constant__ StageArgs A) {
   __shared__ PlaneDF pl[3];
   const Dims& d = A.d;
   const ConstsDF& c = A.c;
-  const int x = threadIdx.x, y = threadIdx.y;
+  const int x = threadIdx.x, y = threadIdx.y + 1;           // column and row of the tile
   const unsigned by = blockIdx.x / A.nbx, bx = blockIdx.x - by * A.nbx;
-  const int i = (int)bx * (VX - 2) - 2 + x, j = (int)by * (VY - 2) - 2 + y;
+  const int i = (int)bx * (VX - 2) - 2 + x, j0 = (int)by * (VY - 2) - 2, j = j0 + y;
   const int k0 = (int)blockIdx.y * A.kchunk - 1, k1 = min(k0 + A.kchunk, d.nk + 1);   // planes [k0, k1) of -1 .. nk
-  const bool inside = i <= d.ni + 1 && j <= d.nj + 1;      // i, j >= -2 by construction
-  const bool inner = x > 0 && x < VX - 1 && y > 0 && y < VY - 1;
-  const bool out = inner && i <= d.ni && j <= d.nj;        // a node this block forms the fluxes of
-  // nodes whose pair copy of Q this thread writes: the block's own and the outermost ghosts
-  const bool own = inside && (x > 0 || i == -2) && (x < VX - 1 || i == d.ni + 1) && (y > 0 || j == -2) &&
-                   (y < VY - 1 || j == d.nj + 1);
+  const bool out = x > 0 && x < VX - 1 && i <= d.ni && j <= d.nj;   // a node this block forms the fluxes of
+  // the halo row whose primitives the first and the last warp form beside their own
+  const int extra = y == 1 ? 0 : (y == VY - 2 ? VY - 1 : -1);
   double rate = 0.0;
   int s0 = 0, s1 = 1, s2 = 2;                               // slots of planes k - 1, k, k + 1
   const unsigned sk = (unsigned)d.sk * 8u;                  // bytes
+  const unsigned sj = (unsigned)d.sj * 8u;
   unsigned p = (unsigned)pidx(d, i, j, k0 - 2) * 8u;        // (k0 - 2 may lie below the array: only p + sk is read then)
   for (int k = k0 - 2; k < k1; ++k, p += sk) {
     dfl S[3][3] = {}, iV = {}, Delta = {};
@@ -165,29 +165,36 @@ __global__ void __launch_bounds__(VX* VY, 3) k_flux_df(const __grid_constant__ S
       iV = ldo(A.invV, p);
       Delta = ldo(A.Delta, p);
     }
-    if (inside) {
-      // primitives of plane k + 1
-      const unsigned pn = p + sk;
-      const dfl rho = df_of(ldo(A.q[0], pn)), m1 = df_of(ldo(A.q[1], pn)), m2 = df_of(ldo(A.q[2], pn)), m3 = df_of(ldo(A.q[3], pn)),
-                e = df_of(ldo(A.q[4], pn));
-      if (own && ((k + 1 >= k0 && k + 1 < k1) || k + 1 == -2 || k + 1 == d.nk + 1)) {
-        sto(A.qdf[0], pn, rho);
-        sto(A.qdf[1], pn, m1);
-        sto(A.qdf[2], pn, m2);
-        sto(A.qdf[3], pn, m3);
-        sto(A.qdf[4], pn, e);
+    // primitives of plane k + 1 in the thread's row and, at the tile's edge, in the halo row
+#pragma unroll 1
+    for (int row = y;; row = extra) {
+      const int jr = j0 + row;
+      if (i <= d.ni + 1 && jr <= d.nj + 1) {               // i, j >= -2 by construction
+        const unsigned pn = p + sk + (unsigned)(row - y) * sj;
+        const dfl rho = df_of(ldo(A.q[0], pn)), m1 = df_of(ldo(A.q[1], pn)), m2 = df_of(ldo(A.q[2], pn)),
+                  m3 = df_of(ldo(A.q[3], pn)), e = df_of(ldo(A.q[4], pn));
+        // the pair copy of Q: the block's own nodes and the outermost ghosts
+        if ((x > 0 || i == -2) && (x < VX - 1 || i == d.ni + 1) && (row > 0 || jr == -2) && (row < VY - 1 || jr == d.nj + 1) &&
+            ((k + 1 >= k0 && k + 1 < k1) || k + 1 == -2 || k + 1 == d.nk + 1)) {
+          sto(A.qdf[0], pn, rho);
+          sto(A.qdf[1], pn, m1);
+          sto(A.qdf[2], pn, m2);
+          sto(A.qdf[3], pn, m3);
+          sto(A.qdf[4], pn, e);
+        }
+        const dfl ir = df_rcp(rho);
+        const dfl u = df_mul(m1, ir), v = df_mul(m2, ir), w = df_mul(m3, ir);
+        const dfl ke = df_fma(m3, w, df_fma(m2, v, df_mul(m1, u)));         // rho |u|^2
+        const dfl pr = df_sub(df_mul(e, c.gm1), df_mul(ke, c.gm1_half));    // (gamma-1)(e - rho|u|^2/2)
+        const dfl T = df_mul(df_mul(pr, c.gamma), ir);
+        PlaneDF& P = pl[s2];
+        P.f[0][row][x] = make_float2(u.hi, u.lo);
+        P.f[1][row][x] = make_float2(v.hi, v.lo);
+        P.f[2][row][x] = make_float2(w.hi, w.lo);
+        P.f[3][row][x] = make_float2(T.hi, T.lo);
+        P.f[4][row][x] = make_float2(pr.hi, pr.lo);
       }
-      const dfl ir = df_rcp(rho);
-      const dfl u = df_mul(m1, ir), v = df_mul(m2, ir), w = df_mul(m3, ir);
-      const dfl ke = df_fma(m3, w, df_fma(m2, v, df_mul(m1, u)));         // rho |u|^2
-      const dfl pr = df_sub(df_mul(e, c.gm1), df_mul(ke, c.gm1_half));    // (gamma-1)(e - rho|u|^2/2)
-      const dfl T = df_mul(df_mul(pr, c.gamma), ir);
-      PlaneDF& P = pl[s2];
-      P.f[0][y][x] = make_float2(u.hi, u.lo);
-      P.f[1][y][x] = make_float2(v.hi, v.lo);
-      P.f[2][y][x] = make_float2(w.hi, w.lo);
-      P.f[3][y][x] = make_float2(T.hi, T.lo);
-      P.f[4][y][x] = make_float2(pr.hi, pr.lo);
+      if (row != y || extra < 0) break;
     }
     if (k >= k0) {
       // plane k + 1 before its neighbours read it one iteration later, and every thread done with
@@ -270,12 +277,12 @@ __global__ void __launch_bounds__(VX* VY, 3) k_flux_df(const __grid_constant__ S
   }
   if (A.rate_max) {
     // block max -> one atomic per block (non-negative doubles order like their bits)
-    __shared__ double redm[VY];
+    __shared__ double redm[VY - 2];
     for (int o = 16; o > 0; o >>= 1) rate = fmax(rate, __shfl_xor_sync(0xffffffffu, rate, o));
-    if (x == 0) redm[y] = rate;
+    if (x == 0) redm[y - 1] = rate;
     __syncthreads();
-    if (x == 0 && y == 0) {
-      for (int n = 1; n < VY; ++n) rate = fmax(rate, redm[n]);
+    if (x == 0 && y == 1) {
+      for (int n = 1; n < VY - 2; ++n) rate = fmax(rate, redm[n]);
       if (rate > 0.0)
         atomicMax(reinterpret_cast<unsigned long long*>(A.rate_max), (unsigned long long)__double_as_longlong(rate));
     }
@@ -498,7 +505,7 @@ cudaError_t flux_df(const Dims& d, const Consts& c, const DFMetrics& M, const Wo
   const long long tiles = (long long)A.nbx * ((d.nj + VY - 1) / (VY - 2));
   A.kchunk = march_kchunk(tiles, d.nk + 2);
   const dim3 gr((unsigned)tiles, (d.nk + 1 + A.kchunk) / A.kchunk);
-  k_flux_df<<<gr, dim3(VX, VY), 0, st>>>(A);
+  k_flux_df<<<gr, dim3(VX, VY - 2), 0, st>>>(A);
   return cudaGetLastError();
 }
 
