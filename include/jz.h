@@ -206,8 +206,12 @@ int jz_rk_step(jz_solver* s, int nsteps, jz_step_stats* out);
  * p~ the pressure on the cylinder r = r_obs (linear in r between the
  * bracketing grid lines), w_ik = r_obs dtheta dx_i (trapezoid in x).
  * The forward sweep stores Q^n every ckpt_every steps; the reverse sweep
- * recomputes each checkpoint segment and each step's five stage states and
- * runs the transposed stage, boundary-condition and ghost-fill kernels.
+ * recomputes each checkpoint segment (the last one is still there) with
+ * every step's five stage states and runs the transposed stage,
+ * boundary-condition and ghost-fill kernels.  Where the stage states of all
+ * steps take less than half of the free device memory they are all kept and
+ * nothing is recomputed (ckpt_every then has no effect); the results do not
+ * depend on the interval.
  * Writes J (*J_out, host) and dJ/dA (grad_out [32], host).  The solver's
  * state and parameters are unchanged on return; device memory for the
  * checkpoints and adjoint arrays is allocated for the call.

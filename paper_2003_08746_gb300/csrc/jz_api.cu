@@ -880,11 +880,10 @@ int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ck
   // The adjoint arrays start at zero; the states are written before they are read.
   DevMem mem;
   mem.used_by(s->st);
-  const int C = ckpt_every;
-  const int nseg = (nsteps + C - 1) / C;
+  int C = 0, nseg = 0;
   const size_t Np = (size_t)d.Np;
   jz::Adj64 a;
-  std::vector<jz::State> ck(nseg), seg(C + 1), stg(4), kept;
+  std::vector<jz::State> ck, seg, stg, kept;
   jz::State wa{}, wb{};
   double* wdev = nullptr;
   // lays the arrays out from base and returns the number of doubles (base null: count only); the
@@ -928,27 +927,40 @@ int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ck
     AS(ck); AS(seg); AS(stg); AS(kept);
     return at;
   };
-  // Where memory allows, the segment recompute keeps the four intermediate stage states of
-  // every step, so that the reverse sweep does not recompute them step by step (one forward
-  // step per step less).  Kept only if they take under half of the device memory that the rest leaves.
-  const size_t base_bytes = layout(nullptr) * sizeof(double);
-  {
-    size_t free_b = 0, total_b = 0;
-    const size_t need = (size_t)C * 4 * 5 * sizeof(double) * Np;
-    if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) {
-      if (base_bytes < free_b && need < (free_b - base_bytes) / 2) kept.resize((size_t)C * 4);
-    } else {
-      cudaGetLastError();
-    }
+  // Segments of `steps` steps, with or without the four intermediate stage states of every step of a
+  // segment; returns the bytes.
+  auto plan = [&](int steps, bool keep) {
+    C = std::min(steps, nsteps);
+    nseg = (nsteps + C - 1) / C;
+    ck.resize(nseg - 1);
+    seg.resize(C + 1);
+    kept.resize(keep ? (size_t)C * 4 : 0);
+    stg.resize(keep ? 0 : 4);
+    return layout(nullptr) * sizeof(double);
+  };
+  // Where memory allows, the stage states of a segment are kept, so that the reverse sweep does not
+  // recompute them step by step (one forward step per step less); and where those of all steps take
+  // under half of the free device memory, there is one segment and nothing is recomputed at all.
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    cudaGetLastError();
+    free_b = 0;
   }
   double* base = nullptr;
-  cudaError_t e = cudaMalloc(&base, layout(nullptr) * sizeof(double));
-  if (e != cudaSuccess && !kept.empty()) {        // not enough after all: run without them
-    cudaGetLastError();
-    kept.clear();
-    e = cudaMalloc(&base, base_bytes);
+  cudaError_t e = cudaErrorMemoryAllocation;
+  auto attempt = [&](size_t bytes) {
+    e = cudaMalloc(&base, bytes);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess;
+  };
+  bool planned = false;
+  if (const size_t all = plan(nsteps, true); all < free_b / 2) planned = attempt(all);
+  if (!planned) {
+    const size_t rest = plan(ckpt_every, false), with = plan(ckpt_every, true);
+    if (rest < free_b && with - rest < (free_b - rest) / 2) planned = attempt(with);
   }
-  if (e != cudaSuccess) return fail(alloc_status(e), "jz_adjoint_step: device allocation failed: %s", cudaGetErrorString(e));
+  if (!planned) planned = attempt(plan(ckpt_every, false));
+  if (!planned) return fail(alloc_status(e), "jz_adjoint_step: device allocation failed: %s", cudaGetErrorString(e));
   mem.blocks.push_back(base);
   layout(base);
   JZ_CK(cudaMemsetAsync(base, 0, zeroed * sizeof(double), s->st));
@@ -986,25 +998,32 @@ int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ck
   // forward sweep with checkpoints; J accumulated on the device
   int r = copy_state(s, wa, s->qn);
   if (r) return r;
+  // One step of a segment, its stage states kept where there is room.
+  auto segment_step = [&](int q, int n) {
+    return kept.empty() ? fwd_step(s, seg[q], seg[q + 1], t0 + n * dt, dt)
+                        : fwd_step_keep(s, seg[q], seg[q + 1], t0 + n * dt, dt, &kept[(size_t)q * 4]);
+  };
+  const int last = (nseg - 1) * C;              // first step of the last segment: advanced in place, not again
   for (int n = 0; n < nsteps; ++n) {
     if (n % C == 0) {
-      r = copy_state(s, ck[n / C], wa);
+      r = copy_state(s, n < last ? ck[n / C] : seg[0], wa);
       if (r) return r;
     }
-    r = fwd_step(s, wa, wb, t0 + n * dt, dt);
+    r = n < last ? fwd_step(s, wa, wb, t0 + n * dt, dt) : segment_step(n - last, n);
     if (r) return r;
-    JZ_RUN(JZ_PROF_ADJOINT, jz::observer(d, s->c, wb, wdev, j0, beta, dt, a, 0, s->st));
+    JZ_RUN(JZ_PROF_ADJOINT, jz::observer(d, s->c, n < last ? wb : seg[n - last + 1], wdev, j0, beta, dt, a, 0, s->st));
     std::swap(wa, wb);
   }
   // reverse sweep, one checkpoint segment at a time
   for (int sg = nseg - 1; sg >= 0; --sg) {
     const int n0 = sg * C, n1 = std::min(n0 + C, nsteps);
-    r = copy_state(s, seg[0], ck[sg]);
-    if (r) return r;
-    for (int q = 0; q < n1 - n0; ++q) {
-      r = kept.empty() ? fwd_step(s, seg[q], seg[q + 1], t0 + (n0 + q) * dt, dt)
-                       : fwd_step_keep(s, seg[q], seg[q + 1], t0 + (n0 + q) * dt, dt, &kept[(size_t)q * 4]);
+    if (n0 < last) {
+      r = copy_state(s, seg[0], ck[sg]);
       if (r) return r;
+      for (int q = 0; q < n1 - n0; ++q) {
+        r = segment_step(q, n0 + q);
+        if (r) return r;
+      }
     }
     for (int n = n1 - 1; n >= n0; --n) {
       const jz::State& Qn = seg[n - n0];

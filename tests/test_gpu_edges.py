@@ -90,3 +90,29 @@ def test_first_step_rate(jz, case):
     grid.close()
     assert rc == jz.JZ_OK or (case == "tiny" and rc == jz.JZ_ERR_NONFINITE)
     assert abs(st.t - dt) <= 1e-13 * dt
+
+
+# the adjoint's three ways to the stage states: all kept, kept per checkpoint segment, recomputed; which
+# one is taken depends on the free memory, the gradient does not (sums with atomics: 1e-12, as between
+# checkpoint intervals)
+def test_adjoint_with_little_memory(jz):
+    g, prm = W.jet_grid(128, 96, 64), W.jet_params(seed=4)
+    grid = jz.Grid.from_workload(g)
+    s = jz.Solver(grid, prm, jz.JZ_PREC_FP64PAIR)
+    s.set_state(W.jet_state(g) + _noise(g, 3, 1e-3), 0.0)
+    A = np.asarray(prm.forcing_amp)
+    state = 5 * 8 * 132 * 100 * 68                                # bytes of one padded state
+    base = (10 + 5 + 3 * 12 + 2) * state // 5                     # the adjoint arrays
+    n, ck = 12, 4
+    torch.cuda.empty_cache()
+    J0, g0 = jz.jz_adjoint_step(s.h, A, n, ck, 0.75)              # all kept
+    for leave in (base + (n * 5 + 4) * state, base + 20 * state):  # not twice all; not twice a segment's
+        free = torch.cuda.mem_get_info()[0]
+        hold = torch.empty(int(free - leave), dtype=torch.uint8, device="cuda")
+        J, gr = jz.jz_adjoint_step(s.h, A, n, ck, 0.75)
+        del hold
+        torch.cuda.empty_cache()
+        assert abs(J - J0) <= 1e-12 * abs(J0)
+        assert np.abs(gr - g0).max() <= 1e-12 * np.abs(g0).max()
+    s.close()
+    grid.close()
