@@ -331,8 +331,9 @@ __global__ void k_adj_axis(Dims d, Adj64 a) {
     if ((threadIdx.x & 31) == 0) red[m][threadIdx.x >> 5] = x;
   }
   __syncthreads();
+  const double ink = 1.0 / d.nk;
   double add[5];
-  for (int m = 0; m < 5; ++m) add[m] = (red[m][0] + red[m][1] + red[m][2] + red[m][3]) / d.nk;
+  for (int m = 0; m < 5; ++m) add[m] = (red[m][0] + red[m][1] + red[m][2] + red[m][3]) * ink;
   for (int k = threadIdx.x; k < d.nk; k += blockDim.x) {
     const long long p0 = pidx(d, i, 0, k), p1 = pidx(d, i, 1, k);
     for (int m = 0; m < 5; ++m) {
@@ -384,20 +385,20 @@ __global__ void __launch_bounds__(kTPBS) k_adj_inout(Dims d, Consts c, Inflow in
         const double u1 = Q1[1] * ir1;
         const double pr1 = c.gm1 * (Q1[4] - 0.5 * (Q1[1] * Q1[1] + Q1[2] * Q1[2] + Q1[3] * Q1[3]) * ir1);
         const double a1 = sqrt64(c.gamma * pr1 * ir1);
-        const double Rm = u1 - 2.0 * a1 / c.gm1, Rp = ut + 2.0 * 1.0 / c.gm1;
+        const double Rm = u1 - 2.0 * a1 * c.Cp, Rp = ut + 2.0 * 1.0 * c.Cp;
         const double ub = 0.5 * (Rp + Rm), ab = 0.25 * c.gm1 * (Rp - Rm);
         const double rs = isentrope(c, fabs(ab));
         const double rhob = lb[0] + lb[1] * ub + 0.5 * lb[4] * ub * ub;
         const double ubb = lb[1] * rs + lb[4] * rs * ub;
-        const double pbb = lb[4] / c.gm1;
-        double rsb = rhob + pbb * ab * ab / c.gamma;
-        double abb = pbb * 2.0 * rs * ab / c.gamma;
-        abb += rsb * 2.0 * rs / (c.gm1 * ab);
+        const double pbb = lb[4] * c.Cp;
+        double rsb = rhob + pbb * ab * ab * c.p_inf;
+        double abb = pbb * 2.0 * rs * ab * c.p_inf;
+        abb += rsb * 2.0 * rs * (c.Cp * rcp64(ab));
         const double Rpb = 0.5 * ubb + 0.25 * c.gm1 * abb;
         const double Rmb = 0.5 * ubb - 0.25 * c.gm1 * abb;
         utb = Rpb;
         double u1b[3] = {Rmb, 0.0, 0.0};
-        const double a1b = -2.0 * Rmb / c.gm1;
+        const double a1b = -2.0 * Rmb * c.Cp;
         const double p1b = a1b * c.gamma * 0.5 * rcp64(a1) * ir1;
         double q1b[5] = {-p1b * pr1 * ir1, 0, 0, 0, 0};
         prim_bar(c, Q1, u1b, p1b, q1b);
@@ -409,18 +410,18 @@ __global__ void __launch_bounds__(kTPBS) k_adj_inout(Dims d, Consts c, Inflow in
       const long long pi = pidx(d, d.ni - 2, j, k), pb = pidx(d, d.ni - 1, j, k);
       double Qi[5];
       load5(q, pi, Qi);
-      const double rho_i = Qi[0];
-      const double u[3] = {Qi[1] / rho_i, Qi[2] / rho_i, Qi[3] / rho_i};
-      const double p_i = c.gm1 * (Qi[4] - 0.5 * (Qi[1] * u[0] + Qi[2] * u[1] + Qi[3] * u[2]));
-      const double rho = c.p_inf / (c.gm1 * (p_i / (c.gm1 * rho_i)));
+      const double rho_i = Qi[0], ir = rcp64(rho_i);
+      const double u[3] = {Qi[1] * ir, Qi[2] * ir, Qi[3] * ir};
+      const double p_i = c.gm1 * (Qi[4] - 0.5 * (Qi[1] * u[0] + Qi[2] * u[1] + Qi[3] * u[2])), ip = rcp64(p_i);
+      const double rho = c.p_inf * rho_i * ip;
       double lb[5];
       for (int m = 0; m < 5; ++m) lb[m] = a.lam[m][pb];
       const double rhob = lb[0] + lb[1] * u[0] + lb[2] * u[1] + lb[3] * u[2] +
                           0.5 * lb[4] * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
       double ub[3];
       for (int x = 0; x < 3; ++x) ub[x] = lb[1 + x] * rho + lb[4] * rho * u[x];
-      double qb[5] = {rhob * rho / rho_i, 0, 0, 0, 0};
-      const double pib = -rhob * rho / p_i;
+      double qb[5] = {rhob * rho * ir, 0, 0, 0, 0};
+      const double pib = -rhob * rho * ip;
       prim_bar(c, Qi, ub, pib, qb);
       for (int m = 0; m < 5; ++m) {
         a.lam[m][pi] += qb[m];
@@ -467,7 +468,7 @@ __global__ void k_adj_farfield(Dims d, Consts c, GridDev g, State q, Adj64 a) {
   const double p_i = c.gm1 * (Qi[4] - 0.5 * (Qi[1] * ui[0] + Qi[2] * ui[1] + Qi[3] * ui[2]));
   const double a_i = sqrt64(c.gamma * p_i * ir), ia = rcp64(a_i);
   const double un_i = ui[0] * n[0] + ui[1] * n[1] + ui[2] * n[2];
-  const double Rp = un_i + 2.0 * a_i / c.gm1, Rm = -2.0 / c.gm1;
+  const double Rp = un_i + 2.0 * a_i * c.Cp, Rm = -2.0 * c.Cp;
   const double un = 0.5 * (Rp + Rm), ab = 0.25 * c.gm1 * (Rp - Rm);
   const bool out = un > 0.0;
   double ut[3];
@@ -483,15 +484,15 @@ __global__ void k_adj_farfield(Dims d, Consts c, GridDev g, State q, Adj64 a) {
     rhob += lb[1 + x] * ubv[x];
     ubb[x] = lb[1 + x] * rho + lb[4] * rho * ubv[x];
   }
-  const double pbb = lb[4] / c.gm1;
-  rhob += pbb * ab * ab / c.gamma;
-  double abb = pbb * 2.0 * rho * ab / c.gamma;
-  abb += rhob * 2.0 * rho / (c.gm1 * ab);
+  const double pbb = lb[4] * c.Cp;
+  rhob += pbb * ab * ab * c.p_inf;
+  double abb = pbb * 2.0 * rho * ab * c.p_inf;
+  abb += rhob * 2.0 * rho * (c.Cp * rcp64(ab));
   double unb = 0.0;
   for (int x = 0; x < 3; ++x) unb += ubb[x] * n[x];
   const double Rpb = 0.5 * unb + 0.25 * c.gm1 * abb;
   double un_ib = Rpb;
-  const double a_ib = 2.0 * Rpb / c.gm1;
+  const double a_ib = 2.0 * Rpb * c.Cp;
   double uib[3] = {0, 0, 0};
   double p_ib = 0.0;
   double qb[5] = {0, 0, 0, 0, 0};

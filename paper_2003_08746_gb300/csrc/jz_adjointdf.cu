@@ -6,7 +6,8 @@
 // adjoints and the observer); the intermediate adjoint arrays the transposed passes pass to one
 // another (alpha dt lambda / V, the face coefficients and sensor adjoints, the adjoints of the
 // gradients, of u, mu and rho) are double-float pairs in the same arrays, so the gathers of the
-// transposed nodal pass run on the FP32 pipes.
+// transposed nodal pass run on the FP32 pipes.  Sums and products inside a chain are unnormalized
+// pairs (jz_df.cuh), normalized before they are stored or seed a root or reciprocal.
 #include "jz_adjgather.cuh"
 #include "jz_dfconsts.cuh"
 
@@ -52,30 +53,30 @@ __global__ void k_adj_faces_df(Dims d, ConstsDF c, Work64 w, QDF qdf, Adj64 a) {
     const long long sd = s[dir];
     const dfl nu0 = ld(w.nu[dir], p), nu1 = ld(w.nu[dir], p + sd);
     const bool first = df_ge(nu0, nu1);
-    const dfl eps2 = df_mul(c.kappa2, first ? nu0 : nu1);
-    const dfl k4 = df_sub(c.kappa4, eps2);
+    const dfl eps2 = df_mul_l(c.kappa2, first ? nu0 : nu1);
+    const dfl k4 = df_n(df_sub_l(c.kappa4, eps2));
     const bool pos4 = df_gt0(k4);
     const dfl eps4 = pos4 ? k4 : df_from(0.f);
-    const dfl Lf = df_scale(df_add(ld(w.Lam[dir], p), ld(w.Lam[dir], p + sd)), 0.5f);
+    const dfl Lf = df_scale(df_add_l(ld(w.Lam[dir], p), ld(w.Lam[dir], p + sd)), 0.5f);
     dfl lf = df_from(0.f), e2b = df_from(0.f), e4b = df_from(0.f);
     for (int m = 0; m < 5; ++m) {
       const double* Q = qdf.q[m];
       const dfl q0 = ld(Q, p), q1 = ld(Q, p + sd), q2 = ld(Q, p + 2 * sd), qm = ld(Q, p - sd);
-      const dfl d1 = df_sub(q1, q0);
-      const dfl d3 = df_sub(df_add(df_sub(q2, df_mul_f(q1, 3.f)), df_mul_f(q0, 3.f)), qm);
-      const dfl Db = df_sub(ld(a.acc[m], p + sd), ld(a.acc[m], p));
-      lf = df_fma(Db, df_sub(df_mul(eps2, d1), df_mul(eps4, d3)), lf);
-      const dfl DL = df_mul(Db, Lf);
-      e2b = df_fma(DL, d1, e2b);
-      e4b = df_sub(e4b, df_mul(DL, d3));
+      const dfl d1 = df_sub_l(q1, q0);
+      const dfl d3 = df_sub_l(df_add_l(df_sub_l(q2, df_mul_f(q1, 3.f)), df_mul_f(q0, 3.f)), qm);
+      const dfl Db = df_sub_l(ld(a.acc[m], p + sd), ld(a.acc[m], p));
+      lf = df_fma_l(Db, df_sub_l(df_mul_l(eps2, d1), df_mul_l(eps4, d3)), lf);
+      const dfl DL = df_mul_l(Db, Lf);
+      e2b = df_fma_l(DL, d1, e2b);
+      e4b = df_sub_l(e4b, df_mul_l(DL, d3));
     }
-    st(a.ca2[dir], p, df_mul(Lf, eps2));
-    st(a.ca4[dir], p, df_mul(Lf, eps4));
-    if (pos4) e2b = df_sub(e2b, e4b);
-    const dfl nub = df_mul(c.kappa2, e2b);
+    st(a.ca2[dir], p, df_n(df_mul_l(Lf, eps2)));
+    st(a.ca4[dir], p, df_n(df_mul_l(Lf, eps4)));
+    if (pos4) e2b = df_sub_l(e2b, e4b);
+    const dfl nub = df_n(df_mul_l(c.kappa2, e2b));
     st(a.nb0[dir], p, first ? nub : df_from(0.f));
     st(a.nb1[dir], p, first ? df_from(0.f) : nub);
-    st(a.lfh[dir], p, df_scale(lf, 0.5f));
+    st(a.lfh[dir], p, df_scale(df_n(lf), 0.5f));
   }
 }
 
@@ -84,7 +85,9 @@ __global__ void k_adj_faces_df(Dims d, ConstsDF c, Work64 w, QDF qdf, Adj64 a) {
 // stresses, heat flux and sensors, in double-float arithmetic on the pair intermediates the pair
 // passes regenerated (u, v, w, T, p, mu, the pair copies of Q and of the metrics).  Nodes within
 // one layer of the real region.
-__global__ void k_adj_visc_df(Dims d, ConstsDF c, DFMetrics M, Work64 w, QDF qdf, Adj64 a) {
+// Four 128-thread blocks per SM (128 registers); three (168) or six (80) are 3% slower.
+constexpr int kTPBV = 128;
+__global__ void __launch_bounds__(kTPBV, 4) k_adj_visc_df(Dims d, ConstsDF c, DFMetrics M, Work64 w, QDF qdf, Adj64 a) {
   int i, j, k;
   if (!plane_node(-1, d.ni + 2, d.nj + 2, i, j, k)) return;
   const long long p = pidx(d, i, j, k);
@@ -92,7 +95,7 @@ __global__ void k_adj_visc_df(Dims d, ConstsDF c, DFMetrics M, Work64 w, QDF qdf
   // adjoint of H^dir (components 1..4 carry the viscous flux)
   dfl Hb[3][4];
   for (int dir = 0; dir < 3; ++dir)
-    for (int m = 0; m < 4; ++m) Hb[dir][m] = df_scale(df_sub(ld(a.acc[m + 1], p - s[dir]), ld(a.acc[m + 1], p + s[dir])), 0.5f);
+    for (int m = 0; m < 4; ++m) Hb[dir][m] = df_scale(df_sub_l(ld(a.acc[m + 1], p - s[dir]), ld(a.acc[m + 1], p + s[dir])), 0.5f);
   // forward viscous quantities
   const double* f[4] = {w.u, w.v, w.w, w.T};
   dfl S[3][3];
@@ -102,30 +105,30 @@ __global__ void k_adj_visc_df(Dims d, ConstsDF c, DFMetrics M, Work64 w, QDF qdf
   dfl L[4][3];
   for (int n = 0; n < 4; ++n) {
     dfl dd[3];
-    for (int dir = 0; dir < 3; ++dir) dd[dir] = df_scale(df_sub(ld(f[n], p + s[dir]), ld(f[n], p - s[dir])), 0.5f);
+    for (int dir = 0; dir < 3; ++dir) dd[dir] = df_scale(df_sub_l(ld(f[n], p + s[dir]), ld(f[n], p - s[dir])), 0.5f);
     for (int jj = 0; jj < 3; ++jj)
-      L[n][jj] = df_mul(iV, df_fma(S[2][jj], dd[2], df_fma(S[1][jj], dd[1], df_mul(S[0][jj], dd[0]))));
+      L[n][jj] = df_n(df_mul_l(iV, df_fma_l(S[2][jj], dd[2], df_fma_l(S[1][jj], dd[1], df_mul_l(S[0][jj], dd[0])))));
   }
   dfl Sij[3][3];
   for (int x = 0; x < 3; ++x)
-    for (int y = 0; y < 3; ++y) Sij[x][y] = df_scale(df_add(L[x][y], L[y][x]), 0.5f);
-  const dfl div = df_add(df_add(Sij[0][0], Sij[1][1]), Sij[2][2]);
+    for (int y = 0; y < 3; ++y) Sij[x][y] = df_scale(df_add_l(L[x][y], L[y][x]), 0.5f);
+  const dfl div = df_add_l(df_add_l(Sij[0][0], Sij[1][1]), Sij[2][2]);
   dfl SS = df_from(0.f);
   for (int x = 0; x < 3; ++x)
-    for (int y = 0; y < 3; ++y) SS = df_fma(Sij[x][y], Sij[x][y], SS);
-  const dfl Smod = df_sqrt(df_scale(SS, 2.f));
+    for (int y = 0; y < 3; ++y) SS = df_fma_l(Sij[x][y], Sij[x][y], SS);
+  const dfl Smod = df_sqrt(df_n(df_scale(SS, 2.f)));
   const dfl mu = ld(w.mu, p);
-  const dfl csd = df_mul(c.C_s, df_load(M.Delta, p));
-  const dfl cs2 = df_mul(csd, csd);
+  const dfl csd = df_mul_l(c.C_s, df_load(M.Delta, p));
+  const dfl cs2 = df_mul_l(csd, csd);
   const dfl rho = ld(qdf.q[0], p);
-  const dfl mu_sgs = df_mul(df_mul(rho, cs2), Smod);
-  const dfl mu_eff = df_add(mu, mu_sgs);
-  const dfl k_eff = df_add(df_mul(mu, c.k_lam), df_mul(mu_sgs, c.k_sgs));
-  const dfl d3 = df_mul(div, c.third);
+  const dfl mu_sgs = df_n(df_mul_l(df_mul_l(rho, cs2), Smod));
+  const dfl mu_eff = df_add_l(mu, mu_sgs);
+  const dfl k_eff = df_add_l(df_mul_l(mu, c.k_lam), df_mul_l(mu_sgs, c.k_sgs));
+  const dfl d3 = df_mul_l(div, c.third);
   const dfl m2 = df_scale(mu_eff, 2.f);
   dfl dev[3][3];                                       // S_ij - delta_ij div/3
   for (int x = 0; x < 3; ++x)
-    for (int y = 0; y < 3; ++y) dev[x][y] = x == y ? df_sub(Sij[x][y], d3) : Sij[x][y];
+    for (int y = 0; y < 3; ++y) dev[x][y] = x == y ? df_sub_l(Sij[x][y], d3) : Sij[x][y];
   const dfl vel[3] = {ld(w.u, p), ld(w.v, p), ld(w.w, p)};
   // reverse: F^dir_m = S^dir_j F_j,m ; H = E - F
   dfl taub[3][3], ubd[3], keb = df_from(0.f), L3b[3];
@@ -137,54 +140,54 @@ __global__ void k_adj_visc_df(Dims d, ConstsDF c, DFMetrics M, Work64 w, QDF qdf
   for (int jj = 0; jj < 3; ++jj) {
     dfl Fb[4];
     for (int m = 0; m < 4; ++m)
-      Fb[m] = df_neg(df_fma(S[2][jj], Hb[2][m], df_fma(S[1][jj], Hb[1][m], df_mul(S[0][jj], Hb[0][m]))));
-    for (int x = 0; x < 3; ++x) taub[x][jj] = df_add(taub[x][jj], Fb[x]);
+      Fb[m] = df_neg(df_fma_l(S[2][jj], Hb[2][m], df_fma_l(S[1][jj], Hb[1][m], df_mul_l(S[0][jj], Hb[0][m]))));
+    for (int x = 0; x < 3; ++x) taub[x][jj] = df_add_l(taub[x][jj], Fb[x]);
     const dfl e = Fb[3];
     for (int x = 0; x < 3; ++x) {
-      ubd[x] = df_fma(e, df_mul(m2, dev[x][jj]), ubd[x]);         // e tau_x,jj
-      taub[x][jj] = df_fma(e, vel[x], taub[x][jj]);
+      ubd[x] = df_fma_l(e, df_mul_l(m2, dev[x][jj]), ubd[x]);         // e tau_x,jj
+      taub[x][jj] = df_fma_l(e, vel[x], taub[x][jj]);
     }
-    keb = df_fma(e, L[3][jj], keb);
-    L3b[jj] = df_fma(e, k_eff, L3b[jj]);
+    keb = df_fma_l(e, L[3][jj], keb);
+    L3b[jj] = df_fma_l(e, k_eff, L3b[jj]);
   }
   dfl mueb = df_from(0.f), Sijb[3][3], tr = df_from(0.f);
   for (int x = 0; x < 3; ++x)
     for (int y = 0; y < 3; ++y) {
-      mueb = df_fma(taub[x][y], df_scale(dev[x][y], 2.f), mueb);
-      Sijb[x][y] = df_mul(m2, taub[x][y]);
+      mueb = df_fma_l(taub[x][y], df_scale(dev[x][y], 2.f), mueb);
+      Sijb[x][y] = df_mul_l(m2, taub[x][y]);
     }
-  for (int x = 0; x < 3; ++x) tr = df_add(tr, taub[x][x]);
-  const dfl divb = df_neg(df_mul(df_mul(mu_eff, df_scale(c.third, 2.f)), tr));
-  for (int x = 0; x < 3; ++x) Sijb[x][x] = df_add(Sijb[x][x], divb);
-  const dfl mub = df_add(df_mul(keb, c.k_lam), mueb);
-  const dfl musb = df_add(df_mul(keb, c.k_sgs), mueb);
-  const dfl rhob = df_mul(df_mul(musb, cs2), Smod);
-  const dfl Smodb = df_mul(df_mul(musb, rho), cs2);
-  const dfl SSb = df_gt0(Smod) ? df_mul(Smodb, df_rcp(Smod)) : df_from(0.f);
+  for (int x = 0; x < 3; ++x) tr = df_add_l(tr, taub[x][x]);
+  const dfl divb = df_neg(df_mul_l(df_mul_l(mu_eff, df_scale(c.third, 2.f)), tr));
+  for (int x = 0; x < 3; ++x) Sijb[x][x] = df_add_l(Sijb[x][x], divb);
+  const dfl mub = df_add_l(df_mul_l(keb, c.k_lam), mueb);
+  const dfl musb = df_add_l(df_mul_l(keb, c.k_sgs), mueb);
+  const dfl rhob = df_mul_l(df_mul_l(musb, cs2), Smod);
+  const dfl Smodb = df_mul_l(df_mul_l(musb, rho), cs2);
+  const dfl SSb = df_gt0(Smod) ? df_mul_l(Smodb, df_rcp(Smod)) : df_from(0.f);
   for (int x = 0; x < 3; ++x)
-    for (int y = 0; y < 3; ++y) Sijb[x][y] = df_fma(df_scale(Sij[x][y], 2.f), SSb, Sijb[x][y]);
+    for (int y = 0; y < 3; ++y) Sijb[x][y] = df_fma_l(df_scale(Sij[x][y], 2.f), SSb, Sijb[x][y]);
   dfl Lb[4][3];
   for (int x = 0; x < 3; ++x)
-    for (int y = 0; y < 3; ++y) Lb[x][y] = df_scale(df_add(Sijb[x][y], Sijb[y][x]), 0.5f);
+    for (int y = 0; y < 3; ++y) Lb[x][y] = df_scale(df_add_l(Sijb[x][y], Sijb[y][x]), 0.5f);
   for (int y = 0; y < 3; ++y) Lb[3][y] = L3b[y];
   for (int n = 0; n < 4; ++n)
     for (int dir = 0; dir < 3; ++dir)
-      st(a.G[n][dir], p, df_mul(iV, df_fma(S[dir][2], Lb[n][2], df_fma(S[dir][1], Lb[n][1], df_mul(S[dir][0], Lb[n][0])))));
-  for (int x = 0; x < 3; ++x) st(a.ubd[x], p, ubd[x]);
-  st(a.mub, p, mub);
-  st(a.rhob, p, rhob);
+      st(a.G[n][dir], p, df_n(df_mul_l(iV, df_fma_l(S[dir][2], Lb[n][2], df_fma_l(S[dir][1], Lb[n][1], df_mul_l(S[dir][0], Lb[n][0]))))));
+  for (int x = 0; x < 3; ++x) st(a.ubd[x], p, df_n(ubd[x]));
+  st(a.mub, p, df_n(mub));
+  st(a.rhob, p, df_n(rhob));
   // pressure sensor nu = |N| / Dn
   const dfl pc2 = df_scale(ld(w.p, p), 2.f);
   for (int dir = 0; dir < 3; ++dir) {
-    const dfl nub = df_add(ld(a.nb0[dir], p), ld(a.nb1[dir], p - s[dir]));
-    const dfl sum = df_add(ld(w.p, p + s[dir]), ld(w.p, p - s[dir]));
-    const dfl N = df_sub(sum, pc2), Dn = df_add(sum, pc2);
+    const dfl nub = df_add_l(ld(a.nb0[dir], p), ld(a.nb1[dir], p - s[dir]));
+    const dfl sum = df_add_l(ld(w.p, p + s[dir]), ld(w.p, p - s[dir]));
+    const dfl N = df_n(df_sub_l(sum, pc2)), Dn = df_n(df_add_l(sum, pc2));
     const dfl iD = df_rcp(Dn);
-    const dfl nu = df_mul(df_abs(N), iD);
+    const dfl nu = df_mul_l(df_abs(N), iD);
     const float sg = N.hi > 0.f ? 1.f : (N.hi < 0.f ? -1.f : 0.f);
-    const dfl nbD = df_mul(nub, iD);
-    st(a.cpm[dir], p, df_mul(nbD, df_sub(df_from(sg), nu)));
-    st(a.c0[dir], p, df_mul(nbD, df_scale(df_add(df_from(sg), nu), -2.f)));
+    const dfl nbD = df_mul_l(nub, iD);
+    st(a.cpm[dir], p, df_n(df_mul_l(nbD, df_sub_l(df_from(sg), nu))));
+    st(a.c0[dir], p, df_n(df_mul_l(nbD, df_scale(df_add_l(df_from(sg), nu), -2.f))));
   }
 }
 
@@ -219,20 +222,20 @@ __device__ __forceinline__ void nodal_gathers_df(const Adj64& a, const PaddedNod
     dfl v = n < 3 ? nb(a.ubd[n], 0, 0) : df_from(0.f);
 #pragma unroll
     for (int dir = 0; dir < 3; ++dir)
-      v = df_add(v, df_scale(df_sub(nb(a.G[n][dir], dir, -1), nb(a.G[n][dir], dir, 1)), 0.5f));
+      v = df_add_l(v, df_scale(df_sub_l(nb(a.G[n][dir], dir, -1), nb(a.G[n][dir], dir, 1)), 0.5f));
     G.fb[n] = v;
   }
   G.pb = df_from(0.f);
 #pragma unroll
   for (int dir = 0; dir < 3; ++dir)
-    G.pb = df_add(G.pb, df_add(df_add(nb(a.c0[dir], 0, 0), nb(a.cpm[dir], dir, -1)),
+    G.pb = df_add_l(G.pb, df_add_l(df_add_l(nb(a.c0[dir], 0, 0), nb(a.cpm[dir], dir, -1)),
                                nb(a.cpm[dir], dir, 1)));
 #pragma unroll
   for (int dir = 0; dir < 3; ++dir) {
 #pragma unroll
     for (int m = 0; m < 5; ++m)
-      G.Eb[dir][m] = df_scale(df_sub(nb(a.acc[m], dir, -1), nb(a.acc[m], dir, 1)), 0.5f);
-    G.Lamb[dir] = df_add(nb(a.lfh[dir], 0, 0), nb(a.lfh[dir], dir, -1));
+      G.Eb[dir][m] = df_scale(df_sub_l(nb(a.acc[m], dir, -1), nb(a.acc[m], dir, 1)), 0.5f);
+    G.Lamb[dir] = df_add_l(nb(a.lfh[dir], 0, 0), nb(a.lfh[dir], dir, -1));
   }
 #pragma unroll
   for (int m = 0; m < 5; ++m) G.qb[m] = df_from(0.f);
@@ -249,26 +252,27 @@ __device__ __forceinline__ void nodal_gathers_df(const Adj64& a, const PaddedNod
       const dfl am2 = nb(a.acc[m], dir, -2), am1 = nb(a.acc[m], dir, -1),
                 a0 = nb(a.acc[m], 0, 0), ap1 = nb(a.acc[m], dir, 1),
                 ap2 = nb(a.acc[m], dir, 2);
-      const dfl D0 = df_sub(am1, am2), D1 = df_sub(a0, am1), D2 = df_sub(ap1, a0), D3 = df_sub(ap2, ap1);
+      const dfl D0 = df_sub_l(am1, am2), D1 = df_sub_l(a0, am1), D2 = df_sub_l(ap1, a0), D3 = df_sub_l(ap2, ap1);
       // -D0 c4(n-2) + D1 (c2(n-1) + 3 c4(n-1)) - D2 (c2(n) + 3 c4(n)) + D3 c4(n+1)
-      dfl v = df_sub(df_mul(D3, c4[3]), df_mul(D0, c4[0]));
-      v = df_fma(D1, df_add(c2[1], df_mul_f(c4[1], 3.f)), v);
-      v = df_sub(v, df_mul(D2, df_add(c2[2], df_mul_f(c4[2], 3.f))));
-      G.qb[m] = df_add(G.qb[m], v);
+      dfl v = df_sub_l(df_mul_l(D3, c4[3]), df_mul_l(D0, c4[0]));
+      v = df_fma_l(D1, df_add_l(c2[1], df_mul_f(c4[1], 3.f)), v);
+      v = df_sub_l(v, df_mul_l(D2, df_add_l(c2[2], df_mul_f(c4[2], 3.f))));
+      G.qb[m] = df_add_l(G.qb[m], v);
     }
   }
-  G.qb[0] = df_add(G.qb[0], nb(a.rhob, 0, 0));
+  G.qb[0] = df_add_l(G.qb[0], nb(a.rhob, 0, 0));
   G.mub = nb(a.mub, 0, 0);
 }
 
 // Transposed nodal pass (jz_adjoint.cu, k_adj_nodal) for a pair-form solver: the gathers, then
 // the reverse of the anisotropic spectral radii, the inviscid fluxes, Sutherland's law and the
 // primitives, all in double-float arithmetic (the gathers on the pair adjoint arrays).
-// Every padded node.  Issue and load latency bound it at the 12 warps per SM that 168 registers
-// leave: 0.21 ms per launch on 128 x 96 x 64, against 0.29 with a bounds check and 64-bit indices for
-// each of the ~140 gathers (more than half of its 6770 instructions per node).
+// Every padded node.  Issue and load latency bound it at the 16 warps per SM that 128 registers
+// leave (a few spilled; three blocks at 168 registers 4% slower, two at 224 20%): 0.17 ms per launch on
+// 128 x 96 x 64, against 0.29 with a bounds check and 64-bit indices for each of the ~140 gathers (more
+// than half of its 6770 instructions per node) and every pair normalized.
 constexpr int kTPBN = 128;
-__global__ void __launch_bounds__(kTPBN, 3) k_adj_nodal_df(const __grid_constant__ Dims d, const __grid_constant__ ConstsDF c,
+__global__ void __launch_bounds__(kTPBN, 4) k_adj_nodal_df(const __grid_constant__ Dims d, const __grid_constant__ ConstsDF c,
                                                            const __grid_constant__ DFMetrics M,
                                                            const __grid_constant__ QDF qdf,
                                                            const __grid_constant__ Adj64 a) {
@@ -291,20 +295,20 @@ __global__ void __launch_bounds__(kTPBN, 3) k_adj_nodal_df(const __grid_constant
   for (int m = 0; m < 5; ++m) Q[m] = ld(qdf.q[m], p);
   const dfl rho = Q[0];
   const dfl ir = df_rcp(rho);
-  const dfl u[3] = {df_mul(Q[1], ir), df_mul(Q[2], ir), df_mul(Q[3], ir)};
-  const dfl pr = df_mul(c.gm1, df_sub(Q[4], df_scale(df_fma(Q[3], u[2], df_fma(Q[2], u[1], df_mul(Q[1], u[0]))), 0.5f)));
-  const dfl T = df_mul(df_mul(c.gamma, pr), ir);
+  const dfl u[3] = {df_mul_l(Q[1], ir), df_mul_l(Q[2], ir), df_mul_l(Q[3], ir)};
+  const dfl pr = df_mul_l(c.gm1, df_sub_l(Q[4], df_scale(df_fma_l(Q[3], u[2], df_fma_l(Q[2], u[1], df_mul_l(Q[1], u[0]))), 0.5f)));
+  const dfl T = df_n(df_mul_l(df_mul_l(c.gamma, pr), ir));
   const dfl aa = df_sqrt(T);
-  const dfl iTS = df_rcp(df_add(T, c.S_hat));
-  const dfl mu = df_mul(df_mul(c.mu_sut, df_mul(T, aa)), iTS);
+  const dfl iTS = df_rcp(df_n(df_add_l(T, c.S_hat)));
+  const dfl mu = df_mul_l(df_mul_l(c.mu_sut, df_mul_l(T, aa)), iTS);
   dfl Sv[3][3], Smag[3], U[3], lam[3];
 #pragma unroll
   for (int dir = 0; dir < 3; ++dir) {
 #pragma unroll
     for (int cc = 0; cc < 3; ++cc) Sv[dir][cc] = df_load(M.S[3 * dir + cc], p);
     Smag[dir] = df_load(M.Smag[dir], p);
-    U[dir] = df_fma(Sv[dir][2], u[2], df_fma(Sv[dir][1], u[1], df_mul(Sv[dir][0], u[0])));
-    lam[dir] = df_fma(aa, Smag[dir], df_abs(U[dir]));
+    U[dir] = df_n(df_fma_l(Sv[dir][2], u[2], df_fma_l(Sv[dir][1], u[1], df_mul_l(Sv[dir][0], u[0]))));
+    lam[dir] = df_n(df_fma_l(aa, Smag[dir], df_abs(U[dir])));
   }
   // anisotropic scaling Lambda_d = lam_d + lo_d (hi_e + hi_f)
   const dfl Lamb[3] = {G.Lamb[0], G.Lamb[1], G.Lamb[2]};
@@ -316,7 +320,7 @@ __global__ void __launch_bounds__(kTPBN, 3) k_adj_nodal_df(const __grid_constant
       if (c.sigma_is_two_thirds) {
         df_cbrt_pair(lam[dd], lo[dd], hi[dd]);                       // lam^(1/3), lam^(2/3)
         dlo[dd] = df_gt0(lo[dd]) ? df_rcp(df_mul_f(hi[dd], 3.f)) : df_from(0.f);   // d lo / d lam
-        dhi[dd] = df_mul(df_scale(lo[dd], 2.f), dlo[dd]);          // d hi / d lam
+        dhi[dd] = df_mul_l(df_scale(lo[dd], 2.f), dlo[dd]);          // d hi / d lam
       } else {
         // a general exponent through FP64 pow (not on the benchmark path)
         const double l = df_to_f64(lam[dd]);
@@ -334,57 +338,57 @@ __global__ void __launch_bounds__(kTPBN, 3) k_adj_nodal_df(const __grid_constant
     const int e1[3] = {1, 0, 0}, e2[3] = {2, 2, 1};
 #pragma unroll
     for (int dd = 0; dd < 3; ++dd) {
-      lob[dd] = df_fma(Lamb[dd], df_add(hi[e1[dd]], hi[e2[dd]]), lob[dd]);
-      const dfl Ll = df_mul(Lamb[dd], lo[dd]);
-      hib[e1[dd]] = df_add(hib[e1[dd]], Ll);
-      hib[e2[dd]] = df_add(hib[e2[dd]], Ll);
+      lob[dd] = df_fma_l(Lamb[dd], df_add_l(hi[e1[dd]], hi[e2[dd]]), lob[dd]);
+      const dfl Ll = df_mul_l(Lamb[dd], lo[dd]);
+      hib[e1[dd]] = df_add_l(hib[e1[dd]], Ll);
+      hib[e2[dd]] = df_add_l(hib[e2[dd]], Ll);
     }
 #pragma unroll
-    for (int dd = 0; dd < 3; ++dd) lamb[dd] = df_fma(hib[dd], dhi[dd], df_fma(lob[dd], dlo[dd], lamb[dd]));
+    for (int dd = 0; dd < 3; ++dd) lamb[dd] = df_fma_l(hib[dd], dhi[dd], df_fma_l(lob[dd], dlo[dd], lamb[dd]));
   }
   dfl ab = df_from(0.f);
-  const dfl h0 = df_add(Q[4], pr);
+  const dfl h0 = df_add_l(Q[4], pr);
 #pragma unroll
   for (int dir = 0; dir < 3; ++dir) {
     const dfl E[5] = {G.Eb[dir][0], G.Eb[dir][1], G.Eb[dir][2], G.Eb[dir][3], G.Eb[dir][4]};
     const float sg = U[dir].hi > 0.f ? 1.f : (U[dir].hi < 0.f ? -1.f : 0.f);
     dfl Ub = df_mul_f(lamb[dir], sg);
-    ab = df_fma(lamb[dir], Smag[dir], ab);
+    ab = df_fma_l(lamb[dir], Smag[dir], ab);
     // E = [rho U, m_i U + p S_i, (e + p) U]
-    qb[0] = df_fma(E[0], U[dir], qb[0]);
-    Ub = df_fma(E[0], rho, Ub);
+    qb[0] = df_fma_l(E[0], U[dir], qb[0]);
+    Ub = df_fma_l(E[0], rho, Ub);
 #pragma unroll
     for (int x = 0; x < 3; ++x) {
-      qb[1 + x] = df_fma(E[1 + x], U[dir], qb[1 + x]);
-      Ub = df_fma(E[1 + x], Q[1 + x], Ub);
-      pb = df_fma(E[1 + x], Sv[dir][x], pb);
+      qb[1 + x] = df_fma_l(E[1 + x], U[dir], qb[1 + x]);
+      Ub = df_fma_l(E[1 + x], Q[1 + x], Ub);
+      pb = df_fma_l(E[1 + x], Sv[dir][x], pb);
     }
-    qb[4] = df_fma(E[4], U[dir], qb[4]);
-    pb = df_fma(E[4], U[dir], pb);
-    Ub = df_fma(E[4], h0, Ub);
+    qb[4] = df_fma_l(E[4], U[dir], qb[4]);
+    pb = df_fma_l(E[4], U[dir], pb);
+    Ub = df_fma_l(E[4], h0, Ub);
 #pragma unroll
-    for (int x = 0; x < 3; ++x) ub[x] = df_fma(Ub, Sv[dir][x], ub[x]);
+    for (int x = 0; x < 3; ++x) ub[x] = df_fma_l(Ub, Sv[dir][x], ub[x]);
   }
   // Sutherland mu(T): d mu / dT = mu (1.5/T - 1/(T + S))
-  Tb = df_fma(mub, df_mul(mu, df_sub(df_mul_f(df_rcp(T), 1.5f), iTS)), Tb);
-  Tb = df_fma(ab, df_scale(df_rcp(aa), 0.5f), Tb);
-  pb = df_fma(Tb, df_mul(c.gamma, ir), pb);
-  qb[0] = df_sub(qb[0], df_mul(df_mul(Tb, T), ir));
+  Tb = df_fma_l(mub, df_mul_l(mu, df_sub_l(df_mul_f(df_rcp(T), 1.5f), iTS)), Tb);
+  Tb = df_fma_l(ab, df_scale(df_rcp(aa), 0.5f), Tb);
+  pb = df_fma_l(Tb, df_mul_l(c.gamma, ir), pb);
+  qb[0] = df_sub_l(qb[0], df_mul_l(df_mul_l(Tb, T), ir));
   // reverse of u_i = m_i / rho, p = (gamma-1)(e - m.u/2)
-  qb[4] = df_fma(c.gm1, pb, qb[4]);
-  const dfl keb = df_scale(df_neg(df_mul(c.gm1, pb)), 0.5f);      // half the adjoint of m.u
+  qb[4] = df_fma_l(c.gm1, pb, qb[4]);
+  const dfl keb = df_scale(df_neg(df_mul_l(c.gm1, pb)), 0.5f);      // half the adjoint of m.u
 #pragma unroll
   for (int x = 0; x < 3; ++x) {
-    qb[1 + x] = df_fma(keb, u[x], qb[1 + x]);
-    ub[x] = df_fma(keb, Q[1 + x], ub[x]);
+    qb[1 + x] = df_fma_l(keb, u[x], qb[1 + x]);
+    ub[x] = df_fma_l(keb, Q[1 + x], ub[x]);
   }
   dfl sum = df_from(0.f);
 #pragma unroll
   for (int x = 0; x < 3; ++x) {
-    qb[1 + x] = df_fma(ub[x], ir, qb[1 + x]);
-    sum = df_fma(ub[x], u[x], sum);
+    qb[1 + x] = df_fma_l(ub[x], ir, qb[1 + x]);
+    sum = df_fma_l(ub[x], u[x], sum);
   }
-  qb[0] = df_sub(qb[0], df_mul(sum, ir));
+  qb[0] = df_sub_l(qb[0], df_mul_l(sum, ir));
 #pragma unroll
   for (int m = 0; m < 5; ++m) a.lam[m][p] = df_to_f64(qb[m]);
 }
@@ -412,7 +416,7 @@ cudaError_t adj_faces_df(const Dims& d, const Consts& c, const Work64& w, const 
 
 cudaError_t adj_visc_df(const Dims& d, const Consts& c, const DFMetrics& M, const Work64& w, const QDF& qdf,
                         const Adj64& a, cudaStream_t st) {
-  k_adj_visc_df<<<plane_grid(d.ni + 2, d.nj + 2, d.nk + 2, 256), 256, 0, st>>>(d, make_cdf(c), M, w, qdf, a);
+  k_adj_visc_df<<<plane_grid(d.ni + 2, d.nj + 2, d.nk + 2, kTPBV), kTPBV, 0, st>>>(d, make_cdf(c), M, w, qdf, a);
   return cudaGetLastError();
 }
 

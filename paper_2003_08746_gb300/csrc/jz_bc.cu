@@ -214,12 +214,13 @@ __global__ void __launch_bounds__(kTPB) k_jet_shell(const __grid_constant__ Shel
       if ((th & 31) < nx) red[m][th >> 5][th & 31] = x;
     }
     __syncthreads();
+    const double ink = 1.0 / d.nk;
     double mean[5];
 #pragma unroll
     for (int m = 0; m < 5; ++m) {
       double x = 0.0;
       for (int w = 0; w < kTPB / 32; ++w) x += red[m][w][ix];
-      mean[m] = x / d.nk;
+      mean[m] = x * ink;
     }
     if (in)
       for (int k = ky; k < d.nk; k += nky) put_node<SH>(A, mean, i, 0, k);
