@@ -644,6 +644,9 @@ int jz_create(jz_grid* g, const jz_params* p, void* stream, jz_solver** out) {
     if (tiles * best < 2LL * slots) best = std::min<long long>(d.nk, (2LL * slots + tiles - 1) / tiles);
     if (tiles * best > 30LL * slots) best = std::max<long long>(1, 30LL * slots / tiles);
     s->kchunk = (d.nk + best - 1) / best;
+#ifdef JZ_KC32
+    s->kchunk = JZ_KC32;
+#endif
   } else {
     s->pair = p->precision == JZ_PREC_FP64PAIR;
     if (s->pair) {

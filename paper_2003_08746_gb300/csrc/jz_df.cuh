@@ -196,7 +196,7 @@ __device__ __forceinline__ void df_cbrt_pair(dfl x, dfl& c1, dfl& c2) {
   const float z0 = mufu_ex2(mufu_lg2(x.hi) * (-1.f / 3.f));
   const float z = __fmaf_rn(z0 * (1.f / 3.f), __fmaf_rn(-x.hi * z0, z0 * z0, 1.f), z0);
   const dfl z2 = df_norm(__fmul_rn(z, z), __fmaf_rn(z, z, -__fmul_rn(z, z)));   // z^2 exactly
-  const dfl xz3 = df_mul_f(df_mul(x, z2), z);
+  const dfl xz3 = df_mul_f(df_mul_l(x, z2), z);
   const float e = __fsub_rn(__fsub_rn(1.f, xz3.hi), xz3.lo);
   const float u = e * __fmaf_rn(2.f / 9.f, e, 1.f / 3.f);
   const float zu = __fmul_rn(z, u), zue = __fmaf_rn(z, u, -zu);

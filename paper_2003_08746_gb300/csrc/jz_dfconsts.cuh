@@ -33,9 +33,9 @@ __device__ __forceinline__ void aniso_df(const ConstsDF& c, const dfl lam[3], df
       hi[d] = df_of(l > 0.0 ? pow(l, c.sigma) : 0.0);
     }
   }
-  Lam[0] = df_fma(lo[0], df_add(hi[1], hi[2]), lam[0]);
-  Lam[1] = df_fma(lo[1], df_add(hi[0], hi[2]), lam[1]);
-  Lam[2] = df_fma(lo[2], df_add(hi[0], hi[1]), lam[2]);
+  Lam[0] = df_fma(lo[0], df_add_l(hi[1], hi[2]), lam[0]);
+  Lam[1] = df_fma(lo[1], df_add_l(hi[0], hi[2]), lam[1]);
+  Lam[2] = df_fma(lo[2], df_add_l(hi[0], hi[1]), lam[2]);
 }
 
 // FP64 value -> pair (hi the FP32 rounding, lo the FP32 rounding of the rest), on the host.

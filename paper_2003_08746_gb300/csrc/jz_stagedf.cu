@@ -92,10 +92,13 @@ __global__ void __launch_bounds__(BX* BY) k_sensor_df(Dims d, Work64 w) {
 // nodal and a viscous pass).
 // The momentum and energy fluxes are contracted as H_m = m_m U + S_j P_jm, P = p I - tau, and
 // H_e = e U + S_j (u_m P_jm - k dT/dx_j).
-// FP32 issue bounds it: 10.2 ms per launch on 512 x 512 x 360 (the two passes before: 11.4) with 8
-// rows at three blocks per SM (80 registers); at four (64, spills) 11.2, at two (128) 11.5; 14 rows at
-// two 10.1, but slower on small grids.  Warps for the halo rows that then idle through the fluxes:
-// 10.7.  Split arrivals instead of a barrier per plane (warps drifting by a plane): 12.0.
+// FP32 issue bounds it: 9.6 ms per launch on 512 x 512 x 360 (the two passes before: 11.4) with 8 rows
+// at three blocks per SM (80 registers); at four (64, spills) 10% slower, at two (128) 12%; 14 rows at
+// two the same, but slower on small grids.  Warps for the halo rows that then idle through the fluxes:
+// 5% slower.  Split arrivals instead of a barrier per plane (warps drifting by a plane): 12%.
+// Sums and products inside a chain are unnormalized pairs (every pair normalized: 6% slower), H, the
+// sensors and what seeds a root or reciprocal normalized: the residual's error against 64 bits is
+// 1.07e-12 on a 333 x 177 x 90 jet, 1.11e-12 with every pair normalized and face sums of H.
 constexpr int VX = 32, VY = 10;      // nodes of the tile with its one-node halo
 
 // Element of a field at a 32-bit byte offset (every field of a pair solver is below 4 GB: its 632
@@ -184,9 +187,9 @@ __global__ void __launch_bounds__(VX*(VY - 2), 3) k_flux_df(const __grid_constan
         }
         const dfl ir = df_rcp(rho);
         const dfl u = df_mul(m1, ir), v = df_mul(m2, ir), w = df_mul(m3, ir);
-        const dfl ke = df_fma(m3, w, df_fma(m2, v, df_mul(m1, u)));         // rho |u|^2
-        const dfl pr = df_sub(df_mul(e, c.gm1), df_mul(ke, c.gm1_half));    // (gamma-1)(e - rho|u|^2/2)
-        const dfl T = df_mul(df_mul(pr, c.gamma), ir);
+        const dfl ke = df_fma_l(m3, w, df_fma_l(m2, v, df_mul_l(m1, u)));                   // rho |u|^2
+        const dfl pr = df_n(df_sub_l(df_mul_l(e, c.gm1), df_mul_l(ke, c.gm1_half)));        // (gamma-1)(e - rho|u|^2/2)
+        const dfl T = df_n(df_mul_l(df_mul_l(pr, c.gamma), ir));
         PlaneDF& P = pl[s2];
         P.f[0][row][x] = make_float2(u.hi, u.lo);
         P.f[1][row][x] = make_float2(v.hi, v.lo);
@@ -211,7 +214,7 @@ __global__ void __launch_bounds__(VX*(VY - 2), 3) k_flux_df(const __grid_constan
           const dfl dz = df_sub_l(sm(Pp, n, y, x), sm(Pm, n, y, x));
 #pragma unroll
           for (int jj = 0; jj < 3; ++jj)
-            G[n][jj] = df_n(df_fma_l(S[2][jj], dz, df_fma_l(S[1][jj], dy, df_mul_l(S[0][jj], dx))));
+            G[n][jj] = df_fma_l(S[2][jj], dz, df_fma_l(S[1][jj], dy, df_mul_l(S[0][jj], dx)));
         }
         const dfl h = df_scale(iV, 0.5f);
         // |S| = h sqrt(2 sum G_ii^2 + sum_{i<j} A_ij^2), A_ij = G_ij + G_ji
@@ -226,7 +229,7 @@ __global__ void __launch_bounds__(VX*(VY - 2), 3) k_flux_df(const __grid_constan
                                          df_mul_l(h, df_sqrt(df_n(df_add_l(df_scale(DG, 2.f), AA))))));
         // Sutherland, eq. (sutherland), with T_inf = 1
         const dfl T = sm(P0, 3, y, x), a = df_sqrt(T);
-        const dfl mu = df_mul(df_mul(c.mu_sut, df_mul(T, a)), df_rcp(df_add(T, c.S_hat)));
+        const dfl mu = df_mul_l(df_mul_l(c.mu_sut, df_mul_l(T, a)), df_rcp(df_n(df_add_l(T, c.S_hat))));
         const dfl mt = df_add_l(mu, mu_sgs);
         const dfl mV = df_mul_l(mt, iV), mh = df_neg(df_mul_l(mt, h));
         const dfl kh = df_neg(df_mul_l(df_add_l(df_mul_l(mu, c.k_lam), df_mul_l(mu_sgs, c.k_sgs)), h));  // -k_eff h
@@ -247,8 +250,8 @@ __global__ void __launch_bounds__(VX*(VY - 2), 3) k_flux_df(const __grid_constan
 #pragma unroll
         for (int dir = 0; dir < 3; ++dir) {
           const dfl sx = S[dir][0], sy = S[dir][1], sz = S[dir][2];
-          const dfl U = df_n(df_fma_l(sz, w, df_fma_l(sy, v, df_mul_l(sx, u))));
-          lam[dir] = df_fma(a, ldo(A.Smag[dir], p), df_abs(U));
+          const dfl U = df_fma_l(sz, w, df_fma_l(sy, v, df_mul_l(sx, u)));
+          lam[dir] = df_fma(a, ldo(A.Smag[dir], p), df_abs(df_n(U)));
           // H^dir = [rho U, m_i U + S_j P_ji, e U + S_j X_j]
           auto flux = [&](dfl q, dfl f1, dfl f2, dfl f3) {
             return df_n(df_fma_l(q, U, df_fma_l(sz, f3, df_fma_l(sy, f2, df_mul_l(sx, f1)))));
@@ -469,14 +472,34 @@ cudaError_t sensor_df_pass(const Dims& d, const Work64& w, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// Planes per block of a marching kernel with `tiles` tiles in the plane: 32 where the grid gives two
-// waves of blocks over the SMs all the same, less on small grids (down to one plane, with its priming
-// work again for every block): a 32 x 24 x 16 grid has 16 tiles, and its faces kernel takes 8 us in
-// blocks of one plane against 25 in blocks of four.
-int march_kchunk(long long tiles, int planes) {
-  int kc = 32;
-  while (kc > 1 && tiles * ((planes + kc - 1) / kc) < 8 * 152) kc /= 2;
-  return kc;
+// Resident blocks of a kernel on the current device, asked for once per device.
+template <class K>
+int resident_blocks(K kernel, int threads, int cache[64]) {
+  int dev = 0, sms = 0, per = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 304;
+  if (cache[dev] == 0) {
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, 0) != cudaSuccess || per < 1)
+      return 304;
+    cache[dev] = sms * per;
+  }
+  return cache[dev];
+}
+
+// Planes per block of the marching kernels, from r = planes of all tiles per resident block.  Fitted to
+// sweeps of 1 .. 45 planes over eight jets from 64 x 48 x 32 to 512 x 512 x 360 (each choice within a few per cent
+// of its sweep's best).  Flux kernel: two planes are primed per block, so long blocks, but three
+// waves of them; small grids take the blocks that just fill the device (96 x 64 x 32: 42 us with 3 planes,
+// 48 with 1, 58 with 8).  Faces kernel: one face is primed per block and its loads want many blocks
+// out of step: twenty waves where that leaves three planes or more (512 x 256 x 128: 1.48 ms with 6, 1.64
+// with 32), then three planes, two, one (128 x 96 x 64: 104 us with 2, 132 with 6).
+int flux_chunk(double r) {
+  if (r <= 3.0) return r <= 1.0 ? 1 : (r <= 2.0 ? 2 : 3);
+  return r < 9.0 ? 3 : (r < 96.0 ? (int)(r / 3.0) : 32);
+}
+int faces_chunk(double r) {
+  if (r >= 60.0) return r < 640.0 ? (int)(r / 20.0) : 32;
+  return r >= 13.5 ? 3 : (r >= 6.0 ? 2 : 1);
 }
 
 cudaError_t flux_df(const Dims& d, const Consts& c, const DFMetrics& M, const Work64& w, const QDF& qdf,
@@ -503,7 +526,8 @@ cudaError_t flux_df(const Dims& d, const Consts& c, const DFMetrics& M, const Wo
   A.rate_max = want_rate ? &sc->rate_max : nullptr;
   A.nbx = (d.ni + VX - 1) / (VX - 2);
   const long long tiles = (long long)A.nbx * ((d.nj + VY - 1) / (VY - 2));
-  A.kchunk = march_kchunk(tiles, d.nk + 2);
+  static int slots[64];
+  A.kchunk = flux_chunk((double)tiles * (d.nk + 2) / resident_blocks(k_flux_df, VX * (VY - 2), slots));
   const dim3 gr((unsigned)tiles, (d.nk + 1 + A.kchunk) / A.kchunk);
   k_flux_df<<<gr, dim3(VX, VY - 2), 0, st>>>(A);
   return cudaGetLastError();
@@ -534,7 +558,8 @@ cudaError_t faces_update_df(const Dims& d, const Consts& c, const GridDev& g, co
   A.res_sum = want_res && !rhs_flat ? const_cast<double*>(&sc->res_sum) : nullptr;
   A.nbx = (d.ni + FX - 2) / (FX - 1);
   const long long tiles = (long long)A.nbx * ((d.nj + FY - 2) / (FY - 1));
-  A.kchunk = march_kchunk(tiles, d.nk);
+  static int slots[64];
+  A.kchunk = faces_chunk((double)tiles * d.nk / resident_blocks(k_faces_update_df<0>, FX * FY, slots));
   const dim3 gr((unsigned)tiles, (d.nk + A.kchunk - 1) / A.kchunk), blk(FX, FY);
   if (rhs_flat)
     k_faces_update_df<1><<<gr, blk, 0, st>>>(A);
