@@ -628,11 +628,11 @@ int jz_create(jz_grid* g, const jz_params* p, void* stream, jz_solver** out) {
       own_mf = reinterpret_cast<float*>(tmp);
       s->Mf = own_mf;
     }
-    // CTAs of 30 x 8 columns marching in k, the k range split into chunks.  Rule fitted to
-    // chunk-count sweeps over eight workloads (box 32x24x16 to jet 1000x400x500): about 32
-    // planes per CTA, but at least two waves of CTAs over the resident slots (small grids are
-    // latency-bound: more, shorter CTAs win even with the 3 priming planes each) and at most
-    // thirty (large grids: longer CTAs amortise the priming).
+    // CTAs of 30 x 8 columns marching in k, the k range split into chunks of kchunk planes, three priming
+    // planes each.  With r planes of all tiles per resident CTA: where the grid can fill the device only
+    // once over, the chunk that just does (64 x 48 x 32: 20 us per stage with 2 planes, 25 with 1, 30 with
+    // 6), else 1.5 sqrt(r), fitted to sweeps of 1 .. 180 planes over ten jets up to 1024 x 512 x 360 (within 4%
+    // of each sweep's best: 300 x 160 x 100 takes 0.33 ms with 8 to 22 planes, 0.37 with 32).
     const int tx = jz::fused32_tile_x(), ty = jz::fused32_tile_y();
     const long long tiles = (long long)((d.ni + tx - 1) / tx) * ((d.nj + ty - 1) / ty);
     int slots = 304;
@@ -640,13 +640,8 @@ int jz_create(jz_grid* g, const jz_params* p, void* stream, jz_solver** out) {
       cudaGetLastError();
       slots = 304;
     }
-    long long best = std::max(1, (d.nk + 16) / 32);
-    if (tiles * best < 2LL * slots) best = std::min<long long>(d.nk, (2LL * slots + tiles - 1) / tiles);
-    if (tiles * best > 30LL * slots) best = std::max<long long>(1, 30LL * slots / tiles);
-    s->kchunk = (d.nk + best - 1) / best;
-#ifdef JZ_KC32
-    s->kchunk = JZ_KC32;
-#endif
+    const double r = (double)tiles * d.nk / slots;
+    s->kchunk = std::min(d.nk, (int)(r <= 4.0 ? std::ceil(r) : 1.5 * std::sqrt(r) + 0.5));
   } else {
     s->pair = p->precision == JZ_PREC_FP64PAIR;
     if (s->pair) {
