@@ -165,33 +165,71 @@ __global__ void k_to_f32(Dims d, Ptrs16 src, float* __restrict__ dst) {
   o[2] = make_float4(r[8], r[9], r[10], r[11]);
 }
 
+// Copies between a padded field and a flat array: 2^sh lanes to a row of real nodes (a warp, or the
+// power of two that covers a row shorter than one), one division per row instead of four 64-bit ones
+// per node.  Memory bandwidth bounds them: 1024 x 512 x 360 in (with the shadow) 5.9 -> 3.6 ms, out
+// 4.2 -> 2.2 ms (6.9 TB/s).
+struct RowLanes {
+  int sh;
+};
+__host__ __forceinline__ RowLanes row_lanes(const Dims& d) {
+  int sh = 0;
+  while (sh < 5 && (1 << sh) < d.ni) ++sh;
+  return {sh};
+}
+__host__ __forceinline__ unsigned row_blocks(const Dims& d) {
+  return blocks_for((long long)d.nj * d.nk, kTPB >> row_lanes(d).sh);
+}
+// The row of this thread: its first elements in a padded field (p) and in the flat array (t), its
+// first node i; false past the last row.
+__device__ __forceinline__ bool my_row(const Dims& d, RowLanes l, long long& p, long long& t, int& i) {
+  const long long row = blockIdx.x * (long long)(kTPB >> l.sh) + (threadIdx.x >> l.sh);
+  if (row >= (long long)d.nj * d.nk) return false;
+  const int k = (int)(row / d.nj), j = (int)(row - (long long)k * d.nj);
+  p = pidx(d, 0, j, k);
+  t = row * d.ni;
+  i = threadIdx.x & ((1 << l.sh) - 1);
+  return true;
+}
+
 // A flat [5][N] array into the real nodes of a state (and their shadow).
-__global__ void k_pack_state(Dims d, ConstsF c, State q, const double* __restrict__ flat) {
-  Box b{0, 0, 0, d.ni, d.nj, d.nk};
-  int i, j, k;
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (!box_coord(b, t, i, j, k)) return;
-  const long long N = (long long)d.ni * d.nj * d.nk, p = pidx(d, i, j, k);
-  double v[5];
+__global__ void __launch_bounds__(kTPB) k_pack_state(Dims d, RowLanes l, ConstsF c, State q,
+                                                     const double* __restrict__ flat) {
+  long long p, t;
+  int i;
+  if (!my_row(d, l, p, t, i)) return;
+  const long long N = (long long)d.ni * d.nj * d.nk;
+#pragma unroll 2
+  for (; i < d.ni; i += 32) {   // a shorter row takes one turn
+    double v[5];
 #pragma unroll
-  for (int m = 0; m < 5; ++m) v[m] = flat[m * N + t];
+    for (int m = 0; m < 5; ++m) v[m] = flat[m * N + t + i];
 #pragma unroll
-  for (int m = 0; m < 5; ++m) q.q[m][p] = v[m];
-  if (q.sh) {
-    float2 s[NSH];
-    shadow_of(c, v, s);
+    for (int m = 0; m < 5; ++m) q.q[m][p + i] = v[m];
+    if (q.sh) {
+      float2 s[NSH];
+      shadow_of(c, v, s);
 #pragma unroll
-    for (int m = 0; m < NSH; ++m) q.sh[m * d.Np + p] = s[m];
+      for (int m = 0; m < NSH; ++m) q.sh[m * d.Np + p + i] = s[m];
+    }
   }
 }
 
-__global__ void k_unpack(Dims d, Ptrs16 padded, double* __restrict__ flat, int nvar) {
-  Box b{0, 0, 0, d.ni, d.nj, d.nk};
-  int i, j, k;
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (!box_coord(b, t, i, j, k)) return;
-  const long long N = (long long)d.ni * d.nj * d.nk, p = pidx(d, i, j, k);
-  for (int v = 0; v < nvar; ++v) flat[v * N + t] = padded.p[v][p];
+// Real nodes of padded fields into a flat [NV][N] array.
+template <int NV>
+__global__ void __launch_bounds__(kTPB) k_unpack(Dims d, RowLanes l, Ptrs16 padded, double* __restrict__ flat) {
+  long long p, t;
+  int i;
+  if (!my_row(d, l, p, t, i)) return;
+  const long long N = (long long)d.ni * d.nj * d.nk;
+#pragma unroll 2
+  for (; i < d.ni; i += 32) {   // a shorter row takes one turn
+    double v[NV];
+#pragma unroll
+    for (int m = 0; m < NV; ++m) v[m] = padded.p[m][p + i];
+#pragma unroll
+    for (int m = 0; m < NV; ++m) flat[m * N + t + i] = v[m];
+  }
 }
 
 __global__ void k_check_volume(Dims d, Ptrs16 M, int* bad) {
@@ -290,8 +328,7 @@ cudaError_t metrics_to_f32(const Dims& d, const GridDev& g, float* Mf, cudaStrea
 }
 
 cudaError_t pack_state(const Dims& d, const Consts& c, const State& q, const double* flat, cudaStream_t st) {
-  const long long nr = (long long)d.ni * d.nj * d.nk;
-  k_pack_state<<<blocks_for(nr, kTPB), kTPB, 0, st>>>(d, make_constsf(c), q, flat);
+  k_pack_state<<<row_blocks(d), kTPB, 0, st>>>(d, row_lanes(d), make_constsf(c), q, flat);
   return cudaGetLastError();
 }
 
@@ -301,8 +338,14 @@ cudaError_t ghost_fill_state(const Dims& d, const State& q, Scalars* advance, cu
 }
 
 cudaError_t unpack_real(const Dims& d, double* const* padded, double* flat, int nvar, cudaStream_t st) {
-  const long long nr = (long long)d.ni * d.nj * d.nk;
-  k_unpack<<<blocks_for(nr, kTPB), kTPB, 0, st>>>(d, ptrs(padded, nvar), flat, nvar);
+  const unsigned n = row_blocks(d);
+  const RowLanes l = row_lanes(d);
+  if (nvar == 5)
+    k_unpack<5><<<n, kTPB, 0, st>>>(d, l, ptrs(padded, 5), flat);
+  else if (nvar == 10)
+    k_unpack<10><<<n, kTPB, 0, st>>>(d, l, ptrs(padded, 10), flat);
+  else
+    return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
 

@@ -318,7 +318,7 @@ cudaError_t ghost_fill_state(const Dims& d, const State& q, Scalars* advance, cu
 // FP32 copy of the metrics S (9) and V; dst_dev is a device array of 10 pointers
 cudaError_t boundary_copies(const Dims& d, const GridDev& g, cudaStream_t st);
 cudaError_t metrics_to_f32(const Dims& d, const GridDev& g, float* Mf, cudaStream_t st);
-// padded real region of nvar fields to a flat [nvar][N] array
+// padded real region of nvar fields (5 or 10) to a flat [nvar][N] array
 cudaError_t unpack_real(const Dims& d, double* const* padded, double* flat, int nvar,
                         cudaStream_t st);
 // real nodes of a state from a flat [5][N] array, with their shadow in the FP32-flux form

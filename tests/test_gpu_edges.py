@@ -116,3 +116,17 @@ def test_adjoint_with_little_memory(jz):
         assert np.abs(gr - g0).max() <= 1e-12 * np.abs(g0).max()
     s.close()
     grid.close()
+
+
+# copies in and out, whole and with part of a warp to a row: a copy is exact
+@pytest.mark.parametrize("ni", [1, 2, 3, 8, 9, 17, 31, 32, 33, 67])
+@pytest.mark.parametrize("form", ["FP64PAIR", "FP32FLUX"])
+def test_state_round_trip(jz, ni, form):
+    g = W.box_grid(ni, 7, 5, h=0.2)
+    q = W.random_state(g, seed=ni, amp=0.05)
+    grid = jz.Grid.from_workload(g)
+    s = jz.Solver(grid, W.box_params(), getattr(jz, "JZ_PREC_" + form))
+    s.set_state(q, 0.0)
+    assert np.array_equal(s.get_state(), q)
+    s.close()
+    grid.close()
