@@ -1,5 +1,5 @@
-// Shared-memory mbarriers (inline PTX) with bounded waits: the fused FP32-flux kernel's TMA copies
-// (jz_stage32.cu) and the pair form's flux kernel (jz_stagedf.cu).
+// Shared-memory mbarriers (inline PTX) with bounded waits, for the fused FP32-flux kernel's TMA copies
+// (jz_stage32.cu).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -26,11 +26,6 @@ __device__ __forceinline__ bool wait_bar(unsigned long long* bar, unsigned parit
     if (ok) return true;
   }
   return false;
-}
-// One arrival on an mbarrier; the caller's earlier shared-memory writes are visible to whoever sees
-// the phase complete.
-__device__ __forceinline__ void bar_arrive(unsigned long long* b) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
 }
 
 }  // namespace jz
