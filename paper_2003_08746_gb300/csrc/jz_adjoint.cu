@@ -345,10 +345,11 @@ __global__ void k_adj_axis(Dims d, Adj64 a) {
 
 // Entrance and exit, blocks of kTPBS threads (a few thousand nodes of long FP64 chains: small blocks
 // spread them over the SMs).  The forcing's temporal factors come from the host, which knows the
-// stage time: sn, and am = amplitude times factor.
+// stage time: the shapes' coefficients co, and for the amplitudes' derivatives each factor times the
+// cosine and (negative) sine of its azimuthal phase.
 constexpr int kTPBS = 64;
 struct ForcingAt {
-  double sn[kNF], am[kNF];
+  double co[kNT], dc[kNF], ds[kNF];
 };
 __global__ void __launch_bounds__(kTPBS) k_adj_inout(Dims d, Consts c, Inflow in, State q, Adj64 a,
                                                      const __grid_constant__ ForcingAt F, unsigned ent_blocks) {
@@ -358,20 +359,20 @@ __global__ void __launch_bounds__(kTPBS) k_adj_inout(Dims d, Consts c, Inflow in
   const bool exit_plane = blockIdx.x >= ent_blocks;
   const long long tt = (blockIdx.x - (exit_plane ? ent_blocks : 0u)) * (long long)kTPBS + threadIdx.x;
   double g0 = 0.0;                 // d J / d u_target (times U_j) at this entrance node
-  __shared__ double Gs[kNF][kTPBS + 1];        // this block's forcing shapes
+  __shared__ double Ts[kNT][kTPBS + 1];        // this block's forcing shapes
   if (tt < nface) {
     const int j = 1 + (int)(tt % nj1), k = (int)(tt / nj1);
     if (!exit_plane) {
       const long long pb = pidx(d, 0, j, k), p1 = pidx(d, 1, j, k);
       const long long tab = (long long)k * d.nj + j;
-      double f[4] = {0.0, 0.0, 0.0, 0.0};
+      double f[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-      for (int mf = 0; mf < kNF; ++mf) {
-        const double G = __ldg(in.Gf + mf * plane + tab);
-        Gs[mf][threadIdx.x] = G;
-        f[mf & 3] = fma(F.am[mf], G, f[mf & 3]);
+      for (int n = 0; n < kNT; ++n) {
+        const double T = __ldg(in.T + n * plane + tab);
+        Ts[n][threadIdx.x] = T;
+        f[n % 5] = fma(F.co[n], T, f[n % 5]);
       }
-      const double ut = in.u0[tab] + c.jet_mach * ((f[0] + f[1]) + (f[2] + f[3]));
+      const double ut = fma(c.jet_mach, ((f[0] + f[1]) + (f[2] + f[3])) + f[4], in.u0[tab]);
       double Q1[5];
       load5(q, p1, Q1);
       double lb[5];
@@ -430,25 +431,31 @@ __global__ void __launch_bounds__(kTPBS) k_adj_inout(Dims d, Consts c, Inflow in
     }
   }
   if (exit_plane) return;
-  // dJ/dA_mf = sum over the entrance of g0 G_mf sin(omega_f t + psi_mf): one parameter per lane, the
-  // block's nodes in halves, one atomic per parameter per block
-  __shared__ double gs[kTPBS], half[kNF];
+  // dJ/dA_mf = sin(omega_f t + psi_mf) (cos phi_mf C_m - sin phi_mf S_m), C_m and S_m the sums of g0 times
+  // the shapes over the entrance: a shape per lane, the block's nodes in quarters, one atomic per
+  // amplitude per block
+  __shared__ double gs[kTPBS], part[kTPBS];
   gs[threadIdx.x] = g0;
   if (tt >= nface)
-    for (int mf = 0; mf < kNF; ++mf) Gs[mf][threadIdx.x] = 0.0;
+    for (int n = 0; n < kNT; ++n) Ts[n][threadIdx.x] = 0.0;
   __syncthreads();
-  const int mf = threadIdx.x % kNF, n0 = threadIdx.x / kNF * (kTPBS / 2);
+  constexpr int NQ = kTPBS / 4;
+  const int sh = threadIdx.x % NQ, n0 = threadIdx.x / NQ * NQ;
   double x = 0.0;
-#pragma unroll 8
-  for (int n = n0; n < n0 + kTPBS / 2; ++n) x = fma(gs[n], Gs[mf][n], x);
-  if (n0) half[mf] = x;
-  __syncthreads();
-  if (n0 == 0) {
-    x = (x + half[mf]) * F.sn[mf];
-    if (x != 0.0) atomicAdd(&a.abar[mf], x);
+  if (sh < kNT) {
+#pragma unroll
+    for (int n = n0; n < n0 + NQ; ++n) x = fma(gs[n], Ts[sh][n], x);
   }
+  part[threadIdx.x] = x;
+  __syncthreads();
+  if (threadIdx.x >= kNF) return;
+  auto sum = [&](int n) { return (part[n] + part[n + NQ]) + (part[n + 2 * NQ] + part[n + 3 * NQ]); };
+  const int mf = threadIdx.x, m = mf / JZ_N_FREQ;
+  x = F.dc[mf] * sum(m);
+  if (m > 0) x = fma(F.ds[mf], sum(JZ_N_MODES + m - 1), x);
+  if (x != 0.0) atomicAdd(&a.abar[mf], x);
 }
-static_assert(kTPBS == 2 * kNF, "two halves of the block's nodes, one lane per parameter");
+static_assert(kNT <= kTPBS / 4 && kNF <= kTPBS, "a lane per shape in each quarter of the block, then one per amplitude");
 
 __global__ void k_adj_farfield(Dims d, Consts c, GridDev g, State q, Adj64 a) {
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -458,9 +465,7 @@ __global__ void k_adj_farfield(Dims d, Consts c, GridDev g, State q, Adj64 a) {
   const int jb = d.nj - 1;
   const long long pb = pidx(d, i, jb, k), pi = pidx(d, i, jb - 1, k);
   const long long nsurf = (long long)d.nk * d.ni, isurf = (long long)k * d.ni + i;
-  const double sx = g.Sb[isurf], sy = g.Sb[nsurf + isurf], sz = g.Sb[2 * nsurf + isurf];
-  const double im = rcp64(sqrt64(sx * sx + sy * sy + sz * sz));
-  const double n[3] = {sx * im, sy * im, sz * im};
+  const double n[3] = {g.Sb[isurf], g.Sb[nsurf + isurf], g.Sb[2 * nsurf + isurf]};
   double Qi[5];
   load5(q, pi, Qi);
   const double rho_i = Qi[0], ir = rcp64(rho_i);
@@ -601,10 +606,14 @@ cudaError_t adj_bcs(const Dims& d, const Consts& c, const GridDev& g, const Infl
   if (d.topo != JZ_TOPO_JET) return cudaSuccess;
   k_adj_axis<<<d.ni, 128, 0, st>>>(d, a);
   ForcingAt F;
+  double am[kNF];
   for (int mf = 0; mf < kNF; ++mf) {
-    F.sn[mf] = std::sin(in.omega[mf % JZ_N_FREQ] * ts + in.psi[mf]);
-    F.am[mf] = in.amp[mf] * F.sn[mf];
+    const double sn = std::sin(in.omega[mf % JZ_N_FREQ] * ts + in.psi[mf]);
+    am[mf] = in.amp[mf] * sn;
+    F.dc[mf] = sn * in.cphi[mf];
+    F.ds[mf] = -sn * in.sphi[mf];
   }
+  for (int n = 0; n < kNT; ++n) F.co[n] = shape_coef(n, am, in.cphi, in.sphi);
   const unsigned nio = blocks_for((long long)(d.nj - 1) * d.nk, kTPBS);
   k_adj_inout<<<2 * nio, kTPBS, 0, st>>>(d, c, in, q, a, F, nio);
   const long long nf = (long long)(d.ni - 2) * d.nk;

@@ -674,8 +674,8 @@ int jz_create(jz_grid* g, const jz_params* p, void* stream, jz_solver** out) {
   A(s->part, 8 * (size_t)jz::stat_partial_count());
   if (d.topo == JZ_TOPO_JET) {
     A(s->in.u0, (size_t)d.nj * d.nk);
-    A(s->in.Gf, (size_t)jz::kNF * d.nj * d.nk);
-    A(s->in.sn, 5 * (size_t)jz::kNF);
+    A(s->in.T, (size_t)jz::kNT * d.nj * d.nk);
+    A(s->in.co, 5 * (size_t)jz::kNT);
   }
   if (e != cudaSuccess) {
     delete s;

@@ -12,6 +12,8 @@
 // shell needs no order between blocks: a thread that owns a boundary node
 // computes it and writes it with all its ghost images, and the ghosts of
 // advanced nodes (across the axis, around the azimuth) are copied beside them.
+#include <cmath>
+
 #include "jz_shadow.cuh"
 
 namespace jz {
@@ -25,12 +27,12 @@ struct ShellArgs {
   Dims d;
   Consts c;
   ConstsF cf;
-  const double* Sb;      // far-field normals [3][nk][ni]
+  const double* Sb;      // far-field unit normals [3][nk][ni]
   const double* u0;      // entrance profile [nk][nj]
-  const double* Gf;      // forcing shapes [32][nk][nj]
-  double amp[kNF];
+  const double* T;       // forcing shapes [15][nk][nj]
+  const double* co;      // their coefficients at this stage's time
+  double ink;            // 1 / nk
   State q;
-  const double* sn;      // temporal factors of the forcing at this stage's time
   Scalars* sc;
   int advance;           // last stage of a step: t += dt
   unsigned bA, bE, bX, bF, bR;   // first block after the axis, entrance, exit, far-field and row roles
@@ -64,9 +66,7 @@ __device__ __forceinline__ void load_q(const State& q, long long p, double v[5])
 __device__ void farfield_value(const ShellArgs& A, int i, int k, const double qi[5], double out[5]) {
   const Consts& c = A.c;
   const long long nb = (long long)A.d.nk * A.d.ni, sb = (long long)k * A.d.ni + i;
-  const double sx = A.Sb[sb], sy = A.Sb[nb + sb], sz = A.Sb[2 * nb + sb];
-  const double im = rcp64(sqrt64(sx * sx + sy * sy + sz * sz));
-  const double n[3] = {sx * im, sy * im, sz * im};
+  const double n[3] = {A.Sb[sb], A.Sb[nb + sb], A.Sb[2 * nb + sb]};
   const Prim r = prim_of(c, qi);
   const double a_i = sqrt64(c.gamma * r.p * r.ir);
   const double un_i = r.u[0] * n[0] + r.u[1] * n[1] + r.u[2] * n[2];
@@ -83,16 +83,16 @@ __device__ void farfield_value(const ShellArgs& A, int i, int k, const double qi
   cons_of(c, rho, v[0], v[1], v[2], pr, out);
 }
 
-// Entrance node (0, j, k) by 1-D characteristics: tanh profile + forcing at the stage time; am the
-// amplitudes times their temporal factors, q1 = Q(1, j, k).
-__device__ void entrance_value(const ShellArgs& A, const double* am, int j, int k, const double q1[5], double out[5]) {
+// Entrance node (0, j, k) by 1-D characteristics: tanh profile + forcing at the stage time,
+// q1 = Q(1, j, k).
+__device__ void entrance_value(const ShellArgs& A, int j, int k, const double q1[5], double out[5]) {
   const Consts& c = A.c;
   const long long tab = (long long)k * A.d.nj + j, plane = (long long)A.d.nk * A.d.nj;
-  // four partial sums: the FP64 latency of one chain of 32 would set the kernel's time
-  double f[4] = {0.0, 0.0, 0.0, 0.0};
+  // five partial sums: the FP64 latency of one chain of 15 would set the kernel's time
+  double f[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-  for (int mf = 0; mf < kNF; ++mf) f[mf & 3] = fma(am[mf], __ldg(A.Gf + mf * plane + tab), f[mf & 3]);
-  const double ut = fma(c.jet_mach, (f[0] + f[1]) + (f[2] + f[3]), A.u0[tab]);
+  for (int n = 0; n < kNT; ++n) f[n % 5] = fma(__ldg(A.co + n), __ldg(A.T + n * plane + tab), f[n % 5]);
+  const double ut = fma(c.jet_mach, ((f[0] + f[1]) + (f[2] + f[3])) + f[4], A.u0[tab]);
   if (ut >= 1.0) {                                          // supersonic: all imposed
     cons_of(c, 1.0, ut, 0.0, 0.0, c.p_inf, out);
     return;
@@ -123,39 +123,38 @@ __device__ __forceinline__ void inner_neighbour(const ShellArgs& A, int i, int j
   }
 }
 
-// Write a value at (i, j, k) and at its azimuthal images.
-template <bool SH>
-__device__ __forceinline__ void put(const ShellArgs& A, const double v[5], const float2 s[NSH], int i, int j, int k) {
-  const Dims& d = A.d;
-  const long long turn = (long long)d.nk * d.sk;
-  long long p = pidx(d, i, j, k);
-  const int before = k >= d.nk - kG, after = k < kG;       // images at k - nk and k + nk
-  if (before) p -= turn;
-  for (int n = 0; n < 1 + before + after; ++n, p += turn) {
-#pragma unroll
-    for (int m = 0; m < 5; ++m) A.q.q[m][p] = v[m];
-    if (SH) {
-#pragma unroll
-      for (int m = 0; m < NSH; ++m) A.q.sh[m * d.Np + p] = s[m];
-    }
-  }
-}
-
-// Write the value of a boundary node (i, j, k), real, with every ghost that copies it: beyond the
-// entrance and exit (zero order in i), beyond the far field (zero order in j), across the axis
-// (rows -1 and -2 hold nodes (i, 1 | 2, k + nk/2)) and around the azimuth.
-template <bool SH>
-__device__ void put_node(const ShellArgs& A, const double v[5], int i, int j, int k) {
+// Write the value of a boundary node at row (j, k), with every ghost that copies it, as NC nodes along
+// i from ia: the entrance and exit with their ghosts beyond (zero order in i), one node elsewhere.  Beyond
+// the far field two more rows take it (zero order in j), across the axis row -j holds it at k + nk/2,
+// and each row has images around the azimuth where k is within two of its ends.
+template <bool SH, int NC>
+__device__ __forceinline__ void put_node(const ShellArgs& A, const double v[5], int ia, int j, int k) {
   const Dims& d = A.d;
   float2 s[NSH];
   if (SH) shadow_of(A.cf, v, s);
-  const int i0 = i == 0 ? -kG : i, i1 = i == d.ni - 1 ? i + kG : i;
-  const int j1 = j == d.nj - 1 ? j + kG : j;
-  const bool mirror = j >= 1 && j <= kG;
-  const int half = d.nk / 2, km = k >= half ? k - half : k + half;
-  for (int ii = i0; ii <= i1; ++ii) {
-    for (int jj = j; jj <= j1; ++jj) put<SH>(A, v, s, ii, jj, k);
-    if (mirror) put<SH>(A, v, s, ii, -j, km);
+  const bool far = j == d.nj - 1, mirror = j >= 1 && j <= kG;
+  const long long turn = (long long)d.nk * d.sk;
+  const int half = d.nk / 2, kf = far ? kG : 0, rows = 1 + kf + (mirror ? 1 : 0);
+#pragma unroll 1
+  for (int r = 0; r < rows; ++r) {
+    const bool m = r > kf;                                 // the row across the axis
+    const int kk = m ? (k >= half ? k - half : k + half) : k;
+    long long p = pidx(d, ia, m ? -j : j + r, kk);
+    const int before = kk >= d.nk - kG, after = kk < kG;   // images at kk - nk and kk + nk
+    if (before) p -= turn;
+#pragma unroll 1
+    for (int n = 0; n < 1 + before + after; ++n, p += turn) {
+#pragma unroll
+      for (int q = 0; q < 5; ++q)
+#pragma unroll
+        for (int x = 0; x < NC; ++x) A.q.q[q][p + x] = v[q];
+      if (SH) {
+#pragma unroll
+        for (int q = 0; q < NSH; ++q)
+#pragma unroll
+          for (int x = 0; x < NC; ++x) A.q.sh[q * d.Np + p + x] = s[q];
+      }
+    }
   }
 }
 
@@ -177,11 +176,6 @@ template <bool SH>
 __global__ void __launch_bounds__(kTPB) k_jet_shell(const __grid_constant__ ShellArgs A) {
   const Dims& d = A.d;
   const unsigned b = blockIdx.x, th = threadIdx.x;
-  __shared__ double am[kNF];
-  if (b < A.bE) {                                          // axis and entrance blocks
-    if (th < kNF) am[th] = A.amp[th] * A.sn[th];
-    __syncthreads();
-  }
   if (b < A.bA) {
     // axis: the ring j = 1 averaged over the azimuth; the two ends, whose ring is entrance and exit
     // nodes, by a block each with all its threads along k, the lines between AXI to a block
@@ -195,7 +189,7 @@ __global__ void __launch_bounds__(kTPB) k_jet_shell(const __grid_constant__ Shel
         double v[5], t[5];
         if (b == 0) {
           inner_neighbour(A, 1, 1, k, t);
-          entrance_value(A, am, 1, k, t, v);
+          entrance_value(A, 1, k, t, v);
         } else if (b == 1) {
           inner_neighbour(A, i - 1, 1, k, t);
           exit_value(A, t, v);
@@ -214,32 +208,34 @@ __global__ void __launch_bounds__(kTPB) k_jet_shell(const __grid_constant__ Shel
       if ((th & 31) < nx) red[m][th >> 5][th & 31] = x;
     }
     __syncthreads();
-    const double ink = 1.0 / d.nk;
     double mean[5];
 #pragma unroll
     for (int m = 0; m < 5; ++m) {
       double x = 0.0;
       for (int w = 0; w < kTPB / 32; ++w) x += red[m][w][ix];
-      mean[m] = x * ink;
+      mean[m] = x * A.ink;
     }
-    if (in)
-      for (int k = ky; k < d.nk; k += nky) put_node<SH>(A, mean, i, 0, k);
+    if (end)
+      for (int k = ky; k < d.nk; k += nky) put_node<SH, 1 + kG>(A, mean, b == 0 ? -kG : i, 0, k);
+    else if (in)
+      for (int k = ky; k < d.nk; k += nky) put_node<SH, 1>(A, mean, i, 0, k);
     if (b == 0 && th == 0 && A.advance) A.sc->t = A.sc->t + A.sc->dt;
     return;
   }
   if (b < A.bX) {
-    // entrance (i = 0) and exit (i = ni-1), 1 <= j <= nj-1
+    // entrance (i = 0) and exit (i = ni-1), 1 <= j <= nj-1; the nodes at j = nj-1, which take the
+    // longest (a far-field value first, three rows of images), last and by warps of their own
     const bool ent = b < A.bE;
-    const unsigned t = (b - (ent ? A.bA : A.bE)) * kTPB + th, nj1 = d.nj - 1;
-    if (t >= nj1 * (unsigned)d.nk) return;
-    const int j = 1 + (int)(t % nj1), k = (int)(t / nj1);
+    const unsigned t = (b - (ent ? A.bA : A.bE)) * kTPB + th, nj2 = d.nj - 2, n = nj2 * (unsigned)d.nk;
+    if (t >= n + (unsigned)d.nk) return;
+    const int k = t < n ? (int)(t / nj2) : (int)(t - n), j = t < n ? 1 + (int)(t - k * nj2) : d.nj - 1;
     double qi[5], v[5];
     inner_neighbour(A, ent ? 1 : d.ni - 2, j, k, qi);
     if (ent)
-      entrance_value(A, am, j, k, qi, v);
+      entrance_value(A, j, k, qi, v);
     else
       exit_value(A, qi, v);
-    put_node<SH>(A, v, ent ? 0 : d.ni - 1, j, k);
+    put_node<SH, 1 + kG>(A, v, ent ? -kG : d.ni - 1, j, k);
     return;
   }
   const unsigned ni2 = d.ni - 2;
@@ -251,7 +247,7 @@ __global__ void __launch_bounds__(kTPB) k_jet_shell(const __grid_constant__ Shel
     double qi[5], v[5];
     load_q(A.q, pidx(d, i, d.nj - 2, k), qi);
     farfield_value(A, i, k, qi, v);
-    put_node<SH>(A, v, i, d.nj - 1, k);
+    put_node<SH, 1>(A, v, i, d.nj - 1, k);
     return;
   }
   if (b < A.bR) {
@@ -276,14 +272,10 @@ __global__ void __launch_bounds__(kTPB) k_jet_shell(const __grid_constant__ Shel
   copy_node<SH>(A, pidx(d, i, j, k), pidx(d, i, j, s < 2 ? k + d.nk : k - d.nk));
 }
 
-struct Phases {
-  double phi[kNF];
-};
-
-// Entrance tables at i = 0: u0 = U_j/2 [1 + tanh((0.5 - r)/(2 theta))] and
-// Gf[m][f] = g(r) cos(m theta + phi_mf), g(r) = exp(-((r - 0.5)/0.1)^2),
-// with r and theta from the node coordinates.
-__global__ void k_build_inflow(Dims d, Consts c, GridDev g, double* u0, double* Gf, Phases ph) {
+// Entrance tables at i = 0: u0 = U_j/2 [1 + tanh((0.5 - r)/(2 theta))] and the forcing shapes
+// g(r) cos m theta, g(r) sin m theta, g(r) = exp(-((r - 0.5)/0.1)^2), with r and theta from the node
+// coordinates.
+__global__ void k_build_inflow(Dims d, Consts c, GridDev g, double* u0, double* T) {
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (t >= (long long)d.nj * d.nk) return;
   const double y = g.Xin[t], z = g.Xin[(long long)d.nj * d.nk + t];   // t = k nj + j
@@ -293,11 +285,10 @@ __global__ void k_build_inflow(Dims d, Consts c, GridDev g, double* u0, double* 
   const double x = (r - 0.5) / 0.1;
   const double gr = exp(-(x * x));
   const long long plane = (long long)d.nk * d.nj;
-  for (int m = 0; m < JZ_N_MODES; ++m)
-    for (int f = 0; f < JZ_N_FREQ; ++f) {
-      const int mf = m * JZ_N_FREQ + f;
-      Gf[mf * plane + t] = gr * cos(m * th + ph.phi[mf]);
-    }
+  for (int n = 0; n < kNT; ++n) {
+    const double a = shape_mode(n) * th;
+    T[n * plane + t] = gr * (shape_sine(n) ? sin(a) : cos(a));
+  }
 }
 
 }  // namespace
@@ -310,11 +301,11 @@ cudaError_t jet_shell(const Dims& d, const Consts& c, const GridDev& g, const In
   A.cf = make_constsf(c);
   A.Sb = g.Sb;
   A.u0 = in.u0;
-  A.Gf = in.Gf;
-  for (int mf = 0; mf < kNF; ++mf) A.amp[mf] = in.amp[mf];
+  A.T = in.T;
+  A.co = in.co + stage * kNT;
+  A.ink = 1.0 / d.nk;
   A.q = q;
   A.sc = sc;
-  A.sn = in.sn + stage * kNF;
   A.advance = advance;
   const long long ni2 = d.ni - 2;
   const unsigned nio = blocks_for((long long)(d.nj - 1) * d.nk, kTPB);
@@ -333,15 +324,15 @@ cudaError_t jet_shell(const Dims& d, const Consts& c, const GridDev& g, const In
 
 cudaError_t build_inflow(const Dims& d, const Consts& c, const GridDev& g, const jz_params& p, Inflow& in,
                          cudaStream_t st) {
-  Phases ph;
   for (int mf = 0; mf < kNF; ++mf) {
-    ph.phi[mf] = p.forcing_phi[mf];
+    in.cphi[mf] = std::cos(p.forcing_phi[mf]);
+    in.sphi[mf] = std::sin(p.forcing_phi[mf]);
     in.amp[mf] = p.forcing_amp[mf];
     in.psi[mf] = p.forcing_psi[mf];
   }
   for (int f = 0; f < JZ_N_FREQ; ++f) in.omega[f] = 2.0 * 3.141592653589793 * p.strouhal[f] * p.jet_mach;
   const long long n = (long long)d.nj * d.nk;
-  k_build_inflow<<<blocks_for(n, kTPB), kTPB, 0, st>>>(d, c, g, in.u0, in.Gf, ph);
+  k_build_inflow<<<blocks_for(n, kTPB), kTPB, 0, st>>>(d, c, g, in.u0, in.T);
   return cudaGetLastError();
 }
 

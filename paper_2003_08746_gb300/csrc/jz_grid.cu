@@ -292,18 +292,21 @@ cudaError_t ghost_fill(const Dims& d, double* const* f, int nvar, cudaStream_t s
   return cudaGetLastError();
 }
 
-// Surface copies: the far-field normals S^eta at j = nj-1 ([3][nk][ni]) and the
+// Surface copies: the far field's unit normals S^eta / |S^eta| at j = nj-1 ([3][nk][ni]) and the
 // entrance-plane coordinates y, z at i = 0 ([2][nk][nj]).
 __global__ void k_boundary_copies(Dims d, GridDev g) {
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long nb = (long long)d.nk * d.ni, ne = (long long)d.nk * d.nj;
-  if (t < 3 * nb) {
-    const int c = (int)(t / nb);
-    const long long r = t % nb;
-    const int k = (int)(r / d.ni), i = (int)(r % d.ni);
-    g.Sb[t] = g.S[3 + c][pidx(d, i, d.nj - 1, k)];
-  } else if (t < 3 * nb + 2 * ne) {
-    const long long u = t - 3 * nb;
+  if (t < nb) {
+    const int k = (int)(t / d.ni), i = (int)(t - (long long)k * d.ni);
+    const long long p = pidx(d, i, d.nj - 1, k);
+    const double sx = g.S[3][p], sy = g.S[4][p], sz = g.S[5][p];
+    const double im = rcp64(sqrt64(sx * sx + sy * sy + sz * sz));
+    g.Sb[t] = sx * im;
+    g.Sb[nb + t] = sy * im;
+    g.Sb[2 * nb + t] = sz * im;
+  } else if (t < nb + 2 * ne) {
+    const long long u = t - nb;
     const int c = (int)(u / ne);
     const long long r = u % ne;
     const int k = (int)(r / d.nj), j = (int)(r % d.nj);
@@ -312,7 +315,7 @@ __global__ void k_boundary_copies(Dims d, GridDev g) {
 }
 
 cudaError_t boundary_copies(const Dims& d, const GridDev& g, cudaStream_t st) {
-  const long long n = 3LL * d.nk * d.ni + 2LL * d.nk * d.nj;
+  const long long n = (long long)d.nk * d.ni + 2LL * d.nk * d.nj;
   k_boundary_copies<<<blocks_for(n, kTPB), kTPB, 0, st>>>(d, g);
   return cudaGetLastError();
 }

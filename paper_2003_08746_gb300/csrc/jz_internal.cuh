@@ -12,6 +12,7 @@ namespace jz {
 
 constexpr int kG = 2;            // ghost layers per side (two-layer ghosts)
 constexpr int kNF = JZ_N_MODES * JZ_N_FREQ;
+constexpr int kNT = 2 * JZ_N_MODES - 1;   // entrance shapes: cos m theta for every mode, sin m theta for m > 0
 
 // Padded box geometry.  Real node (i, j, k), -2 <= i <= ni + 1, sits at
 // element ((k + 2) * Pj + (j + 2)) * Pi + (i + 2).  Pi is rounded up to a
@@ -130,7 +131,7 @@ struct GridDev {
   double* Smag[3];    // |S^dir|
   double* Delta;      // filter width V^(1/3)
   // surface copies kept by every grid (also compact ones)
-  double* Sb;         // far-field normals S^eta at j = nj-1: [3][nk][ni]
+  double* Sb;         // unit normals S^eta / |S^eta| of the far field j = nj-1: [3][nk][ni]
   double* Xin;        // entrance-plane coordinates y, z at i = 0: [2][nk][nj]
   // compact grids (jz_grid_compact): the FP64 arrays above except Sb and Xin are
   // released and the metrics are kept in FP32 only
@@ -296,15 +297,32 @@ struct Adj64 {
 
 // Inflow tables (jet): base profile u0[nk][nj] and forcing shapes
 // Gf[m*4+f][nk][nj] = g(r) cos(m theta + phi_mf), at i = 0.
+// Entrance forcing sum_mf A_mf sin(omega_f t + psi_mf) g(r) cos(m theta + phi_mf) as 15 shapes
+// g cos m theta, g sin m theta with one coefficient each per stage time (the 32 products of an
+// amplitude, its sine and the cosine or sine of its azimuthal phase summed over the frequencies):
+// less than half the table that 32 shapes take, and of the serial sum at each entrance node.
 struct Inflow {
   double* u0;
-  double* Gf;
+  double* T;                     // [15][nk][nj] shapes
   double amp[kNF];
   double psi[kNF];
+  double cphi[kNF], sphi[kNF];   // cosine and sine of the azimuthal phases
   double omega[JZ_N_FREQ];       // 2 pi St_f U_j
-  double* sn;                    // [5][32] temporal factors sin(omega_f (t + alpha_l dt) + psi_mf) of the
-                                 // current step's stages, written with dt (device)
+  double* co;                    // [5][15] the shapes' coefficients at the current step's stage times
+                                 // t + alpha_l dt, written with dt (device)
 };
+// mode of shape n, and whether it is a sine
+__host__ __device__ __forceinline__ int shape_mode(int n) { return n < JZ_N_MODES ? n : n - JZ_N_MODES + 1; }
+__host__ __device__ __forceinline__ bool shape_sine(int n) { return n >= JZ_N_MODES; }
+// coefficient of shape n from am = amplitude times temporal factor
+__host__ __device__ __forceinline__ double shape_coef(int n, const double* am, const double* cphi, const double* sphi) {
+  double x = 0.0;
+  for (int f = 0; f < JZ_N_FREQ; ++f) {
+    const int mf = shape_mode(n) * JZ_N_FREQ + f;
+    x += shape_sine(n) ? -am[mf] * sphi[mf] : am[mf] * cphi[mf];
+  }
+  return x;
+}
 
 // ---- kernels' host launchers -------------------------------------------
 // metrics

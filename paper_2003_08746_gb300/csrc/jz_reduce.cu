@@ -101,20 +101,24 @@ __global__ void __launch_bounds__(kTPB) k_cfl_rate(Dims d, GridDev g, State q, C
   }
 }
 
-// Temporal factors of the entrance forcing at the five stage times of the step (t, dt), one
-// thread each; a step evaluates them once instead of once per entrance block and stage.
+// Coefficients of the entrance shapes at the five stage times of the step (t, dt), one thread for a
+// sine and then one for a coefficient; a step evaluates them once instead of once per entrance
+// block and stage.
 struct Forcing {
-  double psi[kNF], omega[JZ_N_FREQ];
-  double* sn;                    // null off the jet
+  double amp[kNF], psi[kNF], cphi[kNF], sphi[kNF], omega[JZ_N_FREQ];
+  double* co;                    // null off the jet
 };
 constexpr int kForcing = 5 * kNF;
 __device__ __forceinline__ void stage_forcing(const Forcing& f, double t, double dt) {
   const double alpha[5] = {0.25, 1.0 / 6.0, 0.375, 0.5, 1.0};
-  const int l = threadIdx.x / kNF, mf = threadIdx.x % kNF;
-  if (f.sn && l < 5) f.sn[threadIdx.x] = sin(f.omega[mf % JZ_N_FREQ] * (t + alpha[l] * dt) + f.psi[mf]);
+  __shared__ double am[kForcing];
+  const int th = threadIdx.x, l = th / kNF, mf = th % kNF;
+  if (f.co) am[th] = f.amp[mf] * sin(f.omega[mf % JZ_N_FREQ] * (t + alpha[l] * dt) + f.psi[mf]);
+  __syncthreads();
+  if (f.co && th < 5 * kNT) f.co[th] = shape_coef(th % kNT, am + th / kNT * kNF, f.cphi, f.sphi);
 }
 
-__global__ void k_set_dt(Consts c, Forcing f, Scalars* sc) {
+__global__ void __launch_bounds__(kForcing) k_set_dt(Consts c, const __grid_constant__ Forcing f, Scalars* sc) {
   const double dt = c.dt_fixed > 0.0 ? c.dt_fixed : c.cfl / sc->rate_max;
   stage_forcing(f, sc->t, dt);
   __syncthreads();
@@ -124,7 +128,7 @@ __global__ void k_set_dt(Consts c, Forcing f, Scalars* sc) {
   sc->res_sum = 0.0;
 }
 
-__global__ void k_set_time(Forcing f, Scalars* sc, double t, double dt) {
+__global__ void __launch_bounds__(kForcing) k_set_time(const __grid_constant__ Forcing f, Scalars* sc, double t, double dt) {
   stage_forcing(f, t, dt);
   if (threadIdx.x == 0) {
     sc->t = t;
@@ -134,8 +138,13 @@ __global__ void k_set_time(Forcing f, Scalars* sc, double t, double dt) {
 
 Forcing forcing_of(const Inflow& in) {
   Forcing f;
-  f.sn = in.sn;
-  for (int mf = 0; mf < kNF; ++mf) f.psi[mf] = in.psi[mf];
+  f.co = in.co;
+  for (int mf = 0; mf < kNF; ++mf) {
+    f.amp[mf] = in.amp[mf];
+    f.psi[mf] = in.psi[mf];
+    f.cphi[mf] = in.cphi[mf];
+    f.sphi[mf] = in.sphi[mf];
+  }
   for (int q = 0; q < JZ_N_FREQ; ++q) f.omega[q] = in.omega[q];
   return f;
 }
