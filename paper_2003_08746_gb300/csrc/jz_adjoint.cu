@@ -8,7 +8,7 @@
 // two threads write the same address), except the transposed ghost map,
 // which scatter-adds the adjoint of every ghost node onto the real node it
 // copies.  Forward intermediates are recomputed from the stage input with
-// the forward nodal and viscous kernels.  Non-smooth points take the same
+// the forward nodal kernel and the sensors' own.  Non-smooth points take the same
 // branch conventions as the forward code: max() gives its derivative to the
 // first argument on ties, |x| and sqrt(x) at 0 have derivative 0, cbrt'(0)
 // is 0, and the supersonic/subsonic and inflow/outflow switches take the

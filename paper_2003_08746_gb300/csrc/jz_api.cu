@@ -1048,7 +1048,7 @@ int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ck
           JZ_RUN(JZ_PROF_VISCOUS, jz::sensor_df_pass(d, s->w, s->st));
         } else {
           JZ_RUN(JZ_PROF_NODAL, jz::nodal64(d, s->c, g, s->w, *st[l], s->st));
-          JZ_RUN(JZ_PROF_VISCOUS, jz::viscous64(d, s->c, g, s->w, *st[l], s->st));
+          JZ_RUN(JZ_PROF_VISCOUS, jz::sensor64(d, s->w, s->st));
         }
         JZ_RUN(JZ_PROF_ADJOINT, jz::adj_stage(d, s->c, g, s->w, *st[l], a, s->pair ? &s->mdf : nullptr,
                                               s->pair ? &s->qdf : nullptr, s->st));

@@ -348,6 +348,7 @@ cudaError_t nodal64(const Dims& d, const Consts& c, const GridDev& g, const Work
                     cudaStream_t st, double* rate_max = nullptr);
 cudaError_t viscous64(const Dims& d, const Consts& c, const GridDev& g, const Work64& w, const State& qin,
                       cudaStream_t st);
+cudaError_t sensor64(const Dims& d, const Work64& w, cudaStream_t st);
 cudaError_t faces64(const Dims& d, const Consts& c, const Work64& w, const State& qin, cudaStream_t st);
 // stage update (rhs_flat == nullptr) or RHS output to rhs_flat [5][N]
 cudaError_t update64(const Dims& d, const GridDev& g, const Work64& w, const State& qin, const State& qn,
