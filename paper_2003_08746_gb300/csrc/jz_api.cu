@@ -238,21 +238,21 @@ int mark(jz_solver* s, int kind) {
 // cfl_first: stage 1 of a CFL step; the nodal pass reduces the rate of Q^n (Scalars::rate_max
 // is 0 between FP64 steps) and the time step is set from it before the update.
 int run_stage64(jz_solver* s, const jz::State& in, const jz::State& out, double alpha, int want_res,
-                double* rhs_flat, bool cfl_first = false) {
+                double* rhs_flat, bool cfl_first = false, jz::Finish finish = jz::FINISH_NONE) {
   const jz::Dims& d = s->grid->d;
   const jz::GridDev& g = s->grid->g;
   if (s->pair) {
     JZ_RUN(JZ_PROF_VISCOUS, jz::flux_df(d, s->c, s->mdf, s->w, s->qdf, in, s->sc, s->st, cfl_first));
     if (cfl_first) JZ_RUN(JZ_PROF_REDUCE, jz::set_dt(s->c, s->in, s->sc, s->st));
     JZ_RUN(JZ_PROF_FACES, jz::faces_update_df(d, s->c, g, s->w, s->qdf, in, s->qn, out, s->sc, alpha, want_res,
-                                              rhs_flat, s->st));
+                                              rhs_flat, s->st, finish));
     return JZ_OK;
   }
   JZ_RUN(JZ_PROF_NODAL, jz::nodal64(d, s->c, g, s->w, in, s->st, cfl_first ? &s->sc->rate_max : nullptr));
   if (cfl_first) JZ_RUN(JZ_PROF_REDUCE, jz::set_dt(s->c, s->in, s->sc, s->st));
   JZ_RUN(JZ_PROF_VISCOUS, jz::viscous64(d, s->c, g, s->w, in, s->st));
   JZ_RUN(JZ_PROF_FACES, jz::faces64(d, s->c, s->w, in, s->st));
-  JZ_RUN(JZ_PROF_UPDATE, jz::update64(d, g, s->w, in, s->qn, out, s->sc, alpha, want_res, rhs_flat, s->st));
+  JZ_RUN(JZ_PROF_UPDATE, jz::update64(d, g, s->w, in, s->qn, out, s->sc, alpha, want_res, rhs_flat, s->st, finish));
   return JZ_OK;
 }
 
@@ -277,6 +277,8 @@ int run_step(jz_solver* s) {
     if (cfl && !s->rate_ready) JZ_RUN(JZ_PROF_REDUCE, jz::cfl_rate(d, s->c, g, s->Mf, s->qn, s->sc, s->st));
     JZ_RUN(JZ_PROF_REDUCE, jz::set_dt(s->c, s->in, s->sc, s->st));
   }
+  // a box's FP64 and pair updates write its ghosts themselves
+  const bool ghosts = !s->fp32 && d.topo == JZ_TOPO_PERIODIC;
   jz::State in = s->qn;
   for (int l = 0; l < 5; ++l) {
     jz::State out = (l % 2 == 0) ? s->qa : s->qb;
@@ -285,9 +287,10 @@ int run_step(jz_solver* s) {
       JZ_RUN(JZ_PROF_FUSED32, jz::fused32(d, s->c, s->Mf, in, s->tmap_of(in), s->qn, out, s->sc, kAlpha[l], l == 0,
                                           l == 4 && cfl, nullptr, s->kchunk, s->st));
     else
-      r = run_stage64(s, in, out, kAlpha[l], l == 0, nullptr, l == 0 && cfl);
+      r = run_stage64(s, in, out, kAlpha[l], l == 0, nullptr, l == 0 && cfl,
+                      !ghosts ? jz::FINISH_NONE : l == 4 ? jz::FINISH_STEP : jz::FINISH_GHOSTS);
     if (r) return r;
-    r = run_shell(s, out, l, l == 4);
+    if (!ghosts) r = run_shell(s, out, l, l == 4);
     if (r) return r;
     in = out;
   }

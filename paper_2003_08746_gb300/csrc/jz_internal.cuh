@@ -350,10 +350,13 @@ cudaError_t viscous64(const Dims& d, const Consts& c, const GridDev& g, const Wo
                       cudaStream_t st);
 cudaError_t sensor64(const Dims& d, const Work64& w, cudaStream_t st);
 cudaError_t faces64(const Dims& d, const Consts& c, const Work64& w, const State& qin, cudaStream_t st);
+// What the update of a stage does beside the real nodes: nothing (the jet: jet_shell follows), the
+// ghosts of a periodic box, or these and t += dt (the last stage of a step).
+enum Finish { FINISH_NONE = 0, FINISH_GHOSTS = 1, FINISH_STEP = 2 };
 // stage update (rhs_flat == nullptr) or RHS output to rhs_flat [5][N]
 cudaError_t update64(const Dims& d, const GridDev& g, const Work64& w, const State& qin, const State& qn,
-                     const State& qout, const Scalars* sc, double alpha, int want_res, double* rhs_flat,
-                     cudaStream_t st);
+                     const State& qout, Scalars* sc, double alpha, int want_res, double* rhs_flat,
+                     cudaStream_t st, Finish finish = FINISH_NONE);
 // FP32-flux stage (one fused kernel); Mf = the FP32 metric records (kMF floats per padded node);
 // tm_in = the tensor map of qin's shadow (make_shadow_map).  The stage reads qin's shadow and
 // writes qout and its shadow (or, with rhs_flat, the RHS only).
@@ -378,8 +381,9 @@ cudaError_t flux_df(const Dims& d, const Consts& c, const DFMetrics& M, const Wo
                     const State& qin, Scalars* sc, cudaStream_t st, int want_rate = 0);
 cudaError_t sensor_df_pass(const Dims& d, const Work64& w, cudaStream_t st);
 cudaError_t faces_update_df(const Dims& d, const Consts& c, const GridDev& g, const Work64& w, const QDF& qdf,
-                            const State& qin, const State& qn, const State& qout, const Scalars* sc, double alpha,
-                            int want_res, double* rhs_flat, cudaStream_t st);
+                            const State& qin, const State& qn, const State& qout, Scalars* sc, double alpha,
+                            int want_res, double* rhs_flat, cudaStream_t st,
+                            Finish finish = FINISH_NONE);
 // boundary conditions and ghost points of the jet after stage `stage` (one kernel); advance: last
 // stage of a step, t += dt.  Needs the temporal factors that set_dt or set_time left for the step.
 cudaError_t jet_shell(const Dims& d, const Consts& c, const GridDev& g, const Inflow& in, const State& q,
@@ -470,6 +474,27 @@ __host__ __device__ inline void ghost_source(const Dims& d, int i, int j, int k,
   else if (j >= d.nj) { sj = d.nj - 1; }
   else { sj = j; }
   sk = ((kk % d.nk) + d.nk) % d.nk;
+}
+
+// The ghosts of a periodic box that copy the real node (i, j, k): every f(p) of a padded node whose
+// coordinates are its own by whole periods (several where an extent is under two).  The kernel that
+// writes a real node of a box writes them beside it.
+__device__ __forceinline__ bool has_images(const Dims& d, int i, int j, int k) {
+  return i < kG || i >= d.ni - kG || j < kG || j >= d.nj - kG || k < kG || k >= d.nk - kG;
+}
+template <class F>
+__device__ __forceinline__ void for_images(const Dims& d, int i, int j, int k, F f) {
+  int i0 = i, j0 = j, k0 = k;
+  while (i0 - d.ni >= -kG) i0 -= d.ni;
+  while (j0 - d.nj >= -kG) j0 -= d.nj;
+  while (k0 - d.nk >= -kG) k0 -= d.nk;
+#pragma unroll 1
+  for (int kk = k0; kk < d.nk + kG; kk += d.nk)
+#pragma unroll 1
+    for (int jj = j0; jj < d.nj + kG; jj += d.nj)
+#pragma unroll 1
+      for (int ii = i0; ii < d.ni + kG; ii += d.ni)
+        if (ii != i || jj != j || kk != k) f(pidx(d, ii, jj, kk));
 }
 
 // Ghost shell enumerated directly: the four k-ghost planes (with their i/j

@@ -212,11 +212,12 @@ __global__ void __launch_bounds__(kTPB) k_faces(Dims d, Consts c, Work64 w, Stat
   }
 }
 
-// mode 0: stage update; mode 1: write RHS to rhs_flat (unpadded [5][N]).
+// mode 0: stage update; mode 1: write RHS to rhs_flat (unpadded [5][N]); mode 2: stage update of a
+// periodic box with its ghosts.
 template <int MODE>
 __global__ void __launch_bounds__(kTPB) k_update(Dims d, GridDev g, Work64 w, State qin, State qn, State qout,
-                                                 const Scalars* sc, double alpha, int want_res,
-                                                 double* rhs_flat, double* res_sum) {
+                                                 Scalars* sc, double alpha, int want_res,
+                                                 double* rhs_flat, double* res_sum, int last) {
   Box b{0, 0, 0, d.ni, d.nj, d.nk};
   int i, j, k;
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -235,13 +236,18 @@ __global__ void __launch_bounds__(kTPB) k_update(Dims d, GridDev g, Work64 w, St
       const double* G2 = w.G[2][m];
       R[m] = ((G0[p] - G0[p - s[0]]) + (G1[p] - G1[p - s[1]])) + (G2[p] - G2[p - s[2]]);
     }
-    if (MODE == 0) {
+    if (MODE != 1) {
       const double adtV = alpha * sc->dt * hV;
       double qnew[5];
       for (int m = 0; m < 5; ++m) {
         qnew[m] = adv ? qn.q[m][p] - adtV * R[m] : qin.q[m][p];
         qout.q[m][p] = qnew[m];
       }
+      if (MODE == 2 && has_images(d, i, j, k))
+        for_images(d, i, j, k, [&](long long g) {
+          for (int m = 0; m < 5; ++m) qout.q[m][g] = qnew[m];
+        });
+      if (MODE == 2 && last && t == 0) sc->t = sc->t + sc->dt;
     } else {
       const long long N = (long long)d.ni * d.nj * d.nk;
       for (int m = 0; m < 5; ++m) rhs_flat[m * N + t] = adv ? R[m] * hV : 0.0;
@@ -294,15 +300,12 @@ cudaError_t faces64(const Dims& d, const Consts& c, const Work64& w, const State
 }
 
 cudaError_t update64(const Dims& d, const GridDev& g, const Work64& w, const State& qin, const State& qn,
-                     const State& qout, const Scalars* sc, double alpha, int want_res, double* rhs_flat,
-                     cudaStream_t st) {
-  const long long nr = (long long)d.ni * d.nj * d.nk;
-  double* res_sum = const_cast<double*>(&sc->res_sum);
-  if (rhs_flat)
-    k_update<1><<<blocks_for(nr, kTPB), kTPB, 0, st>>>(d, g, w, qin, qn, qout, sc, alpha, 0, rhs_flat, res_sum);
-  else
-    k_update<0><<<blocks_for(nr, kTPB), kTPB, 0, st>>>(d, g, w, qin, qn, qout, sc, alpha, want_res, nullptr,
-                                                       res_sum);
+                     const State& qout, Scalars* sc, double alpha, int want_res, double* rhs_flat,
+                     cudaStream_t st, Finish finish) {
+  const unsigned n = blocks_for((long long)d.ni * d.nj * d.nk, kTPB);
+  const int res = rhs_flat ? 0 : want_res;
+  const auto kernel = rhs_flat ? k_update<1> : finish == FINISH_NONE ? k_update<0> : k_update<2>;
+  kernel<<<n, kTPB, 0, st>>>(d, g, w, qin, qn, qout, sc, alpha, res, rhs_flat, &sc->res_sum, finish == FINISH_STEP);
   return cudaGetLastError();
 }
 

@@ -294,8 +294,8 @@ __global__ void __launch_bounds__(VX*(VY - 2), 3) k_flux_df(const __grid_constan
 
 // C + D: Turkel-Vatsa dissipation, RHS and stage update in one kernel.  Per node and variable
 //   2 V RHS = sum_dir [ H(n+1) - H(n-1) - (D(n+1/2) - D(n-1/2)) ],  D = 2 d,
-// in double-float, then Q^n - alpha dt RHS in FP64 (mode 0) or the RHS itself (mode 1).  Neither the
-// faces nor their sums leave the SM.
+// in double-float, then Q^n - alpha dt RHS in FP64 (mode 0; mode 2: a periodic box, with its ghosts) or
+// the RHS itself (mode 1).  Neither the faces nor their sums leave the SM.
 // 2 d = a32 d1 - b2 e3 on the face between p and p + sd, with d1 and e3 the differences of Q over the
 // face (one and three spacings): Ls = 2 L_f, b2 = Ls eps4, a32 = 3 b2 + Ls eps2, as (a32, b2).
 __device__ __forceinline__ float4 face_coef(const ConstsDF& c, const float2* nu, const float2* Lam, long long p,
@@ -324,8 +324,9 @@ struct FacesArgs {
   const double* qin[5];
   const double* qn[5];
   double* qout[5];
-  const Scalars* sc;
+  Scalars* sc;
   double alpha;
+  int last;              // t += dt (mode 2)
   double* rhs;           // [5][N] (mode 1)
   double* res_sum;       // non-null: add the sum of RHS_rho^2
   int kchunk;
@@ -359,6 +360,7 @@ __global__ void __launch_bounds__(FX* FY, 4) k_faces_update_df(const __grid_cons
   const bool adv = advanced(d, i, j);
   const long long sj = d.sj, sk = d.sk;
   long long p = pidx(d, i, j, k0);
+  const double adt = MODE != 1 ? A.alpha * A.sc->dt : 0.0;
   double r2 = 0.0;
   if (node) {
     const float4 cf = face_coef(c, A.nu[2], A.Lam[2], p - sk, sk);
@@ -414,8 +416,8 @@ __global__ void __launch_bounds__(FX* FY, 4) k_faces_update_df(const __grid_cons
       for (int m = 0; m < 5; ++m) {
         const float2 t1 = g1s[b][m][y][x], t0 = g1s[b][m][y - 1][x];
         const double R64 = df_to_f64(df_sub_l(R[m], df_sub_l(df_make(t1.x, t1.y), df_make(t0.x, t0.y))));
-        if (MODE == 0) {
-          A.qout[m][p] = adv ? fma(-(A.alpha * A.sc->dt * hV), R64, A.qn[m][p]) : A.qin[m][p];
+        if (MODE != 1) {
+          A.qout[m][p] = adv ? fma(-(adt * hV), R64, A.qn[m][p]) : A.qin[m][p];
         } else {
           const long long N = (long long)d.ni * d.nj * d.nk, t = ((long long)k * d.nj + j) * d.ni + i;
           A.rhs[m * N + t] = adv ? R64 * hV : 0.0;
@@ -425,8 +427,20 @@ __global__ void __launch_bounds__(FX* FY, 4) k_faces_update_df(const __grid_cons
           r2 += r0 * r0;
         }
       }
+      // (values read back from what this thread has just written: registers for them would cost
+      // every node)
+      if (MODE == 2 && has_images(d, i, j, k)) {
+        double v[5];
+#pragma unroll
+        for (int m = 0; m < 5; ++m) v[m] = A.qout[m][p];
+        for_images(d, i, j, k, [&](long long g) {
+#pragma unroll
+          for (int m = 0; m < 5; ++m) A.qout[m][g] = v[m];
+        });
+      }
     }
   }
+  if (MODE == 2 && A.last && blockIdx.x == 0 && blockIdx.y == 0 && x == 0 && y == 0) A.sc->t = A.sc->t + A.sc->dt;
   if (A.res_sum) {
     __shared__ double red[FY];
     for (int o = 16; o > 0; o >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, o);
@@ -534,8 +548,8 @@ cudaError_t flux_df(const Dims& d, const Consts& c, const DFMetrics& M, const Wo
 }
 
 cudaError_t faces_update_df(const Dims& d, const Consts& c, const GridDev& g, const Work64& w, const QDF& qdf,
-                            const State& qin, const State& qn, const State& qout, const Scalars* sc, double alpha,
-                            int want_res, double* rhs_flat, cudaStream_t st) {
+                            const State& qin, const State& qn, const State& qout, Scalars* sc, double alpha,
+                            int want_res, double* rhs_flat, cudaStream_t st, Finish finish) {
   FacesArgs A;
   A.d = d;
   A.c = make_cdf(c);
@@ -554,17 +568,16 @@ cudaError_t faces_update_df(const Dims& d, const Consts& c, const GridDev& g, co
   A.invV = g.invV;
   A.sc = sc;
   A.alpha = alpha;
+  A.last = finish == FINISH_STEP;
   A.rhs = rhs_flat;
-  A.res_sum = want_res && !rhs_flat ? const_cast<double*>(&sc->res_sum) : nullptr;
+  A.res_sum = want_res && !rhs_flat ? &sc->res_sum : nullptr;
   A.nbx = (d.ni + FX - 2) / (FX - 1);
   const long long tiles = (long long)A.nbx * ((d.nj + FY - 2) / (FY - 1));
   static int slots[64];
   A.kchunk = faces_chunk((double)tiles * d.nk / resident_blocks(k_faces_update_df<0>, FX * FY, slots));
   const dim3 gr((unsigned)tiles, (d.nk + A.kchunk - 1) / A.kchunk), blk(FX, FY);
-  if (rhs_flat)
-    k_faces_update_df<1><<<gr, blk, 0, st>>>(A);
-  else
-    k_faces_update_df<0><<<gr, blk, 0, st>>>(A);
+  const auto kernel = rhs_flat ? k_faces_update_df<1> : finish == FINISH_NONE ? k_faces_update_df<0> : k_faces_update_df<2>;
+  kernel<<<gr, blk, 0, st>>>(A);
   return cudaGetLastError();
 }
 

@@ -64,6 +64,17 @@ def test_pair_tiles(jz, shape):
     _against_oracle(jz, g, W.random_state(g, seed=9, amp=0.05), W.box_params(), jz.JZ_PREC_FP64PAIR, 2, 1e-12)
 
 
+# a box's update writes its ghosts: extents under two (several images of a node along an axis), and
+# blocks and chunks that hold one edge, both or none
+@pytest.mark.parametrize("shape", [(1, 1, 1), (2, 1, 3), (3, 5, 2), (4, 2, 1), (1, 40, 3), (37, 3, 12), (5, 17, 70)])
+@pytest.mark.parametrize("form", ["FP64", "FP64PAIR"])
+def test_box_ghosts(jz, shape, form):
+    g = W.box_grid(*shape, h=0.21)
+    st, t, _ = _against_oracle(jz, g, W.random_state(g, seed=4, amp=0.05), W.box_params(), getattr(jz, "JZ_PREC_" + form), 3,
+                               1e-12)
+    assert abs(st.t - t) <= 1e-12 * t
+
+
 # the first FP32-flux step's rate: its maximum anywhere in a turn of 32 nodes, ties everywhere,
 # supersonic flow (pressure the small rest of e), and cells too small for FP32 bounds
 @pytest.mark.parametrize("case", ["noise", "uniform", "hypersonic", "tiny", "jet", "one"])
