@@ -366,9 +366,12 @@ struct FacesArgs {
 // Issue-bound (62%) with load latency behind it: 8.1 ms per launch on 512 x 512 x 360 with 32 x 8
 // blocks at four per SM (8.3 for 32 x 16 at two, 8.1 for 32 x 12 at three), 9.2 before with face sums.
 // One variable per thread (five times the threads, coefficients through shared memory) took 16.9.
+// PER blocks per SM: 4, or 2 where every plane of every tile is resident at two: load latency alone is left
+// then, and 128 registers hold more loads in flight than 64 (32 x 24 x 16: 0.9 us per launch less,
+// ten steps 0.98 -> 0.92 ms; with 360 blocks on 304 places 70 x 40 x 20 would take 18.9 us instead of 15.6).
 constexpr int FX = 32, FY = 8;
-template <int MODE>
-__global__ void __launch_bounds__(FX* FY, 4) k_faces_update_df(const __grid_constant__ FacesArgs A) {
+template <int MODE, int PER>
+__global__ void __launch_bounds__(FX* FY, PER) k_faces_update_df(const __grid_constant__ FacesArgs A) {
   const Dims& d = A.d;
   const ConstsDF& c = A.c;
   __shared__ float2 g1s[2][5][FY][FX];   // faces j + 1/2 of the plane, two planes in turn
@@ -595,10 +598,15 @@ cudaError_t faces_update_df(const Dims& d, const Consts& c, const GridDev& g, co
   A.res_sum = want_res && !rhs_flat ? &sc->res_sum : nullptr;
   A.nbx = (d.ni + FX - 2) / (FX - 1);
   const long long tiles = (long long)A.nbx * ((d.nj + FY - 2) / (FY - 1));
-  static int slots[64];
-  A.kchunk = faces_chunk((double)tiles * d.nk / resident_blocks(k_faces_update_df<0>, FX * FY, slots));
+  static int slots[64], slots2[64];
+  const long long planes = tiles * d.nk;
+  const bool small = planes <= resident_blocks(k_faces_update_df<0, 2>, FX * FY, slots2);
+  A.kchunk = small ? 1 : faces_chunk((double)planes / resident_blocks(k_faces_update_df<0, 4>, FX * FY, slots));
   const dim3 gr((unsigned)tiles, (d.nk + A.kchunk - 1) / A.kchunk), blk(FX, FY);
-  const auto kernel = rhs_flat ? k_faces_update_df<1> : finish == FINISH_NONE ? k_faces_update_df<0> : k_faces_update_df<2>;
+  const int mode = rhs_flat ? 1 : finish == FINISH_NONE ? 0 : 2;
+  const auto kernel = mode == 0   ? (small ? k_faces_update_df<0, 2> : k_faces_update_df<0, 4>)
+                      : mode == 1 ? (small ? k_faces_update_df<1, 2> : k_faces_update_df<1, 4>)
+                                  : (small ? k_faces_update_df<2, 2> : k_faces_update_df<2, 4>);
   kernel<<<gr, blk, 0, st>>>(A);
   return cudaGetLastError();
 }
