@@ -96,9 +96,11 @@ __global__ void __launch_bounds__(BX* BY) k_sensor_df(Dims d, Work64 w) {
 // at three blocks per SM (80 registers); at four (64, spills) 10% slower, at two (128) 12%; 14 rows at
 // two the same, but slower on small grids.  Warps for the halo rows that then idle through the fluxes:
 // 5% slower.  Split arrivals instead of a barrier per plane (warps drifting by a plane): 12%.
-// Sums and products inside a chain are unnormalized pairs (every pair normalized: 6% slower), H, the
-// sensors and what seeds a root or reciprocal normalized: the residual's error against 64 bits is
-// 1.07e-12 on a 333 x 177 x 90 jet, 1.11e-12 with every pair normalized and face sums of H.
+// Sums and products inside a chain are unnormalized pairs (every pair normalized: 6% slower); U, H, the
+// sensors, what seeds a root or reciprocal, and in the dissipation the difference over a face (where
+// the leading parts cancel) are normalized.  The residual's error against 64 bits: 9.6e-13 on a
+// 333 x 177 x 90 jet, 1.1e-13 on 40 x 20 x 16; with every pair normalized but face sums of H instead of
+// differences 1.1e-12 and 1.2e-13, without the two last normalizations 1.07e-12 and 1.2e-13 (and 0.6% faster).
 constexpr int VX = 32, VY = 10;      // nodes of the tile with its one-node halo
 
 // Element of a field at a 32-bit byte offset (every field of a pair solver is below 4 GB: its 632
@@ -272,8 +274,8 @@ __global__ void __launch_bounds__(VX*(VY - 2), 3) k_flux_df(const __grid_constan
 #pragma unroll
         for (int dir = 0; dir < 3; ++dir) {
           const dfl sx = S[dir][0], sy = S[dir][1], sz = S[dir][2];
-          const dfl U = df_fma_l(sz, w, df_fma_l(sy, v, df_mul_l(sx, u)));
-          lam[dir] = df_fma(a, ldo(A.Smag[dir], p), df_abs(df_n(U)));
+          const dfl U = df_n(df_fma_l(sz, w, df_fma_l(sy, v, df_mul_l(sx, u))));
+          lam[dir] = df_fma(a, ldo(A.Smag[dir], p), df_abs(U));
           // H^dir = [rho U, m_i U + S_j P_ji, e U + S_j X_j]
           auto flux = [&](dfl q, dfl f1, dfl f2, dfl f3) {
             return df_n(df_fma_l(q, U, df_fma_l(sz, f3, df_fma_l(sy, f2, df_mul_l(sx, f1)))));
@@ -331,7 +333,7 @@ __device__ __forceinline__ float4 face_coef(const ConstsDF& c, const float2* nu,
   return make_float4(a32.hi, a32.lo, b2.hi, b2.lo);
 }
 __device__ __forceinline__ dfl face_diss(float4 k, dfl qm, dfl q0, dfl q1, dfl q2) {
-  const dfl d1 = df_sub_l(q1, q0), e3 = df_sub_l(q2, qm);
+  const dfl d1 = df_n(df_sub_l(q1, q0)), e3 = df_sub_l(q2, qm);
   return df_fma_l(df_make(-k.z, -k.w), e3, df_mul_l(df_make(k.x, k.y), d1));
 }
 
