@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(BX* BY) k_sensor_df(Dims d, Work64 w) {
 // nodal and a viscous pass).
 // The momentum and energy fluxes are contracted as H_m = m_m U + S_j P_jm, P = p I - tau, and
 // H_e = e U + S_j (u_m P_jm - k dT/dx_j).
-// FP32 issue bounds it: 9.6 ms per launch on 512 x 512 x 360 (the two passes before: 11.4) with 8 rows
+// FP32 issue bounds it: 9.5 ms per launch on 512 x 512 x 360 (the two passes before: 11.4) with 8 rows
 // at three blocks per SM (80 registers); at four (64, spills) 10% slower, at two (128) 12%; 14 rows at
 // two the same, but slower on small grids.  Warps for the halo rows that then idle through the fluxes:
 // 5% slower.  Split arrivals instead of a barrier per plane (warps drifting by a plane): 12%.
@@ -202,13 +202,16 @@ __global__ void __launch_bounds__(VX*(VY - 2), 3) k_flux_df(const __grid_constan
     if (row != y || extra < 0) break;
   }
   for (int k = k0; k < k1; ++k, p += sk) {
-    dfl S[3][3] = {}, iV = {}, Delta = {};
+    dfl S[3][3] = {}, Smag[3] = {}, iV = {}, Delta = {};
     if (out) {
-      // the metrics of plane k, requested before the primitives of plane k + 1 that hide their latency
+      // the metrics of plane k, requested before the primitives of plane k + 1 that hide their latency (a load
+      // that follows a store to another array waits for it: |S| read beside its use cost 2.7%)
 #pragma unroll
-      for (int dir = 0; dir < 3; ++dir)
+      for (int dir = 0; dir < 3; ++dir) {
 #pragma unroll
         for (int cc = 0; cc < 3; ++cc) S[dir][cc] = ldo(A.S[3 * dir + cc], p);
+        Smag[dir] = ldo(A.Smag[dir], p);
+      }
       iV = ldo(A.invV, p);
       Delta = ldo(A.Delta, p);
     }
@@ -275,7 +278,7 @@ __global__ void __launch_bounds__(VX*(VY - 2), 3) k_flux_df(const __grid_constan
         for (int dir = 0; dir < 3; ++dir) {
           const dfl sx = S[dir][0], sy = S[dir][1], sz = S[dir][2];
           const dfl U = df_n(df_fma_l(sz, w, df_fma_l(sy, v, df_mul_l(sx, u))));
-          lam[dir] = df_fma(a, ldo(A.Smag[dir], p), df_abs(U));
+          lam[dir] = df_fma(a, Smag[dir], df_abs(U));
           // H^dir = [rho U, m_i U + S_j P_ji, e U + S_j X_j]
           auto flux = [&](dfl q, dfl f1, dfl f2, dfl f3) {
             return df_n(df_fma_l(q, U, df_fma_l(sz, f3, df_fma_l(sy, f2, df_mul_l(sx, f1)))));
@@ -365,8 +368,8 @@ struct FacesArgs {
 // the difference of their neighbours, not as face sums: fewer operations and a smaller rounding
 // error (H(n+1) - H(n-1) cancels before anything is rounded), and the dissipation, small beside the
 // flux, is summed in unnormalized pairs.
-// Issue-bound (62%) with load latency behind it: 8.1 ms per launch on 512 x 512 x 360 with 32 x 8
-// blocks at four per SM (8.3 for 32 x 16 at two, 8.1 for 32 x 12 at three), 9.2 before with face sums.
+// Issue-bound (62%) with load latency behind it: 7.6 ms per launch on 512 x 512 x 360 with 32 x 8
+// blocks at four per SM (when it took 8.1: 8.3 for 32 x 16 at two, 8.1 for 32 x 12 at three; 9.2 with face sums).
 // One variable per thread (five times the threads, coefficients through shared memory) took 16.9.
 // PER blocks per SM: 4, or 2 where every plane of every tile is resident at two: load latency alone is left
 // then, and 128 registers hold more loads in flight than 64 (32 x 24 x 16: 0.9 us per launch less,
@@ -438,13 +441,20 @@ __global__ void __launch_bounds__(FX* FY, PER) k_faces_update_df(const __grid_co
     }
     __syncthreads();
     if (node) {
+      // all of Q^n before the first store (behind it each load would wait for the one before: 5% of the
+      // kernel)
+      double qn[5] = {};
+      if (MODE != 1) {
+#pragma unroll
+        for (int m = 0; m < 5; ++m) qn[m] = A.qn[m][p];
+      }
       const double hV = 0.5 * A.invV[p];
 #pragma unroll
       for (int m = 0; m < 5; ++m) {
         const float2 t1 = g1s[b][m][y][x], t0 = g1s[b][m][y - 1][x];
         const double R64 = df_to_f64(df_sub_l(R[m], df_sub_l(df_make(t1.x, t1.y), df_make(t0.x, t0.y))));
         if (MODE != 1) {
-          A.qout[m][p] = adv ? fma(-(adt * hV), R64, A.qn[m][p]) : A.qin[m][p];
+          A.qout[m][p] = adv ? fma(-(adt * hV), R64, qn[m]) : A.qin[m][p];
         } else {
           const long long N = (long long)d.ni * d.nj * d.nk, t = ((long long)k * d.nj + j) * d.ni + i;
           A.rhs[m * N + t] = adv ? R64 * hV : 0.0;
