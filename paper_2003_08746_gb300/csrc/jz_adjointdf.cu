@@ -13,6 +13,11 @@
 
 namespace jz {
 namespace {
+// an element of an array that the kernel does not write: the load may move before stores to others
+__device__ __forceinline__ dfl ldc(const double* f, long long p) {
+  const float2 v = __ldg(reinterpret_cast<const float2*>(f) + p);
+  return df_make(v.x, v.y);
+}
 
 // Node of a launch over the box [o, o + ei) x [o, o + ej) x [o, o + ek): the plane's nodes in a row
 // along blockIdx.x (no lanes lost to tiles that overhang it: 64 x 4 tiles cost the 130 nodes along i
@@ -34,10 +39,17 @@ __global__ void k_adj_update_df(Dims d, GridDev g, Adj64 a, double adt) {
   const long long p = pidx(d, i, j, k);
   const bool adv = d.topo != JZ_TOPO_JET || (i >= 1 && i <= d.ni - 2 && j >= 1 && j <= d.nj - 2);
   const double f = -adt * g.invV[p];
+  // (every load before the first store: behind it each would wait for the one before)
+  double l[5], qb[5];
+#pragma unroll
   for (int m = 0; m < 5; ++m) {
-    const double l = a.lam[m][p];
-    if (adv) a.qnbar[m][p] += l;
-    st(a.acc[m], p, adv ? df_of(f * l) : df_from(0.f));
+    l[m] = a.lam[m][p];
+    qb[m] = a.qnbar[m][p];
+  }
+#pragma unroll
+  for (int m = 0; m < 5; ++m) {
+    if (adv) a.qnbar[m][p] = qb[m] + l[m];
+    st(a.acc[m], p, adv ? df_of(f * l[m]) : df_from(0.f));
   }
 }
 
@@ -85,7 +97,8 @@ __global__ void k_adj_faces_df(Dims d, ConstsDF c, Work64 w, QDF qdf, Adj64 a) {
 // stresses, heat flux and sensors, in double-float arithmetic on the pair intermediates the pair
 // passes regenerated (u, v, w, T, p, mu, the pair copies of Q and of the metrics).  Nodes within
 // one layer of the real region.
-// Four 128-thread blocks per SM (128 registers); three (168) or six (80) are 3% slower.
+// Four 128-thread blocks per SM (128 registers); three (168) or six (80) are 3% slower.  Loads that may not
+// move before the stores: 2% slower.
 constexpr int kTPBV = 128;
 __global__ void __launch_bounds__(kTPBV, 4) k_adj_visc_df(Dims d, ConstsDF c, DFMetrics M, Work64 w, QDF qdf, Adj64 a) {
   int i, j, k;
@@ -95,7 +108,7 @@ __global__ void __launch_bounds__(kTPBV, 4) k_adj_visc_df(Dims d, ConstsDF c, DF
   // adjoint of H^dir (components 1..4 carry the viscous flux)
   dfl Hb[3][4];
   for (int dir = 0; dir < 3; ++dir)
-    for (int m = 0; m < 4; ++m) Hb[dir][m] = df_scale(df_sub_l(ld(a.acc[m + 1], p - s[dir]), ld(a.acc[m + 1], p + s[dir])), 0.5f);
+    for (int m = 0; m < 4; ++m) Hb[dir][m] = df_scale(df_sub_l(ldc(a.acc[m + 1], p - s[dir]), ldc(a.acc[m + 1], p + s[dir])), 0.5f);
   // forward viscous quantities
   const double* f[4] = {w.u, w.v, w.w, w.T};
   dfl S[3][3];
@@ -105,7 +118,7 @@ __global__ void __launch_bounds__(kTPBV, 4) k_adj_visc_df(Dims d, ConstsDF c, DF
   dfl L[4][3];
   for (int n = 0; n < 4; ++n) {
     dfl dd[3];
-    for (int dir = 0; dir < 3; ++dir) dd[dir] = df_scale(df_sub_l(ld(f[n], p + s[dir]), ld(f[n], p - s[dir])), 0.5f);
+    for (int dir = 0; dir < 3; ++dir) dd[dir] = df_scale(df_sub_l(ldc(f[n], p + s[dir]), ldc(f[n], p - s[dir])), 0.5f);
     for (int jj = 0; jj < 3; ++jj)
       L[n][jj] = df_n(df_mul_l(iV, df_fma_l(S[2][jj], dd[2], df_fma_l(S[1][jj], dd[1], df_mul_l(S[0][jj], dd[0])))));
   }
@@ -117,10 +130,10 @@ __global__ void __launch_bounds__(kTPBV, 4) k_adj_visc_df(Dims d, ConstsDF c, DF
   for (int x = 0; x < 3; ++x)
     for (int y = 0; y < 3; ++y) SS = df_fma_l(Sij[x][y], Sij[x][y], SS);
   const dfl Smod = df_sqrt(df_n(df_scale(SS, 2.f)));
-  const dfl mu = ld(w.mu, p);
+  const dfl mu = ldc(w.mu, p);
   const dfl csd = df_mul_l(c.C_s, df_load(M.Delta, p));
   const dfl cs2 = df_mul_l(csd, csd);
-  const dfl rho = ld(qdf.q[0], p);
+  const dfl rho = ldc(qdf.q[0], p);
   const dfl mu_sgs = df_n(df_mul_l(df_mul_l(rho, cs2), Smod));
   const dfl mu_eff = df_add_l(mu, mu_sgs);
   const dfl k_eff = df_add_l(df_mul_l(mu, c.k_lam), df_mul_l(mu_sgs, c.k_sgs));
@@ -129,7 +142,7 @@ __global__ void __launch_bounds__(kTPBV, 4) k_adj_visc_df(Dims d, ConstsDF c, DF
   dfl dev[3][3];                                       // S_ij - delta_ij div/3
   for (int x = 0; x < 3; ++x)
     for (int y = 0; y < 3; ++y) dev[x][y] = x == y ? df_sub_l(Sij[x][y], d3) : Sij[x][y];
-  const dfl vel[3] = {ld(w.u, p), ld(w.v, p), ld(w.w, p)};
+  const dfl vel[3] = {ldc(w.u, p), ldc(w.v, p), ldc(w.w, p)};
   // reverse: F^dir_m = S^dir_j F_j,m ; H = E - F
   dfl taub[3][3], ubd[3], keb = df_from(0.f), L3b[3];
   for (int x = 0; x < 3; ++x) {
@@ -177,10 +190,10 @@ __global__ void __launch_bounds__(kTPBV, 4) k_adj_visc_df(Dims d, ConstsDF c, DF
   st(a.mub, p, df_n(mub));
   st(a.rhob, p, df_n(rhob));
   // pressure sensor nu = |N| / Dn
-  const dfl pc2 = df_scale(ld(w.p, p), 2.f);
+  const dfl pc2 = df_scale(ldc(w.p, p), 2.f);
   for (int dir = 0; dir < 3; ++dir) {
-    const dfl nub = df_add_l(ld(a.nb0[dir], p), ld(a.nb1[dir], p - s[dir]));
-    const dfl sum = df_add_l(ld(w.p, p + s[dir]), ld(w.p, p - s[dir]));
+    const dfl nub = df_add_l(ldc(a.nb0[dir], p), ldc(a.nb1[dir], p - s[dir]));
+    const dfl sum = df_add_l(ldc(w.p, p + s[dir]), ldc(w.p, p - s[dir]));
     const dfl N = df_n(df_sub_l(sum, pc2)), Dn = df_n(df_add_l(sum, pc2));
     const dfl iD = df_rcp(Dn);
     const dfl nu = df_mul_l(df_abs(N), iD);
