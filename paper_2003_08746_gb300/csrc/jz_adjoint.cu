@@ -58,10 +58,14 @@ __global__ void k_adj_update(Dims d, GridDev g, Adj64 a, double adt) {
   const long long p = pidx(d, i, j, k);
   const bool adv = advanced(d, i, j);
   const double iV = g.invV[p];
+  double l[5], qb[5];
   for (int m = 0; m < 5; ++m) {
-    const double l = a.lam[m][p];
-    if (adv) a.qnbar[m][p] += l;
-    a.acc[m][p] = adv ? -adt * l * iV : 0.0;
+    l[m] = a.lam[m][p];
+    qb[m] = a.qnbar[m][p];
+  }
+  for (int m = 0; m < 5; ++m) {
+    if (adv) a.qnbar[m][p] = qb[m] + l[m];
+    a.acc[m][p] = adv ? -adt * l[m] * iV : 0.0;
   }
 }
 
@@ -299,10 +303,10 @@ __global__ void k_adj_ghost(Dims d, Adj64 a) {
   int si, sj, sk;
   ghost_source(d, i, j, k, si, sj, sk);
   const long long p = pidx(d, i, j, k), q = pidx(d, si, sj, sk);
-  for (int m = 0; m < 5; ++m) {
-    const double v = a.lam[m][p];
-    if (v != 0.0) atomicAdd(&a.lam[m][q], v);
-  }
+  double v[5];
+  for (int m = 0; m < 5; ++m) v[m] = a.lam[m][p];
+  for (int m = 0; m < 5; ++m)
+    if (v[m] != 0.0) atomicAdd(&a.lam[m][q], v[m]);
 }
 
 __global__ void k_adj_addqn(Dims d, Adj64 a) {
@@ -310,8 +314,10 @@ __global__ void k_adj_addqn(Dims d, Adj64 a) {
   int i, j, k;
   if (!box_coord(b, blockIdx.x * (long long)blockDim.x + threadIdx.x, i, j, k)) return;
   const long long p = pidx(d, i, j, k);
+  double v[5];
+  for (int m = 0; m < 5; ++m) v[m] = a.lam[m][p] + a.qnbar[m][p];
   for (int m = 0; m < 5; ++m) {
-    a.lam[m][p] += a.qnbar[m][p];
+    a.lam[m][p] = v[m];
     a.qnbar[m][p] = 0.0;
   }
 }

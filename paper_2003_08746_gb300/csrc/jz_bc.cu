@@ -158,20 +158,32 @@ __device__ __forceinline__ void put_node(const ShellArgs& A, const double v[5], 
   }
 }
 
-// Copy a source node to a ghost (state and shadow as they are).
+// Copy a source node to a ghost (state and shadow as they are), all loads before the first store.
 template <bool SH>
 __device__ __forceinline__ void copy_node(const ShellArgs& A, long long p, long long src) {
-#pragma unroll
-  for (int m = 0; m < 5; ++m) A.q.q[m][p] = A.q.q[m][src];
+  double v[5];
+  float2 s[NSH];
+  load_q(A.q, src, v);
   if (SH) {
 #pragma unroll
-    for (int m = 0; m < NSH; ++m) A.q.sh[m * A.d.Np + p] = A.q.sh[m * A.d.Np + src];
+    for (int m = 0; m < NSH; ++m) s[m] = A.q.sh[m * A.d.Np + src];
+  }
+#pragma unroll
+  for (int m = 0; m < 5; ++m) A.q.q[m][p] = v[m];
+  if (SH) {
+#pragma unroll
+    for (int m = 0; m < NSH; ++m) A.q.sh[m * A.d.Np + p] = s[m];
   }
 }
 
-// Boundary nodes and ghosts of the jet, by block roles: axis, entrance, exit,
-// far field, ghost rows across the axis, ghost planes around the azimuth.  Latency bounds it (a
-// chain of dependent FP64 operations per node on a few thousand nodes).
+// Boundary nodes and ghosts of the jet, by block roles: axis, entrance, exit, far field, ghost rows across the
+// axis, ghost planes around the azimuth.  Every stage waits for it.  On small grids latency bounds it, a chain of
+// dependent FP64 operations per node: 6.6 us per launch on 70 x 33 x 18 (a launch that does nothing 0.7, the
+// copies alone 2.6, the far field 3.9, the exit 5.0, the entrance 6.6), where three kernels for the conditions and
+// one for the ghosts took 4 launches and 57 us; 11 with 32 forcing shapes, the far field's normals normalized at
+// each use, and corner nodes among the others.  On large grids the ghosts' traffic does: 1024 x 512 x 360
+// with the FP32 shadow 0.25 ms (0.32 when each copied value was stored before the next was loaded; 0.64 by the
+// separate kernels).
 template <bool SH>
 __global__ void __launch_bounds__(kTPB) k_jet_shell(const __grid_constant__ ShellArgs A) {
   const Dims& d = A.d;

@@ -145,11 +145,17 @@ __global__ void k_ghost_state(Dims d, State q, Scalars* advance) {
   int si, sj, sk;
   ghost_source(d, i, j, k, si, sj, sk);
   const long long p = pidx(d, i, j, k), s = pidx(d, si, sj, sk);
+  double v[5];
 #pragma unroll
-  for (int m = 0; m < 5; ++m) q.q[m][p] = q.q[m][s];
+  for (int m = 0; m < 5; ++m) v[m] = q.q[m][s];
+#pragma unroll
+  for (int m = 0; m < 5; ++m) q.q[m][p] = v[m];
   if (q.sh) {
+    float2 f[NSH];
 #pragma unroll
-    for (int m = 0; m < NSH; ++m) q.sh[m * d.Np + p] = q.sh[m * d.Np + s];
+    for (int m = 0; m < NSH; ++m) f[m] = q.sh[m * d.Np + s];
+#pragma unroll
+    for (int m = 0; m < NSH; ++m) q.sh[m * d.Np + p] = f[m];
   }
 }
 

@@ -238,9 +238,10 @@ __global__ void __launch_bounds__(kTPB) k_update(Dims d, GridDev g, Work64 w, St
     }
     if (MODE != 1) {
       const double adtV = alpha * sc->dt * hV;
-      double qnew[5];
+      double q0[5], qnew[5];         // (all loads before the first store)
+      for (int m = 0; m < 5; ++m) q0[m] = adv ? qn.q[m][p] : qin.q[m][p];
       for (int m = 0; m < 5; ++m) {
-        qnew[m] = adv ? qn.q[m][p] - adtV * R[m] : qin.q[m][p];
+        qnew[m] = adv ? q0[m] - adtV * R[m] : q0[m];
         qout.q[m][p] = qnew[m];
       }
       if (MODE == 2 && has_images(d, i, j, k))
