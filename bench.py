@@ -41,35 +41,32 @@ FP64_PEAK_TFLOPS = 152 * 4 * 2.07e9 / 1e12
 # fused multiply-add = 2, divide/sqrt/cbrt = 1), counted from the operations
 # the method needs per node (each quantity once).
 # Viscous: 12 differences, 12 metric contractions (60), strain and |S| terms (21), SGS and
-# transport coefficients (12), stresses (9), work + heat flux (21), H^d -= S^d.F (72),
-# sensors (21) = 227.  Faces: 3 faces x (7 per face + 5 x 7 per variable) = 126.
+# transport coefficients (12), pressure minus stresses (12), work + heat flux (21), H^d (87),
+# sensors (21) = 245.  Faces: 3 faces x (7 per face + 5 x 7 per variable) = 126.
 # Update: 5 x (5 differences and sums + 2 for the update) + 5 = 40.
-FLOPS_PER_POINT = {"nodal": 83, "viscous": 227, "faces": 126, "update": 40}
+FLOPS_PER_POINT = {"nodal": 49, "viscous": 245, "faces": 126, "update": 40}
 # DRAM bytes per node of a kernel launch from an ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum / nodes), scaled to the full launch by its node count;
-# profiles/k_viscous_fp64_jet256x128x64.md: (541.0 + 225.7) MB over 258 x 130 x 66 nodes.
-TRAFFIC_PER_NODE = {"viscous": 346.3}
+# profiles/fp64_passes_jet256x128x64_fp64_instructions.md: (457.7 + 274.6) MB over 258 x 130 x 66 nodes.
+TRAFFIC_PER_NODE = {"viscous": 330.8}
 # FP32 instructions per node that the pair form's double-float arithmetic needs in each kernel,
 # counted from the operations of jz_stagedf.cu with the cost of each operation in jz_df.cuh
 # (sum and difference 11, product 7, product by an FP32 number 5, fused multiply-add 15,
 # reciprocal 13, square root 12, cube-root pair 44, |x| 3, max 4, scaling by a power of two 2;
-# in the viscous pass the unnormalized forms: sum 8, product 4, fused multiply-add 12, and 3 for
-# each of the 38 normalizations;
-# conversions and loads not counted).  Nodal: 14 products, 14 fused multiply-adds, 5 sums,
-# 2 reciprocals, 1 square root, 3 |x|, 3 cube-root pairs = 542.  Viscous: 64 products, 76 fused
-# multiply-adds, 45 sums and differences, 38 normalizations, 1 square root, 3 reciprocals, 3 |x|,
-# 3 scalings = 1708 (the inviscid fluxes E^dir are formed here).  Faces: 3 x (max 4, products 7 + 7, difference 11,
-# sum 11, fused multiply-add 15, product by 3 5, select 2 = 62; and 5 x 66 per variable) = 1176.
-# Update: 5 x 5 differences and sums = 275.
-PAIR_INST_PER_POINT = {"nodal": 542, "viscous": 1708, "faces": 1176, "update": 275}
+# unnormalized: sum 8, product 4, fused multiply-add 12, and 3 for each normalization; conversions
+# and loads not counted).  Viscous (the whole flux kernel): primitives 92, gradients 432, strain,
+# viscosities and coefficients 246, stresses with the pressure 72, work and heat flux 120, per
+# direction U 31, lambda 18 and the fluxes 179 (684), anisotropic scaling 210, sensors 161, 2 more
+# scalings = 2017.  Faces: 3 x (max 4, products 7 + 7, difference 11, sum 11, fused multiply-add 15,
+# product by 3 5, select 2 = 62; and 5 x 35 per variable) = 711.  Update: 5 x (6 sums of the flux and
+# 5 of the dissipation differences) x 8 = 440.
+PAIR_INST_PER_POINT = {"viscous": 2017, "faces": 711, "update": 440}
 
 
 def pair_inst_per_launch(g, kind):
-    """Algorithmic FP32 instructions of one launch of a pair-form kernel: the nodal pass over the
-    padded box, the viscous pass over the real box and one layer, and the faces kernel over the
-    faces n + 1/2 (n = -1 .. n_dir - 1) plus the update of every real node, which it also does."""
-    if kind == "nodal":
-        return PAIR_INST_PER_POINT["nodal"] * (g.ni + 4) * (g.nj + 4) * (g.nk + 4)
+    """Algorithmic FP32 instructions of one launch of a pair-form kernel: the flux kernel over the
+    real box and one layer, and the faces kernel over the faces n + 1/2 (n = -1 .. n_dir - 1) plus
+    the update of every real node, which it also does."""
     if kind == "viscous":
         return PAIR_INST_PER_POINT["viscous"] * (g.ni + 2) * (g.nj + 2) * (g.nk + 2)
     return (PAIR_INST_PER_POINT["faces"] * (g.ni + 1) * (g.nj + 1) * (g.nk + 1)
@@ -78,23 +75,21 @@ def pair_inst_per_launch(g, kind):
 
 def pair_launch_nodes(g, kind):
     """Nodes a pair-form kernel launch covers (the faces kernel: the real nodes it updates)."""
-    e = {"nodal": 4, "viscous": 2}.get(kind, 0)
+    e = {"viscous": 2}.get(kind, 0)
     return (g.ni + e) * (g.nj + e) * (g.nk + e)
 
 
 # DRAM bytes per node of a pair-form kernel launch (dram__bytes_read.sum + dram__bytes_write.sum
-# over the launch's nodes), profiles/pair_passes_jet256x128x64.md.
-PAIR_TRAFFIC_PER_NODE = {"nodal": 230.6, "viscous": 316.5, "faces": 338.4}
+# over the launch's nodes), profiles/k_flux_df_jet256x128x64.md and k_faces_update_df_jet256x128x64.md.
+PAIR_TRAFFIC_PER_NODE = {"viscous": 358.9, "faces": 317.8}
 # Algorithmic DRAM bytes per node of each pair-form kernel (every field once, as double-float
-# pairs or FP64): nodal reads Q 40, S 72, |S| 24 and writes the pair copy of Q 40, u, v, w, T, p,
-# mu 48, Lambda 24 = 248; viscous reads S 72, 1/V 8, Delta 8, mu 8, u, v, w, T 32, p 8, the pair
-# copy of Q 40 and writes H 120, the sensors 24 = 320; faces-update reads the sensors 24, Lambda
+# pairs or FP64): viscous reads Q 40, S 72, |S| 24, 1/V 8, Delta 8 and writes the pair copy of Q 40,
+# H 120, Lambda 24, the sensors 24 = 360; faces-update reads the sensors 24, Lambda
 # 24, the pair copy of Q 40, H 120, Q^n 40, 1/V 8 and writes Q^(l) 40 = 296.
-PAIR_ALG_BYTES_PER_NODE = {"nodal": 248, "viscous": 320, "faces": 296}
+PAIR_ALG_BYTES_PER_NODE = {"viscous": 360, "faces": 296}
 FP32_ISSUE_PEAK_TINST = 152 * 128 * 2.07e9 / 1e12      # 152 SMs x 4 x 32 lanes x 2.07 GHz
-# k_fused32: DRAM bytes per node averaged over a step's five launches (stage 1 and stage 2
-# captures of the TMA-fed kernel, profiles/k_fused32_tma_jet256x128x64.md: 179.1 and 180.9 B).
-TRAFFIC_FUSED32_PER_NODE = (179.1 + 4 * 180.9) / 5
+# k_fused32: DRAM bytes per node of a stage whose Q^(l-1) is not Q^n (profiles/k_fused32_jet512x256x128.md).
+TRAFFIC_FUSED32_PER_NODE = 191.4
 
 
 def _dist():

@@ -222,12 +222,12 @@ int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ck
 
 /* ---- kernel timing ---------------------------------------------------- *
  * Kernel kinds of the stage (index of the arrays below). */
-#define JZ_PROF_NODAL    0   /* FP64 nodal pass: primitives, spectral radii, inviscid fluxes */
-#define JZ_PROF_VISCOUS  1   /* FP64 viscous pass: gradients, SGS, viscous fluxes, sensor   */
+#define JZ_PROF_NODAL    0   /* nodal pass: primitives, spectral radii (pair form: adjoint only) */
+#define JZ_PROF_VISCOUS  1   /* gradients, SGS, fluxes, sensors (pair form: with the nodal work) */
 #define JZ_PROF_FACES    2   /* dissipation face fluxes (pair form: with the RHS and update) */
 #define JZ_PROF_UPDATE   3   /* RHS assembly and stage update                              */
-#define JZ_PROF_BC       4   /* boundary-condition kernels                                 */
-#define JZ_PROF_GHOST    5   /* ghost-point fill                                           */
+#define JZ_PROF_BC       4   /* boundary conditions and ghosts of the jet                  */
+#define JZ_PROF_GHOST    5   /* ghost-point fill (FP32-flux boxes; others: in the update)  */
 #define JZ_PROF_REDUCE   6   /* CFL, time, statistics reductions                           */
 #define JZ_PROF_FUSED32  7   /* fused FP32-flux stage kernel                               */
 #define JZ_PROF_ADJOINT  8   /* adjoint stage kernels                                      */

@@ -235,7 +235,7 @@ int mark(jz_solver* s, int kind) {
     if (r_) return r_;              \
   } while (0)
 
-// cfl_first: stage 1 of a CFL step; the nodal pass reduces the rate of Q^n (Scalars::rate_max
+// cfl_first: stage 1 of a CFL step; the nodal pass (pair: flux kernel) reduces the rate of Q^n (Scalars::rate_max
 // is 0 between FP64 steps) and the time step is set from it before the update.
 int run_stage64(jz_solver* s, const jz::State& in, const jz::State& out, double alpha, int want_res,
                 double* rhs_flat, bool cfl_first = false, jz::Finish finish = jz::FINISH_NONE) {
@@ -376,7 +376,7 @@ int stats_sample(jz_solver* s) {
 
 // ---- discrete adjoint: forward stages from an explicit Q^n --------------------------
 // A pair-form solver advances the states in pair arithmetic (its reverse sweep also regenerates
-// the intermediates the transposed kernels read with the pair nodal and viscous passes).
+// the intermediates the transposed kernels read with the pair nodal and sensor passes).
 int fwd_stage(jz_solver* s, const jz::State& in, const jz::State& qn, const jz::State& out, int l) {
   const jz::Dims& d = s->grid->d;
   const jz::GridDev& g = s->grid->g;

@@ -219,8 +219,8 @@ struct Scalars {
 // CFL rate of one node, (lambda_xi + lambda_eta + lambda_zeta) / V with
 // lambda_d = |S^d . u| + a |S^d|, from its conserved variables: the stand-alone
 // reduction (first FP32-flux step after jz_set_state, the adjoint's frozen step).
-// The FP64 form's stage-1 nodal pass forms the same expressions from the same
-// primitives.
+// The FP64 form's stage-1 nodal pass and the pair form's flux kernel form the same from the
+// same primitives.
 __device__ __forceinline__ double node_rate(const GridDev& g, const Consts& c, long long p, double rho, double m1,
                                             double m2, double m3, double e) {
   const double ir = rcp64(rho);
@@ -295,9 +295,7 @@ struct Adj64 {
   double* J;               // [1] functional accumulator
 };
 
-// Inflow tables (jet): base profile u0[nk][nj] and forcing shapes
-// Gf[m*4+f][nk][nj] = g(r) cos(m theta + phi_mf), at i = 0.
-// Entrance forcing sum_mf A_mf sin(omega_f t + psi_mf) g(r) cos(m theta + phi_mf) as 15 shapes
+// Entrance (i = 0) of a jet: base profile u0[nk][nj] and the forcing sum_mf A_mf sin(omega_f t + psi_mf) g(r) cos(m theta + phi_mf) as 15 shapes
 // g cos m theta, g sin m theta with one coefficient each per stage time (the 32 products of an
 // amplitude, its sine and the cosine or sine of its azimuthal phase summed over the frequencies):
 // less than half the table that 32 shapes take, and of the serial sum at each entrance node.
@@ -385,7 +383,7 @@ cudaError_t faces_update_df(const Dims& d, const Consts& c, const GridDev& g, co
                             int want_res, double* rhs_flat, cudaStream_t st,
                             Finish finish = FINISH_NONE);
 // boundary conditions and ghost points of the jet after stage `stage` (one kernel); advance: last
-// stage of a step, t += dt.  Needs the temporal factors that set_dt or set_time left for the step.
+// stage of a step, t += dt.  Needs the shapes' coefficients that set_dt or set_time left for the step.
 cudaError_t jet_shell(const Dims& d, const Consts& c, const GridDev& g, const Inflow& in, const State& q,
                       Scalars* sc, int stage, int advance, cudaStream_t st);
 cudaError_t build_inflow(const Dims& d, const Consts& c, const GridDev& g, const jz_params& p,
@@ -395,9 +393,9 @@ cudaError_t build_inflow(const Dims& d, const Consts& c, const GridDev& g, const
 // records, null: none at hand
 cudaError_t cfl_rate(const Dims& d, const Consts& c, const GridDev& g, const float* Mf, const State& q, Scalars* sc,
                      cudaStream_t st);
-// time step of the current step from the reduced rate (or dt_fixed), and the forcing's temporal factors
+// time step of the current step from the reduced rate (or dt_fixed), and the forcing shapes' coefficients
 cudaError_t set_dt(const Consts& c, const Inflow& in, Scalars* sc, cudaStream_t st);
-// t and dt given (the adjoint's sweeps), and the forcing's temporal factors
+// t and dt given (the adjoint's sweeps), and the forcing shapes' coefficients
 cudaError_t set_time(const Inflow& in, Scalars* sc, double t, double dt, cudaStream_t st);
 int stat_partial_count();
 cudaError_t stats_with(const Dims& d, const Consts& c, const GridDev& g, const State& q, Scalars* sc,

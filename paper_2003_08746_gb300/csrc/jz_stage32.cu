@@ -296,7 +296,7 @@ __device__ __forceinline__ void nodal(const Args& A, const Smem& sm, const float
   N.iV = iV;
 }
 
-// Latency and issue bound it (58% of the cycles issue, 20 warps per SM): 9.9 ms per launch on
+// Latency and issue bound it (56% of the cycles issue, 20 warps per SM): 9.9 ms per launch on
 // 1024 x 512 x 360, 2.9 TB/s of algorithmic bytes, against 13.0 with the zeta and xi quantities and
 // the faces in shared memory too and two barriers per plane.  Rows per tile: 8 (96 registers, two
 // CTAs per SM); 6: 11.7, 9 (88 registers, spills): 17.5, 12 at one CTA: 12.8.  H^zeta(p-1) in shared
