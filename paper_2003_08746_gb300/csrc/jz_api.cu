@@ -645,6 +645,7 @@ int jz_create(jz_grid* g, const jz_params* p, void* stream, jz_solver** out) {
     }
     const double r = (double)tiles * d.nk / slots;
     s->kchunk = std::min(d.nk, (int)(r <= 4.0 ? std::ceil(r) : 1.5 * std::sqrt(r) + 0.5));
+    s->kchunk = std::max(s->kchunk, (d.nk + 65534) / 65535);      // the launch's chunks along z
   } else {
     s->pair = p->precision == JZ_PREC_FP64PAIR;
     if (s->pair) {
