@@ -16,37 +16,50 @@ constexpr int kStatBlocks = 1216;   // 8 x 152 SMs; fixed so the sums are reprod
 // So every node gets an interval [lo, hi] around its rate in FP32, and only nodes whose interval
 // reaches the largest rate known so far (this warp's lower bounds, its exact values, what other
 // warps have published) are evaluated exactly: the node of the maximum is always among them, so the
-// result is the plain sweep's bit for bit.  Values outside FP32's range and NaN count as reaching it.
+// result is the plain sweep's bit for bit.  A node whose quantities leave the ranges in which the
+// bounds' errors are known (values that FP32 flushes, overflows or holds as subnormals, squares of
+// metrics among them; NaN) is open: it claims nothing and is always evaluated.
 struct RateBounds {
   float lo, hi;
 };
+__device__ __forceinline__ float f32_or_inf(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7FFFFFFFu) < 0x45E00000u ? f64_to_f32(x) : __int_as_float(0x7F800000);   // |x| < 2^95
+}
 __device__ __forceinline__ RateBounds rate_bounds(const ConstsF& c, const double q[5], const float S[9], float iV) {
+  const RateBounds open{0.f, __int_as_float(0x7F800000)};
   unsigned big = 0;
 #pragma unroll
   for (int m = 0; m < 5; ++m) big = max(big, (unsigned)__double2hiint(q[m]) & 0x7FFFFFFFu);
-  if (big >= 0x45E00000u) return RateBounds{0.f, __int_as_float(0x7F800000)};   // some |q| >= 2^95
+  if (big >= 0x45E00000u) return open;   // some |q| >= 2^95
   // each quantity below is within kRel of its FP64 value relative to the magnitudes summed in it:
   // truncated conversions (2^-23 each), a few roundings, one hardware reciprocal and square root
   constexpr float kRel = 4e-6f;
-  const float ir = f_rcp(f64_to_f32(q[0]));
+  const float rho = f64_to_f32(q[0]);
+  if (!(rho > 1e-8f && rho < 1e8f) || !(iV > 1e-30f && iV < 1e30f)) return open;
+  const float ir = f_rcp(rho);
   const float m1 = f64_to_f32(q[1]), m2 = f64_to_f32(q[2]), m3 = f64_to_f32(q[3]), e = f64_to_f32(q[4]);
   const float u = m1 * ir, v = m2 * ir, w = m3 * ir;
   const float ke = 0.5f * (m1 * u + m2 * v + m3 * w);
-  const float p = c.gm1 * (e - ke), dp = kRel * c.gm1 * (fabsf(e) + fabsf(ke));
-  const float a_hi = sqrtf(c.gamma * fabsf(ir) * (fabsf(p) + dp)), a_lo = ir > 0.f ? sqrtf(fmaxf(c.gamma * ir * (p - dp), 0.f)) : 0.f;
-  float lo = 0.f, hi = 0.f;
+  const float p = c.gm1 * (e - ke), dp = kRel * c.gm1 * (fabsf(e) + fabsf(ke)), p_lo = p - dp, p_hi = p + dp;
+  if (!(p_hi > 1e-20f && p_hi < 1e20f)) return open;
+  const float a_hi = sqrtf(c.gamma * ir * p_hi), a_lo = sqrtf(c.gamma * ir * fmaxf(p_lo, 0.f));
+  float lo = 0.f, hi = 0.f, s_min = 1.f, s_max = 1.f;
 #pragma unroll
   for (int dir = 0; dir < 3; ++dir) {
     const float sx = S[3 * dir], sy = S[3 * dir + 1], sz = S[3 * dir + 2];
     const float U = fabsf(sx * u + sy * v + sz * w), dU = kRel * (fabsf(sx * u) + fabsf(sy * v) + fabsf(sz * w));
-    const float smag = sqrtf(sx * sx + sy * sy + sz * sz);
+    const float s2 = sx * sx + sy * sy + sz * sz, smag = sqrtf(s2);
+    s_min = fminf(s_min, s2);
+    s_max = fmaxf(s_max, s2);
     lo += fmaxf(U - dU, 0.f) + a_lo * smag;
     hi += U + dU + a_hi * smag;
   }
-  const float inf = __int_as_float(0x7F800000), top = hi * iV * (1.f + kRel);
-  // (sums so small that flushed conversions could matter decide nothing)
-  if (!(hi > 1e-25f) || !(top > 1e-25f)) return RateBounds{0.f, inf};
-  return RateBounds{lo * iV * (1.f - kRel), top};
+  // |S|^2 below this holds squares of its parts that FP32 rounds as subnormals or drops
+  if (!(s_min > 1e-30f && s_max < 1e30f)) return open;
+  const float top = hi * iV * (1.f + kRel);
+  if (!(top > 1e-25f && top < 1e30f)) return open;
+  // (a node whose pressure may be negative has no rate to claim: FP64 gives NaN, which the maximum drops)
+  return RateBounds{p_lo > 0.f ? lo * iV * (1.f - kRel) : 0.f, top};
 }
 
 // Mf: FP32 metric records where the solver or the grid has them, else the FP64 metrics.
@@ -79,9 +92,8 @@ __global__ void __launch_bounds__(kTPB) k_cfl_rate(Dims d, GridDev g, State q, C
       iV = e.z;
     } else {
 #pragma unroll
-      for (int m = 0; m < 9; ++m) S[m] = f64_to_f32(g.S[m][p]);
-      const double w = g.invV[p];
-      iV = w < 1e30 ? f64_to_f32(w) : __int_as_float(0x7F800000);
+      for (int m = 0; m < 9; ++m) S[m] = f32_or_inf(g.S[m][p]);
+      iV = f32_or_inf(g.invV[p]);
     }
     cut = fmax(cut, *known);
     const RateBounds b = rate_bounds(cf, v, S, iV);
