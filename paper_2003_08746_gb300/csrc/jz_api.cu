@@ -844,8 +844,9 @@ int jz_rk_step(jz_solver* s, int nsteps, jz_step_stats* out) {
   return JZ_OK;
 }
 
-int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ckpt_every, double r_obs,
-                    double* J_out, double* grad_out) {
+// The work of jz_adjoint_step (may throw std::bad_alloc).
+static int adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ckpt_every, double r_obs, double* J_out,
+                        double* grad_out) {
   if (!s || !forcing_amps || !J_out || !grad_out) return fail(JZ_ERR_ARG, "jz_adjoint_step: NULL argument");
   if (nsteps < 1 || ckpt_every < 1) return fail(JZ_ERR_ARG, "jz_adjoint_step: nsteps and ckpt_every must be >= 1");
   if (s->fp32) return fail(JZ_ERR_ARG, "jz_adjoint_step: the adjoint is available for the FP64 form");
@@ -883,14 +884,15 @@ int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ck
   // The adjoint arrays start at zero; the states are written before they are read.
   DevMem mem;
   mem.used_by(s->st);
-  int C = 0, nseg = 0;
+  mem.blocks.reserve(1);
+  long long C = 0, nseg = 0;      // steps per segment, segments
   const size_t Np = (size_t)d.Np;
   jz::Adj64 a;
   std::vector<jz::State> ck, seg, stg, kept;
   jz::State wa{}, wb{};
   double* wdev = nullptr;
-  // lays the arrays out from base and returns the number of doubles (base null: count only); the
-  // first `zeroed` of them are the adjoint arrays
+  // lays the arrays out from base and returns the number of doubles (base null: count only; without
+  // the lists of states); the first `zeroed` of them are the adjoint arrays
   size_t zeroed = 0;
   auto layout = [&](double* base) {
     size_t at = 0;
@@ -931,15 +933,18 @@ int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ck
     return at;
   };
   // Segments of `steps` steps, with or without the four intermediate stage states of every step of a
-  // segment; returns the bytes.
-  auto plan = [&](int steps, bool keep) {
+  // segment; returns the bytes (the most a size_t holds if they are more).  Counted, not listed: the lists
+  // of the plan that is taken are made below, so that a long run with short segments asks the host for no more
+  // than its own plan does.
+  const size_t fixed = (layout(nullptr) + 31) / 32 * 32, per_state = 5 * ((Np + 31) / 32 * 32);
+  bool keep = false;
+  auto plan = [&](int steps, bool with_stages) {
     C = std::min(steps, nsteps);
     nseg = (nsteps + C - 1) / C;
-    ck.resize(nseg - 1);
-    seg.resize(C + 1);
-    kept.resize(keep ? (size_t)C * 4 : 0);
-    stg.resize(keep ? 0 : 4);
-    return layout(nullptr) * sizeof(double);
+    keep = with_stages;
+    const size_t states = (size_t)(nseg - 1) + (size_t)(C + 1) + (keep ? 4 * (size_t)C : 4);
+    const size_t most = (size_t)-1 / sizeof(double);
+    return states > (most - fixed) / per_state ? (size_t)-1 : (fixed + states * per_state) * sizeof(double);
   };
   // Where memory allows, the stage states of a segment are kept, so that the reverse sweep does not
   // recompute them step by step (one forward step per step less); and where those of all steps take
@@ -952,7 +957,7 @@ int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ck
   double* base = nullptr;
   cudaError_t e = cudaErrorMemoryAllocation;
   auto attempt = [&](size_t bytes) {
-    e = cudaMalloc(&base, bytes);
+    e = bytes == (size_t)-1 ? cudaErrorMemoryAllocation : cudaMalloc(&base, bytes);
     if (e != cudaSuccess) cudaGetLastError();
     return e == cudaSuccess;
   };
@@ -965,6 +970,10 @@ int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ck
   if (!planned) planned = attempt(plan(ckpt_every, false));
   if (!planned) return fail(alloc_status(e), "jz_adjoint_step: device allocation failed: %s", cudaGetErrorString(e));
   mem.blocks.push_back(base);
+  ck.resize(nseg - 1);
+  seg.resize(C + 1);
+  kept.resize(keep ? 4 * C : 0);
+  stg.resize(keep ? 0 : 4);
   layout(base);
   JZ_CK(cudaMemsetAsync(base, 0, zeroed * sizeof(double), s->st));
   JZ_CK(cudaMemcpyAsync(wdev, w.data(), sizeof(double) * d.ni, cudaMemcpyHostToDevice, s->st));
@@ -1006,7 +1015,7 @@ int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ck
     return kept.empty() ? fwd_step(s, seg[q], seg[q + 1], t0 + n * dt, dt)
                         : fwd_step_keep(s, seg[q], seg[q + 1], t0 + n * dt, dt, &kept[(size_t)q * 4]);
   };
-  const int last = (nseg - 1) * C;              // first step of the last segment: advanced in place, not again
+  const int last = (int)((nseg - 1) * C);       // first step of the last segment: advanced in place, not again
   for (int n = 0; n < nsteps; ++n) {
     if (n % C == 0) {
       r = copy_state(s, n < last ? ck[n / C] : seg[0], wa);
@@ -1018,8 +1027,8 @@ int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ck
     std::swap(wa, wb);
   }
   // reverse sweep, one checkpoint segment at a time
-  for (int sg = nseg - 1; sg >= 0; --sg) {
-    const int n0 = sg * C, n1 = std::min(n0 + C, nsteps);
+  for (long long sg = nseg - 1; sg >= 0; --sg) {
+    const int n0 = (int)(sg * C), n1 = (int)std::min<long long>(n0 + C, nsteps);
     if (n0 < last) {
       r = copy_state(s, seg[0], ck[sg]);
       if (r) return r;
@@ -1067,6 +1076,15 @@ int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ck
   JZ_CK(cudaStreamSynchronize(s->st));
   *J_out = Jh;
   return JZ_OK;
+}
+
+int jz_adjoint_step(jz_solver* s, const double* forcing_amps, int nsteps, int ckpt_every, double r_obs,
+                    double* J_out, double* grad_out) {
+  try {
+    return adjoint_step(s, forcing_amps, nsteps, ckpt_every, r_obs, J_out, grad_out);
+  } catch (const std::bad_alloc&) {          // the lists of stage states, on the host
+    return fail(JZ_ERR_OOM, "jz_adjoint_step: host allocation failed");
+  }
 }
 
 int jz_profile(jz_solver* s, int enable) {
