@@ -208,9 +208,14 @@ int jz_rk_step(jz_solver* s, int nsteps, jz_step_stats* out);
  * The forward sweep stores Q^n every ckpt_every steps; the reverse sweep
  * recomputes each checkpoint segment (the last one is still there) with
  * every step's five stage states and runs the transposed stage,
- * boundary-condition and ghost-fill kernels.  Where the stage states of all
- * steps take less than half of the free device memory they are all kept and
- * nothing is recomputed (ckpt_every then has no effect); the results do not
+ * boundary-condition and ghost-fill kernels.  ckpt_every sets the memory of
+ * the call, in states of 40 bytes per padded node: one per segment but the
+ * last, ckpt_every + 1 for a segment, 4 ckpt_every for its stage states where
+ * these are under half of what is still free (else 4, and the stages of
+ * each step are computed once more), and 13 for the sweeps.  Only where the
+ * stage states of all steps and these 13 take at most 1/32 of the free device memory
+ * are they all kept and nothing is recomputed, whatever ckpt_every
+ * (ckpt_every = nsteps asks for that at any size).  The results do not
  * depend on the interval.
  * Writes J (*J_out, host) and dJ/dA (grad_out [32], host).  The solver's
  * state and parameters are unchanged on return; device memory for the
