@@ -42,6 +42,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 
 #include "jz_mbar.cuh"
@@ -553,14 +554,14 @@ static_assert(TX % 2 == 0, "the TMA box must start on a 16-byte boundary (x0 = i
 
 // The dynamic shared-memory size above 48 KB must be allowed once per device.
 cudaError_t allow_smem() {
-  static bool attr[64] = {false};
+  static std::atomic<bool> attr[64];
   int dev = 0;
   cudaError_t e0 = cudaGetDevice(&dev);
   if (e0 != cudaSuccess) return e0;
-  if (dev < 0 || dev >= 64 || !attr[dev]) {
+  if (dev < 0 || dev >= 64 || !attr[dev].load(std::memory_order_relaxed)) {
     cudaError_t e = cudaFuncSetAttribute(k_fused32, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) attr[dev] = true;
+    if (dev >= 0 && dev < 64) attr[dev].store(true, std::memory_order_relaxed);
   }
   return cudaSuccess;
 }
@@ -581,7 +582,8 @@ cudaError_t fused32_slots(int* slots) {
 }
 
 cudaError_t make_shadow_map(const Dims& d, float2* sh, void* tmap128) {
-  static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
+  static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> known{nullptr};
+  PFN_cuTensorMapEncodeTiled_v12000 encode = known.load(std::memory_order_relaxed);
   if (!encode) {
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q;
@@ -589,6 +591,7 @@ cudaError_t make_shadow_map(const Dims& d, float2* sh, void* tmap128) {
     if (e != cudaSuccess) return e;
     if (q != cudaDriverEntryPointSuccess || !fn) return cudaErrorInvalidValue;
     encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+    known.store(encode, std::memory_order_relaxed);
   }
   // 8-byte elements (one float2 pair each); rows of Pi, planes of Pi x Pj, three arrays of Np
   const cuuint64_t dims[4] = {(cuuint64_t)d.Pi, (cuuint64_t)d.Pj, (cuuint64_t)d.Pk, (cuuint64_t)NSH};

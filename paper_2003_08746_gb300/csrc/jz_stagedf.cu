@@ -11,6 +11,8 @@
 // The adjoint of a pair-form solver regenerates the primitives, spectral radii and sensors of a
 // stage with the nodal and sensor passes below, on 3-D launches (64 x 4 threads per block along i
 // and j, one block row per k), so that no pass divides a flat index.
+#include <atomic>
+
 #include "jz_dfconsts.cuh"
 
 namespace jz {
@@ -523,18 +525,22 @@ cudaError_t sensor_df_pass(const Dims& d, const Work64& w, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// Resident blocks of a kernel on the current device, asked for once per device.
+// Resident blocks of a kernel on the current device, asked for once per device (by any host thread: all
+// store the same value).
+using SlotCache = std::atomic<int>[64];
 template <class K>
-int resident_blocks(K kernel, int threads, int cache[64]) {
+int resident_blocks(K kernel, int threads, SlotCache& cache) {
   int dev = 0, sms = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 304;
-  if (cache[dev] == 0) {
+  int n = cache[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, 0) != cudaSuccess || per < 1)
       return 304;
-    cache[dev] = sms * per;
+    n = sms * per;
+    cache[dev].store(n, std::memory_order_relaxed);
   }
-  return cache[dev];
+  return n;
 }
 
 // Planes per block of the marching kernels, from r = planes of all tiles per resident block.  Fitted to
@@ -577,7 +583,7 @@ cudaError_t flux_df(const Dims& d, const Consts& c, const DFMetrics& M, const Wo
   A.rate_max = want_rate ? &sc->rate_max : nullptr;
   A.nbx = (d.ni + VX - 1) / (VX - 2);
   const long long tiles = (long long)A.nbx * ((d.nj + VY - 1) / (VY - 2));
-  static int slots[64];
+  static SlotCache slots;
   A.kchunk = flux_chunk((double)tiles * (d.nk + 2) / resident_blocks(k_flux_df, VX * (VY - 2), slots));
   const dim3 gr((unsigned)tiles, (d.nk + 1 + A.kchunk) / A.kchunk);
   k_flux_df<<<gr, dim3(VX, VY - 2), 0, st>>>(A);
@@ -610,7 +616,7 @@ cudaError_t faces_update_df(const Dims& d, const Consts& c, const GridDev& g, co
   A.res_sum = want_res && !rhs_flat ? &sc->res_sum : nullptr;
   A.nbx = (d.ni + FX - 2) / (FX - 1);
   const long long tiles = (long long)A.nbx * ((d.nj + FY - 2) / (FY - 1));
-  static int slots[64], slots2[64];
+  static SlotCache slots, slots2;
   const long long planes = tiles * d.nk;
   const bool small = planes <= resident_blocks(k_faces_update_df<0, 2>, FX * FY, slots2);
   A.kchunk = small ? 1 : faces_chunk((double)planes / resident_blocks(k_faces_update_df<0, 4>, FX * FY, slots));
