@@ -1,6 +1,6 @@
 // Transposed passes of the discrete adjoint for a pair-form solver (see jz_adjoint.cu for the
 // FP64 form and the structure of the reverse sweep): the face, viscous-and-sensor and nodal
-// passes in double-float arithmetic on the pair intermediates that the pair nodal and viscous
+// passes in double-float arithmetic on the pair intermediates that the pair nodal and sensor
 // passes regenerated (u, v, w, T, p, mu, the sensors, Lambda, the pair copies of Q and of the
 // metrics).  The running adjoint lambda and Q^n's adjoint stay FP64 (as do the boundary-condition
 // adjoints and the observer); the intermediate adjoint arrays the transposed passes pass to one

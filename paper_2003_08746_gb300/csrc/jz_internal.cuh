@@ -250,7 +250,7 @@ __device__ __forceinline__ double node_rate(const GridDev& g, const Consts& c, l
 struct Work64 {
   double* u; double* v; double* w; double* T; double* p; double* mu;
   double* Lam[3];
-  double* H[3][5];    // transformed inviscid flux, then inviscid - viscous
+  double* H[3][5];    // transformed fluxes (inviscid - viscous); H[dir][0] holds U^dir between the FP64 nodal and viscous passes
   double* nu[3];      // pressure sensor per direction
   double* G[3][5];    // twice the total face flux at n + 1/2: H_n + H_(n+1) - 2 d_(n+1/2)
 };
@@ -331,8 +331,9 @@ cudaError_t compute_metrics(const Dims& d, GridDev& g, double* scratch9[9], cuda
 cudaError_t ghost_fill(const Dims& d, double* const* f, int nvar, cudaStream_t st);
 // ghosts of a state and of its shadow; advance: the scalars of a solver whose step ends here, t += dt
 cudaError_t ghost_fill_state(const Dims& d, const State& q, Scalars* advance, cudaStream_t st);
-// FP32 copy of the metrics S (9) and V; dst_dev is a device array of 10 pointers
+// far-field unit normals and entrance coordinates (GridDev::Sb, Xin)
 cudaError_t boundary_copies(const Dims& d, const GridDev& g, cudaStream_t st);
+// FP32 metric records of every padded node
 cudaError_t metrics_to_f32(const Dims& d, const GridDev& g, float* Mf, cudaStream_t st);
 // padded real region of nvar fields (5 or 10) to a flat [nvar][N] array
 cudaError_t unpack_real(const Dims& d, double* const* padded, double* flat, int nvar,

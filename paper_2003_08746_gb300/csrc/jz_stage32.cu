@@ -324,8 +324,8 @@ __global__ void __launch_bounds__(NT, 2) k_fused32(const __grid_constant__ Args 
   // the halo-2 box starts at real (i0 - 2, j0 - 2): padded (i0, j0); x0 * 8 bytes is a multiple
   // of 16 because TX is even
   const int x0 = i0, y0 = j0;
-  // its element in plane p of a padded field (32 bits: a field's Np nodes at 168 bytes each reach the
-  // GPU's memory before 2^32), here for p = k0 - 2
+  // its element in plane p of a padded field (32 bits: a field's Np nodes at 240 bytes each, three
+  // states with their shadows and the metric records, reach the GPU's memory before 2^32), here for p = k0 - 2
   const unsigned sk = (unsigned)d.sk;
   unsigned pp = (unsigned)(valid ? pidx(d, oi, oj, k0 - 2) : 0);
   // prime: mbarriers, then planes k0-2 .. k0 requested; k0-2 and k0-1 waited for
@@ -416,7 +416,6 @@ __global__ void __launch_bounds__(NT, 2) k_fused32(const __grid_constant__ Args 
       request_plane(A, sm, ring(p + 3), x0, y0, p + 3);
       last_req = p + 3;
     }
-    // metrics of plane p+2 (those of plane p+1 have been used)
     if (rowt) {
       // (c) zeta face p+1/2, RHS and update of plane p
       float q0[5], q1[5], q2[5], Dz[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
@@ -429,7 +428,7 @@ __global__ void __launch_bounds__(NT, 2) k_fused32(const __grid_constant__ Args 
 #pragma unroll
         for (int m = 0; m < 5; ++m) {
           float a = acc[m];
-                    a += 0.5f * (N.H[2][m] - sm.carry[m][t]) - (Dz[m] - Dz_prev[m]);
+          a += 0.5f * (N.H[2][m] - sm.carry[m][t]) - (Dz[m] - Dz_prev[m]);
           R[m] = a * iV0;
         }
         if (A.rhs) {

@@ -374,7 +374,7 @@ struct FacesArgs {
 // blocks at four per SM (when it took 8.1: 8.3 for 32 x 16 at two, 8.1 for 32 x 12 at three; 9.2 with face sums).
 // One variable per thread (five times the threads, coefficients through shared memory) took 16.9.
 // PER blocks per SM: 4, or 2 where every plane of every tile is resident at two: load latency alone is left
-// then, and 128 registers hold more loads in flight than 64 (32 x 24 x 16: 0.9 us per launch less,
+// then, and 108 to 119 registers (of the 128 that two blocks leave) hold more loads in flight than 64 (32 x 24 x 16: 0.9 us per launch less,
 // ten steps 0.98 -> 0.92 ms; with 360 blocks on 304 places 70 x 40 x 20 would take 18.9 us instead of 15.6).
 constexpr int FX = 32, FY = 8;
 template <int MODE, int PER>
